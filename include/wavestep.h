@@ -392,8 +392,8 @@ int ws_test_stall(ws_t ws, int item);
  * patterns); it synchronizes the handle's stream. With the padding filled,
  * the interior results must not change: nothing beyond the halo may reach
  * a result. Calls that zero whole state buffers clear their canaries, so
- * fill after them: ws_write_field, ws_forward and ws_adjoint_gradient
- * (which restart from rest) and ws_set_storage (which allocates the 16-bit
+ * fill after them: ws_write_field with a NULL level, ws_forward and
+ * ws_adjoint_gradient (which restart from rest) and ws_set_storage (which allocates the 16-bit
  * buffers); the model setters write the interior only. Errors: BADARG
  * (NULL), CUDA, OOM. */
 int ws_test_fill_padding(ws_t ws);

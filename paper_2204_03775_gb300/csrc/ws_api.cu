@@ -213,9 +213,19 @@ int build_rec_tiles(ws_t ws, const ws::StreamTiling &t, int rows) {
     return WS_OK;
 }
 
-// Copy an unpadded [nz][ny][nx] array into the interior of a padded buffer.
-int copy_in(ws_t ws, float *dst, const float *src, int on_device) {
+// Whether the copy kernels may take a device array: float elements on their
+// natural alignment (a 2D copy takes any address).
+static bool kernel_copyable(const void *p) { return (reinterpret_cast<uintptr_t>(p) & 3u) == 0; }
+
+// Copy unpadded [nz][ny][nx] arrays into the interiors of padded buffers:
+// device arrays by one kernel, host arrays plane by plane.
+int copy_in(ws_t ws, float *dst, const float *src, int on_device, float *dst2, const float *src2) {
     const ws::Geom &g = ws->g;
+    if (on_device && kernel_copyable(src) && kernel_copyable(src2)) {
+        WS_CUDA(ws::launch_copy_in(src, src2, dst, dst2, g, ws->stream), "copy into the padded field");
+        ws->launches++;
+        return WS_OK;
+    }
     const cudaMemcpyKind kind = on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice;
     for (int k = 0; k < g.nz; ++k) {
         WS_CUDA(cudaMemcpy2DAsync(dst + ws::pidx(g, 0, 0, k), size_t(g.pnx) * 4,
@@ -223,11 +233,21 @@ int copy_in(ws_t ws, float *dst, const float *src, int on_device) {
                                   size_t(g.nx) * 4, g.ny, kind, ws->stream),
                 "copy into the padded field");
     }
-    return WS_OK;
+    return src2 ? copy_in(ws, dst2, src2, on_device) : WS_OK;
 }
 
-int copy_out(ws_t ws, float *dst, const float *src, int on_device) {
+int copy_out(ws_t ws, float *dst, const float *src, int on_device, float *dst2, const float *src2) {
     const ws::Geom &g = ws->g;
+    if (on_device && kernel_copyable(dst) && kernel_copyable(dst2)) {
+        // outputs that overlap get their copies one after the other
+        const size_t n = size_t(g.nx) * g.ny * g.nz;
+        const bool both = src2 && (dst2 >= dst + n || dst >= dst2 + n);
+        WS_CUDA(ws::launch_copy_out(src, both ? src2 : nullptr, dst, both ? dst2 : nullptr, g,
+                                    ws->stream),
+                "copy out of the padded field");
+        ws->launches++;
+        return src2 && !both ? copy_out(ws, dst2, src2, on_device) : WS_OK;
+    }
     const cudaMemcpyKind kind = on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost;
     for (int k = 0; k < g.nz; ++k) {
         WS_CUDA(cudaMemcpy2DAsync(dst + size_t(k) * g.ny * g.nx, size_t(g.nx) * 4,
@@ -235,7 +255,7 @@ int copy_out(ws_t ws, float *dst, const float *src, int on_device) {
                                   size_t(g.nx) * 4, g.ny, kind, ws->stream),
                 "copy out of the padded field");
     }
-    return WS_OK;
+    return src2 ? copy_out(ws, dst2, src2, on_device) : WS_OK;
 }
 
 int upload_profiles(ws_t ws) {
@@ -838,8 +858,11 @@ int ws_read_field(ws_t ws, float *u, float *u_prev, int on_device) {
         rc = decode_state16(ws);
         if (rc != WS_OK) return rc;
     }
-    if (u) rc = copy_out(ws, u, ws->buf[ws->cur], on_device);
-    if (rc == WS_OK && u_prev) rc = copy_out(ws, u_prev, ws->buf[1 - ws->cur], on_device);
+    const float *un = ws->buf[ws->cur], *um = ws->buf[1 - ws->cur];
+    if (u)
+        rc = copy_out(ws, u, un, on_device, u_prev, u_prev ? um : nullptr);
+    else if (u_prev)
+        rc = copy_out(ws, u_prev, um, on_device);
     if (rc != WS_OK) return rc;
     if (!on_device) WS_CUDA(cudaStreamSynchronize(ws->stream), "ws_read_field");
     return WS_OK;
@@ -848,19 +871,21 @@ int ws_read_field(ws_t ws, float *u, float *u_prev, int on_device) {
 int ws_write_field(ws_t ws, const float *u, const float *u_prev, long long step, int on_device) {
     if (!ws) return fail(WS_ERR_BADARG, "ws_write_field: NULL handle");
     if (step < 0) return fail(WS_ERR_BADARG, "ws_write_field: step must be >= 0");
+    // everything outside the interior is zero from the start and stays so:
+    // only a missing level needs its buffer cleared
     const size_t fb = field_bytes(ws->g);
-    float *dst[2] = {ws->buf[ws->cur], ws->buf[1 - ws->cur]};
-    const float *srcs[2] = {u, u_prev};
-    for (int b = 0; b < 2; ++b) {
-        WS_CUDA(cudaMemsetAsync(dst[b], 0, fb, ws->stream), "ws_write_field");
-        if (srcs[b]) {
-            int rc = copy_in(ws, dst[b], srcs[b], on_device);
-            if (rc != WS_OK) return rc;
-        }
-    }
+    float *un = ws->buf[ws->cur], *um = ws->buf[1 - ws->cur];
+    if (!u) WS_CUDA(cudaMemsetAsync(un, 0, fb, ws->stream), "ws_write_field");
+    if (!u_prev) WS_CUDA(cudaMemsetAsync(um, 0, fb, ws->stream), "ws_write_field");
+    int rc = WS_OK;
+    if (u)
+        rc = copy_in(ws, un, u, on_device, u_prev ? um : nullptr, u_prev);
+    else if (u_prev)
+        rc = copy_in(ws, um, u_prev, on_device);
+    if (rc != WS_OK) return rc;
     ws->step = step;
     if (ws->storage != WS_STORAGE_FP32) {
-        int rc = encode_state16(ws);
+        rc = encode_state16(ws);
         if (rc != WS_OK) return rc;
     }
     if (!on_device) WS_CUDA(cudaStreamSynchronize(ws->stream), "ws_write_field");

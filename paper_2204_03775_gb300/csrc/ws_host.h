@@ -155,9 +155,12 @@ void free_receivers(ws_t ws);
 // Receiver table of the streaming kernels for tile t, whose consumer threads
 // own 4 x-cells of `rows` consecutive rows (FP32 kernels 1, 16-bit kernel 2).
 int build_rec_tiles(ws_t ws, const ws::StreamTiling &t, int rows = 1);
-// Unpadded [nz][ny][nx] user array <-> interior of a padded field.
-int copy_in(ws_t ws, float *dst, const float *src, int on_device);
-int copy_out(ws_t ws, float *dst, const float *src, int on_device);
+// Unpadded [nz][ny][nx] user arrays <-> interiors of padded fields, one or
+// two fields a call (src2 / dst2 null: one).
+int copy_in(ws_t ws, float *dst, const float *src, int on_device, float *dst2 = nullptr,
+            const float *src2 = nullptr);
+int copy_out(ws_t ws, float *dst, const float *src, int on_device, float *dst2 = nullptr,
+             const float *src2 = nullptr);
 int upload_profiles(ws_t ws);
 // The tile of the 16-bit streaming kernel (64 x ty) and the rows each of its
 // threads computes. The default tile height is the first of kTile16Ys that

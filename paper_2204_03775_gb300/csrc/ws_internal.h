@@ -111,6 +111,14 @@ cudaError_t launch_slowness2_to_w(float *w, const Geom &g, double dt_over_h2,
                                   unsigned *extrema /* [2]: max m bits, min m bits */,
                                   cudaStream_t s);
 
+// Unpadded device arrays a, b [nz][ny][nx] -> interiors of the padded fields
+// A, B, and back; b (B for the way out) null: one field. The two outputs must
+// not overlap. Pointers are aligned to 4 bytes.
+cudaError_t launch_copy_in(const float *a, const float *b, float *A, float *B, const Geom &g,
+                           cudaStream_t s);
+cudaError_t launch_copy_out(const float *A, const float *B, float *a, float *b, const Geom &g,
+                            cudaStream_t s);
+
 struct StreamTiling {
     int tx, ty, zb;
 };

@@ -1,0 +1,56 @@
+"""State copies between user arrays and the padded fields (GPU).
+
+Device arrays go through the copy kernels, host arrays through plane copies;
+the two must agree byte for byte, whatever the row length (whole vectors, a
+ragged tail, single cells), the alignment of the device array, one field or
+both, and nothing outside the interior may change.
+"""
+
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+import paper_2204_03775_gb300 as wsb  # noqa: E402
+
+
+def device_copy(a, offset):
+    """The array on the GPU, its first element `offset` elements into an allocation."""
+    t = torch.empty(a.size + offset, dtype=torch.float32, device="cuda")
+    v = t[offset:].view(a.shape)
+    v.copy_(torch.from_numpy(a))
+    return v
+
+
+@pytest.mark.parametrize("shape", [(1, 1, 1), (3, 2, 3), (2, 5, 4), (7, 3, 36), (5, 9, 101),
+                                   (4, 33, 130), (3, 8, 1028), (6, 400, 64)])
+@pytest.mark.parametrize("offset", [0, 1, 2])
+def test_device_copies_equal_host_copies(shape, offset):
+    nz, ny, nx = shape
+    rng = np.random.default_rng(nx)
+    u, p = (rng.standard_normal(shape).astype(np.float32) for _ in range(2))
+    h = wsb.ws_create(nx, ny, nz, 10.0, 1e-3)
+    wsb.ws_test_fill_padding(h)
+    du, dp = device_copy(u, offset), device_copy(p, offset)
+    for first, second in ((u, p), (u, None), (None, p)):
+        wsb.ws_write_field(h, None, None, 0)
+        wsb.ws_write_field(h, None if first is None else du, None if second is None else dp, 0)
+        ref = [np.zeros(shape, np.float32) if a is None else a for a in (first, second)]
+        hu, hp = wsb.ws_read_field(h)          # host copies
+        assert np.array_equal(hu, ref[0]) and np.array_equal(hp, ref[1])
+        ou, op = device_copy(np.full(shape, 7, np.float32), offset), \
+            device_copy(np.full(shape, 7, np.float32), offset)
+        wsb.ws_read_field(h, ou, op)
+        assert np.array_equal(ou.cpu().numpy(), ref[0]) and np.array_equal(op.cpu().numpy(), ref[1])
+        ou.fill_(7)
+        wsb.ws_read_field(h, None, ou, new=False)
+        assert np.array_equal(ou.cpu().numpy(), ref[1])
+    # the same array for both levels: the copies run one after the other
+    wsb.ws_write_field(h, du, dp, 0)
+    wsb.ws_read_field(h, ou, ou)
+    assert np.array_equal(ou.cpu().numpy(), p)
+    # nothing outside the interior was written
+    wsb.ws_test_fill_padding(h)
+    wsb.ws_write_field(h, du, dp, 0)
+    assert wsb.ws_test_check_padding(h) == 0
