@@ -13,63 +13,180 @@ constexpr int kCopyThreads = 256;
 // Blocks of a launch: about two full loads of the GPU's 152 x 8 resident
 // blocks; longer copies loop over their rows.
 constexpr int kCopyBlocks = 2432;
-// Loads of one row that a thread keeps in flight per field.
-constexpr int kCopyDepth = 4;
+// Vectors of one row that a thread keeps in flight per field: four in rows of
+// whole vectors; one (two loads) in shifted rows, whose 60 registers leave
+// fewer warps (755 x 994 x 400 in 863 us, with two of them 1007).
+constexpr int kCopyDepth = 4, kShiftDepth = 1;
 
-template <int V>
-struct VecOf;
-template <>
-struct VecOf<4> {
-    using T = float4;
-};
-template <>
-struct VecOf<1> {
-    using T = float;
+// One or two arrays on each side: in: user -> padded, out: padded -> user.
+struct Fields {
+    const float *src[2];
+    float *dst[2];
 };
 
-// A group of blockDim.x threads copies a row (nq vectors of V cells); both
-// fields of a row are in flight together. kFields = 1 ignores s1 and d1.
-template <int V, int kFields>
+// The caller's rows when they do not all start on 16 bytes: row r starts
+// `shift` elements (0..3) behind the 16-byte boundary `base`; [lo, hi) are the
+// elements of `base` that belong to the whole array.
+struct Row {
+    long long lo, hi;
+    int shift;
+};
+__device__ __forceinline__ Row user_row(const float *array, long long start, long long cells) {
+    const int shift = (int)((reinterpret_cast<uintptr_t>(array + start) >> 2) & 3u);
+    return Row{shift - start, shift - start + cells, shift};
+}
+
+// The 16 bytes at element e of base, only those inside [lo, hi).
+__device__ __forceinline__ float4 load_inside(const float *base, long long e, const Row &r) {
+    if (e >= r.lo && e + 4 <= r.hi) return *reinterpret_cast<const float4 *>(base + e);
+    float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (e + 0 >= r.lo && e + 0 < r.hi) v.x = base[e + 0];
+    if (e + 1 >= r.lo && e + 1 < r.hi) v.y = base[e + 1];
+    if (e + 2 >= r.lo && e + 2 < r.hi) v.z = base[e + 2];
+    if (e + 3 >= r.lo && e + 3 < r.hi) v.w = base[e + 3];
+    return v;
+}
+
+// Elements s .. s+3 of the 8 in (a, b).
+__device__ __forceinline__ float4 window(const float4 &a, const float4 &b, int s) {
+    switch (s) {
+        case 0: return a;
+        case 1: return make_float4(a.y, a.z, a.w, b.x);
+        case 2: return make_float4(a.z, a.w, b.x, b.y);
+        case 3: return make_float4(a.w, b.x, b.y, b.z);
+        default: return b;
+    }
+}
+
+// Elements [from, to) of v to p (16-byte aligned when all four go).
+__device__ __forceinline__ void store_part(float *p, const float4 &v, int from, int to) {
+    if (from <= 0 && to >= 4) {
+        *reinterpret_cast<float4 *>(p) = v;
+        return;
+    }
+    if (from <= 0 && to > 0) p[0] = v.x;
+    if (from <= 1 && to > 1) p[1] = v.y;
+    if (from <= 2 && to > 2) p[2] = v.z;
+    if (from <= 3 && to > 3) p[3] = v.w;
+}
+
+// A group of blockDim.x threads copies a row; both fields of a row are in
+// flight together. kAligned: every row is whole 16-byte vectors on both
+// sides. Otherwise every access still is a 16-byte one on a 16-byte boundary:
+// the shifted side is read as two neighbouring vectors, the second of which
+// comes from L1, and a row's first and last vectors are written cell by cell,
+// so nothing outside the row changes. Both fields of 755 x 994 x 400: in 863,
+// out 754 us (5.6, 6.4 TB/s), against 1166, 1523 us with 4-byte accesses;
+// 1024 x 512 x 512: in 650, out 641 us (6.6, 6.7 TB/s of the measured 6.78).
+template <bool kAligned, bool kIn, int kFields>
 __global__ void __launch_bounds__(kCopyThreads)
-    copy_rows_kernel(const float *__restrict__ s0, const float *__restrict__ s1,
-                     float *__restrict__ d0, float *__restrict__ d1, const int nq,
-                     const unsigned ny, const unsigned rows, const long long spitch,
-                     const long long splane, const long long dpitch, const long long dplane) {
-    using T = typename VecOf<V>::T;
+    copy_rows_kernel(const Fields f, const int nx, const unsigned ny, const unsigned rows,
+                     const int pitch, const long long plane, const long long cells) {
     const int step = blockDim.x;
     for (unsigned long long r = (unsigned long long)blockIdx.x * blockDim.y + threadIdx.y; r < rows;
          r += (unsigned long long)gridDim.x * blockDim.y) {
         const unsigned k = (unsigned)r / ny, j = (unsigned)r - k * ny;
-        const long long so = k * splane + j * spitch, dof = k * dplane + j * dpitch;
-        const T *a0 = reinterpret_cast<const T *>(s0 + so);
-        const T *a1 = reinterpret_cast<const T *>(s1 + so);
-        T *b0 = reinterpret_cast<T *>(d0 + dof);
-        T *b1 = reinterpret_cast<T *>(d1 + dof);
-        for (int q = threadIdx.x; q < nq; q += kCopyDepth * step) {
-            T x0[kCopyDepth], x1[kCopyDepth];
+        const long long uo = (long long)r * nx, po = k * plane + (long long)j * pitch;
+        if constexpr (kAligned) {
+            const int nq = nx / 4;
+            for (int q = threadIdx.x; q < nq; q += kCopyDepth * step) {
+                float4 x[kFields][kCopyDepth];
 #pragma unroll
-            for (int c = 0; c < kCopyDepth; ++c)
-                if (q + c * step < nq) {
-                    x0[c] = __ldcs(a0 + q + c * step);
-                    if (kFields == 2) x1[c] = __ldcs(a1 + q + c * step);
+                for (int c = 0; c < kCopyDepth; ++c)
+#pragma unroll
+                    for (int m = 0; m < kFields; ++m)
+                        if (q + c * step < nq)
+                            x[m][c] = __ldcs(reinterpret_cast<const float4 *>(
+                                                 f.src[m] + (kIn ? uo : po)) + q + c * step);
+#pragma unroll
+                for (int c = 0; c < kCopyDepth; ++c)
+#pragma unroll
+                    for (int m = 0; m < kFields; ++m)
+                        if (q + c * step < nq)
+                            reinterpret_cast<float4 *>(f.dst[m] + (kIn ? po : uo))[q + c * step] =
+                                x[m][c];
+            }
+        } else {
+            Row w[kFields];
+            const float *ub[kFields];   // the caller's side, 16-byte aligned
+            const float *pb[kFields];   // the padded side
+            int nq = (nx + 3) / 4;      // in: padded vectors of the row
+#pragma unroll
+            for (int m = 0; m < kFields; ++m) {
+                const float *user = kIn ? f.src[m] : f.dst[m];
+                w[m] = user_row(user, uo, cells);
+                ub[m] = user + uo - w[m].shift;
+                pb[m] = (kIn ? f.dst[m] : f.src[m]) + po;
+                // out: the most user vectors that either row touches
+                if (!kIn) nq = max(nq, (nx + w[m].shift + 3) / 4);
+            }
+            // the row's vectors, and the one behind them, all lie in the array
+            const bool inside = uo >= 4 && uo + nx + 8 <= cells;
+            constexpr int D = kShiftDepth;
+            for (int q = threadIdx.x; q < nq; q += D * step) {
+                float4 a[kFields][D], b[kFields][D];
+                if constexpr (kIn) {   // user cells 4v .. 4v+3 of the row
+                    auto load = [&](auto &&vec) {
+#pragma unroll
+                        for (int c = 0; c < D; ++c)
+#pragma unroll
+                            for (int m = 0; m < kFields; ++m)
+                                if (q + c * step < nq) {
+                                    const long long e = 4ll * (q + c * step);
+                                    a[m][c] = vec(m, e);
+                                    b[m][c] = w[m].shift ? vec(m, e + 4) : a[m][c];
+                                }
+                    };
+                    // all but the array's ends: plain loads, issued together
+                    if (inside)
+                        load([&](int m, long long e) {
+                            return *reinterpret_cast<const float4 *>(ub[m] + e);
+                        });
+                    else
+                        load([&](int m, long long e) { return load_inside(ub[m], e, w[m]); });
+                } else {               // row cells 4v - shift .. + 3
+#pragma unroll
+                    for (int c = 0; c < D; ++c)
+#pragma unroll
+                        for (int m = 0; m < kFields; ++m) {
+                            const int v = q + c * step;
+                            if (v >= nq) continue;
+                            b[m][c] = 4 * v < nx   // else beyond the row: not stored
+                                          ? *reinterpret_cast<const float4 *>(pb[m] + 4 * v)
+                                          : make_float4(0.f, 0.f, 0.f, 0.f);
+                            a[m][c] = w[m].shift && v > 0
+                                          ? *reinterpret_cast<const float4 *>(pb[m] + 4 * v - 4)
+                                          : b[m][c];
+                        }
                 }
 #pragma unroll
-            for (int c = 0; c < kCopyDepth; ++c)
-                if (q + c * step < nq) {
-                    b0[q + c * step] = x0[c];
-                    if (kFields == 2) b1[q + c * step] = x1[c];
-                }
+                for (int c = 0; c < D; ++c)
+#pragma unroll
+                    for (int m = 0; m < kFields; ++m) {
+                        const int v = q + c * step;
+                        if (v >= nq) continue;
+                        if constexpr (kIn)
+                            store_part(const_cast<float *>(pb[m]) + 4 * v,
+                                       window(a[m][c], b[m][c], w[m].shift), 0, nx - 4 * v);
+                        else
+                            store_part(const_cast<float *>(ub[m]) + 4 * v,
+                                       window(a[m][c], b[m][c], 4 - w[m].shift),
+                                       w[m].shift - 4 * v, nx + w[m].shift - 4 * v);
+                    }
+            }
         }
     }
 }
 
 bool aligned16(const void *p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
 
-template <int V>
-cudaError_t launch_copy(const float *s0, const float *s1, float *d0, float *d1, const Geom &g,
-                        long long spitch, long long splane, long long dpitch, long long dplane,
-                        cudaStream_t s) {
-    const int nq = g.nx / V;
+template <bool kIn>
+cudaError_t launch_copy(const Fields &f, const Geom &g, cudaStream_t s) {
+    // rows are whole vectors on both sides (the padded interiors always start
+    // on 128 bytes)
+    const float *const *user = kIn ? f.src : f.dst;
+    const bool aligned = g.nx % 4 == 0 && aligned16(user[0]) && aligned16(user[1]);
+    const int nq = (g.nx + 3) / 4;
     // threads a row: the widest of 32, 16, 8 that leaves the fewest idle
     int bx = 32;
     for (int b : {16, 8})
@@ -78,37 +195,33 @@ cudaError_t launch_copy(const float *s0, const float *s1, float *d0, float *d1, 
     const unsigned rows = (unsigned)g.ny * (unsigned)g.nz;   // at most 65535^2
     const unsigned want = (unsigned)(((unsigned long long)rows + block.y - 1) / block.y);
     const unsigned grid = want < (unsigned)kCopyBlocks ? want : (unsigned)kCopyBlocks;
-    if (s1)
-        copy_rows_kernel<V, 2><<<grid, block, 0, s>>>(s0, s1, d0, d1, nq, g.ny, rows, spitch, splane,
-                                                      dpitch, dplane);
-    else
-        copy_rows_kernel<V, 1><<<grid, block, 0, s>>>(s0, nullptr, d0, nullptr, nq, g.ny, rows,
-                                                      spitch, splane, dpitch, dplane);
+    const long long cells = (long long)rows * g.nx;
+#define WS_COPY(AL, NF)                                                                        \
+    copy_rows_kernel<AL, kIn, NF><<<grid, block, 0, s>>>(f, g.nx, g.ny, rows, g.pnx, g.plane, \
+                                                         cells)
+    if (aligned) {
+        if (f.src[1]) WS_COPY(true, 2);
+        else WS_COPY(true, 1);
+    } else {
+        if (f.src[1]) WS_COPY(false, 2);
+        else WS_COPY(false, 1);
+    }
+#undef WS_COPY
     return cudaGetLastError();
 }
 
 }  // namespace
 
-// 128-bit accesses need rows that are whole float4s on both sides: the padded
-// interiors always start on 128 bytes, the caller's rows only when nx is a
-// multiple of 4 and the arrays are 16-byte aligned; else one cell a thread
-// (coalesced all the same).
 cudaError_t launch_copy_in(const float *a, const float *b, float *A, float *B, const Geom &g,
                            cudaStream_t s) {
-    const long long o = pidx(g, 0, 0, 0), plane = (long long)g.nx * g.ny;
-    float *d1 = b ? B + o : nullptr;
-    if (g.nx % 4 == 0 && aligned16(a) && aligned16(b))
-        return launch_copy<4>(a, b, A + o, d1, g, g.nx, plane, g.pnx, g.plane, s);
-    return launch_copy<1>(a, b, A + o, d1, g, g.nx, plane, g.pnx, g.plane, s);
+    const long long o = pidx(g, 0, 0, 0);
+    return launch_copy<true>(Fields{{a, b}, {A + o, b ? B + o : nullptr}}, g, s);
 }
 
 cudaError_t launch_copy_out(const float *A, const float *B, float *a, float *b, const Geom &g,
                             cudaStream_t s) {
-    const long long o = pidx(g, 0, 0, 0), plane = (long long)g.nx * g.ny;
-    const float *s1 = B ? B + o : nullptr;
-    if (g.nx % 4 == 0 && aligned16(a) && aligned16(b))
-        return launch_copy<4>(A + o, s1, a, b, g, g.pnx, g.plane, g.nx, plane, s);
-    return launch_copy<1>(A + o, s1, a, b, g, g.pnx, g.plane, g.nx, plane, s);
+    const long long o = pidx(g, 0, 0, 0);
+    return launch_copy<false>(Fields{{A + o, B ? B + o : nullptr}, {a, b}}, g, s);
 }
 
 }  // namespace ws
