@@ -577,12 +577,16 @@ int ws_set_velocity(ws_t ws, const float *v, int on_device) {
     if (!ws || !v) return fail(WS_ERR_BADARG, "ws_set_velocity: NULL argument");
     ws->model_version++;
     ws->vel_ok = false;
-    int rc = copy_in(ws, ws->w, v, on_device);
-    if (rc != WS_OK) return rc;
+    const bool direct = on_device && kernel_copyable(v);
+    if (!direct) {
+        int rc = copy_in(ws, ws->w, v, on_device);
+        if (rc != WS_OK) return rc;
+    }
     static const unsigned init[2] = {0u, 0x7f800000u};
     WS_CUDA(cudaMemcpyAsync(ws->status + 1, init, sizeof init, cudaMemcpyHostToDevice, ws->stream),
             "ws_set_velocity");
-    WS_CUDA(ws::launch_velocity_to_w(ws->w, ws->g, ws->dt / ws->h, ws->status + 1, ws->stream),
+    WS_CUDA(ws::launch_velocity_to_w(direct ? v : nullptr, ws->w, ws->g, ws->dt / ws->h,
+                                     ws->status + 1, ws->stream),
             "velocity conversion kernel");
     ws->launches++;
     unsigned ext[2];
@@ -607,13 +611,17 @@ int ws_set_slowness2(ws_t ws, const float *m, int on_device) {
     if (!ws || !m) return fail(WS_ERR_BADARG, "ws_set_slowness2: NULL argument");
     ws->model_version++;
     ws->vel_ok = false;
-    int rc = copy_in(ws, ws->w, m, on_device);
-    if (rc != WS_OK) return rc;
+    const bool direct = on_device && kernel_copyable(m);
+    if (!direct) {
+        int rc = copy_in(ws, ws->w, m, on_device);
+        if (rc != WS_OK) return rc;
+    }
     static const unsigned init[2] = {0u, 0x7f800000u};
     WS_CUDA(cudaMemcpyAsync(ws->status + 1, init, sizeof init, cudaMemcpyHostToDevice, ws->stream),
             "ws_set_slowness2");
     const double r = ws->dt / ws->h;
-    WS_CUDA(ws::launch_slowness2_to_w(ws->w, ws->g, r * r, ws->status + 1, ws->stream),
+    WS_CUDA(ws::launch_slowness2_to_w(direct ? m : nullptr, ws->w, ws->g, r * r, ws->status + 1,
+                                      ws->stream),
             "slowness conversion kernel");
     ws->launches++;
     unsigned ext[2];

@@ -104,12 +104,14 @@ cudaError_t launch_step_direct(const float *u, const float *up, float *out, cons
 cudaError_t launch_gather_receivers(const float *u_next, const long long *rec_pidx, int nrec,
                                     float *traces, int nt_max, long long trace_step,
                                     cudaStream_t s);
-cudaError_t launch_velocity_to_w(float *w, const Geom &g, double dt_over_h,
-                                 unsigned *extrema /* [2]: max bits, min bits */,
-                                 cudaStream_t s);
-cudaError_t launch_slowness2_to_w(float *w, const Geom &g, double dt_over_h2,
-                                  unsigned *extrema /* [2]: max m bits, min m bits */,
-                                  cudaStream_t s);
+// The model (device array [nz][ny][nx], or null: already in w's interior) into
+// the padded w: V -> (V dt / h)^2, m = 1/V^2 -> (dt / h)^2 / m, in double,
+// rounded once. extrema collects {max, min} of the values as float bits; a
+// value that is not finite and > 0 counts as 0 in the minimum.
+cudaError_t launch_velocity_to_w(const float *v, float *w, const Geom &g, double dt_over_h,
+                                 unsigned *extrema, cudaStream_t s);
+cudaError_t launch_slowness2_to_w(const float *m, float *w, const Geom &g, double dt_over_h2,
+                                  unsigned *extrema, cudaStream_t s);
 
 // Unpadded device arrays a, b [nz][ny][nx] -> interiors of the padded fields
 // A, B, and back; b (B for the way out) null: one field. The two outputs must

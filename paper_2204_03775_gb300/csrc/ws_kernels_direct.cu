@@ -78,86 +78,4 @@ cudaError_t launch_gather_receivers(const float *u_next, const long long *rec_pi
     return cudaGetLastError();
 }
 
-// In place over the interior of the padded buffer: V -> (V dt / h)^2,
-// computed in double and rounded once. extrema[0] collects max(V) and
-// extrema[1] min(V) as float bit patterns (their unsigned order is the float
-// order for V >= 0). A value that is not finite and > 0 contributes 0 to the
-// minimum, which the host rejects.
-__global__ void velocity_to_w_kernel(float *__restrict__ w, Geom g, double dt_over_h,
-                                     unsigned *__restrict__ extrema) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    const int j = blockIdx.y;
-    const int k = blockIdx.z;
-    unsigned vmax = 0u, vmin = 0x7f800000u;
-    if (i < g.nx) {
-        const long long p = pidx(g, i, j, k);
-        const float v = w[p];
-        if (v > 0.0f && isfinite(v)) {
-            vmax = __float_as_uint(v);
-            vmin = vmax;
-        } else {
-            vmin = 0u;
-        }
-        const double r = __dmul_rn((double)v, dt_over_h);   // as ws_energy_noalloc forms it
-        w[p] = (float)__dmul_rn(r, r);
-    }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        vmax = max(vmax, __shfl_xor_sync(0xffffffffu, vmax, o));
-        vmin = min(vmin, __shfl_xor_sync(0xffffffffu, vmin, o));
-    }
-    if ((threadIdx.x & 31) == 0) {
-        atomicMax(&extrema[0], vmax);
-        atomicMin(&extrema[1], vmin);
-    }
-}
-
-// In place: m (squared slowness, s^2/m^2) -> (V dt / h)^2 = (dt / h)^2 / m,
-// in double, rounded once. extrema[0] / extrema[1] collect max(m) / min(m)
-// as float bits; a value that is not finite and > 0 contributes 0 to the
-// minimum, which the host rejects.
-__global__ void slowness2_to_w_kernel(float *__restrict__ w, Geom g, double dt_over_h2,
-                                      unsigned *__restrict__ extrema) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    const int j = blockIdx.y;
-    const int k = blockIdx.z;
-    unsigned mmax = 0u, mmin = 0x7f800000u;
-    if (i < g.nx) {
-        const long long p = pidx(g, i, j, k);
-        const float m = w[p];
-        if (m > 0.0f && isfinite(m)) {
-            mmax = __float_as_uint(m);
-            mmin = mmax;
-        } else {
-            mmin = 0u;
-        }
-        w[p] = (float)(dt_over_h2 / (double)m);
-    }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        mmax = max(mmax, __shfl_xor_sync(0xffffffffu, mmax, o));
-        mmin = min(mmin, __shfl_xor_sync(0xffffffffu, mmin, o));
-    }
-    if ((threadIdx.x & 31) == 0) {
-        atomicMax(&extrema[0], mmax);
-        atomicMin(&extrema[1], mmin);
-    }
-}
-
-cudaError_t launch_slowness2_to_w(float *w, const Geom &g, double dt_over_h2, unsigned *extrema,
-                                  cudaStream_t s) {
-    dim3 block(128, 1, 1);
-    dim3 grid((g.nx + 127) / 128, g.ny, g.nz);
-    slowness2_to_w_kernel<<<grid, block, 0, s>>>(w, g, dt_over_h2, extrema);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_velocity_to_w(float *w, const Geom &g, double dt_over_h, unsigned *extrema,
-                                 cudaStream_t s) {
-    dim3 block(128, 1, 1);
-    dim3 grid((g.nx + 127) / 128, g.ny, g.nz);
-    velocity_to_w_kernel<<<grid, block, 0, s>>>(w, g, dt_over_h, extrema);
-    return cudaGetLastError();
-}
-
 }  // namespace ws

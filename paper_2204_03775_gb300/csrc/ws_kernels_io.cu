@@ -1,7 +1,7 @@
 // Copies between the caller's unpadded [nz][ny][nx] device arrays and the
-// interiors of the padded fields.
+// interiors of the padded fields, and the conversion of the caller's model.
 //
-// Bound: HBM, 8 bytes a cell and field. One launch moves both time levels.
+// Copies: bound by HBM, 8 bytes a cell and field. One launch moves both time levels.
 // (One 2D copy per plane and field, which this replaces, cost 4 to 8 us a
 // plane whatever its size: 256^3 in and out 4.2 ms, 1024^3 35 ms.)
 #include "ws_internal.h"
@@ -178,6 +178,19 @@ __global__ void __launch_bounds__(kCopyThreads)
     }
 }
 
+// Blocks and threads of a kernel that walks the grid's rows in vectors of 4
+// cells: threads a row: the widest of 32, 16, 8 that leaves the fewest idle.
+unsigned row_grid(const Geom &g, dim3 *block) {
+    const int nq = (g.nx + 3) / 4;
+    int bx = 32;
+    for (int b : {16, 8})
+        if ((nq + b - 1) / b * b < (nq + bx - 1) / bx * bx) bx = b;
+    *block = dim3(bx, kCopyThreads / bx);
+    const unsigned long long rows = (unsigned long long)g.ny * g.nz;
+    const unsigned long long want = (rows + block->y - 1) / block->y;
+    return (unsigned)(want < kCopyBlocks ? want : kCopyBlocks);
+}
+
 bool aligned16(const void *p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
 
 template <bool kIn>
@@ -186,15 +199,9 @@ cudaError_t launch_copy(const Fields &f, const Geom &g, cudaStream_t s) {
     // on 128 bytes)
     const float *const *user = kIn ? f.src : f.dst;
     const bool aligned = g.nx % 4 == 0 && aligned16(user[0]) && aligned16(user[1]);
-    const int nq = (g.nx + 3) / 4;
-    // threads a row: the widest of 32, 16, 8 that leaves the fewest idle
-    int bx = 32;
-    for (int b : {16, 8})
-        if ((nq + b - 1) / b * b < (nq + bx - 1) / bx * bx) bx = b;
-    const dim3 block(bx, kCopyThreads / bx);
     const unsigned rows = (unsigned)g.ny * (unsigned)g.nz;   // at most 65535^2
-    const unsigned want = (unsigned)(((unsigned long long)rows + block.y - 1) / block.y);
-    const unsigned grid = want < (unsigned)kCopyBlocks ? want : (unsigned)kCopyBlocks;
+    dim3 block;
+    const unsigned grid = row_grid(g, &block);
     const long long cells = (long long)rows * g.nx;
 #define WS_COPY(AL, NF)                                                                        \
     copy_rows_kernel<AL, kIn, NF><<<grid, block, 0, s>>>(f, g.nx, g.ny, rows, g.pnx, g.plane, \
@@ -222,6 +229,178 @@ cudaError_t launch_copy_out(const float *A, const float *B, float *a, float *b, 
                             cudaStream_t s) {
     const long long o = pidx(g, 0, 0, 0);
     return launch_copy<false>(Fields{{A + o, B ? B + o : nullptr}, {a, b}}, g, s);
+}
+
+// ------------------------------------------------------------ model
+
+namespace {
+
+// (V dt / h)^2 from V, and (dt / h)^2 / m from m = 1/V^2, each the double
+// result rounded to float. GB300 runs FP64 at a small fraction of FP32, so
+// the value is formed as a sum q + q2 of two floats (error below 2^-44 of it:
+// the scale as two floats, products and remainders exact through fma), whose
+// nearest float is that of the double result unless both lie within 2^-42 of
+// a tie between two floats; then, and outside the range in which no term
+// underflows, the double expression itself is evaluated (about one cell in
+// 2^18). The stored floats are the same bits either way.
+struct Scale {
+    double c;       // dt / h, or (dt / h)^2
+    float hi, lo;   // c as two floats
+    bool fast;      // hi in [2^-60, 2^60]
+};
+
+Scale scale_of(double c) {
+    Scale s{c, (float)c, 0.0f, false};
+    s.lo = (float)(c - (double)s.hi);
+    s.fast = s.hi >= 0x1p-60f && s.hi <= 0x1p60f;
+    return s;
+}
+
+// The nearest float of q + q2 if the sum moved by +-2^-42 q rounds alike.
+__device__ __forceinline__ bool round_sum(float q, float q2, float *w) {
+    const float a = q + fmaf(q, 0x1p-42f, q2), b = q + fmaf(q, -0x1p-42f, q2);
+    *w = a;
+    return a == b && q >= 0x1p-60f && q <= 0x1p60f;
+}
+
+struct FromVelocity {
+    // (a call: inlined, its two products were issued for every cell)
+    static __device__ __noinline__ float slow(float v, double c) {
+        const double r = __dmul_rn((double)v, c);   // as ws_energy_noalloc forms it
+        return (float)__dmul_rn(r, r);
+    }
+    static __device__ __forceinline__ bool fast(float v, const Scale &k, float *w) {
+        const float p = __fmul_rn(v, k.hi);
+        const float l = fmaf(v, k.lo, fmaf(v, k.hi, -p));
+        const float s = __fadd_rn(p, l), t = __fsub_rn(l, __fsub_rn(s, p));   // V dt / h = s + t
+        const float q = __fmul_rn(s, s);
+        return round_sum(q, fmaf(2.0f * s, t, fmaf(s, s, -q)), w) && k.fast;
+    }
+};
+
+struct FromSlowness2 {
+    static __device__ __noinline__ float slow(float m, double c) {
+        return (float)(c / (double)m);
+    }
+    static __device__ __forceinline__ bool fast(float m, const Scale &k, float *w) {
+        const float q = __fdiv_rn(k.hi, m);
+        const float r = __fadd_rn(fmaf(-q, m, k.hi), k.lo);   // c - q m
+        return round_sum(q, __fdividef(r, m), w) && k.fast && m >= 0x1p-100f && m <= 0x1p100f;
+    }
+};
+
+struct Extrema {
+    unsigned hi, lo;
+    // max and min as float bit patterns (their unsigned order is the float
+    // order for x >= 0); a value that is not finite and > 0 counts as 0 in
+    // the minimum, which the host rejects
+    __device__ __forceinline__ void take(float x) {
+        const bool good = x > 0.0f && isfinite(x);
+        const unsigned b = __float_as_uint(x);
+        hi = max(hi, good ? b : 0u);
+        lo = min(lo, good ? b : 0u);
+    }
+};
+
+template <class Conv>
+__device__ __forceinline__ float convert(float x, const Scale &k, Extrema &e) {
+    float w;
+    e.take(x);
+    if (!Conv::fast(x, k, &w)) w = Conv::slow(x, k.c);
+    return w;
+}
+
+// The model into the padded field w: from the caller's array (rows that are
+// whole 16-byte vectors) or, src null, in place. Bound: HBM, 8 bytes a cell.
+// Extrema meet in the block before its one atomic pair: one pair a warp, all
+// on two words, took 0.67 ms at 256^3 and 44 ms at 1024^3; this takes 0.026
+// and 1.43 ms from a velocity (6.0 TB/s), 0.035 and 1.73 from a slowness
+// (one float division a cell); with the double products issued for every
+// cell 7.8 ms at 1024^3.
+template <class Conv>
+__global__ void __launch_bounds__(kCopyThreads)
+    model_kernel(const float *src, float *w, const int nx, const unsigned ny, const unsigned rows,
+                 const int pitch, const long long plane, const Scale scale,
+                 unsigned *__restrict__ extrema) {
+    Extrema e{0u, 0x7f800000u};
+    const int step = blockDim.x;
+    for (unsigned long long r = (unsigned long long)blockIdx.x * blockDim.y + threadIdx.y; r < rows;
+         r += (unsigned long long)gridDim.x * blockDim.y) {
+        const unsigned k = (unsigned)r / ny, j = (unsigned)r - k * ny;
+        float *out = w + k * plane + (long long)j * pitch;
+        const float *in = src ? src + (long long)r * nx : out;
+        for (int i = 4 * threadIdx.x; i < nx; i += 8 * step) {
+            // two vectors in flight (in place, the last one may reach into
+            // the halo of its row)
+            const int i2 = i + 4 * step;
+            const float4 x = *reinterpret_cast<const float4 *>(in + i);
+            const float4 y = i2 < nx ? *reinterpret_cast<const float4 *>(in + i2) : x;
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const int at = h ? i2 : i;
+                const float4 v = h ? y : x;
+                if (at + 4 <= nx) {
+                    float4 o;
+                    o.x = convert<Conv>(v.x, scale, e);
+                    o.y = convert<Conv>(v.y, scale, e);
+                    o.z = convert<Conv>(v.z, scale, e);
+                    o.w = convert<Conv>(v.w, scale, e);
+                    *reinterpret_cast<float4 *>(out + at) = o;
+                } else if (at < nx) {
+                    out[at] = convert<Conv>(v.x, scale, e);
+                    if (at + 1 < nx) out[at + 1] = convert<Conv>(v.y, scale, e);
+                    if (at + 2 < nx) out[at + 2] = convert<Conv>(v.z, scale, e);
+                }
+            }
+        }
+    }
+    __shared__ unsigned hi, lo;
+    if (threadIdx.x == 0 && threadIdx.y == 0) {
+        hi = 0u;
+        lo = 0x7f800000u;
+    }
+    __syncthreads();
+    const unsigned whi = __reduce_max_sync(0xffffffffu, e.hi);
+    const unsigned wlo = __reduce_min_sync(0xffffffffu, e.lo);
+    if (((threadIdx.y * blockDim.x + threadIdx.x) & 31) == 0) {
+        atomicMax(&hi, whi);
+        atomicMin(&lo, wlo);
+    }
+    __syncthreads();
+    if (threadIdx.x == 0 && threadIdx.y == 0) {
+        atomicMax(&extrema[0], hi);
+        atomicMin(&extrema[1], lo);
+    }
+}
+
+// v may be null (the values are in w already). Rows that are not whole
+// vectors are brought into the padded field first.
+template <class Conv>
+cudaError_t launch_model(const float *v, float *w, const Geom &g, double c, unsigned *extrema,
+                         cudaStream_t s) {
+    if (v && (g.nx % 4 != 0 || !aligned16(v))) {
+        const cudaError_t e = launch_copy_in(v, nullptr, w, nullptr, g, s);
+        if (e != cudaSuccess) return e;
+        v = nullptr;
+    }
+    dim3 block;
+    const unsigned grid = row_grid(g, &block);
+    model_kernel<Conv><<<grid, block, 0, s>>>(v, w + pidx(g, 0, 0, 0), g.nx, g.ny,
+                                              (unsigned)g.ny * (unsigned)g.nz, g.pnx, g.plane,
+                                              scale_of(c), extrema);
+    return cudaGetLastError();
+}
+
+}  // namespace
+
+cudaError_t launch_velocity_to_w(const float *v, float *w, const Geom &g, double dt_over_h,
+                                 unsigned *extrema, cudaStream_t s) {
+    return launch_model<FromVelocity>(v, w, g, dt_over_h, extrema, s);
+}
+
+cudaError_t launch_slowness2_to_w(const float *m, float *w, const Geom &g, double dt_over_h2,
+                                  unsigned *extrema, cudaStream_t s) {
+    return launch_model<FromSlowness2>(m, w, g, dt_over_h2, extrema, s);
 }
 
 }  // namespace ws

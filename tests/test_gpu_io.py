@@ -54,3 +54,52 @@ def test_device_copies_equal_host_copies(shape, offset):
     wsb.ws_test_fill_padding(h)
     wsb.ws_write_field(h, du, dp, 0)
     assert wsb.ws_test_check_padding(h) == 0
+
+
+def near_ties(values, of):
+    """The values whose double result lies closest to the middle of two floats."""
+    x = of(values.astype(np.float64))
+    f = x.astype(np.float32)
+    gap = np.abs(np.abs(x - f.astype(np.float64)) - 0.5 * np.spacing(f).astype(np.float64))
+    return values[np.argsort(gap / x)[:8]]
+
+
+@pytest.mark.parametrize("slowness", [False, True])
+@pytest.mark.parametrize("nx,offset", [(64, 0), (64, 1), (67, 0), (5, 0)])
+def test_model_is_the_rounded_double(slowness, nx, offset):
+    """The stored model is (V dt/h)^2, formed in double and rounded once, also
+    where the double lies next to a tie between two floats: read back exactly
+    as one step from rest under sources of amplitude 1 with h = 1."""
+    ny, nz, dt = 3, 5, 0.4 / 4500.0
+    rng = np.random.default_rng(nx + offset)
+    many = rng.uniform(1500.0, 4500.0, 1 << 20).astype(np.float32)
+    if slowness:
+        many = (1.0 / many.astype(np.float64) ** 2).astype(np.float32)
+        of = lambda m: (dt * dt) / m                      # noqa: E731
+    else:
+        of = lambda v: (v * dt) * (v * dt)                # noqa: E731
+    vals = np.concatenate([near_ties(many, of), many[:8]])
+    model = np.full((nz, ny, nx), vals[0], np.float32)
+    cells = [tuple(int(c) for c in np.unravel_index(q, model.shape))
+             for q in rng.choice(model.size, 16, replace=False)]
+    cells[0] = (nz - 1, ny - 1, nx - 1)
+    for c, v in zip(cells, vals):
+        model[c] = v
+    expected = np.zeros(model.shape, np.float32)
+    for c in set(cells):
+        expected[c] = np.float32(of(np.float64(model[c])))
+    for on_device in (True, False):
+        h = wsb.ws_create(nx, ny, nz, 1.0, dt)
+        wsb.ws_test_fill_padding(h)
+        setter = wsb.ws_set_slowness2 if slowness else wsb.ws_set_velocity
+        setter(h, device_copy(model, offset) if on_device else model)
+        for k, j, i in set(cells):
+            wsb.ws_add_source(h, i, j, k, 10.0, 0.0, 1.0)
+        wsb.ws_step(h, 1)
+        u, _ = wsb.ws_read_field(h)
+        assert np.array_equal(u, expected)
+        assert wsb.ws_test_check_padding(h) == 0
+        bad = model.copy()
+        bad[nz // 2, 0, nx - 1] = np.nan
+        with pytest.raises(wsb.WaveStepError):
+            setter(h, device_copy(bad, offset) if on_device else bad)
