@@ -319,12 +319,12 @@ int default_zblock16(const ws::Geom &g, int ty) {
     return std::min(zb, std::min(zs, g.nz));
 }
 
-// FP32 buffers -> the 16-bit state (U = u^n, D = u^n - u^{n-1}), exponents
-// in the step's slot.
-int encode_state16(ws_t ws) {
+// FP32 levels (the handle's buffers, or device arrays) -> the 16-bit state
+// (U = u^n, D = u^n - u^{n-1}), exponents in the step's slot.
+int encode_state16(ws_t ws, const ws::Fp32Fields &f) {
     const int sn = (int)(ws->step & 3), so = (int)((ws->step + 1) & 3);
-    WS_CUDA(ws::launch_encode16(ws->storage, ws->buf[ws->cur], ws->buf[1 - ws->cur],
-                                ws->buf16[ws->cur], ws->d16, ws->g, ws->scale, sn, ws->stream),
+    WS_CUDA(ws::launch_encode16(ws->storage, f, ws->buf16[ws->cur], ws->d16, ws->g, ws->scale, sn,
+                                ws->stream),
             "encode field");
     // the next step accumulates max |u^{n+1}| into slot (step + 1) & 3
     WS_CUDA(cudaMemsetAsync(&ws->scale->amax[so], 0, sizeof(unsigned), ws->stream), "encode field");
@@ -332,14 +332,23 @@ int encode_state16(ws_t ws) {
     return WS_OK;
 }
 
-// The 16-bit state -> FP32 buffers (u^n, u^{n-1}).
-int decode_state16(ws_t ws) {
+int encode_state16(ws_t ws) {
+    const float *un = ws->buf[ws->cur], *um = ws->buf[1 - ws->cur];
+    return encode_state16(ws, ws::padded_pair(un, um, ws->g));
+}
+
+// The 16-bit state -> FP32 levels.
+int decode_state16(ws_t ws, const ws::Fp32Out &f) {
     const int sn = (int)(ws->step & 3);
-    WS_CUDA(ws::launch_decode16(ws->storage, ws->buf16[ws->cur], ws->d16, ws->buf[ws->cur],
-                                ws->buf[1 - ws->cur], ws->g, ws->scale, sn, ws->stream),
+    WS_CUDA(ws::launch_decode16(ws->storage, ws->buf16[ws->cur], ws->d16, f, ws->g, ws->scale, sn,
+                                ws->stream),
             "decode field");
     ws->launches += 1;
     return WS_OK;
+}
+
+int decode_state16(ws_t ws) {
+    return decode_state16(ws, ws::padded_pair(ws->buf[ws->cur], ws->buf[1 - ws->cur], ws->g));
 }
 
 // Point sources of step n: (V_s dt)^2 s(t_n) is added at each source cell,
@@ -863,6 +872,16 @@ int ws_read_field(ws_t ws, float *u, float *u_prev, int on_device) {
     if (!ws) return fail(WS_ERR_BADARG, "ws_read_field: NULL handle");
     int rc = WS_OK;
     if (ws->storage != WS_STORAGE_FP32) {
+        if (on_device && kernel_copyable(u) && kernel_copyable(u_prev)) {
+            // straight into the caller's arrays; outputs that overlap one
+            // after the other
+            const size_t n = size_t(ws->g.nx) * ws->g.ny * ws->g.nz;
+            const bool both = !u || !u_prev || u_prev >= u + n || u >= u_prev + n;
+            if (both) return decode_state16(ws, ws::dense_pair(u, u_prev, ws->g));
+            rc = decode_state16(ws, ws::dense_pair<float>(u, nullptr, ws->g));
+            if (rc == WS_OK) rc = decode_state16(ws, ws::dense_pair<float>(nullptr, u_prev, ws->g));
+            return rc;
+        }
         rc = decode_state16(ws);
         if (rc != WS_OK) return rc;
     }
@@ -879,6 +898,11 @@ int ws_read_field(ws_t ws, float *u, float *u_prev, int on_device) {
 int ws_write_field(ws_t ws, const float *u, const float *u_prev, long long step, int on_device) {
     if (!ws) return fail(WS_ERR_BADARG, "ws_write_field: NULL handle");
     if (step < 0) return fail(WS_ERR_BADARG, "ws_write_field: step must be >= 0");
+    if (ws->storage != WS_STORAGE_FP32 && on_device && (u || u_prev) && kernel_copyable(u) &&
+        kernel_copyable(u_prev)) {
+        ws->step = step;   // straight from the caller's arrays
+        return encode_state16(ws, ws::dense_pair(u, u_prev, ws->g));
+    }
     // everything outside the interior is zero from the start and stays so:
     // only a missing level needs its buffer cleared
     const size_t fb = field_bytes(ws->g);

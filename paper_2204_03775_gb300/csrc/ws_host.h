@@ -173,7 +173,10 @@ constexpr int kNumTile16Ys = 2;
 int pick_tile16(const ws_t ws);
 int default_zblock16(const ws::Geom &g, int ty);
 int encode_maps16(ws_t ws, int ty);
+// FP32 levels (by default the handle's buffers) <-> the 16-bit state.
+int encode_state16(ws_t ws, const ws::Fp32Fields &f);
 int encode_state16(ws_t ws);
+int decode_state16(ws_t ws, const ws::Fp32Out &f);
 int decode_state16(ws_t ws);
 // Point sources of step n (amp = h^2 s(t_n)).
 void sources_of_step(const ws_t ws, long long n, ws::Sources *out);

@@ -113,6 +113,33 @@ cudaError_t launch_velocity_to_w(const float *v, float *w, const Geom &g, double
 cudaError_t launch_slowness2_to_w(const float *m, float *w, const Geom &g, double dt_over_h2,
                                   unsigned *extrema, cudaStream_t s);
 
+// Kernels that walk the rows of a grid in vectors of 4 cells: blocks of
+// kRowThreads = block->x threads a row x rows; the number of blocks.
+constexpr int kRowThreads = 256;
+unsigned row_grid(const Geom &g, dim3 *block);
+
+// The two FP32 levels from interior cell (0, 0, 0) on, cell (i, j, k) at
+// k * plane + j * pitch + i; null: zeros (as input), not wanted (as output).
+// vec: every row is readable in whole 16-byte vectors up to its last cell.
+template <class T>
+struct Fp32Pair {
+    T *u, *up;
+    long long pitch, plane;
+    bool vec;
+};
+using Fp32Fields = Fp32Pair<const float>;
+using Fp32Out = Fp32Pair<float>;
+template <class T>
+inline Fp32Pair<T> padded_pair(T *u, T *up, const Geom &g) {
+    const long long o = pidx(g, 0, 0, 0);
+    return {u ? u + o : nullptr, up ? up + o : nullptr, g.pnx, g.plane, true};
+}
+template <class T>
+inline Fp32Pair<T> dense_pair(T *u, T *up, const Geom &g) {
+    const bool al = ((reinterpret_cast<uintptr_t>(u) | reinterpret_cast<uintptr_t>(up)) & 15u) == 0;
+    return {u, up, g.nx, (long long)g.nx * g.ny, g.nx % 4 == 0 && al};
+}
+
 // Unpadded device arrays a, b [nz][ny][nx] -> interiors of the padded fields
 // A, B, and back; b (B for the way out) null: one field. The two outputs must
 // not overlap. Pointers are aligned to 4 bytes.
@@ -200,10 +227,11 @@ cudaError_t launch_step_stream16(int storage, const Maps16In &m, const StepArgs 
                                  long long step, float src_hint, const Free16 &fr,
                                  const StreamTiling &t, const int *rec_ptr, const RecEntry *rec,
                                  cudaStream_t s);
-// FP32 padded (u^n, u^{n-1}) <-> 16-bit padded (U, D) (interior), exponent slot `slot`.
-cudaError_t launch_encode16(int storage, const float *u, const float *up, uint16_t *U, uint16_t *D,
+// FP32 (u^n, u^{n-1}), padded or the caller's, <-> 16-bit padded (U, D)
+// (interior), exponent slot `slot`.
+cudaError_t launch_encode16(int storage, const Fp32Fields &f, uint16_t *U, uint16_t *D,
                             const Geom &g, Scale16 *sc, int slot, cudaStream_t s);
-cudaError_t launch_decode16(int storage, const uint16_t *U, const uint16_t *D, float *u, float *up,
+cudaError_t launch_decode16(int storage, const uint16_t *U, const uint16_t *D, const Fp32Out &f,
                             const Geom &g, const Scale16 *sc, int slot, cudaStream_t s);
 // (V dt/h)^2 (FP32 padded) -> the 16-bit model.
 cudaError_t launch_model16(const float *w, uint16_t *w16, const Geom &g, cudaStream_t s);

@@ -7,12 +7,25 @@
 #include "ws_internal.h"
 
 namespace ws {
-namespace {
 
-constexpr int kCopyThreads = 256;
 // Blocks of a launch: about two full loads of the GPU's 152 x 8 resident
 // blocks; longer copies loop over their rows.
 constexpr int kCopyBlocks = 2432;
+
+// Threads a row: the widest of 32, 16, 8 that leaves the fewest idle.
+unsigned row_grid(const Geom &g, dim3 *block) {
+    const int nq = (g.nx + 3) / 4;
+    int bx = 32;
+    for (int b : {16, 8})
+        if ((nq + b - 1) / b * b < (nq + bx - 1) / bx * bx) bx = b;
+    *block = dim3(bx, kRowThreads / bx);
+    const unsigned long long rows = (unsigned long long)g.ny * g.nz;
+    const unsigned long long want = (rows + block->y - 1) / block->y;
+    return (unsigned)(want < kCopyBlocks ? want : kCopyBlocks);
+}
+
+namespace {
+
 // Vectors of one row that a thread keeps in flight per field: four in rows of
 // whole vectors; one (two loads) in shifted rows, whose 60 registers leave
 // fewer warps (755 x 994 x 400 in 863 us, with two of them 1007).
@@ -79,7 +92,7 @@ __device__ __forceinline__ void store_part(float *p, const float4 &v, int from, 
 // out 754 us (5.6, 6.4 TB/s), against 1166, 1523 us with 4-byte accesses;
 // 1024 x 512 x 512: in 650, out 641 us (6.6, 6.7 TB/s of the measured 6.78).
 template <bool kAligned, bool kIn, int kFields>
-__global__ void __launch_bounds__(kCopyThreads)
+__global__ void __launch_bounds__(kRowThreads)
     copy_rows_kernel(const Fields f, const int nx, const unsigned ny, const unsigned rows,
                      const int pitch, const long long plane, const long long cells) {
     const int step = blockDim.x;
@@ -176,19 +189,6 @@ __global__ void __launch_bounds__(kCopyThreads)
             }
         }
     }
-}
-
-// Blocks and threads of a kernel that walks the grid's rows in vectors of 4
-// cells: threads a row: the widest of 32, 16, 8 that leaves the fewest idle.
-unsigned row_grid(const Geom &g, dim3 *block) {
-    const int nq = (g.nx + 3) / 4;
-    int bx = 32;
-    for (int b : {16, 8})
-        if ((nq + b - 1) / b * b < (nq + bx - 1) / bx * bx) bx = b;
-    *block = dim3(bx, kCopyThreads / bx);
-    const unsigned long long rows = (unsigned long long)g.ny * g.nz;
-    const unsigned long long want = (rows + block->y - 1) / block->y;
-    return (unsigned)(want < kCopyBlocks ? want : kCopyBlocks);
 }
 
 bool aligned16(const void *p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
@@ -318,7 +318,7 @@ __device__ __forceinline__ float convert(float x, const Scale &k, Extrema &e) {
 // (one float division a cell); with the double products issued for every
 // cell 7.8 ms at 1024^3.
 template <class Conv>
-__global__ void __launch_bounds__(kCopyThreads)
+__global__ void __launch_bounds__(kRowThreads)
     model_kernel(const float *src, float *w, const int nx, const unsigned ny, const unsigned rows,
                  const int pitch, const long long plane, const Scale scale,
                  unsigned *__restrict__ extrema) {

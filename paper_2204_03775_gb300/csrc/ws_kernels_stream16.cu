@@ -991,97 +991,217 @@ cudaError_t launch_step_stream16(int storage, const Maps16In &m, const StepArgs 
 }
 
 // ------------------------------------------------------------ conversions
+//
+// Bound: HBM. Every kernel walks the rows (row_grid) in vectors of 4 cells,
+// one 8-byte access a 16-bit field and vector, and reads or writes the
+// caller's unpadded arrays or the padded FP32 fields alike (Fp32Fields). One
+// cell a thread, through the padded fields, with one atomic a warp for the
+// maximum, a 1024^3 state took 32.9 ms in, 6.8 out and its model 4.2; now 1.19
+// (amax2, 7.2 TB/s) + 1.91 (encode, 6.8), 2.10 (decode, 6.1), 0.96 ms.
 
 namespace {
 
-// max |u| and max |u - up| over the interior into *amax (float bits).
-__global__ void amax2_kernel(const float *__restrict__ u, const float *__restrict__ up, Geom g,
-                             unsigned *__restrict__ amax) {
-    const int j = blockIdx.y, k = blockIdx.z;
-    float m = 0.0f;
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < g.nx; i += gridDim.x * blockDim.x) {
-        const long long p = pidx(g, i, j, k);
-        m = fmaxf(m, fmaxf(fabsf(u[p]), fabsf(u[p] - up[p])));
-    }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
-    if ((threadIdx.x & 31) == 0) atomicMax(amax, __float_as_uint(m));
+// Row j of plane k: 4 cells from cell i on, zeros beyond nx or without a field.
+template <bool kVec>
+__device__ __forceinline__ float4 row_load(const float *row, int i, int nx) {
+    float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (!row) return v;
+    if constexpr (kVec) return *reinterpret_cast<const float4 *>(row + i);
+    v.x = row[i];
+    if (i + 1 < nx) v.y = row[i + 1];
+    if (i + 2 < nx) v.z = row[i + 2];
+    if (i + 3 < nx) v.w = row[i + 3];
+    return v;
 }
 
-// FP32 (u^n, u^{n-1}) -> U = u^n, D = u^n - u^{n-1} (16-bit, interior), with
-// the exponent from the maximum of slot `slot`; block (0,0,0) records it.
-template <class Fmt>
-__global__ void encode_kernel(const float *__restrict__ u, const float *__restrict__ up,
-                              uint16_t *__restrict__ U, uint16_t *__restrict__ D, Geom g,
-                              Scale16 *__restrict__ sc, int slot) {
+template <bool kVec>
+__device__ __forceinline__ void row_store(float *row, int i, int nx, const float4 &v) {
+    if (!row) return;
+    if (kVec && i + 4 <= nx) {
+        *reinterpret_cast<float4 *>(row + i) = v;
+        return;
+    }
+    row[i] = v.x;
+    if (i + 1 < nx) row[i + 1] = v.y;
+    if (i + 2 < nx) row[i + 2] = v.z;
+    if (i + 3 < nx) row[i + 3] = v.w;
+}
+
+// 4 packed 16-bit values to cells i .. of a padded row, none beyond nx.
+__device__ __forceinline__ void row_store16(uint16_t *row, int i, int nx, uint2 v) {
+    if (i + 4 <= nx) {
+        *reinterpret_cast<uint2 *>(row + i) = v;
+        return;
+    }
+    row[i] = (uint16_t)(v.x & 0xffffu);
+    if (i + 1 < nx) row[i + 1] = (uint16_t)(v.x >> 16);
+    if (i + 2 < nx) row[i + 2] = (uint16_t)(v.y & 0xffffu);
+}
+
+// This thread group's rows: calls fn(k, j) for each.
+template <class F>
+__device__ __forceinline__ void for_rows(unsigned ny, unsigned rows, F &&fn) {
+    for (unsigned long long r = (unsigned long long)blockIdx.x * blockDim.y + threadIdx.y; r < rows;
+         r += (unsigned long long)gridDim.x * blockDim.y) {
+        const unsigned k = (unsigned)r / ny;
+        fn(k, (unsigned)r - k * ny);
+    }
+}
+
+__device__ __forceinline__ float amax_of(const float4 &u, const float4 &p) {
+    const float a = fmaxf(fmaxf(fabsf(u.x), fabsf(u.y)), fmaxf(fabsf(u.z), fabsf(u.w)));
+    const float d = fmaxf(fmaxf(fabsf(u.x - p.x), fabsf(u.y - p.y)),
+                          fmaxf(fabsf(u.z - p.z), fabsf(u.w - p.w)));
+    return fmaxf(a, d);
+}
+
+// max |u| and max |u - up| over the grid into *amax (float bits).
+template <bool kVec>
+__global__ void __launch_bounds__(kRowThreads)
+    amax2_kernel(const Fp32Fields f, const int nx, const unsigned ny, const unsigned rows,
+                 unsigned *__restrict__ amax) {
+    float m = 0.0f;
+    const int step = 4 * blockDim.x;
+    for_rows(ny, rows, [&](unsigned k, unsigned j) {
+        const long long o = k * f.plane + (long long)j * f.pitch;
+        const float *u = f.u ? f.u + o : nullptr, *p = f.up ? f.up + o : nullptr;
+        for (int i = 4 * threadIdx.x; i < nx; i += 2 * step) {
+            const int i2 = i + step < nx ? i + step : i;   // two vectors in flight
+            const float4 u0 = row_load<kVec>(u, i, nx), u1 = row_load<kVec>(u, i2, nx);
+            const float4 p0 = row_load<kVec>(p, i, nx), p1 = row_load<kVec>(p, i2, nx);
+            m = fmaxf(m, fmaxf(amax_of(u0, p0), amax_of(u1, p1)));
+        }
+    });
+    __shared__ unsigned best;
+    const int tid = threadIdx.y * blockDim.x + threadIdx.x;
+    if (tid == 0) best = 0u;
+    __syncthreads();
+    const unsigned w = __reduce_max_sync(0xffffffffu, __float_as_uint(m));   // m >= 0
+    if ((tid & 31) == 0) atomicMax(&best, w);
+    __syncthreads();
+    if (tid == 0) atomicMax(amax, best);
+}
+
+__device__ __forceinline__ float4 scale4(const float4 &x, float f0, float f1) {
+    return make_float4(x.x * f0 * f1, x.y * f0 * f1, x.z * f0 * f1, x.w * f0 * f1);
+}
+
+// FP32 (u^n, u^{n-1}) -> U = u^n, D = u^n - u^{n-1} (16-bit, interior; U and D
+// at interior cell 0), with the exponent from the maximum of slot `slot`;
+// block 0 records it.
+template <class Fmt, bool kVec>
+__global__ void __launch_bounds__(kRowThreads)
+    encode_kernel(const Fp32Fields f, uint16_t *__restrict__ U, uint16_t *__restrict__ D,
+                  const int nx, const unsigned ny, const unsigned rows, const int pitch,
+                  const long long plane, Scale16 *__restrict__ sc, int slot) {
     const int e = scale_exponent(__uint_as_float(sc->amax[slot]));
-    const int j = blockIdx.y, k = blockIdx.z;
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (blockIdx.x == 0 && j == 0 && k == 0 && threadIdx.x == 0) sc->e[slot] = e;
-    if (i >= g.nx) return;
-    const long long p = pidx(g, i, j, k);
-    const uint2 v = Fmt::encode(make_float4(scale2(u[p], e), scale2(u[p] - up[p], e), 0.f, 0.f));
-    U[p] = (uint16_t)(v.x & 0xffffu);
-    D[p] = (uint16_t)(v.x >> 16);
+    const float f0 = pow2f(e / 2), f1 = pow2f(e - e / 2);   // the factors of scale2
+    if (blockIdx.x == 0 && threadIdx.x == 0 && threadIdx.y == 0) sc->e[slot] = e;
+    for_rows(ny, rows, [&](unsigned k, unsigned j) {
+        const long long o = k * f.plane + (long long)j * f.pitch;
+        const float *u = f.u ? f.u + o : nullptr, *p = f.up ? f.up + o : nullptr;
+        const long long q = k * plane + (long long)j * pitch;
+        for (int i = 4 * threadIdx.x; i < nx; i += 4 * blockDim.x) {
+            const float4 a = row_load<kVec>(u, i, nx), b = row_load<kVec>(p, i, nx);
+            const float4 d = make_float4(a.x - b.x, a.y - b.y, a.z - b.z, a.w - b.w);
+            row_store16(U + q, i, nx, Fmt::encode(scale4(a, f0, f1)));
+            row_store16(D + q, i, nx, Fmt::encode(scale4(d, f0, f1)));
+        }
+    });
 }
 
 // U, D (16-bit) -> FP32 u^n = U, u^{n-1} = U - D (interior).
-template <class Fmt>
-__global__ void decode_kernel(const uint16_t *__restrict__ U, const uint16_t *__restrict__ D,
-                              float *__restrict__ u, float *__restrict__ up, Geom g,
-                              const Scale16 *__restrict__ sc, int slot) {
-    const int j = blockIdx.y, k = blockIdx.z;
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= g.nx) return;
-    const long long p = pidx(g, i, j, k);
-    const float4 v = Fmt::decode(make_uint2((unsigned)U[p] | ((unsigned)D[p] << 16), 0u));
-    const float un = scale2(v.x, -sc->e[slot]);
-    const float dn = scale2(v.y, -sc->e[slot]);
-    u[p] = un;
-    up[p] = un - dn;
+template <class Fmt, bool kVec>
+__global__ void __launch_bounds__(kRowThreads)
+    decode_kernel(const uint16_t *__restrict__ U, const uint16_t *__restrict__ D, const Fp32Out f,
+                  const int nx, const unsigned ny, const unsigned rows, const int pitch,
+                  const long long plane, const Scale16 *__restrict__ sc, int slot) {
+    const int e = -sc->e[slot];
+    const float f0 = pow2f(e / 2), f1 = pow2f(e - e / 2);
+    for_rows(ny, rows, [&](unsigned k, unsigned j) {
+        const long long o = k * f.plane + (long long)j * f.pitch;
+        float *u = f.u ? f.u + o : nullptr, *p = f.up ? f.up + o : nullptr;
+        const long long q = k * plane + (long long)j * pitch;
+        for (int i = 4 * threadIdx.x; i < nx; i += 4 * blockDim.x) {
+            // a ragged row's last vector reaches into its halo
+            const float4 a = scale4(Fmt::decode(*reinterpret_cast<const uint2 *>(U + q + i)), f0, f1);
+            const float4 d = scale4(Fmt::decode(*reinterpret_cast<const uint2 *>(D + q + i)), f0, f1);
+            row_store<kVec>(u, i, nx, a);
+            row_store<kVec>(p, i, nx, make_float4(a.x - d.x, a.y - d.y, a.z - d.z, a.w - d.w));
+        }
+    });
 }
 
-// (V dt/h)^2 (FP32 padded) -> FP16 of value * 2^kW16Exp (interior).
-__global__ void model16_kernel(const float *__restrict__ w, uint16_t *__restrict__ w16, Geom g) {
-    const int j = blockIdx.y, k = blockIdx.z;
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= g.nx) return;
-    const long long p = pidx(g, i, j, k);
-    unsigned short h;
-    asm("cvt.rn.f16.f32 %0, %1;" : "=h"(h) : "f"(w[p] * (float)(1 << kW16Exp)));
-    w16[p] = h;
+// (V dt/h)^2 (FP32 padded) -> FP16 of value * 2^kW16Exp (interior; both at
+// interior cell 0).
+__global__ void __launch_bounds__(kRowThreads)
+    model16_kernel(const float *__restrict__ w, uint16_t *__restrict__ w16, const int nx,
+                   const unsigned ny, const unsigned rows, const int pitch, const long long plane) {
+    for_rows(ny, rows, [&](unsigned k, unsigned j) {
+        const long long q = k * plane + (long long)j * pitch;
+        for (int i = 4 * threadIdx.x; i < nx; i += 4 * blockDim.x) {
+            const float4 v = *reinterpret_cast<const float4 *>(w + q + i);
+            row_store16(w16 + q, i, nx, Fp16Fmt::encode(mul4(v, (float)(1 << kW16Exp))));
+        }
+    });
 }
 
 }  // namespace
 
-cudaError_t launch_encode16(int storage, const float *u, const float *up, uint16_t *U, uint16_t *D,
+cudaError_t launch_encode16(int storage, const Fp32Fields &f, uint16_t *U, uint16_t *D,
                             const Geom &g, Scale16 *sc, int slot, cudaStream_t s) {
     cudaError_t e = cudaMemsetAsync(&sc->amax[slot], 0, sizeof(unsigned), s);
     if (e != cudaSuccess) return e;
-    amax2_kernel<<<dim3((g.nx + 255) / 256, g.ny, g.nz), 256, 0, s>>>(u, up, g, &sc->amax[slot]);
+    const unsigned rows = (unsigned)g.ny * (unsigned)g.nz;
+    const long long o = pidx(g, 0, 0, 0);
+    dim3 block;
+    const unsigned grid = row_grid(g, &block);
+    if (f.vec)
+        amax2_kernel<true><<<grid, block, 0, s>>>(f, g.nx, g.ny, rows, &sc->amax[slot]);
+    else
+        amax2_kernel<false><<<grid, block, 0, s>>>(f, g.nx, g.ny, rows, &sc->amax[slot]);
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    dim3 grid((g.nx + 127) / 128, g.ny, g.nz);
-    if (storage == WS_STORAGE_BF16)
-        encode_kernel<Bf16Fmt><<<grid, 128, 0, s>>>(u, up, U, D, g, sc, slot);
-    else
-        encode_kernel<Fp16Fmt><<<grid, 128, 0, s>>>(u, up, U, D, g, sc, slot);
+#define WS_ENCODE(FMT, V)                                                                       \
+    encode_kernel<FMT, V><<<grid, block, 0, s>>>(f, U + o, D + o, g.nx, g.ny, rows, g.pnx, \
+                                                 g.plane, sc, slot)
+    if (storage == WS_STORAGE_BF16) {
+        if (f.vec) WS_ENCODE(Bf16Fmt, true);
+        else WS_ENCODE(Bf16Fmt, false);
+    } else {
+        if (f.vec) WS_ENCODE(Fp16Fmt, true);
+        else WS_ENCODE(Fp16Fmt, false);
+    }
+#undef WS_ENCODE
     return cudaGetLastError();
 }
 
-cudaError_t launch_decode16(int storage, const uint16_t *U, const uint16_t *D, float *u, float *up,
+cudaError_t launch_decode16(int storage, const uint16_t *U, const uint16_t *D, const Fp32Out &f,
                             const Geom &g, const Scale16 *sc, int slot, cudaStream_t s) {
-    dim3 grid((g.nx + 127) / 128, g.ny, g.nz);
-    if (storage == WS_STORAGE_BF16)
-        decode_kernel<Bf16Fmt><<<grid, 128, 0, s>>>(U, D, u, up, g, sc, slot);
-    else
-        decode_kernel<Fp16Fmt><<<grid, 128, 0, s>>>(U, D, u, up, g, sc, slot);
+    const unsigned rows = (unsigned)g.ny * (unsigned)g.nz;
+    const long long o = pidx(g, 0, 0, 0);
+    dim3 block;
+    const unsigned grid = row_grid(g, &block);
+#define WS_DECODE(FMT, V)                                                                       \
+    decode_kernel<FMT, V><<<grid, block, 0, s>>>(U + o, D + o, f, g.nx, g.ny, rows, g.pnx, \
+                                                 g.plane, sc, slot)
+    if (storage == WS_STORAGE_BF16) {
+        if (f.vec) WS_DECODE(Bf16Fmt, true);
+        else WS_DECODE(Bf16Fmt, false);
+    } else {
+        if (f.vec) WS_DECODE(Fp16Fmt, true);
+        else WS_DECODE(Fp16Fmt, false);
+    }
+#undef WS_DECODE
     return cudaGetLastError();
 }
 
 cudaError_t launch_model16(const float *w, uint16_t *w16, const Geom &g, cudaStream_t s) {
-    dim3 grid((g.nx + 127) / 128, g.ny, g.nz);
-    model16_kernel<<<grid, 128, 0, s>>>(w, w16, g);
+    const long long o = pidx(g, 0, 0, 0);
+    dim3 block;
+    const unsigned grid = row_grid(g, &block);
+    model16_kernel<<<grid, block, 0, s>>>(w + o, w16 + o, g.nx, g.ny,
+                                          (unsigned)g.ny * (unsigned)g.nz, g.pnx, g.plane);
     return cudaGetLastError();
 }
 

@@ -103,3 +103,33 @@ def test_model_is_the_rounded_double(slowness, nx, offset):
         bad[nz // 2, 0, nx - 1] = np.nan
         with pytest.raises(wsb.WaveStepError):
             setter(h, device_copy(bad, offset) if on_device else bad)
+
+
+@pytest.mark.parametrize("storage", [wsb.WS_STORAGE_FP16, wsb.WS_STORAGE_BF16])
+@pytest.mark.parametrize("nx,offset", [(64, 0), (64, 1), (67, 0), (130, 2), (101, 3)])
+def test_16bit_state_of_device_and_host_arrays(storage, nx, offset):
+    """The 16-bit state made from device arrays is the one made from host
+    arrays, and comes back alike to both; a missing level counts as zero."""
+    shape = (5, 17, nx)
+    nz, ny, _ = shape
+    rng = np.random.default_rng(nx)
+    u, p = (rng.standard_normal(shape).astype(np.float32) * 0.3 for _ in range(2))
+    h = wsb.ws_create(nx, ny, nz, 10.0, 1e-3)
+    wsb.ws_set_storage(h, storage)
+    wsb.ws_test_fill_padding(h)
+    du, dp = device_copy(u, offset), device_copy(p, offset)
+    zero = np.zeros(shape, np.float32)
+    for first, second, hf, hs in ((du, dp, u, p), (du, None, u, zero), (None, dp, zero, p)):
+        wsb.ws_write_field(h, hf, hs, 5)
+        wsb.ws_test_fill_padding(h)
+        ref = wsb.ws_read_field(h)
+        assert np.abs(ref[0] - hf).max() < 4e-3
+        wsb.ws_write_field(h, first, second, 6)
+        got = wsb.ws_read_field(h)
+        ou, op = (device_copy(np.full(shape, 7, np.float32), offset) for _ in range(2))
+        wsb.ws_read_field(h, ou, op)
+        for r, g, o in zip(ref, got, (ou, op)):
+            assert np.array_equal(r, g) and np.array_equal(r, o.cpu().numpy())
+        wsb.ws_read_field(h, ou, ou)
+        assert np.array_equal(ou.cpu().numpy(), ref[1])
+        assert wsb.ws_test_check_padding(h) == 0
