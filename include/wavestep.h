@@ -54,7 +54,7 @@ extern "C" {
 #define WS_ERR_STATE    -6  /* call not valid in the handle's current state */
 
 /* Step kernels selectable with ws_set_kernel. */
-#define WS_KERNEL_AUTO    0  /* the streaming kernel when the grid fits its tile, else DIRECT */
+#define WS_KERNEL_AUTO    0  /* the streaming kernel when the grid fits its tile and is not tiny, else DIRECT */
 #define WS_KERNEL_DIRECT  1  /* one thread per cell, neighbours loaded from global memory */
 #define WS_KERNEL_STREAM  2  /* z-streaming: TMA rings + 9-plane register queue, one CTA per item */
 
@@ -288,20 +288,22 @@ int ws_set_storage(ws_t ws, int storage);
 
 /* Choose the step kernel (WS_KERNEL_*) and, for WS_KERNEL_STREAM, its tile:
  * tile_x x tile_y in {32x8, 32x16, 64x8, 64x16, 64x32} for the FP32 kernel
- * (0, 0 = keep the current tile; the default is 64x8) or in {64x16, 64x24,
- * 64x48} for the 16-bit kernel (64x16 selects both; a 16-bit tile leaves the
- * FP32 tile unchanged and needs nx >= 64 and ny >= tile_y), zblock >= 1 planes
- * per work item (0 = default: blocks of about 200 planes with a last block
- * about a quarter as long, so that the last items of a launch are short;
- * fewer planes on small grids).
- * WS_KERNEL_STREAM needs nx >= tile_x and ny >= tile_y; else BADARG. */
+ * (0, 0 = keep the chosen tile; while none is chosen the step takes 64x16, or
+ * 32x16 where 64-cell tiles would be mostly empty, or 8 rows on low grids, and
+ * AUTO runs grids of at most 200000 cells with the direct kernel) or in {64x16,
+ * 64x24, 64x48} for the 16-bit kernel (64x16 selects both; a 16-bit tile leaves
+ * the FP32 tile unchanged and needs nx >= 64 and ny >= tile_y), zblock >= 1
+ * planes per work item (0 = default: for FP32 the block whose waves of resident
+ * CTAs are estimated to finish first; for 16-bit storage blocks of about 200
+ * planes with a last block about a quarter as long, fewer on small grids).
+ * WS_KERNEL_STREAM needs nx >= tile_x and ny >= tile_y (64 x 8 while no tile is
+ * chosen); else BADARG. */
 int ws_set_kernel(ws_t ws, int kernel, int tile_x, int tile_y, int zblock);
 
 /* Pick the streaming kernel's tile and z-block for this handle's grid by
- * timing the candidates (every tile of 64x8, 32x8, 32x16 that fits: 64x16
- * and 64x32 hold too few registers per thread and are never faster; z-blocks giving the default
- * length and item counts just below and just above 1 .. 8 waves of the
- * resident CTAs) on
+ * timing the candidates (every tile of 64x16, 32x16, 64x8, 32x8 that fits;
+ * z-blocks giving the default length and item counts just below and just above
+ * 1 .. 8 waves of the resident CTAs) on
  * steps written to a scratch field, so the state is unchanged; then select
  * WS_KERNEL_STREAM with the fastest (WS_KERNEL_DIRECT if no tile fits).
  * Results are cached by (GPU name, storage, nx, ny, nz) in the process and

@@ -117,24 +117,90 @@ int default_zblock(int nz) {
     return (4 * nz + 4 * blocks - 4) / (4 * blocks - 3);   // ceil(nz / (blocks - 3/4))
 }
 
-// The default, shortened on small grids to about two full waves of items
-// over the resident CTAs (a 256^3 grid in 64 x 8 tiles has 128 tiles for 456
-// CTAs: one 256-plane block per tile ran at 139 Gcell/s, short blocks at
-// more than twice that); the count is rounded down so the last wave is full.
+// The FP32 streaming kernel's default for a grid and tile: the z block of the
+// smallest estimated step, in units of one plane of a full SM (about 1 us for
+// 64 x 16 tiles). An item of p planes takes kItem + p on a full SM; a CTA alone
+// on its SM walks a plane in kAlone of that, in between it is interpolated.
+//  - Up to kWaves waves of resident CTAs: the waves one after the other, the
+//    last one at the speed of its fewer CTAs. Small grids end up with one or
+//    two nearly full waves: 192 x 160 x 144 in 64 x 16 tiles, 10-plane blocks
+//    (0.99 of a wave) 13.1 us, 8 (1.2 waves) 17.0, 5 (1.9) 14.2; 128^3 5-plane
+//    blocks 7.9 us, the former 8-plane minimum 10.5.
+//  - More waves blur into one another: the work divided by the CTAs, and a
+//    tail that grows with the length of the last items. Blocks are also tried
+//    with a last one about a quarter as long, so that a launch ends on short
+//    items (755 x 994 x 200: blocks of 160 and 40 planes 369 us, of 67 376;
+//    384^3: 128 147 us, 96 195).
+// Over 33 grids of 16 thousand to 270 million cells the chosen block was within
+// 2 % (geometric mean) of the best of any tile and block. At least 2 planes
+// (fewer only repeat the 8-plane prologue), at most 256.
 int default_zblock(const ws::Geom &g, int tx, int ty) {
-    int zb = default_zblock(g.nz), slots = 0;
-    if (ws::stream_slots(tx, ty, false, &slots) != cudaSuccess) return zb;
+    constexpr double kItem = 2.5, kAlone = 0.62, kWaves = 3.0, kTail = 0.2;
+    constexpr int kMin = 2, kMax = 256;
+    int slots = 0, sms = 0;
+    if (ws::stream_slots(tx, ty, false, &slots, &sms) != cudaSuccess || g.nz <= kMin)
+        return default_zblock(g.nz);
+    const int ctas = slots / sms;
     const long long tiles = (long long)((g.nx + tx - 1) / tx) * ((g.ny + ty - 1) / ty);
-    const long long blocks = std::max<long long>(1, 2LL * slots / tiles);
-    const int zs = (int)std::max<long long>(8, (g.nz + blocks - 1) / blocks);
-    return std::min(zb, std::min(zs, g.nz));
+    auto cost = [&](int zb) {
+        const long long blocks = (g.nz + zb - 1) / zb, n = tiles * blocks;
+        const int last = g.nz - (int)(blocks - 1) * zb;
+        if (n > kWaves * slots)
+            return tiles * (blocks * kItem + g.nz) / slots +
+                   kTail * (kItem + (tiles >= slots / 2 ? last : zb));
+        const long long full = n / slots, rem = n % slots;
+        if (rem == 0) return full * (kItem + zb) - (tiles >= slots ? zb - last : 0);
+        const double share = ctas > 1 ? double((rem + sms - 1) / sms - 1) / (ctas - 1) : 1.0;
+        return full * (kItem + zb) + kItem +
+               (rem <= tiles ? last : zb) * (kAlone + (1.0 - kAlone) * share);
+    };
+    int best = 0;
+    double best_cost = 0.0;
+    auto consider = [&](int zb) {
+        if (zb < kMin || zb > kMax || zb > g.nz) return;
+        const double c = cost(zb);
+        if (best == 0 || c < best_cost - 1e-9) {
+            best = zb;
+            best_cost = c;
+        }
+    };
+    for (int b = 1, zb; (zb = (g.nz + b - 1) / b) >= kMin; ++b) {
+        if (b > 1) consider((4 * g.nz + 4 * b - 4) / (4 * b - 3));   // the last a quarter as long
+        consider(zb);
+        if (zb == kMin) break;
+    }
+    return best > 0 ? best : std::min(g.nz, kMax);
+}
+
+// The tile of a grid for which none was chosen: 64 x 16 is the fastest, 32 x 16
+// takes about 1.2 times as long per cell of its tiles (256^3 52.3 against 47.7
+// us), so it is taken where 64-wide tiles would be emptier than that (70 x 900
+// x 300: 73 against 82 us; 221 x 293 x 338 stays at 64: 63 against 67). Low
+// grids get 8-row tiles. False if no tile fits.
+bool default_tile(const ws::Geom &g, ws::StreamTiling *t) {
+    if (g.nx < 32 || g.ny < 8) return false;
+    t->ty = g.ny >= 16 ? 16 : 8;
+    const int w64 = (g.nx + 63) / 64 * 64, w32 = (g.nx + 31) / 32 * 32;
+    t->tx = g.nx >= 64 && 5 * w64 <= 6 * w32 ? 64 : 32;
+    return true;
 }
 
 // Choose the kernel for the next steps; fills *tiling for the streaming one.
+// Grids of at most kDirectCells cells, left to choose by themselves, take the
+// direct kernel: 101 x 37 x 45 in 2.9 us a step against 3.5 in stream tiles,
+// 48 x 40 x 40 2.3 against 3.4, 191 x 25 x 43 (205 thousand cells) 3.4 either
+// way, 64^3 3.5 against 3.3, 138 x 55 x 138 9.2 against 7.1.
 int pick_kernel(ws_t ws, ws::StreamTiling *tiling) {
+    constexpr long long kDirectCells = 200000;
     if (ws->kernel == WS_KERNEL_DIRECT) return WS_KERNEL_DIRECT;
+    const ws::Geom &g = ws->g;
     ws::StreamTiling t = ws->tiling;
-    if (ws->kernel == WS_KERNEL_AUTO && !stream_fits(ws, t)) {
+    if (!ws->tile_chosen) {
+        const bool automatic = ws->kernel == WS_KERNEL_AUTO;
+        if (!default_tile(g, &t)) return WS_KERNEL_DIRECT;   // AUTO only: STREAM needs 64 x 8
+        if (automatic && t.zb <= 0 && (long long)g.nx * g.ny * g.nz <= kDirectCells)
+            return WS_KERNEL_DIRECT;
+    } else if (ws->kernel == WS_KERNEL_AUTO && !stream_fits(ws, t)) {
         const ws::StreamTiling cands[3] = {{32, 16, 0}, {32, 8, 0}, {64, 16, 0}};
         bool found = false;
         for (const auto &c : cands)
@@ -146,41 +212,48 @@ int pick_kernel(ws_t ws, ws::StreamTiling *tiling) {
             }
         if (!found) return WS_KERNEL_DIRECT;
     }
-    if (t.zb <= 0) t.zb = default_zblock(ws->g, t.tx, t.ty);
+    if (t.zb <= 0) {
+        if (ws->auto_zb.tx != t.tx || ws->auto_zb.ty != t.ty)
+            ws->auto_zb = ws::StreamTiling{t.tx, t.ty, default_zblock(g, t.tx, t.ty)};
+        t.zb = ws->auto_zb.zb;
+    }
     *tiling = t;
     return WS_KERNEL_STREAM;
 }
 
 void free_receivers(ws_t ws) {
     cudaFree(ws->traces);
-    cudaFree(ws->rec_pidx);
     cudaFree(ws->rec_ptr);
     cudaFree(ws->rec_entries);
     ws->traces = nullptr;
-    ws->rec_pidx = nullptr;
     ws->rec_ptr = nullptr;
     ws->rec_entries = nullptr;
-    ws->rec_tiling_tx = ws->rec_tiling_ty = ws->rec_tiling_rows = 0;
+    ws->rec_tiling_tx = ws->rec_tiling_ty = 0;
 }
 
-// Receiver table of the streaming kernels for tile t: per (tile, consumer
-// warp) a range of entries sorted by k. Thread owner = (row pair) * tx/4 + x
-// quad, lane = 4 * (row within the thread's rows) + x cell.
-int build_rec_tiles(ws_t ws, const ws::StreamTiling &t, int rows) {
+// Receiver table for tile t. Streaming kernels: per (tile, warp) a range of
+// entries sorted by k; thread owner = (row pair) * tx/4 + x quad, lane = 4 *
+// (row of the pair) + x cell. Direct kernel (direct): per tile, owner = row,
+// lane = x cell.
+int build_rec_tiles(ws_t ws, const ws::StreamTiling &t, bool direct) {
     if (ws->nrec == 0) return WS_OK;
-    if (ws->rec_tiling_tx == t.tx && ws->rec_tiling_ty == t.ty && ws->rec_tiling_rows == rows)
+    if (ws->rec_tiling_tx == t.tx && ws->rec_tiling_ty == t.ty && ws->rec_direct == direct)
         return WS_OK;
     const int tiles_x = (ws->g.nx + t.tx - 1) / t.tx;
     const int tiles_y = (ws->g.ny + t.ty - 1) / t.ty;
-    const int warps = t.tx / 4 * (t.ty / rows) / 32;   // consumer warps of a CTA
+    const int warps = direct ? 1 : t.tx / 4 * (t.ty / 2) / 32;
     const int ntiles = tiles_x * tiles_y * warps;   // (tile, warp) ranges
     std::vector<std::pair<int, ws::RecEntry>> e(ws->nrec);
     for (int r = 0; r < ws->nrec; ++r) {
         const int i = ws->rec_ijk[3 * r], j = ws->rec_ijk[3 * r + 1], k = ws->rec_ijk[3 * r + 2];
         const int tile = (j / t.ty) * tiles_x + (i / t.tx);
         const int li = i - (i / t.tx) * t.tx, lj = j - (j / t.ty) * t.ty;
-        const int owner = (lj / rows) * (t.tx / 4) + li / 4;
-        e[r] = {tile * warps + owner / 32, ws::RecEntry{k, owner, (lj % rows) * 4 + li % 4, r}};
+        if (direct) {
+            e[r] = {tile, ws::RecEntry{k, lj, li, r}};
+            continue;
+        }
+        const int owner = (lj / 2) * (t.tx / 4) + li / 4;
+        e[r] = {tile * warps + owner / 32, ws::RecEntry{k, owner, (lj % 2) * 4 + li % 4, r}};
     }
     std::stable_sort(e.begin(), e.end(), [](const auto &x, const auto &y) {
         return x.first != y.first ? x.first < y.first : x.second.k < y.second.k;
@@ -209,7 +282,7 @@ int build_rec_tiles(ws_t ws, const ws::StreamTiling &t, int rows) {
     WS_CUDA(cudaStreamSynchronize(ws->stream), "upload receiver table");
     ws->rec_tiling_tx = t.tx;
     ws->rec_tiling_ty = t.ty;
-    ws->rec_tiling_rows = rows;
+    ws->rec_direct = direct;
     return WS_OK;
 }
 
@@ -275,9 +348,9 @@ int upload_profiles(ws_t ws) {
         *lo = a;
         *hi = b;
     };
-    ones(px, &ws->free16.x0, &ws->free16.x1);
-    ones(py, &ws->free16.y0, &ws->free16.y1);
-    ones(pz, &ws->free16.z0, &ws->free16.z1);
+    ones(px, &ws->free_box.x0, &ws->free_box.x1);
+    ones(py, &ws->free_box.y0, &ws->free_box.y1);
+    ones(pz, &ws->free_box.z0, &ws->free_box.z1);
     WS_CUDA(cudaMemcpyAsync(ws->gx, px.data(), 4 * px.size(), cudaMemcpyHostToDevice, ws->stream),
             "upload taper");
     WS_CUDA(cudaMemcpyAsync(ws->gy, py.data(), 4 * py.size(), cudaMemcpyHostToDevice, ws->stream),
@@ -375,6 +448,7 @@ ws::StepArgs base_args(const ws_t ws) {
     a.gx = ws->gx;
     a.gy = ws->gy;
     a.gz = ws->gz;
+    a.fr = ws->free_box;
     a.traces = ws->traces;
     a.nt_max = ws->nt_max;
     a.status = ws->status;
@@ -395,17 +469,13 @@ int step_fp32(ws_t ws, ws::StepArgs &a, int kern, const ws::StreamTiling &tiling
     a.trace_step = n - ws->trace_start;
     cudaError_t e;
     if (kern == WS_KERNEL_STREAM) {
-        e = ws::launch_step_stream(un_halo, unm1_tile, &ws->tmap_w, out, a, tiling,
+        e = ws::launch_step_stream(un_halo, unm1_tile, &ws->tmap_w, un, out, a, tiling,
                                    record ? ws->rec_ptr : nullptr, ws->rec_entries, ws->stream);
         ws->launches++;
     } else {
-        e = ws::launch_step_direct(un, unm1, out, ws->w, a, ws->stream);
+        e = ws::launch_step_direct(un, unm1, out, ws->w, a, record ? ws->rec_ptr : nullptr,
+                                   ws->rec_entries, ws->stream);
         ws->launches++;
-        if (e == cudaSuccess && record) {
-            e = ws::launch_gather_receivers(out, ws->rec_pidx, ws->nrec, ws->traces, ws->nt_max,
-                                            a.trace_step, ws->stream);
-            ws->launches++;
-        }
     }
     if (e != cudaSuccess) return cuda_fail(e, "step launch");
     return WS_OK;
@@ -415,7 +485,8 @@ int step_fp32(ws_t ws, ws::StepArgs &a, int kern, const ws::StreamTiling &tiling
 // the receiver table in line with its tiling.
 int prepare_fp32(ws_t ws, int *kern, ws::StreamTiling *tiling) {
     *kern = pick_kernel(ws, tiling);
-    if (*kern != WS_KERNEL_STREAM) return WS_OK;
+    if (*kern != WS_KERNEL_STREAM)
+        return build_rec_tiles(ws, ws::StreamTiling{ws::kDirectX, ws::kDirectY, 0}, true);
     if (tiling->tx != ws->tiling.tx || tiling->ty != ws->tiling.ty) {
         ws->tiling.tx = tiling->tx;
         ws->tiling.ty = tiling->ty;
@@ -706,13 +777,6 @@ int ws_set_receivers(ws_t ws, int nrec, const int *ijk, int nt_max) {
     WS_CUDA(cudaMalloc(&ws->traces, sizeof(float) * size_t(nrec) * nt_max), "cudaMalloc traces");
     WS_CUDA(cudaMemsetAsync(ws->traces, 0, sizeof(float) * size_t(nrec) * nt_max, ws->stream),
             "zero traces");
-    std::vector<long long> pid(nrec);
-    for (int r = 0; r < nrec; ++r) pid[r] = ws::pidx(g, ijk[3 * r], ijk[3 * r + 1], ijk[3 * r + 2]);
-    WS_CUDA(cudaMalloc(&ws->rec_pidx, sizeof(long long) * nrec), "cudaMalloc receivers");
-    WS_CUDA(cudaMemcpyAsync(ws->rec_pidx, pid.data(), sizeof(long long) * nrec,
-                            cudaMemcpyHostToDevice, ws->stream),
-            "upload receivers");
-    WS_CUDA(cudaStreamSynchronize(ws->stream), "upload receivers");
     ws->nrec = nrec;
     ws->nt_max = nt_max;
     return WS_OK;
@@ -761,7 +825,10 @@ int ws_set_kernel(ws_t ws, int kernel, int tile_x, int tile_y, int zblock) {
     if (kernel != WS_KERNEL_AUTO && kernel != WS_KERNEL_DIRECT && kernel != WS_KERNEL_STREAM)
         return fail(WS_ERR_BADARG, "ws_set_kernel: unknown kernel %d", kernel);
     if (zblock < 0) return fail(WS_ERR_BADARG, "ws_set_kernel: zblock must be >= 0");
-    ws::StreamTiling t = ws->tiling;
+    // the streaming tile that must fit: the chosen one, else 64 x 8 (the
+    // smallest that a default may come down to)
+    ws::StreamTiling t = ws->tile_chosen ? ws->tiling : ws::StreamTiling{64, 8, 0};
+    bool chosen = ws->tile_chosen;
     if (tile_x != 0 || tile_y != 0) {
         const bool fp32 = ws::stream_tiling_supported(tile_x, tile_y);
         const bool t16 = ws::stream16_tiling_supported(tile_x, tile_y);
@@ -777,15 +844,19 @@ int ws_set_kernel(ws_t ws, int kernel, int tile_x, int tile_y, int zblock) {
         if (fp32) {
             t.tx = tile_x;
             t.ty = tile_y;
+            chosen = true;
         }
     }
     t.zb = zblock;
     if (kernel == WS_KERNEL_STREAM && !stream_fits(ws, t))
         return fail(WS_ERR_BADARG, "ws_set_kernel: grid %d x %d is smaller than the tile %d x %d",
                     ws->g.nx, ws->g.ny, t.tx, t.ty);
-    const bool box_changed = t.tx != ws->tiling.tx || t.ty != ws->tiling.ty;
     ws->kernel = kernel;
+    ws->tiling.zb = zblock;
+    if (!chosen) return WS_OK;   // the step picks the tile
+    const bool box_changed = t.tx != ws->tiling.tx || t.ty != ws->tiling.ty;
     ws->tiling = t;
+    ws->tile_chosen = true;
     if (box_changed) return encode_maps(ws);
     return WS_OK;
 }
@@ -812,7 +883,7 @@ int ws_step(ws_t ws, int nsteps) {
             int rc = encode_maps16(ws, tiling.ty);
             if (rc != WS_OK) return rc;
         }
-        int rc = build_rec_tiles(ws, tiling, kRows16);
+        int rc = build_rec_tiles(ws, tiling);
         if (rc != WS_OK) return rc;
         if (!ws->w16_ok) {
             WS_CUDA(ws::launch_model16(ws->w, ws->w16, ws->g, ws->stream), "16-bit model");
@@ -836,7 +907,7 @@ int ws_step(ws_t ws, int nsteps) {
             const ws::Maps16In maps{&ws->t16_halo[ws->cur], &ws->t16_d, &ws->t16_w,
                                     ws->buf16[1 - ws->cur], ws->d16};
             cudaError_t e = ws::launch_step_stream16(
-                ws->storage, maps, a, ws->scale, ws->step, (float)hint, ws->free16, tiling,
+                ws->storage, maps, a, ws->scale, ws->step, (float)hint, tiling,
                 ws->nrec > 0 ? ws->rec_ptr : nullptr, ws->rec_entries, ws->stream);
             a.stall_item = -1;
             ws->launches++;

@@ -34,6 +34,7 @@ struct ws_batch {
     std::vector<Cand> todo;
     bool tuned = false, fixed = false;
     Cand best{0, 0, 0};
+    Cand untuned{0, 0, 2};             // before any candidate is timed
     Cand cfg{0, 0, -1};                // what the item table was built for
     float best_ms = 1e30f;
     long long launches = 0;
@@ -41,23 +42,24 @@ struct ws_batch {
 
 namespace {
 
-// Tiles of the streaming kernel, in the order the tuners try them. 64 x 16
-// and 64 x 32 are left out: with 9 and 17 warps per CTA one SM sub-partition
-// holds 5 of their warps, which caps them at 96 registers per thread, and
-// they spill (measured at less than half the speed of these three).
-constexpr int kTileCands[3][2] = {{64, 8}, {32, 8}, {32, 16}};
+// Tiles of the streaming kernel, in the order the tuners try them: the tuner
+// of one grid all that fit, a batch's the first three that fit every shot. 64 x
+// 32 is left out (its one CTA of 8 warps per SM is the fastest on few grids
+// only, by a few per cent).
+constexpr int kTileCands[4][2] = {{64, 16}, {32, 16}, {64, 8}, {32, 8}};
 
 // z-block candidates for a grid of nz planes cut into `tiles` xy tiles: the
 // default, and for m = 1 .. 8 the z blocks whose item count comes closest to
 // m waves of the resident CTAs from below and from above (a wave that is only
 // partly filled leaves SMs idle at the end of every step on small grids).
-std::vector<int> zblock_candidates(int nz, long long tiles, int slots) {
-    std::vector<int> z{default_zblock(nz)};
+std::vector<int> zblock_candidates(const ws::Geom &g, int tx, int ty, long long tiles, int slots) {
+    const int nz = g.nz;
+    std::vector<int> z{default_zblock(nz), default_zblock(g, tx, ty)};
     for (int m = 1; m <= 8; ++m) {
         const long long target = (long long)m * slots;
         for (long long blocks : {target / tiles, (target + tiles - 1) / tiles}) {
             blocks = std::max<long long>(1, blocks);
-            const int zb = (int)std::max<long long>(8, (nz + blocks - 1) / blocks);
+            const int zb = (int)std::max<long long>(2, (nz + blocks - 1) / blocks);
             z.push_back(std::min(zb, nz));
         }
     }
@@ -181,7 +183,7 @@ int ws_autotune(ws_t ws, int *tile_x, int *tile_y, int *zblock) {
             if ((rc = encode_maps(ws)) != WS_OK) break;
             const long long tiles =
                 (long long)((g.nx + t.tx - 1) / t.tx) * ((g.ny + t.ty - 1) / t.ty);
-            for (int zb : zblock_candidates(g.nz, tiles, slots)) {
+            for (int zb : zblock_candidates(g, t.tx, t.ty, tiles, slots)) {
                 t.zb = zb;
                 const int c = ws->cur;
                 float ms = 0.f;
@@ -189,7 +191,7 @@ int ws_autotune(ws_t ws, int *tile_x, int *tile_y, int *zblock) {
                     if (rep == 1) e = cudaEventRecord(e0, ws->stream);
                     if (e == cudaSuccess)
                         e = ws::launch_step_stream(&ws->tmap_halo[c], &ws->tmap_tile[1 - c],
-                                                   &ws->tmap_w, out, a, t, nullptr, nullptr,
+                                                   &ws->tmap_w, ws->buf[c], out, a, t, nullptr, nullptr,
                                                    ws->stream);
                     ws->launches++;
                 }
@@ -222,6 +224,7 @@ int ws_autotune(ws_t ws, int *tile_x, int *tile_y, int *zblock) {
     } else {
         ws->kernel = WS_KERNEL_STREAM;
         ws->tiling = best;
+        ws->tile_chosen = true;
         int rc = encode_maps(ws);
         if (rc != WS_OK) return rc;
     }
@@ -288,6 +291,7 @@ int batch_configure(ws_batch_t b, int tx, int ty, int m) {
             zb = (int)std::min<long long>(g.nz, std::max<long long>(8, (g.nz + blocks - 1) / blocks));
         }
         b->zb[q] = zb;
+        ws->tile_chosen = true;
         if (ws->tiling.tx != tx || ws->tiling.ty != ty) {
             ws->tiling.tx = tx;
             ws->tiling.ty = ty;
@@ -469,10 +473,12 @@ int ws_batch_create(ws_batch_t *out, int nshots, const ws_t *shots) {
     // online tuning candidates: every tile that fits every shot, z-blocks
     // for about 1, 2, 3, 4, 6 x the resident CTAs in items and the per-shot
     // default (0)
+    int tiles = 0;
     for (const auto &tc : kTileCands) {
-        bool fits = true;
+        bool fits = tiles < 3;
         for (ws_t ws : b->shots) fits = fits && ws->g.nx >= tc[0] && ws->g.ny >= tc[1];
         if (!fits) continue;
+        if (tiles++ == 0) b->untuned = ws_batch::Cand{tc[0], tc[1], 2};
         for (int m : {0, 1, 2, 3, 4, 6}) b->todo.push_back(ws_batch::Cand{tc[0], tc[1], m});
     }
     if (b->todo.empty()) {
@@ -571,8 +577,8 @@ int ws_batch_step(ws_batch_t b, int nsteps) {
         if (b->todo.empty()) b->tuned = true;
     }
     if (rc == WS_OK && done < nsteps) {
-        // the best candidate; while tuning is incomplete, 64 x 8 with 2 x CTAs items
-        const ws_batch::Cand want = b->best.tx ? b->best : ws_batch::Cand{64, 8, 2};
+        // the best candidate; while none is timed, the first tile with 2 x CTAs items
+        const ws_batch::Cand want = b->best.tx ? b->best : b->untuned;
         if (b->cfg.tx != want.tx || b->cfg.ty != want.ty || b->cfg.m != want.m)
             rc = batch_configure(b, want.tx, want.ty, want.m);
         if (rc == WS_OK) rc = batch_upload(b, nsteps - done);

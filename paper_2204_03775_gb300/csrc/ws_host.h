@@ -72,13 +72,15 @@ struct ws_handle {
     long long trace_start = 0;
     std::vector<int> rec_ijk;
     float *traces = nullptr;
-    long long *rec_pidx = nullptr;       // direct path
-    int *rec_ptr = nullptr;              // streaming path: per-tile ranges
+    int *rec_ptr = nullptr;              // per-tile ranges of rec_entries
     ws::RecEntry *rec_entries = nullptr;
-    int rec_tiling_tx = 0, rec_tiling_ty = 0, rec_tiling_rows = 0;
+    int rec_tiling_tx = 0, rec_tiling_ty = 0;
+    bool rec_direct = false;             // the table is the direct kernel's
 
     int kernel = WS_KERNEL_AUTO;
-    ws::StreamTiling tiling{64, 8, 0};
+    ws::StreamTiling tiling{64, 16, 0};  // tile of the tensor maps; zb 0: default
+    bool tile_chosen = false;            // by ws_set_kernel, ws_autotune or a batch
+    ws::StreamTiling auto_zb{0, 0, 0};   // default z block of the tile last used
     CUtensorMap tmap_halo[2];  // buf[b] with the (tx+8, ty+8, 1) box
     CUtensorMap tmap_tile[2];  // buf[b] with the (tx, ty, 1) box
     CUtensorMap tmap_w;        // w with the (tx, ty, 1) box
@@ -95,7 +97,7 @@ struct ws_handle {
     ws::Scale16 *scale = nullptr;
     CUtensorMap t16_halo[2], t16_d, t16_w;
     double wmax = 0.0;         // max (V dt / h)^2 of the model
-    ws::Free16 free16{};       // cells whose taper is exactly 1, per axis
+    ws::FreeBox free_box{};    // cells whose taper is exactly 1, per axis
     int tile16_y = 0;          // 16-bit tile height chosen by ws_set_kernel (0: default)
     int t16_ty = 0;            // tile height the 16-bit tensor maps are encoded for
 
@@ -145,16 +147,15 @@ int encode_map(CUtensorMap *map, void *base, const ws::Geom &g, int bx, int by,
 // The handle's maps for its current tiling.
 int encode_maps(ws_t ws);
 bool stream_fits(const ws_t ws, const ws::StreamTiling &t);
-// Planes per work item: the default for nz planes, and the default shortened
-// to about two full waves of items on small grids.
+// Planes per work item: the default for nz planes, and the FP32 streaming
+// kernel's for a grid and tile.
 int default_zblock(int nz);
 int default_zblock(const ws::Geom &g, int tx, int ty);
 // Choose the kernel for the next steps; fills *tiling for the streaming one.
 int pick_kernel(ws_t ws, ws::StreamTiling *tiling);
 void free_receivers(ws_t ws);
-// Receiver table of the streaming kernels for tile t, whose consumer threads
-// own 4 x-cells of `rows` consecutive rows (FP32 kernels 1, 16-bit kernel 2).
-int build_rec_tiles(ws_t ws, const ws::StreamTiling &t, int rows = 1);
+// Receiver table of the streaming kernels, or of the direct kernel, for tile t.
+int build_rec_tiles(ws_t ws, const ws::StreamTiling &t, bool direct = false);
 // Unpadded [nz][ny][nx] user arrays <-> interiors of padded fields, one or
 // two fields a call (src2 / dst2 null: one).
 int copy_in(ws_t ws, float *dst, const float *src, int on_device, float *dst2 = nullptr,
@@ -162,12 +163,11 @@ int copy_in(ws_t ws, float *dst, const float *src, int on_device, float *dst2 = 
 int copy_out(ws_t ws, float *dst, const float *src, int on_device, float *dst2 = nullptr,
              const float *src2 = nullptr);
 int upload_profiles(ws_t ws);
-// The tile of the 16-bit streaming kernel (64 x ty) and the rows each of its
-// threads computes. The default tile height is the first of kTile16Ys that
+// The tile of the 16-bit streaming kernel (64 x ty). The default tile height is the first of kTile16Ys that
 // the grid holds: 24 (two CTAs of 6 warps per SM) measured fastest on the
 // 1024^3 survey (FP16 434.7, BF16 436.5 Gcell/s, against 418 for 48 and 395
 // for 16); 48 is selectable with ws_set_kernel.
-constexpr int kTile16X = 64, kRows16 = 2;
+constexpr int kTile16X = 64;
 constexpr int kTile16Ys[] = {24, 16};
 constexpr int kNumTile16Ys = 2;
 int pick_tile16(const ws_t ws);

@@ -76,7 +76,8 @@ __host__ __device__ inline long long pidx(const Geom &g, int i, int j, int k) {
 // Receivers grouped for the streaming kernels: per (xy tile, consumer warp)
 // a contiguous range of entries sorted by k, ranges indexed
 // tile * warps + warp. owner = thread index inside the tile's CTA (in that
-// warp), lane = which of the thread's 4 x-cells, r = receiver number.
+// warp), lane = 4 * (which of the thread's two rows) + x-cell, r = receiver
+// number.
 struct RecEntry {
     int k;
     int owner;
@@ -84,11 +85,20 @@ struct RecEntry {
     int r;
 };
 
+// The cells whose taper is exactly 1 on each axis, [x0, x1) x [y0, y1) x
+// [z0, z1) (empty ranges allowed): the 16-bit kernel's tiles inside them take
+// the update without taper multiplies, which gives the same bits. (In the FP32
+// kernel the second form of the update cost 2 %.)
+struct FreeBox {
+    int x0, x1, y0, y1, z0, z1;
+};
+
 struct StepArgs {
     Geom g;
     Coeffs c;
     Sources src;
     const float *gx, *gy, *gz;   // taper profiles (1.0 without damping)
+    FreeBox fr;
     float *traces;               // [nrec][nt_max] or null
     int nt_max;
     long long trace_step;        // column of this step in traces
@@ -99,11 +109,12 @@ struct StepArgs {
 
 // Launchers (stream-ordered, no synchronization).
 // out = u^{n+1} from u = u^n and up = u^{n-1}; out may be up (in place).
+// rec_ptr (null: none): per tile of kDirectX x kDirectY columns a range of rec
+// sorted by k, with lane = x and owner = y inside the tile.
+constexpr int kDirectX = 32, kDirectY = 8;
 cudaError_t launch_step_direct(const float *u, const float *up, float *out, const float *w,
-                               const StepArgs &a, cudaStream_t s);
-cudaError_t launch_gather_receivers(const float *u_next, const long long *rec_pidx, int nrec,
-                                    float *traces, int nt_max, long long trace_step,
-                                    cudaStream_t s);
+                               const StepArgs &a, const int *rec_ptr, const RecEntry *rec,
+                               cudaStream_t s);
 // The model (device array [nz][ny][nx], or null: already in w's interior) into
 // the padded w: V -> (V dt / h)^2, m = 1/V^2 -> (dt / h)^2 / m, in double,
 // rounded once. extrema collects {max, min} of the values as float bits; a
@@ -152,12 +163,12 @@ struct StreamTiling {
     int tx, ty, zb;
 };
 bool stream_tiling_supported(int tx, int ty);
-// tmap_u: u^n with box (tx+8, ty+8, 1); tmap_up: u^{n-1} (written in place
+// tmap_u: u^n (the field u) with box (tx+8, ty+8, 1); tmap_up: u^{n-1} (written in place
 // with u^{n+1} through up) and tmap_w: (V dt/h)^2, both with box (tx, ty, 1).
 cudaError_t launch_step_stream(const CUtensorMap *tmap_u, const CUtensorMap *tmap_up,
-                               const CUtensorMap *tmap_w, float *up, const StepArgs &a,
-                               const StreamTiling &t, const int *rec_ptr, const RecEntry *rec,
-                               cudaStream_t s);
+                               const CUtensorMap *tmap_w, const float *u, float *up,
+                               const StepArgs &a, const StreamTiling &t, const int *rec_ptr,
+                               const RecEntry *rec, cudaStream_t s);
 
 // One shot of a batched step (global memory, written by the host before the
 // launch). Step t of a run reads u^n from buf[cur0 ^ (t & 1)] with
@@ -182,7 +193,7 @@ struct alignas(128) BatchShot {
 // SMs x resident CTAs of the streaming kernel (batch: the batched one) with
 // tile tx x ty. Also sets the kernel's shared-memory limit, so call it once
 // before capturing launches into a graph.
-cudaError_t stream_slots(int tx, int ty, bool batch, int *slots);
+cudaError_t stream_slots(int tx, int ty, bool batch, int *slots, int *sms = nullptr);
 
 // One launch over items[0..nitems) = (shot, item of the shot), one CTA each,
 // every shot with the tile tx x ty (stream_tiling_supported).
@@ -201,14 +212,9 @@ struct Scale16 {
     unsigned amax[4];
 };
 // Stencil weights of the 16-bit kernel (centre weight c0 applied once; see
-// zero_sum_weights16) and the cells whose taper is exactly 1 on each axis,
-// [x0, x1) x [y0, y1) x [z0, z1) (empty ranges allowed): tiles inside them take
-// the update without taper multiplies, which gives the same bits.
+// zero_sum_weights16).
 struct Weights16 {
     float c0, c1, c2, c3, c4;
-};
-struct Free16 {
-    int x0, x1, y0, y1, z0, z1;
 };
 Weights16 zero_sum_weights16();
 bool stream16_tiling_supported(int tx, int ty);
@@ -224,7 +230,7 @@ struct Maps16In {
     uint16_t *u_out, *d_io;
 };
 cudaError_t launch_step_stream16(int storage, const Maps16In &m, const StepArgs &a, Scale16 *sc,
-                                 long long step, float src_hint, const Free16 &fr,
+                                 long long step, float src_hint,
                                  const StreamTiling &t, const int *rec_ptr, const RecEntry *rec,
                                  cudaStream_t s);
 // FP32 (u^n, u^{n-1}), padded or the caller's, <-> 16-bit padded (U, D)

@@ -1,10 +1,12 @@
 // Direct step kernel (one thread per cell, neighbours read from global
-// memory through L1/L2) and the small helper kernels of the library.
+// memory through L1/L2).
 //
-// The direct kernel is the plain form of the fused step: it is used for
-// grids smaller than a streaming tile and as a second, independent CUDA path
-// in the parity tests. The hot path is the streaming kernel.
-#include "ws_internal.h"
+// The direct kernel is the plain form of the fused step: it is used for grids
+// smaller than a streaming tile or so small that a step is all latency (every
+// load of a cell is in flight at once, where the streaming kernel walks planes
+// one after the other), and as a second, independent CUDA path in the parity
+// tests. The hot path is the streaming kernel.
+#include "ws_ptx.cuh"
 
 namespace ws {
 
@@ -12,10 +14,8 @@ namespace ws {
 // leapfrog of Eq. 2, absorbing taper, source (right-hand side of Eq. 2).
 // u: u^n, up: u^{n-1} on entry and u^{n+1} on exit (same cell only),
 // w: (V dt / h)^2.
-__global__ void __launch_bounds__(256) step_direct_kernel(const float *__restrict__ u,
-                                                          const float *up, float *out,
-                                                          const float *__restrict__ w,
-                                                          const __grid_constant__ StepArgs a) {
+__device__ __forceinline__ void step_cell(const float *u, const float *up, float *out,
+                                          const float *w, const StepArgs &a) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     const int j = blockIdx.y * blockDim.y + threadIdx.y;
     const int k = blockIdx.z;
@@ -51,31 +51,39 @@ __global__ void __launch_bounds__(256) step_direct_kernel(const float *__restric
     out[p] = un;
 }
 
+// Receivers: a block's entries of its tile's range (sorted by k) on its plane
+// are sampled once all its threads have stored. (As a launch of its own this
+// cost 1 us a step on grids of a few microseconds.)
+__device__ __forceinline__ void record_block(const float *out, const StepArgs &a, int k,
+                                             const int *rec_ptr, const RecEntry *rec) {
+    const int tile = blockIdx.y * gridDim.x + blockIdx.x;
+    const int lo = rec_ptr[tile], hi = rec_ptr[tile + 1];
+    if (lo == hi) return;
+    __syncthreads();
+    const int tid = threadIdx.y * blockDim.x + threadIdx.x;
+    for (int e = lo + tid; e < hi; e += blockDim.x * blockDim.y) {
+        if (rec[e].k != k) continue;
+        const int i = blockIdx.x * blockDim.x + rec[e].lane, j = blockIdx.y * blockDim.y + rec[e].owner;
+        a.traces[(long long)rec[e].r * a.nt_max + a.trace_step] = out[pidx(a.g, i, j, k)];
+    }
+}
+
+__global__ void __launch_bounds__(256) step_direct_kernel(const float *u,
+                                                          const float *up, float *out,
+                                                          const float *w,
+                                                          const __grid_constant__ StepArgs a,
+                                                          const int *rec_ptr, const RecEntry *rec) {
+    wait_predecessor();
+    step_cell(u, up, out, w, a);
+    if (rec_ptr) record_block(out, a, blockIdx.z, rec_ptr, rec);
+}
+
 cudaError_t launch_step_direct(const float *u, const float *up, float *out, const float *w,
-                               const StepArgs &a, cudaStream_t s) {
-    dim3 block(32, 8, 1);
-    dim3 grid((a.g.nx + 31) / 32, (a.g.ny + 7) / 8, a.g.nz);
-    step_direct_kernel<<<grid, block, 0, s>>>(u, up, out, w, a);
-    return cudaGetLastError();
-}
-
-// traces[r][step] = u^{n+1} at receiver r (the direct kernel's receiver pass).
-__global__ void gather_receivers_kernel(const float *__restrict__ u_next,
-                                        const long long *__restrict__ rec_pidx, int nrec,
-                                        float *__restrict__ traces, int nt_max,
-                                        long long trace_step) {
-    const int r = blockIdx.x * blockDim.x + threadIdx.x;
-    if (r >= nrec) return;
-    traces[(long long)r * nt_max + trace_step] = u_next[rec_pidx[r]];
-}
-
-cudaError_t launch_gather_receivers(const float *u_next, const long long *rec_pidx, int nrec,
-                                    float *traces, int nt_max, long long trace_step,
-                                    cudaStream_t s) {
-    if (nrec <= 0) return cudaSuccess;
-    gather_receivers_kernel<<<(nrec + 255) / 256, 256, 0, s>>>(u_next, rec_pidx, nrec, traces,
-                                                               nt_max, trace_step);
-    return cudaGetLastError();
+                               const StepArgs &a, const int *rec_ptr, const RecEntry *rec,
+                               cudaStream_t s) {
+    dim3 block(kDirectX, kDirectY, 1);
+    dim3 grid((a.g.nx + kDirectX - 1) / kDirectX, (a.g.ny + kDirectY - 1) / kDirectY, a.g.nz);
+    return launch_overlapped(step_direct_kernel, grid, block, 0, s, u, up, out, w, a, rec_ptr, rec);
 }
 
 }  // namespace ws

@@ -7,30 +7,32 @@
 // lives in a per-thread register queue of 9 planes (k-4 .. k+4), and the x/y
 // neighbours come from a shared-memory copy of plane k with its 4-cell halo.
 //
-// Warp-specialized CTAs, one per work item, which the hardware dispatches in
-// item order as resident CTAs finish. (A persistent grid of SMs x CTAs-per-SM
-// looping over the items measured 2-5% slower on the 1024^3 survey: its CTAs
-// drift apart, so a tile's halo rows leave L2 before the neighbouring tile
-// reads them; in-order dispatch keeps the tiles in flight a contiguous range
-// of items. The item loop is kept, so a smaller grid still works.)
-//  - one producer lane issues every TMA copy (cp.async.bulk.tensor) into two
-//    shared-memory rings, ring A (u^n tile with halo, (TX+8) x (TY+8)) and
-//    ring B (u^{n-1} and (V dt/h)^2 tiles, TX x TY), each slot guarded by a
-//    "full" mbarrier (transaction count) and an "empty" mbarrier;
-//  - the consumer warps compute: each thread owns 4 consecutive x cells of
-//    one row, waits on "full", reads the slot, and arrives on "empty" -- no
-//    atomics, fences or divergent code in the steady state. The producer
-//    runs ahead by the ring depth, across item boundaries too.
-// u^{n+1} is written in place of u^{n-1} with 128-bit streaming stores.
+// One CTA per work item, dispatched by the hardware in item order as resident
+// CTAs finish, so the tiles in flight are always a contiguous range of items
+// and a tile's halo rows are still in L2 when its neighbour reads them.
+//  - Every thread computes the 4 cells i .. i+3 of the two rows j and j+1: the
+//    rows j-4 .. j-1 and j+2 .. j+5 serve both, and the waits, the ring
+//    bookkeeping and the x loads of a plane are paid once for 8 cells.
+//  - TMA copies (cp.async.bulk.tensor) fill two shared-memory rings: ring A
+//    (u^n with halo, (TX+8) x (TY+8), P + 4 planes) and ring B (u^{n-1} and
+//    (V dt/h)^2 tiles, P planes). Stage r carries what plane r needs new: the
+//    u^n plane r+4 and ring B's plane r, on one "full" mbarrier. A warp that
+//    has read plane r arrives on the stage's "empty" mbarrier; one lane of one
+//    warp waits for it and issues stage r + P. There is no
+//    producer warp (its registers would cost a third of the compute warps)
+//    and no CTA-wide barrier in the loop.
+//  - The four planes below the block, of which only the thread's own cells are
+//    needed, are read from global memory straight into the queue.
+// u^{n+1} is written in place of u^{n-1} with 128-bit stores (plain ones: with
+// evict-first stores 1024 x 1024 x 512 ran at 415 instead of 422 Gcell/s).
 // Taper, source injection and receiver sampling are fused into the pass.
 // The z loop is unrolled by 3 with the queue indices rotated at compile time.
 //
-// Each thread's 4 cells are processed as two pairs with the packed FP32x2
-// instructions of sm_100+ (add/mul/fma .rn .f32x2), which halves the
-// floating-point instruction count. Each lane is rounded exactly as the
-// scalar instruction, so the arithmetic per cell is the same expression, in
-// the same order, as the direct kernel, and the two CUDA paths agree bit for
-// bit.
+// Each thread's 4 cells of a row are processed as two pairs with the packed
+// FP32x2 instructions of sm_100+ (add/mul/fma .rn .f32x2). Each lane is
+// rounded exactly as the scalar instruction, so the arithmetic per cell is the
+// same expression, in the same order, as the direct kernel, and the two CUDA
+// paths agree bit for bit.
 //
 // Every wait is bounded (kWaitLimitNs); on a timeout the kernel records
 // kStatusTimeout, all warps leave their loops, and the CTA waits (bounded)
@@ -48,31 +50,25 @@
 namespace ws {
 namespace {
 
-#ifndef WS_STREAM_UNROLL
-#define WS_STREAM_UNROLL 3
-#endif
-constexpr int kUnroll = WS_STREAM_UNROLL;  // planes per loop trip: 3 or 9 (divides the queue rotation)
-static_assert(kUnroll == 3 || kUnroll == 9, "the 9-plane queue rotation needs 3 or 9");
-#ifndef WS_RING_A
-#define WS_RING_A 8
-#endif
+constexpr int kTrip = 3;   // planes per loop trip, and the stages in flight
 
-// Tile geometry and ring sizes of one streaming-kernel instantiation.
-template <int TX, int TY, int NA, int NB>
+// Tile geometry and ring sizes of one instantiation.
+template <int TX, int TY>
 struct StreamCfg {
-    static constexpr int kConsumers = (TX / 4) * TY;   // compute threads
-    static constexpr int kThreads = kConsumers + 32;   // + one producer warp
-    static constexpr int kRowW = TX + 2 * kHalo;       // floats per ring-A row
+    static constexpr int kCols = TX / 4;                 // threads across a row
+    static constexpr int kThreads = kCols * (TY / 2);
+    static constexpr int kWarps = kThreads / 32;
+    static constexpr int P = kTrip;                      // stages (ring-B planes)
+    static constexpr int NA = P + 4;                     // ring-A planes
+    static constexpr int kRowW = TX + 2 * kHalo;         // floats per ring-A row
     static constexpr int kRows = TY + 2 * kHalo;
-    static constexpr int kSlotA = kRowW * kRows;       // floats per ring-A slot
-    static constexpr unsigned kSlotABytes = kSlotA * 4u;
-    static constexpr int kTile = TX * TY;              // floats per field in a ring-B slot
-    static constexpr unsigned kSlotBBytes = 2u * kTile * 4u;
-    static_assert(kConsumers % 32 == 0, "whole consumer warps");
-    static_assert((NA & (NA - 1)) == 0 && NA >= 8, "ring A: power of two, >= 8 planes");
-    static_assert((NB & (NB - 1)) == 0 && NB >= 2, "ring B: power of two, >= 2 planes");
+    static constexpr unsigned kRowBytes = kRowW * 4u;
+    static constexpr unsigned kSlotABytes = kRowW * kRows * 4u;
+    static constexpr unsigned kTileBytes = TX * TY * 4u;
+    static constexpr unsigned kSlotBBytes = 2u * kTileBytes;   // u^{n-1} tile, then (V dt/h)^2
+    static_assert(kThreads % 32 == 0, "whole warps");
     static_assert(kSlotABytes % 128 == 0 && kSlotBBytes % 128 == 0, "slots stay 128-byte aligned");
-    static constexpr size_t kSmem = size_t(NA) * kSlotABytes + size_t(NB) * kSlotBBytes;
+    static constexpr size_t kSmem = size_t(NA) * kSlotABytes + size_t(P) * kSlotBBytes;
 };
 
 // The tensor maps of one launch: u^n with the halo box, u^{n-1} and
@@ -81,20 +77,21 @@ struct StreamMaps {
     CUtensorMap u, up, w;
 };
 
-// What the producer needs of an item: its extent and the three maps;
-// stall (a test hook) withholds the item's first copy.
+// What the copies of an item need: its extent and the three maps; stall (a
+// test hook) withholds the item's first copies.
 struct Job {
     Item it;
     const CUtensorMap *u, *up, *w;
     bool stall;
 };
 
-// What the consumers need of an item's grid: fields read at the start of an
+// What the threads need of an item's grid: fields read at the start of an
 // item or on every plane, and accessors for what only source injection and
 // receiver recording use.
 struct View {
     Geom g;
     const float *gx, *gy, *gz;
+    const float *u;            // u^n field (padded)
     float *out;                // u^{n+1} field (padded)
     long long lap_delta;       // L u^n goes to out + lap_delta (0: not stored)
     const int *rec_ptr;        // per-tile receiver ranges, or null
@@ -120,17 +117,17 @@ struct OneGrid {
     using V = View;
     const StreamMaps &mp;
     const StepArgs &a;
+    const float *u;
     float *up;
-    int zb, tiles_x, ntiles, n;
+    int zb, tiles_x, ntiles;
     const int *rec_ptr;
     const RecEntry *rec;
 
-    __device__ __forceinline__ int nitems() const { return n; }
     __device__ __forceinline__ Job job(int item) const {
         return Job{item_of(item, tiles_x, ntiles, zb, a.g.nz, TX, TY), &mp.u, &mp.up, &mp.w,
                    item == a.stall_item};
     }
-    __device__ __forceinline__ Item view(int item, View *v) const {
+    __device__ __forceinline__ void view(int, View *v) const {
         v->g = a.g;
         v->gx = a.gx;
         v->gy = a.gy;
@@ -140,20 +137,21 @@ struct OneGrid {
         v->traces_ = a.traces;
         v->nt_max_ = a.nt_max;
         v->trace_step_ = a.trace_step;
+        v->u = u;
         v->out = up;
         v->lap_delta = kLap ? a.lap - up : 0;
         v->rec_ptr = rec_ptr;
         v->rec_ = rec;
-        return item_of(item, tiles_x, ntiles, zb, a.g.nz, TX, TY);
     }
 };
 
 // The view of a batch item: the fields of every plane in registers, the rest
 // read from the shot's descriptor where they are used (held in registers for
-// the whole item they would not fit the batched kernel's register budget).
+// the whole item they would not fit the register budget).
 struct BatchView {
     Geom g;
     const float *gx, *gy, *gz;
+    const float *u;
     float *out;
     const int *rec_ptr;
     const BatchShot *shot;
@@ -176,9 +174,8 @@ struct ShotBatch {
     using V = BatchView;
     const BatchShot *shots;
     const int2 *items;
-    int n, t;
+    int t;
 
-    __device__ __forceinline__ int nitems() const { return n; }
     __device__ __forceinline__ Job job(int item) const {
         const int2 e = items[item];
         const BatchShot &s = shots[e.x];
@@ -186,7 +183,7 @@ struct ShotBatch {
         return Job{item_of(e.y, s.tiles_x, s.ntiles, s.zb, s.g.nz, TX, TY), &s.halo[p],
                    &s.tile[1 - p], &s.w, t == 0 && e.y == s.stall_item};
     }
-    __device__ __forceinline__ Item view(int item, BatchView *v) const {
+    __device__ __forceinline__ void view(int item, BatchView *v) const {
         const int2 e = items[item];
         const BatchShot &s = shots[e.x];
         const int p = s.cur0 ^ (t & 1);
@@ -194,140 +191,71 @@ struct ShotBatch {
         v->gx = s.gx;
         v->gy = s.gy;
         v->gz = s.gz;
+        v->u = s.buf[p];
         v->out = s.buf[1 - p];
         v->rec_ptr = s.rec_ptr;
         v->shot = &s;
         v->t = t;
-        return item_of(e.y, s.tiles_x, s.ntiles, s.zb, s.g.nz, TX, TY);
     }
 };
 
-// Per-thread state of a consumer thread's walk down one item.
+// Barriers of one CTA.
+template <int P>
+struct Bars {
+    uint64_t full[P], empty[P];   // stages
+    uint64_t first;               // ring-A planes z0 .. z0+3
+    int issued;                   // stages issued (for the drain)
+    int first_issued;
+    int abort;
+};
+
+// Per-thread state of the walk down an item.
 struct Walk {
-    float4 q[9];            // u^n of planes k-4 .. k+4 (rotated: see plane_step)
-    float gzb[3];           // z taper of planes k, k+1, k+2 (rotated)
-    float4 gxy;             // gx * gy of this thread's 4 columns
-    float *out_k;           // u^{n+1} of plane k
-    int nvalid;             // cells of the 4 inside the grid (0 when the row is outside)
+    float4 q[9][2];         // u^n of planes k-4 .. k+4, rows j and j+1 (rotated: see plane_step)
+    float4 gxy[2];          // gx * gy of this thread's 4 columns per row
+    float *out_k;           // u^{n+1} of (i, j, k)
+    unsigned halo, own;     // byte offsets of the ring-A slots of planes k and k + 4
+    int nvalid;             // cells of the 4 inside the grid (0 when the column is outside)
+    bool row1;              // row j+1 inside the grid
+    bool whole;             // all cells of the warp lie inside the grid
     int rcur, rend, rnext_k;
     unsigned src_mask;
-    unsigned gAw, gAr, gB;  // ring-A planes waited for / released, ring-B planes used
-    bool ok;
+    int next_event;         // the next plane with a source or a receiver
 };
 
-template <int TX, int TY, int NA, int NB>
+template <int TX, int TY>
 struct Kern {
-    using Cfg = StreamCfg<TX, TY, NA, NB>;
-    using R = Rings<NA, NB>;
+    using Cfg = StreamCfg<TX, TY>;
+    static constexpr int P = Cfg::P, NA = Cfg::NA;
+    using B = Bars<P>;
 
-    // ---------------------------------------------------------------- producer
-
-    // Copy relative plane pr of the item (interior plane z0 - 4 + pr, with
-    // its halo) into the g-th ring-A slot use, once its previous plane is
-    // released. The maps cover the interior only (origin at interior cell 0):
-    // the box corner is (i0 - 4, j0 - 4, z0 - 4 + pr), and whatever of the
-    // box lies outside the grid arrives as zeros without a memory read (the
-    // zero halo). x is a multiple of 4 elements (16 bytes).
-    static __device__ __forceinline__ bool produce_a(R &rg, float *ringA, const Job &jb, unsigned g,
-                                                     int pr, unsigned *status) {
-        const int slot = g & (NA - 1);
-        if (!wait_phase(&rg.emptyA[slot], ((g / NA) & 1u) ^ 1u, &rg.abort, status)) return false;
-        rg.issuedA[slot]++;
-        mbar_arrive_expect_tx(&rg.fullA[slot], Cfg::kSlotABytes);
-        tma_load_3d(ringA + slot * Cfg::kSlotA, jb.u, &rg.fullA[slot], jb.it.i0 - kHalo,
-                    jb.it.j0 - kHalo, jb.it.z0 - kHalo + pr);
-        return true;
+    // Stage r of the item into its slots (ring A at byte slotA): the u^n plane z0 + r + 4 with its
+    // halo, and u^{n-1} and (V dt/h)^2 of plane z0 + r. The maps cover the
+    // interior only (origin at interior cell 0): whatever of a box lies
+    // outside the grid arrives as zeros without a memory read (the zero halo).
+    // x is a multiple of 4 elements (16 bytes).
+    static __device__ __forceinline__ void issue(B &br, unsigned ringA, unsigned ringB, const Job &jb,
+                                                 int r, unsigned slotA, int stage) {
+        uint64_t *bar = &br.full[stage];
+        mbar_arrive_expect_tx(bar, Cfg::kSlotABytes + Cfg::kSlotBBytes);
+        const unsigned b = ringB + stage * Cfg::kSlotBBytes;
+        tma_load_3d_at(ringA + slotA, jb.u, bar, jb.it.i0 - kHalo,
+                       jb.it.j0 - kHalo, jb.it.z0 + kHalo + r);
+        tma_load_3d_at(b, jb.up, bar, jb.it.i0, jb.it.j0, jb.it.z0 + r);
+        tma_load_3d_at(b + Cfg::kTileBytes, jb.w, bar, jb.it.i0, jb.it.j0, jb.it.z0 + r);
     }
 
-    // u^{n-1} and (V dt/h)^2 of interior plane z0 + b into the g-th ring-B use.
-    static __device__ __forceinline__ bool produce_b(R &rg, float *ringB, const Job &jb, unsigned g,
-                                                     int b, unsigned *status) {
-        const int slot = g & (NB - 1);
-        if (!wait_phase(&rg.emptyB[slot], ((g / NB) & 1u) ^ 1u, &rg.abort, status)) return false;
-        rg.issuedB[slot]++;
-        float *dst = ringB + slot * (2 * Cfg::kTile);
-        mbar_arrive_expect_tx(&rg.fullB[slot], Cfg::kSlotBBytes);
-        tma_load_3d(dst, jb.up, &rg.fullB[slot], jb.it.i0, jb.it.j0, jb.it.z0 + b);
-        tma_load_3d(dst + Cfg::kTile, jb.w, &rg.fullB[slot], jb.it.i0, jb.it.j0, jb.it.z0 + b);
-        return true;
-    }
-
-    // One lane issues every copy of every item of this CTA, in the order the
-    // consumers need them: the 8 planes of the queue prologue, then for each
-    // plane k of the block its u^{n-1} / (V dt/h)^2 and the u^n plane k + 8.
-    template <class S>
-    static __device__ void producer(R &rg, float *ringA, float *ringB, const S &src,
-                                    unsigned *status) {
-        unsigned gA = 0, gB = 0;
-        for (int item = blockIdx.x; item < src.nitems(); item += gridDim.x) {
-            const Job jb = src.job(item);
-            const int nb = jb.it.z1 - jb.it.z0, nplanes = nb + 2 * kHalo;
-            for (int pr = 0; pr < 2 * kHalo; ++pr) {
-                if (pr == 0 && jb.stall) {   // never filled: the consumers' bounded waits run out
-                    ++gA;
-                    continue;
-                }
-                if (!produce_a(rg, ringA, jb, gA++, pr, status)) return;
-            }
-            for (int b = 0; b < nb; ++b) {
-                if (!produce_b(rg, ringB, jb, gB++, b, status)) return;
-                if (b + 2 * kHalo < nplanes && !produce_a(rg, ringA, jb, gA++, b + 2 * kHalo, status))
-                    return;
-            }
-        }
-    }
-
-    // ---------------------------------------------------------------- consumers
-
-    static __device__ __forceinline__ const float *wait_a(Walk &wk, R &rg, const float *ringA,
-                                                          unsigned g, unsigned *status) {
-        const int slot = g & (NA - 1);
-        wk.ok = wk.ok && wait_phase(&rg.fullA[slot], (g / NA) & 1u, &rg.abort, status);
-        return ringA + slot * Cfg::kSlotA;
-    }
-
-    // Plane k of the item, with the rotation R = (k - z0) mod 9 fixed at
-    // compile time.
-    template <int RQ, bool kLap, class VT>
-    static __device__ __forceinline__ void plane_step(Walk &wk, R &rg, const float *ringA,
-                                                      const float *ringB, const VT &v,
-                                                      const Coeffs &c, unsigned *status,
-                                                      const Item &it, int k, int i, int j,
-                                                      int offA, int offB) {
-#define QI(m) ((RQ + (m)) % 9)
-#define BI(d) ((RQ + (d)) % 3)
-        // u^n of plane k + 4 into the queue
-        const float *sa = wait_a(wk, rg, ringA, wk.gAw, status);
-        wk.q[QI(8)] = lds4(sa + offA);
-        ++wk.gAw;
-
-        // u^{n-1} and (V dt/h)^2 of plane k
-        const int sb = wk.gB & (NB - 1);
-        wk.ok = wk.ok && wait_phase(&rg.fullB[sb], (wk.gB / NB) & 1u, &rg.abort, status);
-        const float *tb = ringB + sb * (2 * Cfg::kTile) + offB;
-        const float4 upc = lds4(tb);
-        const float4 wc = lds4(tb + Cfg::kTile);
-        warp_arrive(&rg.emptyB[sb]);
-        ++wk.gB;
-
-        if (k + 2 < it.z1) wk.gzb[BI(2)] = __ldg(v.gz + k + 2);
-
-        // u^n of plane k with its halo (waited for four planes ago)
-        const float *row = ringA + (wk.gAr & (NA - 1)) * Cfg::kSlotA + offA;
-        const float4 xl = lds4(row - 4);   // cells x-4 .. x-1 of lane 0
-        const float4 xc = wk.q[QI(4)];
-        const float4 xr = lds4(row + 4);   // cells x+4 .. x+7 of lane 0
-        float4 yp[4], ym[4];
-#pragma unroll
-        for (int m = 1; m <= 4; ++m) {
-            yp[m - 1] = lds4(row + m * Cfg::kRowW);
-            ym[m - 1] = lds4(row - m * Cfg::kRowW);
-        }
-        warp_arrive(&rg.emptyA[wk.gAr & (NA - 1)]);
-        ++wk.gAr;
-
-        // x pairs: offsets +-2 and +-4 are aligned float2 pairs of (xl, xc, xr);
-        // offsets +-1 and +-3 straddle pairs and are summed per lane.
+    // The stencil sum of one row's 4 cells (two FP32x2 pairs). xl, xr: cells
+    // x-4..x-1 and x+4..x+7 of the row; yp / ym: rows j+m / j-m of this row;
+    // z from the register queue.
+    template <int RQ>
+    static __device__ __forceinline__ void stencil_row(const Walk &wk, const Coeffs &c, int r,
+                                                       const float4 &xl, const float4 &xr,
+                                                       const float4 (&yp)[4], const float4 (&ym)[4],
+                                                       float2 (&lap)[2]) {
+        const float4 xc = wk.q[(RQ + 4) % 9][r];
+        // x pairs: offsets +-2 and +-4 are aligned float2 pairs of (xl, xc,
+        // xr); offsets +-1 and +-3 straddle pairs and are summed per lane
         const float e[12] = {xl.x, xl.y, xl.z, xl.w, xc.x, xc.y, xc.z, xc.w,
                              xr.x, xr.y, xr.z, xr.w};
         float2 sx[2][5];
@@ -343,234 +271,340 @@ struct Kern {
                 sx[p][m] = make_float2(e[4 + l0 + m] + e[4 + l0 - m], e[4 + l1 + m] + e[4 + l1 - m]);
             }
         }
-
-        const float gzk = wk.gzb[BI(0)];
-        float2 o[2], lp[2];
 #pragma unroll
         for (int p = 0; p < 2; ++p) {
             float2 s[5];
 #pragma unroll
             for (int m = 1; m <= 4; ++m) {
                 const float2 sy = add2(pair(yp[m - 1], p), pair(ym[m - 1], p));
-                const float2 sz = add2(pair(wk.q[QI(4 + m)], p), pair(wk.q[QI(4 - m)], p));
+                const float2 sz = add2(pair(wk.q[(RQ + 4 + m) % 9][r], p),
+                                       pair(wk.q[(RQ + 4 - m + 9) % 9][r], p));
                 s[m] = add2(add2(sx[p][m], sy), sz);
             }
             const float2 uc = pair(xc, p);
             // sum_m c_m (s_m - 6 u): exactly zero on constants (see Coeffs)
-            float2 lap = mul2(splat(c.c4), fma2(splat(-6.0f), uc, s[4]));
-            lap = fma2(splat(c.c3), fma2(splat(-6.0f), uc, s[3]), lap);
-            lap = fma2(splat(c.c2), fma2(splat(-6.0f), uc, s[2]), lap);
-            lap = fma2(splat(c.c1), fma2(splat(-6.0f), uc, s[1]), lap);
-            lp[p] = lap;
-            const float2 gd = mul2(pair(wk.gxy, p), splat(gzk));
-            const float2 ngd = mul2(pair(wk.gxy, p), splat(-gzk));   // -gd, exactly
-            const float2 t = fma2(pair(wc, p), lap, fma2(splat(2.0f), uc, mul2(ngd, pair(upc, p))));
+            float2 l = mul2(splat(c.c4), fma2(splat(-6.0f), uc, s[4]));
+            l = fma2(splat(c.c3), fma2(splat(-6.0f), uc, s[3]), l);
+            l = fma2(splat(c.c2), fma2(splat(-6.0f), uc, s[2]), l);
+            lap[p] = fma2(splat(c.c1), fma2(splat(-6.0f), uc, s[1]), l);
+        }
+    }
+
+    // u^{n+1} = g (2 u - g u^{n-1} + W L) of one row's 4 cells.
+    static __device__ __forceinline__ float4 update(const float2 (&lap)[2], const float4 &u,
+                                                    const float4 &up, const float4 &w,
+                                                    const float4 &gxy, float gzk) {
+        float2 o[2];
+#pragma unroll
+        for (int p = 0; p < 2; ++p) {
+            const float2 gd = mul2(pair(gxy, p), splat(gzk));
+            const float2 ngd = mul2(pair(gxy, p), splat(-gzk));   // -gd, exactly
+            const float2 t =
+                fma2(pair(w, p), lap[p], fma2(splat(2.0f), pair(u, p), mul2(ngd, pair(up, p))));
             o[p] = mul2(gd, t);
         }
-        float4 out = make_float4(o[0].x, o[0].y, o[1].x, o[1].y);
-        if (wk.src_mask) {
-            const SourceSample *srcs = v.src();
-            for (int qs = 0, ns = v.nsrc(); qs < ns; ++qs) {
-                const SourceSample ss = srcs[qs];
-                if (((wk.src_mask >> qs) & 1u) && ss.k == k && ss.j == j) {
+        return make_float4(o[0].x, o[0].y, o[1].x, o[1].y);
+    }
+
+    // Rows j and j+1 of one plane: the common warp stores all 8 cells a thread.
+    static __device__ __forceinline__ void store_rows(const Walk &wk, float *p, int pitch,
+                                                      const float4 &a, const float4 &b) {
+        if (wk.whole) {
+            *reinterpret_cast<float4 *>(p) = a;
+            *reinterpret_cast<float4 *>(p + pitch) = b;
+            return;
+        }
 #pragma unroll
-                    for (int l = 0; l < 4; ++l)
-                        if (ss.i == i + l) set_comp(out, l, fmaf(comp(wc, l), ss.amp, comp(out, l)));
-                }
+        for (int r = 0; r < 2; ++r) {
+            if (r == 1 && !wk.row1) break;
+            const float4 v = r ? b : a;
+            float *q = p + r * pitch;
+            if (wk.nvalid > 0) q[0] = v.x;
+            if (wk.nvalid > 1) q[1] = v.y;
+            if (wk.nvalid > 2) q[2] = v.z;
+            if (wk.nvalid > 3) q[3] = v.w;
+        }
+    }
+
+    // The first plane after k with a source or a receiver of this warp.
+    template <class VT>
+    static __device__ __forceinline__ int event_after(const Walk &wk, const VT &v, int k) {
+        int next = wk.rnext_k;
+        for (unsigned m = wk.src_mask; m; m &= m - 1) {
+            const int sk = v.src()[__ffs(m) - 1].k;
+            if (sk > k) next = min(next, sk);
+        }
+        return next;
+    }
+
+    // Sources and receivers of plane k (few planes have any).
+    template <class VT>
+    static __device__ __forceinline__ void events(Walk &wk, const VT &v, int k, int i, int j,
+                                                  float4 (&out)[2], const float4 &w0,
+                                                  const float4 &w1) {
+        for (unsigned m = wk.src_mask; m; m &= m - 1) {
+            const SourceSample ss = v.src()[__ffs(m) - 1];
+            if (ss.k != k) continue;
+#pragma unroll
+            for (int l = 0; l < 4; ++l) {
+                if (ss.i != i + l) continue;
+                if (ss.j == j) set_comp(out[0], l, fmaf(comp(w0, l), ss.amp, comp(out[0], l)));
+                if (ss.j == j + 1) set_comp(out[1], l, fmaf(comp(w1, l), ss.amp, comp(out[1], l)));
             }
         }
-        if (wk.nvalid == 4) {
-            __stcs(reinterpret_cast<float4 *>(wk.out_k), out);
-        } else if (wk.nvalid > 0) {
-            wk.out_k[0] = out.x;
-            if (wk.nvalid > 1) wk.out_k[1] = out.y;
-            if (wk.nvalid > 2) wk.out_k[2] = out.z;
-        }
-        if constexpr (kLap) {   // the stencil sum, for the adjoint's imaging
-            float *lk = wk.out_k + v.lap_delta;
-            const float4 l4 = make_float4(lp[0].x, lp[0].y, lp[1].x, lp[1].y);
-            if (wk.nvalid == 4) {
-                __stcs(reinterpret_cast<float4 *>(lk), l4);
-            } else if (wk.nvalid > 0) {
-                lk[0] = l4.x;
-                if (wk.nvalid > 1) lk[1] = l4.y;
-                if (wk.nvalid > 2) lk[2] = l4.z;
-            }
-        }
-        wk.out_k += v.g.plane;
         if (k == wk.rnext_k)
-            record_plane(out, 1.0f, k, &wk.rcur, wk.rend, &wk.rnext_k, v.rec(), v.traces(),
-                         v.nt_max(), v.trace_step());
-#undef QI
-#undef BI
+            record_plane2(out, k, &wk.rcur, wk.rend, &wk.rnext_k, v.rec(), v.traces(), v.nt_max(),
+                          v.trace_step());
+        wk.next_event = event_after(wk, v, k);
     }
 
-    // After kUnroll planes the queue is rotated by kUnroll; rename it back.
-    static __device__ __forceinline__ void rotate_queue(Walk &wk) {
-        if constexpr (kUnroll % 9 != 0) {
-            float4 t[9];
-#pragma unroll
-            for (int m = 0; m < 9; ++m) t[m] = wk.q[(m + kUnroll) % 9];
-#pragma unroll
-            for (int m = 0; m < 9; ++m) wk.q[m] = t[m];
+    // Plane k of the item, RQ = (k - z0) mod kTrip (also the stage); parity:
+    // of the trip. Returns false when a bounded wait ran out.
+    template <int RQ, bool kLap, class VT>
+    static __device__ __forceinline__ bool plane_step(Walk &wk, B &br, unsigned aOwn, unsigned bOwn,
+                                                      unsigned ringA, unsigned ringB, const Job &jb,
+                                                      const VT &v, const Coeffs &c, unsigned *status,
+                                                      int k, int i, int j, unsigned parity,
+                                                      bool issuer_warp) {
+        constexpr int Q8 = (RQ + 8) % 9, Q4 = (RQ + 4) % 9;
+        constexpr unsigned RS = Cfg::kRowBytes, TB = Cfg::kTileBytes;
+        if (!__all_sync(0xffffffffu, mbar_try_wait(&br.full[RQ], parity))) {
+            const bool ok = wait_phase(&br.full[RQ], parity, &br.abort, status);
+            if (!__all_sync(0xffffffffu, ok)) return false;
         }
+        // u^n of plane k + 4 into the queue
+        wk.q[Q8][0] = lds4_at<0>(aOwn + wk.own);
+        wk.q[Q8][1] = lds4_at<RS>(aOwn + wk.own);
+        // u^n of plane k with its halo (in ring A for four planes already)
+        const unsigned h = aOwn + wk.halo;
+        const float4 xl0 = lds4_at<-16>(h), xr0 = lds4_at<16>(h);
+        const float4 xl1 = lds4_at<(int)RS - 16>(h), xr1 = lds4_at<(int)RS + 16>(h);
+        const float4 lm[4] = {lds4_at<-(int)RS>(h), lds4_at<-2 * (int)RS>(h),
+                              lds4_at<-3 * (int)RS>(h), lds4_at<-4 * (int)RS>(h)};
+        const float4 lp[4] = {lds4_at<2 * (int)RS>(h), lds4_at<3 * (int)RS>(h),
+                              lds4_at<4 * (int)RS>(h), lds4_at<5 * (int)RS>(h)};
+        // u^{n-1} and (V dt/h)^2 of plane k
+        constexpr int OB = RQ * Cfg::kSlotBBytes;
+        const float4 up0 = lds4_at<OB>(bOwn), up1 = lds4_at<OB + TX * 4>(bOwn);
+        const float4 w0 = lds4_at<OB + (int)TB>(bOwn), w1 = lds4_at<OB + (int)TB + TX * 4>(bOwn);
+        warp_arrive(&br.empty[RQ]);
+
+        float2 lap0[2], lap1[2];
+        {
+            const float4 yp[4] = {wk.q[Q4][1], lp[0], lp[1], lp[2]};
+            stencil_row<RQ>(wk, c, 0, xl0, xr0, yp, lm, lap0);
+        }
+        // Refill plane k's stage (and the ring-A slot of plane k) for plane
+        // k + P as soon as every warp has read it. Half way through the
+        // arithmetic the others usually have, so the lane does not wait, and
+        // the copy has 2 1/2 planes of time: 384^3 at 381 Gcell/s, against 366
+        // issued one plane later (the copy then has one), 358 right after the
+        // arrive (the lane waits for its neighbours) and 371 after the
+        // arithmetic. The vote that ends a failed walk is taken here, by this
+        // warp alone: at the end of every plane, by all warps, the CTAs drifted
+        // apart and it ran at 260.
+        if (issuer_warp && k + P < jb.it.z1) {
+            bool ok = true;
+            if ((threadIdx.x & 31) == 0) {
+                ok = wait_phase(&br.empty[RQ], parity, &br.abort, status);
+                if (ok) {
+                    br.issued++;
+                    issue(br, ringA, ringB, jb, k + P - jb.it.z0, wk.halo, RQ);
+                }
+            }
+            if (!__all_sync(0xffffffffu, ok)) return false;
+        }
+        {
+            const float4 ym[4] = {wk.q[Q4][0], lm[0], lm[1], lm[2]};
+            stencil_row<RQ>(wk, c, 1, xl1, xr1, lp, ym, lap1);
+        }
+        const float gzk = v.gz[k];
+        float4 out[2] = {update(lap0, wk.q[Q4][0], up0, w0, wk.gxy[0], gzk),
+                         update(lap1, wk.q[Q4][1], up1, w1, wk.gxy[1], gzk)};
+        if (k == wk.next_event) events(wk, v, k, i, j, out, w0, w1);
+        store_rows(wk, wk.out_k, v.g.pnx, out[0], out[1]);
+        if constexpr (kLap)   // the stencil sum, for the adjoint's imaging
+            store_rows(wk, wk.out_k + v.lap_delta, v.g.pnx,
+                       make_float4(lap0[0].x, lap0[0].y, lap0[1].x, lap0[1].y),
+                       make_float4(lap1[0].x, lap1[0].y, lap1[1].x, lap1[1].y));
+        wk.out_k += v.g.plane;
+        wk.halo = wk.halo == (NA - 1) * Cfg::kSlotABytes ? 0u : wk.halo + Cfg::kSlotABytes;
+        wk.own = wk.own == (NA - 1) * Cfg::kSlotABytes ? 0u : wk.own + Cfg::kSlotABytes;
+        return true;
     }
 
-    template <class S>
-    static __device__ void consumer(R &rg, const float *ringA, const float *ringB, const S &src,
-                                    const Coeffs &c, unsigned *status) {
-        const int tid = threadIdx.x;
-        const int tx = tid % (TX / 4);
-        const int ty = tid / (TX / 4);
-        const int offA = (kHalo + ty) * Cfg::kRowW + kHalo + 4 * tx;
-        const int offB = ty * TX + 4 * tx;
-        Walk wk;
-        wk.gAw = wk.gAr = wk.gB = 0;
-        wk.ok = true;
-        for (int item = blockIdx.x; item < src.nitems() && wk.ok; item += gridDim.x) {
-            typename S::V v;
-            const Item it = src.view(item, &v);
-            const Geom &g = v.g;
-            const int i = it.i0 + 4 * tx;
-            const int j = it.j0 + ty;
-            const bool col_ok = (j < g.ny) && (i < g.nx);
-            wk.nvalid = col_ok ? min(4, g.nx - i) : 0;
-            wk.gxy = make_float4(0.f, 0.f, 0.f, 0.f);
-            if (col_ok) {
-                const float gyj = v.gy[j];
-                wk.gxy.x = v.gx[i] * gyj;
-                if (wk.nvalid > 1) wk.gxy.y = v.gx[i + 1] * gyj;
-                if (wk.nvalid > 2) wk.gxy.z = v.gx[i + 2] * gyj;
-                if (wk.nvalid > 3) wk.gxy.w = v.gx[i + 3] * gyj;
-            }
-            wk.src_mask = 0u;
-            const SourceSample *srcs = v.src();
-            for (int qs = 0, ns = v.nsrc(); qs < ns; ++qs) {
-                const SourceSample ss = srcs[qs];
-                if (ss.i >= it.i0 && ss.i < it.i0 + TX && ss.j >= it.j0 && ss.j < it.j0 + TY &&
-                    ss.k >= it.z0 && ss.k < it.z1)
-                    wk.src_mask |= 1u << qs;
-            }
-            wk.rcur = wk.rend = 0;
-            if (v.rec_ptr != nullptr) {
-                const int r = it.tile * (Cfg::kConsumers / 32) + (tid >> 5);
-                wk.rend = v.rec_ptr[r + 1];
-                wk.rcur = first_entry(v.rec(), v.rec_ptr[r], wk.rend, it.z0);
-            }
-            wk.rnext_k = wk.rcur < wk.rend ? v.rec()[wk.rcur].k : INT_MAX;
-            wk.out_k = v.out + pidx(g, col_ok ? i : 0, col_ok ? j : 0, it.z0);
+    // After a trip of kTrip planes the queue is rotated by kTrip; rename it.
+    static __device__ __forceinline__ void rotate_queue(Walk &wk) {
+        float4 t[9][2];
 #pragma unroll
-            for (int d = 0; d < 2; ++d)
-                wk.gzb[d] = (it.z0 + d < it.z1) ? __ldg(v.gz + it.z0 + d) : 1.0f;
-
-            // queue prologue: planes z0-4 .. z0+3; the first four are only
-            // needed here and are released at once
+        for (int m = 0; m < 9; ++m) {
+            t[m][0] = wk.q[(m + kTrip) % 9][0];
+            t[m][1] = wk.q[(m + kTrip) % 9][1];
+        }
 #pragma unroll
-            for (int m = 0; m < 2 * kHalo; ++m) {
-                const float *sa = wait_a(wk, rg, ringA, wk.gAw, status);
-                wk.q[m] = lds4(sa + offA);
-                ++wk.gAw;
-            }
-#pragma unroll
-            for (int m = 0; m < kHalo; ++m) {
-                warp_arrive(&rg.emptyA[wk.gAr & (NA - 1)]);
-                ++wk.gAr;
-            }
-            if (!warp_all_ok(wk)) break;
-
-            for (int kb = it.z0; kb < it.z1; kb += kUnroll) {
-#define WS_PLANE(RQ)                                                                         \
-    if (kb + (RQ) >= it.z1) break;                                                           \
-    plane_step<RQ, S::kStoreLap>(wk, rg, ringA, ringB, v, c, status, it, kb + (RQ), i, j, offA, \
-                                 offB);                                                     \
-    if (!warp_all_ok(wk)) break;
-                WS_PLANE(0)
-                WS_PLANE(1)
-                WS_PLANE(2)
-                if constexpr (kUnroll == 9) {
-                    WS_PLANE(3)
-                    WS_PLANE(4)
-                    WS_PLANE(5)
-                    WS_PLANE(6)
-                    WS_PLANE(7)
-                    WS_PLANE(8)
-                }
-#undef WS_PLANE
-                rotate_queue(wk);
-            }
-            // the last four planes (z1 .. z1+3) were needed only for the queue
-#pragma unroll
-            for (int m = 0; m < kHalo; ++m) {
-                warp_arrive(&rg.emptyA[wk.gAr & (NA - 1)]);
-                ++wk.gAr;
-            }
+        for (int m = 0; m < 9; ++m) {
+            wk.q[m][0] = t[m][0];
+            wk.q[m][1] = t[m][1];
         }
     }
 };
 
-// The body of a launch: ring set-up, the warp roles, and the drain.
-template <int TX, int TY, int NA, int NB, class S>
+// The body of a launch: one CTA's item.
+template <int TX, int TY, class S>
 __device__ __forceinline__ void stream_body(const S &src, const Coeffs &c, unsigned *status) {
-    using K = Kern<TX, TY, NA, NB>;
+    using K = Kern<TX, TY>;
     using Cfg = typename K::Cfg;
+    constexpr int P = Cfg::P;
     extern __shared__ __align__(128) float smem[];
-    __shared__ Rings<NA, NB> rg;
-    float *ringA = smem;
-    float *ringB = smem + NA * Cfg::kSlotA;
+    __shared__ Bars<P> br;
+    const unsigned ringA = smem_addr(smem);
+    const unsigned ringB = ringA + Cfg::NA * Cfg::kSlotABytes;
+    const int tid = threadIdx.x;
+    // the copies' lane: of a warp that differs between neighbouring CTAs, so
+    // that the SM's sub-partitions share this work
+    const bool issuer_warp = tid / 32 == (int)(blockIdx.x % Cfg::kWarps);
+    const bool issuer = issuer_warp && (tid & 31) == 0;
 
-    if (threadIdx.x == 0) {
-        for (int s = 0; s < NA; ++s) {
-            mbar_init(&rg.fullA[s], 1);
-            mbar_init(&rg.emptyA[s], Cfg::kConsumers / 32);
-            rg.issuedA[s] = 0;
+    if (issuer) {
+        for (int s = 0; s < P; ++s) {
+            mbar_init(&br.full[s], 1);
+            mbar_init(&br.empty[s], Cfg::kWarps);
         }
-        for (int s = 0; s < NB; ++s) {
-            mbar_init(&rg.fullB[s], 1);
-            mbar_init(&rg.emptyB[s], Cfg::kConsumers / 32);
-            rg.issuedB[s] = 0;
-        }
-        rg.abort = 0;
+        mbar_init(&br.first, 1);
+        br.issued = 0;
+        br.first_issued = 0;
+        br.abort = 0;
         fence_mbar_init();
     }
     __syncthreads();
-
-    if (threadIdx.x >= Cfg::kConsumers) {
-        if (threadIdx.x == Cfg::kConsumers) K::producer(rg, ringA, ringB, src, status);
-    } else {
-        K::consumer(rg, ringA, ringB, src, c, status);
+    wait_predecessor();
+    const Job jb = src.job(blockIdx.x);
+    const Item &it = jb.it;
+    const int nb = it.z1 - it.z0;
+    if (issuer) {
+        if (!jb.stall) {   // else never filled: the bounded waits run out
+            br.first_issued = 1;
+            mbar_arrive_expect_tx(&br.first, kHalo * Cfg::kSlotABytes);
+            for (int m = 0; m < kHalo; ++m)
+                tma_load_3d_at(ringA + m * Cfg::kSlotABytes, jb.u, &br.first, it.i0 - kHalo,
+                               it.j0 - kHalo, it.z0 + m);
+        }
+        const int n = min(P, nb);
+        br.issued = n;
+        for (int r = 0; r < n; ++r) 
+            K::issue(br, ringA, ringB, jb, r, (kHalo + r) * Cfg::kSlotABytes, r);
     }
 
-    // After an abort, wait (bounded) for the last copy issued into each slot
-    // to land before the CTA exits.
+    typename S::V v;
+    src.view(blockIdx.x, &v);
+    const Geom &g = v.g;
+    const int tx = tid % Cfg::kCols, py = tid / Cfg::kCols;
+    const int i = it.i0 + 4 * tx, j = it.j0 + 2 * py;
+    const unsigned aOwn = ringA + 4u * ((kHalo + 2 * py) * Cfg::kRowW + kHalo + 4 * tx);
+    const unsigned bOwn = ringB + 4u * (2 * py * TX + 4 * tx);
+    const bool col_ok = (j < g.ny) && (i < g.nx);
+    Walk wk;
+    wk.nvalid = col_ok ? min(4, g.nx - i) : 0;
+    wk.row1 = col_ok && j + 1 < g.ny;
+    const long long at = pidx(g, col_ok ? i : 0, col_ok ? j : 0, it.z0);
+    // the queue's planes z0-4 .. z0-1: this thread's own cells only, from
+    // global memory (the planes below the grid are its zero halo)
+#pragma unroll
+    for (int m = 0; m < kHalo; ++m) {
+        const float *p = v.u + at + (m - kHalo) * g.plane;
+        const float4 z = make_float4(0.f, 0.f, 0.f, 0.f);
+        wk.q[m][0] = col_ok ? __ldcg(reinterpret_cast<const float4 *>(p)) : z;
+        wk.q[m][1] = wk.row1 ? __ldcg(reinterpret_cast<const float4 *>(p + g.pnx)) : z;
+    }
+#pragma unroll
+    for (int r = 0; r < 2; ++r) {
+        wk.gxy[r] = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (col_ok && (r == 0 || wk.row1)) {
+            const float gyj = v.gy[j + r];
+            wk.gxy[r].x = v.gx[i] * gyj;
+            if (wk.nvalid > 1) wk.gxy[r].y = v.gx[i + 1] * gyj;
+            if (wk.nvalid > 2) wk.gxy[r].z = v.gx[i + 2] * gyj;
+            if (wk.nvalid > 3) wk.gxy[r].w = v.gx[i + 3] * gyj;
+        }
+    }
+    wk.src_mask = 0u;
+    {
+        const SourceSample *srcs = v.src();
+        for (int qs = 0, ns = v.nsrc(); qs < ns; ++qs) {
+            const SourceSample ss = srcs[qs];
+            if (ss.i >= it.i0 && ss.i < it.i0 + TX && ss.j >= it.j0 && ss.j < it.j0 + TY &&
+                ss.k >= it.z0 && ss.k < it.z1)
+                wk.src_mask |= 1u << qs;
+        }
+    }
+    wk.rcur = wk.rend = 0;
+    if (v.rec_ptr != nullptr) {
+        const int r = it.tile * Cfg::kWarps + (tid >> 5);
+        wk.rend = v.rec_ptr[r + 1];
+        wk.rcur = first_entry(v.rec(), v.rec_ptr[r], wk.rend, it.z0);
+    }
+    wk.rnext_k = wk.rcur < wk.rend ? v.rec()[wk.rcur].k : INT_MAX;
+    wk.out_k = v.out + at;
+    wk.whole = __all_sync(0xffffffffu, wk.nvalid == 4 && wk.row1);
+    wk.next_event = K::event_after(wk, v, it.z0 - 1);
+    wk.halo = 0u;
+    wk.own = kHalo * Cfg::kSlotABytes;
+
+    bool ok = wait_phase(&br.first, 0u, &br.abort, status);
+    ok = __all_sync(0xffffffffu, ok);
+    if (ok) {
+#pragma unroll
+        for (int m = 0; m < kHalo; ++m) {   // planes z0 .. z0+3
+            wk.q[kHalo + m][0] = lds4_dyn(aOwn + m * Cfg::kSlotABytes);
+            wk.q[kHalo + m][1] = lds4_dyn(aOwn + m * Cfg::kSlotABytes + Cfg::kRowBytes);
+        }
+        unsigned parity = 0;
+        for (int kb = it.z0;; kb += kTrip, parity ^= 1u) {
+#define WS_PLANE(RQ)                                                                              \
+    if (kb + (RQ) >= it.z1 ||                                                                     \
+        !K::template plane_step<RQ, S::kStoreLap>(wk, br, aOwn, bOwn, ringA, ringB, jb, v, c,     \
+                                                  status, kb + (RQ), i, j, parity, issuer_warp))  \
+        break;
+            WS_PLANE(0)
+            WS_PLANE(1)
+            WS_PLANE(2)
+#undef WS_PLANE
+            K::rotate_queue(wk);
+        }
+    }
+
+    // After an abort, wait (bounded) for the last copies issued into each
+    // stage to land before the CTA exits.
     __syncthreads();
-    if (rg.abort && threadIdx.x == 0) {
-        for (int s = 0; s < NA + NB; ++s) {
-            const int cnt = s < NA ? rg.issuedA[s] : rg.issuedB[s - NA];
-            uint64_t *bar = s < NA ? &rg.fullA[s] : &rg.fullB[s - NA];
-            if (cnt == 0) continue;
+    if (br.abort && tid == 0) {
+        for (int s = 0; s <= P; ++s) {
+            // fills of stage s; the first planes as one more stage
+            const int n = s < P ? (br.issued + P - 1 - s) / P : br.first_issued;
+            uint64_t *bar = s < P ? &br.full[s] : &br.first;
+            if (n == 0) continue;
             const unsigned long long t0 = global_ns();
-            while (!mbar_try_wait(bar, (unsigned)(cnt - 1) & 1u) && global_ns() - t0 < kWaitLimitNs) {
+            while (!mbar_try_wait(bar, (unsigned)(n - 1) & 1u) && global_ns() - t0 < kWaitLimitNs) {
             }
         }
     }
 }
 
-template <int TX, int TY, int NA, int NB, int MINB, bool kLap>
-__global__ void __launch_bounds__(StreamCfg<TX, TY, NA, NB>::kThreads, MINB)
-    step_stream_kernel(const __grid_constant__ StreamMaps maps, float *__restrict__ up,
+template <int TX, int TY, int MINB, bool kLap>
+__global__ void __launch_bounds__(StreamCfg<TX, TY>::kThreads, MINB)
+    step_stream_kernel(const __grid_constant__ StreamMaps maps, const float *u, float *up,
                        const __grid_constant__ StepArgs a, const int zb, const int tiles_x,
-                       const int ntiles, const int nitems, const int *__restrict__ rec_ptr,
+                       const int ntiles, const int *__restrict__ rec_ptr,
                        const RecEntry *__restrict__ rec) {
-    const OneGrid<TX, TY, kLap> src{maps, a, up, zb, tiles_x, ntiles, nitems, rec_ptr, rec};
-    stream_body<TX, TY, NA, NB>(src, a.c, a.status);
+    const OneGrid<TX, TY, kLap> src{maps, a, u, up, zb, tiles_x, ntiles, rec_ptr, rec};
+    stream_body<TX, TY>(src, a.c, a.status);
 }
 
-template <int TX, int TY, int NA, int NB, int MINB>
-__global__ void __launch_bounds__(StreamCfg<TX, TY, NA, NB>::kThreads, MINB)
+template <int TX, int TY, int MINB>
+__global__ void __launch_bounds__(StreamCfg<TX, TY>::kThreads, MINB)
     step_batch_kernel(const BatchShot *__restrict__ shots, const int2 *__restrict__ items,
-                      const int nitems, const int t, const Coeffs c, unsigned *status) {
-    const ShotBatch<TX, TY> src{shots, items, nitems, t};
-    stream_body<TX, TY, NA, NB>(src, c, status);
+                      const int t, const Coeffs c, unsigned *status) {
+    const ShotBatch<TX, TY> src{shots, items, t};
+    stream_body<TX, TY>(src, c, status);
 }
 
 // Resident CTAs per SM and SM count of a kernel on the current device,
@@ -598,55 +632,44 @@ cudaError_t occupancy(KernFn kern, int threads, size_t smem, LaunchFacts &lf, in
     return cudaSuccess;
 }
 
-template <int TX, int TY, int NA, int NB, int MINB, bool kLap>
-cudaError_t launch_tile_as(const StreamMaps &maps, float *up, const StepArgs &a, int zb,
-                           const int *rec_ptr, const RecEntry *rec, cudaStream_t s) {
-    using Cfg = StreamCfg<TX, TY, NA, NB>;
-    auto kern = step_stream_kernel<TX, TY, NA, NB, MINB, kLap>;
-    static LaunchFacts lf;
-    int ctas_per_sm = 0, sms = 0;
-    cudaError_t e = occupancy(kern, Cfg::kThreads, Cfg::kSmem, lf, &ctas_per_sm, &sms);
-    if (e != cudaSuccess) return e;
-    const int tiles_x = (a.g.nx + TX - 1) / TX;
-    const int ntiles = tiles_x * ((a.g.ny + TY - 1) / TY);
-    const int nitems = ntiles * ((a.g.nz + zb - 1) / zb);
-    // one CTA per item (see the header: in-order dispatch keeps neighbours' halos in L2)
-    kern<<<nitems, Cfg::kThreads, Cfg::kSmem, s>>>(maps, up, a, zb, tiles_x, ntiles, nitems, rec_ptr,
-                                                   rec);
-    return cudaGetLastError();
+// Calls fn with the configuration of tile tx x ty: (TX, TY, resident CTAs per
+// SM that its registers and rings allow).
+template <int TX, int TY, int MINB>
+struct TileTag {
+    static constexpr int kX = TX, kY = TY, kMin = MINB;
+};
+template <class F>
+cudaError_t with_tile(int tx, int ty, F &&fn) {
+    if (tx == 64 && ty == 32) return fn(TileTag<64, 32, 1>{});
+    if (tx == 64 && ty == 16) return fn(TileTag<64, 16, 3>{});
+    if (tx == 64 && ty == 8) return fn(TileTag<64, 8, 5>{});
+    if (tx == 32 && ty == 16) return fn(TileTag<32, 16, 5>{});
+    if (tx == 32 && ty == 8) return fn(TileTag<32, 8, 8>{});
+    return cudaErrorInvalidValue;
 }
 
-template <int TX, int TY, int NA, int NB, int MINB>
-cudaError_t launch_tile(const StreamMaps &maps, float *up, const StepArgs &a, int zb,
+template <class T, bool kLap>
+cudaError_t launch_grid(const StreamMaps &maps, const float *u, float *up, const StepArgs &a, int zb,
                         const int *rec_ptr, const RecEntry *rec, cudaStream_t s) {
-    if (a.lap) return launch_tile_as<TX, TY, NA, NB, MINB, true>(maps, up, a, zb, rec_ptr, rec, s);
-    return launch_tile_as<TX, TY, NA, NB, MINB, false>(maps, up, a, zb, rec_ptr, rec, s);
-}
-
-template <int TX, int TY, int NA, int NB, int MINB>
-cudaError_t slots_of(bool batch, int *slots) {
-    using Cfg = StreamCfg<TX, TY, NA, NB>;
-    static LaunchFacts lf_grid, lf_batch;
-    int c = 0, n = 0;
-    cudaError_t e = batch ? occupancy(step_batch_kernel<TX, TY, NA, NB, MINB>, Cfg::kThreads,
-                                      Cfg::kSmem, lf_batch, &c, &n)
-                          : occupancy(step_stream_kernel<TX, TY, NA, NB, MINB, false>,
-                                      Cfg::kThreads, Cfg::kSmem, lf_grid, &c, &n);
-    if (e == cudaSuccess) *slots = c * n;
-    return e;
-}
-
-template <int TX, int TY, int NA, int NB, int MINB>
-cudaError_t launch_batch_tile(const BatchShot *shots, const int2 *items, int nitems, int t,
-                              const Coeffs &c, unsigned *status, cudaStream_t s) {
-    using Cfg = StreamCfg<TX, TY, NA, NB>;
-    auto kern = step_batch_kernel<TX, TY, NA, NB, MINB>;
+    using Cfg = StreamCfg<T::kX, T::kY>;
+    auto kern = step_stream_kernel<T::kX, T::kY, T::kMin, kLap>;
     static LaunchFacts lf;
     int ctas_per_sm = 0, sms = 0;
     cudaError_t e = occupancy(kern, Cfg::kThreads, Cfg::kSmem, lf, &ctas_per_sm, &sms);
     if (e != cudaSuccess) return e;
-    kern<<<nitems, Cfg::kThreads, Cfg::kSmem, s>>>(shots, items, nitems, t, c, status);
-    return cudaGetLastError();
+    const int tiles_x = (a.g.nx + T::kX - 1) / T::kX;
+    const int ntiles = tiles_x * ((a.g.ny + T::kY - 1) / T::kY);
+    const int nitems = ntiles * ((a.g.nz + zb - 1) / zb);
+    return launch_overlapped(kern, nitems, Cfg::kThreads, Cfg::kSmem, s, maps, u, up, a, zb, tiles_x,
+                             ntiles, rec_ptr, rec);
+}
+
+template <class T>
+cudaError_t batch_facts(int *ctas_per_sm, int *sms) {
+    static LaunchFacts lf;
+    using Cfg = StreamCfg<T::kX, T::kY>;
+    return occupancy(step_batch_kernel<T::kX, T::kY, T::kMin>, Cfg::kThreads, Cfg::kSmem, lf,
+                     ctas_per_sm, sms);
 }
 
 }  // namespace
@@ -656,46 +679,47 @@ bool stream_tiling_supported(int tx, int ty) {
 }
 
 cudaError_t launch_step_stream(const CUtensorMap *tmap_u, const CUtensorMap *tmap_up,
-                               const CUtensorMap *tmap_w, float *up, const StepArgs &a,
-                               const StreamTiling &t, const int *rec_ptr, const RecEntry *rec,
-                               cudaStream_t s) {
+                               const CUtensorMap *tmap_w, const float *u, float *up,
+                               const StepArgs &a, const StreamTiling &t, const int *rec_ptr,
+                               const RecEntry *rec, cudaStream_t s) {
     StreamMaps maps;
     maps.u = *tmap_u;
     maps.up = *tmap_up;
     maps.w = *tmap_w;
-    // ring sizes chosen so that the CTAs of one SM fit in its shared memory
-    if (t.tx == 64 && t.ty == 32) return launch_tile<64, 32, 8, 4, 1>(maps, up, a, t.zb, rec_ptr, rec, s);
-    if (t.tx == 64 && t.ty == 16) return launch_tile<64, 16, 8, 4, 2>(maps, up, a, t.zb, rec_ptr, rec, s);
-    if (t.tx == 64 && t.ty == 8) return launch_tile<64, 8, 8, 4, 3>(maps, up, a, t.zb, rec_ptr, rec, s);
-    if (t.tx == 32 && t.ty == 16)
-        return launch_tile<32, 16, WS_RING_A, 4, 3>(maps, up, a, t.zb, rec_ptr, rec, s);
-    if (t.tx == 32 && t.ty == 8) return launch_tile<32, 8, 8, 4, 4>(maps, up, a, t.zb, rec_ptr, rec, s);
-    return cudaErrorInvalidValue;
+    return with_tile(t.tx, t.ty, [&](auto tag) {
+        using T = decltype(tag);
+        if (a.lap) return launch_grid<T, true>(maps, u, up, a, t.zb, rec_ptr, rec, s);
+        return launch_grid<T, false>(maps, u, up, a, t.zb, rec_ptr, rec, s);
+    });
 }
 
-}  // namespace ws
-
-namespace ws {
-
-cudaError_t stream_slots(int tx, int ty, bool batch, int *slots) {
-    if (tx == 64 && ty == 32) return slots_of<64, 32, 8, 4, 1>(batch, slots);
-    if (tx == 64 && ty == 16) return slots_of<64, 16, 8, 4, 2>(batch, slots);
-    if (tx == 64 && ty == 8) return slots_of<64, 8, 8, 4, 3>(batch, slots);
-    if (tx == 32 && ty == 16) return slots_of<32, 16, WS_RING_A, 4, 3>(batch, slots);
-    if (tx == 32 && ty == 8) return slots_of<32, 8, 8, 4, 4>(batch, slots);
-    return cudaErrorInvalidValue;
+cudaError_t stream_slots(int tx, int ty, bool batch, int *slots, int *sms) {
+    return with_tile(tx, ty, [&](auto tag) {
+        using T = decltype(tag);
+        using Cfg = StreamCfg<T::kX, T::kY>;
+        static LaunchFacts lf;
+        int c = 0, n = 0;
+        cudaError_t e = batch ? batch_facts<T>(&c, &n)
+                              : occupancy(step_stream_kernel<T::kX, T::kY, T::kMin, false>,
+                                          Cfg::kThreads, Cfg::kSmem, lf, &c, &n);
+        if (e == cudaSuccess) *slots = c * n;
+        if (e == cudaSuccess && sms) *sms = n;
+        return e;
+    });
 }
 
 cudaError_t launch_step_batch(const BatchShot *shots, const int2 *items, int nitems, int t,
                               const Coeffs &c, unsigned *status, int tx, int ty, cudaStream_t s) {
     if (nitems <= 0) return cudaSuccess;
-    if (tx == 64 && ty == 32) return launch_batch_tile<64, 32, 8, 4, 1>(shots, items, nitems, t, c, status, s);
-    if (tx == 64 && ty == 16) return launch_batch_tile<64, 16, 8, 4, 2>(shots, items, nitems, t, c, status, s);
-    if (tx == 64 && ty == 8) return launch_batch_tile<64, 8, 8, 4, 3>(shots, items, nitems, t, c, status, s);
-    if (tx == 32 && ty == 16)
-        return launch_batch_tile<32, 16, WS_RING_A, 4, 3>(shots, items, nitems, t, c, status, s);
-    if (tx == 32 && ty == 8) return launch_batch_tile<32, 8, 8, 4, 4>(shots, items, nitems, t, c, status, s);
-    return cudaErrorInvalidValue;
+    return with_tile(tx, ty, [&](auto tag) {
+        using T = decltype(tag);
+        using Cfg = StreamCfg<T::kX, T::kY>;
+        int ctas_per_sm = 0, sms = 0;
+        cudaError_t e = batch_facts<T>(&ctas_per_sm, &sms);
+        if (e != cudaSuccess) return e;
+        return launch_overlapped(step_batch_kernel<T::kX, T::kY, T::kMin>, nitems, Cfg::kThreads,
+                                 Cfg::kSmem, s, shots, items, t, c, status);
+    });
 }
 
 }  // namespace ws

@@ -198,14 +198,6 @@ __device__ __forceinline__ uint2 lds2_at(unsigned a) {
     return v;
 }
 template <int OFF>
-__device__ __forceinline__ float4 lds4_at(unsigned a) {
-    float4 v;
-    asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];"
-                 : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
-                 : "r"(a + static_cast<unsigned>(OFF)));
-    return v;
-}
-template <int OFF>
 __device__ __forceinline__ void sts4_at(unsigned a, float4 v) {
     asm volatile("st.shared.v4.f32 [%0+%1], {%2, %3, %4, %5};" ::"r"(a), "n"(OFF), "f"(v.x),
                  "f"(v.y), "f"(v.z), "f"(v.w)
@@ -245,43 +237,6 @@ __device__ __forceinline__ int scale_exponent(float a) {
     int k;
     frexpf(a, &k);
     return max(-100, min(100, 12 - k));
-}
-
-// Receivers of a two-row thread: RecEntry.lane = 4 * row + x cell. Lane q of
-// the warp takes entry cur + q, fetches the owner's 8 values by shuffle and
-// stores the one it names.
-__device__ __forceinline__ void record_plane2(const float4 (&out)[2], int k, int *rcur, int rend,
-                                              int *rnext_k, const RecEntry *rec, float *traces,
-                                              int nt_max, long long trace_step) {
-    const int lane = threadIdx.x & 31;
-    int cur = *rcur;
-    for (;;) {
-        const int idx = cur + lane;
-        RecEntry e{INT_MAX, 0, 0, 0};
-        if (idx < rend) e = rec[idx];
-        const bool take = e.k == k;
-        const int src = e.owner & 31;
-        float v[8];
-#pragma unroll
-        for (int r = 0; r < 2; ++r) {
-            v[4 * r + 0] = __shfl_sync(0xffffffffu, out[r].x, src);
-            v[4 * r + 1] = __shfl_sync(0xffffffffu, out[r].y, src);
-            v[4 * r + 2] = __shfl_sync(0xffffffffu, out[r].z, src);
-            v[4 * r + 3] = __shfl_sync(0xffffffffu, out[r].w, src);
-        }
-        if (take) {
-            float x = v[0];
-#pragma unroll
-            for (int l = 1; l < 8; ++l)
-                if (e.lane == l) x = v[l];
-            traces[(long long)e.r * nt_max + trace_step] = x;
-        }
-        const int n = __popc(__ballot_sync(0xffffffffu, take));
-        cur += n;
-        if (n < 32) break;
-    }
-    *rcur = cur;
-    *rnext_k = cur < rend ? rec[cur].k : INT_MAX;
 }
 
 // Rarely taken paths of a plane, kept as small inlined helpers.
@@ -604,7 +559,7 @@ struct Kern16 {
             dn[0] = delta_fast(lap0, d0, w0);
             dn[1] = delta_fast(lap1, d1, w1);
         } else {
-            const float gzk = __ldg(cx.gz + k);
+            const float gzk = cx.gz[k];
             dn[0] = delta_taper(lap0, d0, w0, wk.q[Q4][0], cx.gxy[0], gzk);
             dn[1] = delta_taper(lap1, d1, w1, wk.q[Q4][1], cx.gxy[1], gzk);
         }
@@ -689,8 +644,8 @@ template <class Fmt, int TX, int TY, int NA, int NB>
 __global__ void __launch_bounds__(Cfg16<TX, TY, NA, NB>::kThreads, Cfg16<TX, TY, NA, NB>::kMinBlocks)
     step_stream16_kernel(const __grid_constant__ Maps16 maps, uint16_t *u_out, uint16_t *d_io,
                          const __grid_constant__ StepArgs a,
-                         Scale16 *__restrict__ sc, const long long step, const float src_hint,
-                         const Free16 fr, const int zb, const int tiles_x, const int ntiles,
+                         Scale16 *sc, const long long step, const float src_hint,
+                         const int zb, const int tiles_x, const int ntiles,
                          const int *__restrict__ rec_ptr, const RecEntry *__restrict__ rec) {
     using K = Kern16<Fmt, TX, TY, NA, NB>;
     using Cfg = typename K::Cfg;
@@ -700,8 +655,10 @@ __global__ void __launch_bounds__(Cfg16<TX, TY, NA, NB>::kThreads, Cfg16<TX, TY,
     uint16_t *ringA = reinterpret_cast<uint16_t *>(smem16 + 2 * Cfg::kStage);
     uint16_t *ringB = ringA + NA * Cfg::kSlotA;
     const Geom &g = a.g;
+    const FreeBox &fr = a.fr;
     const int tid = threadIdx.x;
 
+    wait_predecessor();
     // scale of this step: U, D of step n have e; U', D' get e_o
     const int sn = (int)(step & 3), so = (int)((step + 1) & 3);
     const int e = sc->e[sn];
@@ -903,7 +860,7 @@ cudaError_t facts16(int *ctas, int *sms) {
 
 template <class Fmt, int TX, int TY, int NA, int NB>
 cudaError_t launch16(const Maps16 &maps, uint16_t *u_out, uint16_t *d_io, const StepArgs &a,
-                     Scale16 *sc, long long step, float src_hint, const Free16 &fr, int zb,
+                     Scale16 *sc, long long step, float src_hint, int zb,
                      const int *rec_ptr, const RecEntry *rec, cudaStream_t s) {
     using Cfg = Cfg16<TX, TY, NA, NB>;
     auto kern = step_stream16_kernel<Fmt, TX, TY, NA, NB>;
@@ -913,9 +870,8 @@ cudaError_t launch16(const Maps16 &maps, uint16_t *u_out, uint16_t *d_io, const 
     const int tiles_x = (a.g.nx + TX - 1) / TX;
     const int ntiles = tiles_x * ((a.g.ny + TY - 1) / TY);
     const int nitems = ntiles * ((a.g.nz + zb - 1) / zb);
-    kern<<<nitems, Cfg::kThreads, Cfg::kSmem, s>>>(maps, u_out, d_io, a, sc, step, src_hint, fr,
-                                                   zb, tiles_x, ntiles, rec_ptr, rec);
-    return cudaGetLastError();
+    return launch_overlapped(kern, nitems, Cfg::kThreads, Cfg::kSmem, s, maps, u_out, d_io, a, sc,
+                             step, src_hint, zb, tiles_x, ntiles, rec_ptr, rec);
 }
 
 }  // namespace
@@ -956,8 +912,8 @@ Weights16 zero_sum_weights16() {
 }
 
 cudaError_t launch_step_stream16(int storage, const Maps16In &m, const StepArgs &a, Scale16 *sc,
-                                 long long step, float src_hint, const Free16 &fr,
-                                 const StreamTiling &t, const int *rec_ptr, const RecEntry *rec,
+                                 long long step, float src_hint, const StreamTiling &t,
+                                 const int *rec_ptr, const RecEntry *rec,
                                  cudaStream_t s) {
     // the kernel's compile-time weights must be those of zero_sum_weights16
     static const bool weights_ok = [] {
@@ -974,7 +930,7 @@ cudaError_t launch_step_stream16(int storage, const Maps16In &m, const StepArgs 
     // ring A 9 slots (the planes of one loop trip), ring B 3; 64 x 16 tiles
     // run 3 CTAs per SM, 64 x 24 two, 64 x 48 one (12 warps in all)
 #define WS_LAUNCH16(FMT, TY)                                                                     \
-    return launch16<FMT, 64, TY, 9, 3>(maps, m.u_out, m.d_io, a, sc, step, src_hint, fr, t.zb, \
+    return launch16<FMT, 64, TY, 9, 3>(maps, m.u_out, m.d_io, a, sc, step, src_hint, t.zb, \
                                        rec_ptr, rec, s)
     if (storage == WS_STORAGE_BF16) {
         if (t.ty == 16) WS_LAUNCH16(Bf16Fmt, 16);

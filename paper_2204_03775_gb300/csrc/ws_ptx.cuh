@@ -3,6 +3,7 @@
 #pragma once
 
 #include <climits>
+#include <utility>
 
 #include "ws_internal.h"
 
@@ -14,6 +15,39 @@ struct LaunchFacts {
     int ctas[kMaxDevices] = {};
     int sms[kMaxDevices] = {};
 };
+
+// Overlap of a step with the end of the one before it on the same stream
+// (programmatic dependent launch). A kernel launched with launch_overlapped
+// may start while its predecessor still runs: every thread calls
+// wait_predecessor before it touches global memory (it returns once all
+// earlier work of the stream is complete and visible), then lets its own
+// successor start, whose blocks fill the slots that the last wave leaves free.
+// Since the release comes after the wait, at most two kernels of a stream
+// overlap and a successor never runs ahead of anything but its predecessor.
+// Loads of what a predecessor writes are plain or L2 ones, never read-only
+// (nc) ones, which may not see writes made during the kernel's lifetime.
+// What it saves is the launch latency between two dependent kernels, a few
+// microseconds a step: see the rule at each launch.
+static __device__ __forceinline__ void wait_predecessor() {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
+template <class... Params, class... Args>
+static cudaError_t launch_overlapped(void (*kern)(Params...), dim3 grid, dim3 block, size_t smem,
+                                     cudaStream_t s, Args &&...args) {
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t c{};
+    c.gridDim = grid;
+    c.blockDim = block;
+    c.dynamicSmemBytes = smem;
+    c.stream = s;
+    c.attrs = &at;
+    c.numAttrs = 1;
+    return cudaLaunchKernelEx(&c, kern, std::forward<Args>(args)...);
+}
 
 static __device__ __forceinline__ unsigned smem_addr(const void *p) {
     return static_cast<unsigned>(__cvta_generic_to_shared(p));
@@ -61,16 +95,31 @@ static __device__ __forceinline__ void tma_load_3d(void *dst, const CUtensorMap 
         : "memory");
 }
 
+static __device__ __forceinline__ void tma_load_3d_at(unsigned dst, const CUtensorMap *map,
+                                               uint64_t *bar, int x, int y, int z) {
+    asm volatile(
+        "cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes"
+        " [%0], [%1, {%2, %3, %4}], [%5];" ::"r"(dst),
+        "l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y), "r"(z), "r"(smem_addr(bar))
+        : "memory");
+}
+
 // 128-bit shared-memory load, kept whole: a warp reading 16-byte cells at
 // 16-byte stride is conflict-free only as one 128-bit access per thread (two
 // 64-bit halves would each hit every bank twice). Volatile, so it stays after
 // the barrier wait that guards the data.
-static __device__ __forceinline__ float4 lds4(const float *p) {
+static __device__ __forceinline__ float4 lds4_dyn(unsigned a) {
     float4 v;
     asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];"
                  : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
-                 : "r"(smem_addr(p)));
+                 : "r"(a));
     return v;
+}
+// The same at a 32-bit shared address plus a compile-time byte offset
+// (negative offsets wrap modulo 2^32, which is the same address).
+template <int OFF>
+static __device__ __forceinline__ float4 lds4_at(unsigned a) {
+    return lds4_dyn(a + static_cast<unsigned>(OFF));
 }
 
 static __device__ __forceinline__ float comp(const float4 &v, int l) {
@@ -150,9 +199,8 @@ static __device__ __forceinline__ Item item_of(int item, int tiles_x, int ntiles
 // Receivers: each warp of a streaming CTA owns a range of the receiver
 // table sorted by plane k (the receivers whose cell one of its threads
 // computes). first_entry skips to the first entry at or below plane z0 by
-// binary search; record_plane stores the values of plane k: lane q takes
-// entry cur + q, fetches the owning thread's cell by shuffle, and stores it.
-// Every lane of the warp calls both with the same range.
+// binary search; record_plane2 stores the values of plane k. Every lane of the
+// warp calls both with the same range.
 static __device__ __forceinline__ int first_entry(const RecEntry *rec, int lo, int hi, int z0) {
     while (lo < hi) {
         const int mid = (lo + hi) >> 1;
@@ -164,10 +212,12 @@ static __device__ __forceinline__ int first_entry(const RecEntry *rec, int lo, i
     return lo;
 }
 
-static __device__ __forceinline__ void record_plane(const float4 &out, float scale, int k,
-                                                    int *rcur, int rend, int *rnext_k,
-                                                    const RecEntry *rec, float *traces, int nt_max,
-                                                    long long trace_step) {
+// Receivers of a two-row thread: RecEntry.lane = 4 * row + x cell. Lane q of
+// the warp takes entry cur + q, fetches the owner's 8 values by shuffle and
+// stores the one it names.
+static __device__ __forceinline__ void record_plane2(const float4 (&out)[2], int k, int *rcur, int rend,
+                                              int *rnext_k, const RecEntry *rec, float *traces,
+                                              int nt_max, long long trace_step) {
     const int lane = threadIdx.x & 31;
     int cur = *rcur;
     for (;;) {
@@ -176,13 +226,20 @@ static __device__ __forceinline__ void record_plane(const float4 &out, float sca
         if (idx < rend) e = rec[idx];
         const bool take = e.k == k;
         const int src = e.owner & 31;
-        const float v0 = __shfl_sync(0xffffffffu, out.x, src);
-        const float v1 = __shfl_sync(0xffffffffu, out.y, src);
-        const float v2 = __shfl_sync(0xffffffffu, out.z, src);
-        const float v3 = __shfl_sync(0xffffffffu, out.w, src);
+        float v[8];
+#pragma unroll
+        for (int r = 0; r < 2; ++r) {
+            v[4 * r + 0] = __shfl_sync(0xffffffffu, out[r].x, src);
+            v[4 * r + 1] = __shfl_sync(0xffffffffu, out[r].y, src);
+            v[4 * r + 2] = __shfl_sync(0xffffffffu, out[r].z, src);
+            v[4 * r + 3] = __shfl_sync(0xffffffffu, out[r].w, src);
+        }
         if (take) {
-            const float v = e.lane == 0 ? v0 : e.lane == 1 ? v1 : e.lane == 2 ? v2 : v3;
-            traces[(long long)e.r * nt_max + trace_step] = v * scale;
+            float x = v[0];
+#pragma unroll
+            for (int l = 1; l < 8; ++l)
+                if (e.lane == l) x = v[l];
+            traces[(long long)e.r * nt_max + trace_step] = x;
         }
         const int n = __popc(__ballot_sync(0xffffffffu, take));
         cur += n;
@@ -191,23 +248,6 @@ static __device__ __forceinline__ void record_plane(const float4 &out, float sca
     *rcur = cur;
     *rnext_k = cur < rend ? rec[cur].k : INT_MAX;
 }
-
-// A consumer leaves its loops only together with its whole warp (the
-// receiver shuffles and the warp-wide arrives need every lane): after a
-// failed wait in any lane, every lane's walk stops.
-template <class W>
-static __device__ __forceinline__ bool warp_all_ok(W &wk) {
-    wk.ok = __all_sync(0xffffffffu, wk.ok);
-    return wk.ok;
-}
-
-// Shared-memory state of one CTA.
-template <int NA, int NB>
-struct Rings {
-    uint64_t fullA[NA], emptyA[NA], fullB[NB], emptyB[NB];
-    int issuedA[NA], issuedB[NB];   // copies issued into each slot (for the drain)
-    int abort;
-};
 
 // Bounded wait for a phase of an mbarrier. Gives up after kWaitLimitNs, or
 // early once another warp has aborted; returns false then.

@@ -1,0 +1,63 @@
+"""Kernel and tiling choice (GPU): whatever kernel, tile and z block a step
+takes, the fields and the traces are the same bits."""
+
+import numpy as np
+import pytest
+
+import paper_2204_03775_gb300 as wsb
+from paper_2204_03775_gb300 import synthetic
+
+pytestmark = pytest.mark.gpu
+
+NT = 14
+
+
+def _run(shape, kernel, tile=(0, 0), zblock=0):
+    """Fields and traces after NT steps of a tapered model with sources and
+    receivers on faces, edges, tile borders and in one column."""
+    nz, ny, nx = shape
+    vel = synthetic.smooth_random_velocity(shape, 11, 1500.0, 4500.0, spacing=4)
+    h = wsb.ws_create(nx, ny, nz, 10.0, synthetic.cfl_dt(4500.0, 10.0))
+    wsb.ws_set_kernel(h, kernel, *tile, zblock)
+    wsb.ws_set_velocity(h, vel)
+    wsb.ws_set_sponge(h, 3, 0.2)
+    cells = [(0, 0, 0), (nx - 1, ny - 1, nz - 1), (nx // 2, ny // 2, nz // 2),
+             (min(63, nx - 1), min(15, ny - 1), 0), (min(64, nx - 1), min(16, ny - 1), nz - 1),
+             (nx // 2, min(7, ny - 1), nz // 3), (nx // 2, min(8, ny - 1), nz // 3)]
+    for n, c in enumerate(cells):
+        wsb.ws_add_source(h, *c, 20.0, 0.01 + 0.001 * n, 1.0 + n)
+    rec = cells + cells[:2] + [(nx // 2, ny // 2, k) for k in range(nz)] \
+        + [(i, ny // 2, nz // 2) for i in range(0, nx, 3)]
+    wsb.ws_set_receivers(h, np.array(rec, np.int32), NT)
+    wsb.ws_step(h, 5)
+    wsb.ws_step(h, NT - 5)
+    wsb.ws_synchronize(h)
+    u, p = wsb.ws_read_field(h)
+    return u, p, wsb.ws_read_traces(h)
+
+
+@pytest.mark.parametrize("tile", [(64, 16), (64, 8), (64, 32), (32, 16), (32, 8)])
+@pytest.mark.parametrize("shape", [(9, 32, 64), (10, 33, 65), (13, 47, 131), (5, 34, 98)])
+def test_every_tile_gives_the_direct_kernels_bits(tile, shape):
+    ref = _run(shape, wsb.WS_KERNEL_DIRECT)
+    assert np.abs(ref[2]).max() > 0
+    for zblock in (0, 1, 2, 3, 4, 7, shape[0]):
+        for r, x in zip(ref, _run(shape, wsb.WS_KERNEL_STREAM, tile, zblock)):
+            assert np.array_equal(r, x)
+
+
+@pytest.mark.parametrize("shape", [(20, 99, 101), (20, 100, 101), (40, 40, 48), (6, 12, 80),
+                                   (7, 40, 33), (3, 5, 300)])
+def test_default_choice_gives_the_direct_kernels_bits(shape):
+    """Grids on both sides of the direct kernel's limit, low and narrow ones."""
+    ref = _run(shape, wsb.WS_KERNEL_DIRECT)
+    for r, x in zip(ref, _run(shape, wsb.WS_KERNEL_AUTO)):
+        assert np.array_equal(r, x)
+    nz, ny, nx = shape
+    if nx >= 64 and ny >= 8:      # STREAM without a tile needs 64 x 8, as ever
+        for r, x in zip(ref, _run(shape, wsb.WS_KERNEL_STREAM)):
+            assert np.array_equal(r, x)
+    else:
+        h = wsb.ws_create(nx, ny, nz, 10.0, 1e-3)
+        with pytest.raises(wsb.WaveStepError):
+            wsb.ws_set_kernel(h, wsb.WS_KERNEL_STREAM)
