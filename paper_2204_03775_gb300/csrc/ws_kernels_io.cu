@@ -4,7 +4,7 @@
 // Copies: bound by HBM, 8 bytes a cell and field. One launch moves both time levels.
 // (One 2D copy per plane and field, which this replaces, cost 4 to 8 us a
 // plane whatever its size: 256^3 in and out 4.2 ms, 1024^3 35 ms.)
-#include "ws_internal.h"
+#include "ws_model.cuh"
 
 namespace ws {
 
@@ -235,60 +235,6 @@ cudaError_t launch_copy_out(const float *A, const float *B, float *a, float *b, 
 
 namespace {
 
-// (V dt / h)^2 from V, and (dt / h)^2 / m from m = 1/V^2, each the double
-// result rounded to float. GB300 runs FP64 at a small fraction of FP32, so
-// the value is formed as a sum q + q2 of two floats (error below 2^-44 of it:
-// the scale as two floats, products and remainders exact through fma), whose
-// nearest float is that of the double result unless both lie within 2^-42 of
-// a tie between two floats; then, and outside the range in which no term
-// underflows, the double expression itself is evaluated (about one cell in
-// 2^18). The stored floats are the same bits either way.
-struct Scale {
-    double c;       // dt / h, or (dt / h)^2
-    float hi, lo;   // c as two floats
-    bool fast;      // hi in [2^-60, 2^60]
-};
-
-Scale scale_of(double c) {
-    Scale s{c, (float)c, 0.0f, false};
-    s.lo = (float)(c - (double)s.hi);
-    s.fast = s.hi >= 0x1p-60f && s.hi <= 0x1p60f;
-    return s;
-}
-
-// The nearest float of q + q2 if the sum moved by +-2^-42 q rounds alike.
-__device__ __forceinline__ bool round_sum(float q, float q2, float *w) {
-    const float a = q + fmaf(q, 0x1p-42f, q2), b = q + fmaf(q, -0x1p-42f, q2);
-    *w = a;
-    return a == b && q >= 0x1p-60f && q <= 0x1p60f;
-}
-
-struct FromVelocity {
-    // (a call: inlined, its two products were issued for every cell)
-    static __device__ __noinline__ float slow(float v, double c) {
-        const double r = __dmul_rn((double)v, c);   // as ws_energy_noalloc forms it
-        return (float)__dmul_rn(r, r);
-    }
-    static __device__ __forceinline__ bool fast(float v, const Scale &k, float *w) {
-        const float p = __fmul_rn(v, k.hi);
-        const float l = fmaf(v, k.lo, fmaf(v, k.hi, -p));
-        const float s = __fadd_rn(p, l), t = __fsub_rn(l, __fsub_rn(s, p));   // V dt / h = s + t
-        const float q = __fmul_rn(s, s);
-        return round_sum(q, fmaf(2.0f * s, t, fmaf(s, s, -q)), w) && k.fast;
-    }
-};
-
-struct FromSlowness2 {
-    static __device__ __noinline__ float slow(float m, double c) {
-        return (float)(c / (double)m);
-    }
-    static __device__ __forceinline__ bool fast(float m, const Scale &k, float *w) {
-        const float q = __fdiv_rn(k.hi, m);
-        const float r = __fadd_rn(fmaf(-q, m, k.hi), k.lo);   // c - q m
-        return round_sum(q, __fdividef(r, m), w) && k.fast && m >= 0x1p-100f && m <= 0x1p100f;
-    }
-};
-
 struct Extrema {
     unsigned hi, lo;
     // max and min as float bit patterns (their unsigned order is the float
@@ -303,11 +249,9 @@ struct Extrema {
 };
 
 template <class Conv>
-__device__ __forceinline__ float convert(float x, const Scale &k, Extrema &e) {
-    float w;
+__device__ __forceinline__ float convert(float x, const ModelScale &k, Extrema &e) {
     e.take(x);
-    if (!Conv::fast(x, k, &w)) w = Conv::slow(x, k.c);
-    return w;
+    return to_model<Conv>(x, k);
 }
 
 // The model into the padded field w: from the caller's array (rows that are
@@ -320,7 +264,7 @@ __device__ __forceinline__ float convert(float x, const Scale &k, Extrema &e) {
 template <class Conv>
 __global__ void __launch_bounds__(kRowThreads)
     model_kernel(const float *src, float *w, const int nx, const unsigned ny, const unsigned rows,
-                 const int pitch, const long long plane, const Scale scale,
+                 const int pitch, const long long plane, const ModelScale scale,
                  unsigned *__restrict__ extrema) {
     Extrema e{0u, 0x7f800000u};
     const int step = blockDim.x;
@@ -387,7 +331,7 @@ cudaError_t launch_model(const float *v, float *w, const Geom &g, double c, unsi
     const unsigned grid = row_grid(g, &block);
     model_kernel<Conv><<<grid, block, 0, s>>>(v, w + pidx(g, 0, 0, 0), g.nx, g.ny,
                                               (unsigned)g.ny * (unsigned)g.nz, g.pnx, g.plane,
-                                              scale_of(c), extrema);
+                                              model_scale(c), extrema);
     return cudaGetLastError();
 }
 

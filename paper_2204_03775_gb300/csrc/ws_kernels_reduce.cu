@@ -1,20 +1,35 @@
-// FP64 reduction of the discrete energy of the leapfrog scheme.
+// Reduction of the discrete energy of the leapfrog scheme.
 //
 // With M = 1/(V dt)^2 and L the 25-point Laplacian (zero outside the grid),
 // the recurrence of Eq. 2 without source or damping is
 // M (u^{n+1} - 2 u^n + u^{n-1}) = L u^n; multiplying by u^{n+1} - u^{n-1}
 // and summing over the grid telescopes (L is symmetric), so
 //     E^{n-1/2} = sum (u^n - u^{n-1})^2 / (V dt)^2 - sum u^n (L u^{n-1})
-// is the same for every n. The kernels evaluate it in double precision from
-// the float fields: each block sums a fixed set of rows into one partial,
-// and one block adds the partials in a fixed order, so the result does not
-// depend on scheduling.
-#include "ws_internal.h"
+// is the same for every n. The kernels evaluate it from the float fields: each
+// block sums a fixed set of rows into one partial, and one block adds the
+// partials in a fixed order, so the result does not depend on scheduling.
+//
+// GB300 runs FP64 at a 64th of its FP32 rate, and evaluated in FP64 (some 90
+// operations and conversions a cell) the kernel was bound by that pipe: 3.7 ms
+// at 320 x 288 x 256. Instead each cell is summed as pairs of floats, hi + lo,
+// through error-free sums and products (Dekker, Knuth), about 270 FP32
+// operations a cell, and only the threads' totals are FP64:
+//  - 5040 h^2 L p = 8064 d1 - 1008 d2 + 128 d3 - 9 d4, d_m the six neighbours at
+//    distance m less 6 p: whole weights, so none is rounded. The pairs p(+m) +
+//    p(-m) and their difference to 2 p are error-free, and on smooth fields the
+//    difference is a single float.
+//  - Values are scaled by a power of two that brings the block's largest to
+//    about 1, so no product underflows that matters.
+// The error of the sum against 80-bit arithmetic, both forms emulated on the
+// CPU, on smooth fields of 40^3 to 96^3 cells: at most 1.6e-16, FP64 3.0e-16
+// (whose weights are rounded); on white noise both 1 to 3e-16. Blocks out of the scaled range, and threads that meet a
+// value that is not finite or a model below 2^-60, take the FP64 form.
+#include "ws_model.cuh"
 
 namespace ws {
 namespace {
 
-constexpr int kThreads = 256;
+constexpr int kThreads = 256;   // 8 warps, each a row at a time
 
 // Scratch of the allocation-free entry point: the per-block partial sums,
 // one array per device that loads the library, held until the process exits.
@@ -24,9 +39,12 @@ static __device__ __align__(256) double g_noalloc_partials[kNoAllocMaxPartials];
 struct PaddedFields {
     const float *u, *p, *w;
     Geom g;
-    __device__ float u_at(int i, int j, int k) const { return u[pidx(g, i, j, k)]; }
-    __device__ float p_at(int i, int j, int k) const { return p[pidx(g, i, j, k)]; }
-    __device__ float w_at(int i, int j, int k) const { return w[pidx(g, i, j, k)]; }
+    __device__ long long at(int i, int j, int k) const { return pidx(g, i, j, k); }
+    __device__ long long row() const { return g.pnx; }
+    __device__ long long plane() const { return g.plane; }
+    // p at offset o from cell e of the array; in: whether that is in the grid
+    __device__ float p_near(long long e, long long o, bool) const { return p[e + o]; }
+    __device__ float w_at(long long e) const { return w[e]; }
 };
 
 // Unpadded [nz][ny][nx] caller arrays; (V dt / h)^2 is formed from the
@@ -36,54 +54,172 @@ struct PaddedFields {
 struct DenseFields {
     const float *u, *p, *v;
     int nx, ny, nz;
-    double dt_over_h;
+    ModelScale scale;
     __device__ long long at(int i, int j, int k) const { return ((long long)k * ny + j) * nx + i; }
-    __device__ float u_at(int i, int j, int k) const { return u[at(i, j, k)]; }
-    __device__ float p_at(int i, int j, int k) const {
-        const bool in = i >= 0 && i < nx && j >= 0 && j < ny && k >= 0 && k < nz;
-        return in ? p[at(i, j, k)] : 0.0f;
-    }
-    __device__ float w_at(int i, int j, int k) const {
-        const double r = __dmul_rn((double)v[at(i, j, k)], dt_over_h);
-        return (float)__dmul_rn(r, r);
-    }
+    __device__ long long row() const { return nx; }
+    __device__ long long plane() const { return (long long)nx * ny; }
+    __device__ float p_near(long long e, long long o, bool in) const { return in ? p[e + o] : 0.0f; }
+    __device__ float w_at(long long e) const { return to_model<FromVelocity>(v[e], scale); }
 };
 
-// Block (x = row block jb, y = plane k) sums rows [jb*rows, jb*rows+rows) of
-// plane k into partials[k * gridDim.x + jb].
+// hi + lo, lo below half an ulp of hi or so.
+struct Pair {
+    float hi, lo;
+};
+__device__ __forceinline__ Pair two_sum(float a, float b) {   // a + b exactly
+    const float s = __fadd_rn(a, b), t = __fsub_rn(s, a);
+    return Pair{s, __fadd_rn(__fsub_rn(a, __fsub_rn(s, t)), __fsub_rn(b, t))};
+}
+__device__ __forceinline__ Pair two_prod(float a, float b) {   // a b exactly
+    const float p = __fmul_rn(a, b);
+    return Pair{p, __fmaf_rn(a, b, -p)};
+}
+__device__ __forceinline__ Pair add(Pair a, Pair b) {
+    const Pair s = two_sum(a.hi, b.hi);
+    const float l = __fadd_rn(s.lo, __fadd_rn(a.lo, b.lo));
+    const float h = __fadd_rn(s.hi, l);   // renormalized
+    return Pair{h, __fadd_rn(__fsub_rn(s.hi, h), l)};
+}
+__device__ __forceinline__ Pair mul(Pair a, float b) {
+    const Pair p = two_prod(a.hi, b);
+    return Pair{p.hi, __fmaf_rn(a.lo, b, p.lo)};
+}
+
+// p(+m) + p(-m) - 2 p on one axis.
+__device__ __forceinline__ Pair second_difference(float plus, float minus, float p2) {
+    const Pair s = two_sum(plus, minus);
+    const Pair d = two_sum(s.hi, -p2);
+    return Pair{d.hi, __fadd_rn(d.lo, s.lo)};
+}
+
+// The values that a cell's term needs.
+struct Cell {
+    float u, p, w;
+    float n[4][6];   // p at distance 1 .. 4 on x+, x-, y+, y-, z+, z-
+};
+
 template <class F>
-__global__ void __launch_bounds__(kThreads) energy_partials_kernel(F f, int nx, int ny, int rows,
-                                                                   double h2, Coeffs64 c,
-                                                                   double *__restrict__ partials) {
+__device__ __forceinline__ Cell load_cell(const F &f, int i, int j, int k, int nx, int ny, int nz) {
+    Cell c;
+    const long long e = f.at(i, j, k), sy = f.row(), sz = f.plane();
+    c.u = f.u[e];
+    c.p = f.p[e];
+    c.w = f.w_at(e);
+#pragma unroll
+    for (int m = 1; m <= 4; ++m) {
+        c.n[m - 1][0] = f.p_near(e, m, i + m < nx);
+        c.n[m - 1][1] = f.p_near(e, -m, i - m >= 0);
+        c.n[m - 1][2] = f.p_near(e, m * sy, j + m < ny);
+        c.n[m - 1][3] = f.p_near(e, -m * sy, j - m >= 0);
+        c.n[m - 1][4] = f.p_near(e, m * sz, k + m < nz);
+        c.n[m - 1][5] = f.p_near(e, -m * sz, k - m >= 0);
+    }
+    return c;
+}
+
+// Adds (u - p)^2 / w to *kin + *kin2 and 5040 u h^2 L p to *pot, of the values
+// times s (a power of two).
+__device__ __forceinline__ void add_cell(const Cell &c, float s, Pair *kin, float *kin2, Pair *pot) {
+    const float u = c.u * s, p = c.p * s, p2 = 2.0f * p;
+    Pair lap{0.0f, 0.0f};
+#pragma unroll
+    for (int m = 4; m >= 1; --m) {
+        const float *n = c.n[m - 1];
+        Pair d = second_difference(n[0] * s, n[1] * s, p2);
+        d = add(d, second_difference(n[2] * s, n[3] * s, p2));
+        d = add(d, second_difference(n[4] * s, n[5] * s, p2));
+        const Pair t = mul(d, m == 1 ? 8064.0f : m == 2 ? -1008.0f : m == 3 ? 128.0f : -9.0f);
+        lap = m == 4 ? t : add(lap, t);
+    }
+    *pot = add(*pot, mul(lap, u));
+    // u - p = d exactly; (u - p)^2 = q + d.lo^2, the last below 2^-50 of q but
+    // never negative, so it is summed apart
+    const Pair d = two_sum(u, -p);
+    Pair q = two_prod(d.hi, d.hi);
+    q.lo = __fmaf_rn(2.0f * d.hi, d.lo, q.lo);
+    // q / w: the nearest quotient, its exact remainder, that one's quotient
+    const float a = __fdiv_rn(q.hi, c.w);
+    const float r = __fadd_rn(__fmaf_rn(-a, c.w, q.hi), q.lo);
+    *kin = add(*kin, Pair{a, __fdividef(r, c.w)});
+    *kin2 = __fadd_rn(*kin2, __fdividef(__fmul_rn(d.lo, d.lo), c.w));
+}
+
+// The term of one cell in FP64: (u - p)^2 / (V dt)^2 - u (L p), every
+// operation explicitly rounded (no contraction left to the compiler), so each
+// field layout gives the same bits.
+__device__ __noinline__ double cell_fp64(const Cell &c, const Coeffs64 &w, double h2) {
+    const double pc = c.p;
+    double l[3];
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+        l[a] = __dmul_rn(w.c0, pc);
+#pragma unroll
+        for (int m = 1; m <= 4; ++m) {
+            const double cm = m == 1 ? w.c1 : m == 2 ? w.c2 : m == 3 ? w.c3 : w.c4;
+            l[a] = __fma_rn(cm, __dadd_rn((double)c.n[m - 1][2 * a], (double)c.n[m - 1][2 * a + 1]),
+                            l[a]);
+        }
+    }
+    const double lap = __ddiv_rn(__dadd_rn(__dadd_rn(l[0], l[1]), l[2]), h2);
+    const double uc = c.u;
+    const double d = __dsub_rn(uc, pc);
+    const double vdt2 = __dmul_rn((double)c.w, h2);   // (V dt)^2
+    return __fma_rn(-uc, lap, __ddiv_rn(__dmul_rn(d, d), vdt2));
+}
+
+// Block (x = row block jb, y = plane k) sums rows [jb*rows, jb*rows+rows) of
+// plane k into partials[k * gridDim.x + jb]; a warp takes whole rows.
+template <class F>
+__global__ void __launch_bounds__(kThreads)
+    energy_partials_kernel(F f, int nx, int ny, int nz, int rows, double h2, Coeffs64 c,
+                           double *__restrict__ partials) {
     const int k = blockIdx.y;
     const int j0 = blockIdx.x * rows;
     const int j1 = min(j0 + rows, ny);
-    double acc = 0.0;
-    for (int j = j0; j < j1; ++j) {
-        for (int i = threadIdx.x; i < nx; i += blockDim.x) {
-            // every operation explicitly rounded (no contraction left to the
-            // compiler), so each field layout gives the same bits
-            const double pc = f.p_at(i, j, k);
-            double lx = __dmul_rn(c.c0, pc), ly = lx, lz = lx;
-#pragma unroll
-            for (int m = 1; m <= 4; ++m) {
-                const double cm = m == 1 ? c.c1 : m == 2 ? c.c2 : m == 3 ? c.c3 : c.c4;
-                lx = __fma_rn(cm, __dadd_rn(f.p_at(i + m, j, k), f.p_at(i - m, j, k)), lx);
-                ly = __fma_rn(cm, __dadd_rn(f.p_at(i, j + m, k), f.p_at(i, j - m, k)), ly);
-                lz = __fma_rn(cm, __dadd_rn(f.p_at(i, j, k + m), f.p_at(i, j, k - m)), lz);
-            }
-            const double lap = __ddiv_rn(__dadd_rn(__dadd_rn(lx, ly), lz), h2);
-            const double uc = f.u_at(i, j, k);
-            const double d = __dsub_rn(uc, pc);
-            const double vdt2 = __dmul_rn((double)f.w_at(i, j, k), h2);   // (V dt)^2
-            acc = __dadd_rn(acc, __fma_rn(-uc, lap, __ddiv_rn(__dmul_rn(d, d), vdt2)));
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    // the block's largest magnitude (bit patterns: NaN above infinity)
+    unsigned big = 0u;
+    for (int j = j0 + warp; j < j1; j += kThreads / 32)
+        for (int i = lane; i < nx; i += 32) {
+            const long long e = f.at(i, j, k);
+            big = max(big, max(__float_as_uint(f.u[e]) & 0x7fffffffu,
+                               __float_as_uint(f.p[e]) & 0x7fffffffu));
         }
+    __shared__ unsigned s_big;
+    __shared__ double warp_sum[kThreads / 32];
+    if (threadIdx.x == 0) s_big = 0u;
+    __syncthreads();
+    big = __reduce_max_sync(0xffffffffu, big);
+    if (lane == 0) atomicMax(&s_big, big);
+    __syncthreads();
+    big = s_big;
+    double acc = 0.0;
+    if (big != 0u) {   // else every term is zero
+        const int ex = (int)(big >> 23) - 127;
+        const int se = max(-60, min(60, -ex));
+        const float s = __int_as_float((se + 127) << 23);
+        Pair kin{0.0f, 0.0f}, pot{0.0f, 0.0f};
+        float kin2 = 0.0f;
+        bool fast = abs(ex + se) <= 30;
+        if (fast)
+            for (int j = j0 + warp; j < j1; j += kThreads / 32)
+                for (int i = lane; i < nx; i += 32) {
+                    const Cell q = load_cell(f, i, j, k, nx, ny, nz);
+                    fast = fast && q.w >= 0x1p-60f;
+                    add_cell(q, s, &kin, &kin2, &pot);
+                }
+        const double K = (double)kin.hi + ((double)kin.lo + (double)kin2), Q = (double)pot.hi + (double)pot.lo;
+        if (fast && isfinite(K) && isfinite(Q))
+            acc = (K - Q / 5040.0) * scalbn(1.0, -2 * se) / h2;
+        else
+            for (int j = j0 + warp; j < j1; j += kThreads / 32)
+                for (int i = lane; i < nx; i += 32)
+                    acc = __dadd_rn(acc, cell_fp64(load_cell(f, i, j, k, nx, ny, nz), c, h2));
     }
     // fixed-order block reduction: warp shuffles, then warp 0
-    __shared__ double warp_sum[kThreads / 32];
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, o);
-    if ((threadIdx.x & 31) == 0) warp_sum[threadIdx.x >> 5] = acc;
+    if (lane == 0) warp_sum[warp] = acc;
     __syncthreads();
     if (threadIdx.x < 32) {
         acc = threadIdx.x < kThreads / 32 ? warp_sum[threadIdx.x] : 0.0;
@@ -116,7 +252,7 @@ cudaError_t launch_energy(const F &f, int nx, int ny, int nz, double h, const Co
                           double *partials, double *out, cudaStream_t s) {
     const int rows = energy_rows_per_block();
     dim3 grid((ny + rows - 1) / rows, nz, 1);
-    energy_partials_kernel<F><<<grid, kThreads, 0, s>>>(f, nx, ny, rows, h * h, c, partials);
+    energy_partials_kernel<F><<<grid, kThreads, 0, s>>>(f, nx, ny, nz, rows, h * h, c, partials);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     sum_partials_kernel<<<1, kThreads, 0, s>>>(partials, (int)(grid.x * grid.y), out);
@@ -150,7 +286,7 @@ cudaError_t launch_energy_noalloc(const float *u, const float *p, const float *v
     cudaError_t e = cudaGetSymbolAddress(&ptr, g_noalloc_partials);
     if (e != cudaSuccess) return e;
     double *partials = static_cast<double *>(ptr);
-    DenseFields f{u, p, v, nx, ny, nz, dt / h};
+    DenseFields f{u, p, v, nx, ny, nz, model_scale(dt / h)};
     return launch_energy(f, nx, ny, nz, h, c, partials, out, s);
 }
 
