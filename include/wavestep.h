@@ -272,8 +272,8 @@ int ws_forward(ws_t ws);
  * sits near 2^12 (16x under the FP16 limit); FP16 then holds values down to
  * ~2^-36 of that maximum and smaller ones as zero. The current state is converted
  * (rounded once). 16-bit storage runs its own streaming kernel with a 64 x ty
- * tile (ty = 24 by default, 16 on grids with ny < 24; 16, 24 or 48 through
- * ws_set_kernel), single grids only (batches and the adjoint gradient need
+ * tile (ty = 24 or 16 by default, whichever is estimated to be faster on the
+ * grid; 16, 24 or 48 through ws_set_kernel), single grids only (batches and the adjoint gradient need
  * FP32 storage), and needs nx >= 64, ny >= 16, else BADARG. ws_read_field,
  * ws_write_field and ws_energy convert to and from FP32 (ws_energy then uses
  * the FP32 model). Relative L2 error against the FP64 oracle, measured on the
@@ -293,9 +293,9 @@ int ws_set_storage(ws_t ws, int storage);
  * AUTO runs grids of at most 200000 cells with the direct kernel) or in {64x16,
  * 64x24, 64x48} for the 16-bit kernel (64x16 selects both; a 16-bit tile leaves
  * the FP32 tile unchanged and needs nx >= 64 and ny >= tile_y), zblock >= 1
- * planes per work item (0 = default: for FP32 the block whose waves of resident
- * CTAs are estimated to finish first; for 16-bit storage blocks of about 200
- * planes with a last block about a quarter as long, fewer on small grids).
+ * planes per work item (0 = default: the block, and for 16-bit storage the tile
+ * height of 24 or 16 rows, whose waves of resident CTAs are estimated to finish
+ * first).
  * WS_KERNEL_STREAM needs nx >= tile_x and ny >= tile_y (64 x 8 while no tile is
  * chosen); else BADARG. */
 int ws_set_kernel(ws_t ws, int kernel, int tile_x, int tile_y, int zblock);

@@ -117,59 +117,72 @@ int default_zblock(int nz) {
     return (4 * nz + 4 * blocks - 4) / (4 * blocks - 3);   // ceil(nz / (blocks - 3/4))
 }
 
-// The FP32 streaming kernel's default for a grid and tile: the z block of the
+// The default z block of a streaming kernel for a grid and tile: the one of the
 // smallest estimated step, in units of one plane of a full SM (about 1 us for
-// 64 x 16 tiles). An item of p planes takes kItem + p on a full SM; a CTA alone
-// on its SM walks a plane in kAlone of that, in between it is interpolated.
-//  - Up to kWaves waves of resident CTAs: the waves one after the other, the
+// FP32 64 x 16 tiles). An item of p planes takes item + p on a full SM; a CTA
+// alone on its SM walks a plane in `alone` of that, in between it is
+// interpolated.
+//  - Up to `waves` waves of resident CTAs: the waves one after the other, the
 //    last one at the speed of its fewer CTAs. Small grids end up with one or
-//    two nearly full waves: 192 x 160 x 144 in 64 x 16 tiles, 10-plane blocks
-//    (0.99 of a wave) 13.1 us, 8 (1.2 waves) 17.0, 5 (1.9) 14.2; 128^3 5-plane
-//    blocks 7.9 us, the former 8-plane minimum 10.5.
+//    two nearly full waves: FP32 192 x 160 x 144 in 64 x 16 tiles, 10-plane
+//    blocks (0.99 of a wave) 13.1 us, 8 (1.2 waves) 17.0, 5 (1.9) 14.2; 128^3
+//    5-plane blocks 7.9 us, the former 8-plane minimum 10.5.
 //  - More waves blur into one another: the work divided by the CTAs, and a
 //    tail that grows with the length of the last items. Blocks are also tried
 //    with a last one about a quarter as long, so that a launch ends on short
-//    items (755 x 994 x 200: blocks of 160 and 40 planes 369 us, of 67 376;
-//    384^3: 128 147 us, 96 195).
-// Over 33 grids of 16 thousand to 270 million cells the chosen block was within
-// 2 % (geometric mean) of the best of any tile and block. At least 2 planes
-// (fewer only repeat the 8-plane prologue), at most 256.
-int default_zblock(const ws::Geom &g, int tx, int ty) {
-    constexpr double kItem = 2.5, kAlone = 0.62, kWaves = 3.0, kTail = 0.2;
+//    items (FP32 755 x 994 x 200: blocks of 160 and 40 planes 369 us, of 67
+//    376; 384^3: 128 147 us, 96 195).
+// The constants were fitted to step times over z blocks and tiles: FP32, 33
+// grids of 16 thousand to 270 million cells, the choice within 2 % (geometric
+// mean) of the best of any tile and block; 16-bit, 22 grids, within 1.3 % (a
+// 200-plane default, shortened to two waves, was 37 % off: 512^3 359 us, now
+// 302). At least 2 planes (fewer only repeat the prologue), at most 256.
+struct BlockModel {
+    double item, alone, waves;
+};
+constexpr BlockModel kModel32{2.5, 0.62, 3.0}, kModel16{3.0, 0.6, 4.0};
+
+int best_zblock(int nz, long long tiles, int slots, int sms, const BlockModel &m, double *best_cost) {
+    constexpr double kTail = 0.2;
     constexpr int kMin = 2, kMax = 256;
-    int slots = 0, sms = 0;
-    if (ws::stream_slots(tx, ty, false, &slots, &sms) != cudaSuccess || g.nz <= kMin)
-        return default_zblock(g.nz);
     const int ctas = slots / sms;
-    const long long tiles = (long long)((g.nx + tx - 1) / tx) * ((g.ny + ty - 1) / ty);
     auto cost = [&](int zb) {
-        const long long blocks = (g.nz + zb - 1) / zb, n = tiles * blocks;
-        const int last = g.nz - (int)(blocks - 1) * zb;
-        if (n > kWaves * slots)
-            return tiles * (blocks * kItem + g.nz) / slots +
-                   kTail * (kItem + (tiles >= slots / 2 ? last : zb));
+        const long long blocks = (nz + zb - 1) / zb, n = tiles * blocks;
+        const int last = nz - (int)(blocks - 1) * zb;
+        if (n > m.waves * slots)
+            return tiles * (blocks * m.item + nz) / slots +
+                   kTail * (m.item + (tiles >= slots / 2 ? last : zb));
         const long long full = n / slots, rem = n % slots;
-        if (rem == 0) return full * (kItem + zb) - (tiles >= slots ? zb - last : 0);
+        if (rem == 0) return full * (m.item + zb) - (tiles >= slots ? zb - last : 0);
         const double share = ctas > 1 ? double((rem + sms - 1) / sms - 1) / (ctas - 1) : 1.0;
-        return full * (kItem + zb) + kItem +
-               (rem <= tiles ? last : zb) * (kAlone + (1.0 - kAlone) * share);
+        return full * (m.item + zb) + m.item +
+               (rem <= tiles ? last : zb) * (m.alone + (1.0 - m.alone) * share);
     };
     int best = 0;
-    double best_cost = 0.0;
     auto consider = [&](int zb) {
-        if (zb < kMin || zb > kMax || zb > g.nz) return;
+        if (zb < 1 || zb > kMax || zb > nz) return;
         const double c = cost(zb);
-        if (best == 0 || c < best_cost - 1e-9) {
+        if (best == 0 || c < *best_cost - 1e-9) {
             best = zb;
-            best_cost = c;
+            *best_cost = c;
         }
     };
-    for (int b = 1, zb; (zb = (g.nz + b - 1) / b) >= kMin; ++b) {
-        if (b > 1) consider((4 * g.nz + 4 * b - 4) / (4 * b - 3));   // the last a quarter as long
+    for (int b = 1;; ++b) {
+        const int zb = (nz + b - 1) / b;
+        if (b > 1 && zb < kMin) break;
+        if (b > 1) consider((4 * nz + 4 * b - 4) / (4 * b - 3));   // the last a quarter as long
         consider(zb);
-        if (zb == kMin) break;
+        if (zb <= kMin) break;
     }
-    return best > 0 ? best : std::min(g.nz, kMax);
+    return best;
+}
+
+int default_zblock(const ws::Geom &g, int tx, int ty) {
+    int slots = 0, sms = 0;
+    if (ws::stream_slots(tx, ty, false, &slots, &sms) != cudaSuccess) return default_zblock(g.nz);
+    const long long tiles = (long long)((g.nx + tx - 1) / tx) * ((g.ny + ty - 1) / ty);
+    double cost = 0.0;
+    return best_zblock(g.nz, tiles, slots, sms, kModel32, &cost);
 }
 
 // The tile of a grid for which none was chosen: 64 x 16 is the fastest, 32 x 16
@@ -372,8 +385,9 @@ int encode_maps16(ws_t ws, int ty) {
     return rc;
 }
 
-// The 16-bit kernel's tile height for this grid: the one ws_set_kernel chose
-// if the grid holds it, else the first of kTile16Ys that the grid holds.
+// A tile height of the 16-bit kernel for this grid: the one ws_set_kernel chose
+// if the grid holds it, else the first of kTile16Ys that the grid holds (0:
+// none).
 int pick_tile16(const ws_t ws) {
     if (ws->tile16_y > 0 && ws->g.ny >= ws->tile16_y) return ws->tile16_y;
     for (int ty : kTile16Ys)
@@ -381,15 +395,35 @@ int pick_tile16(const ws_t ws) {
     return 0;
 }
 
-// Planes per work item of the 16-bit kernel: the FP32 kernel's default,
-// shortened on small grids to about two full waves of the resident CTAs.
-int default_zblock16(const ws::Geom &g, int ty) {
-    int zb = default_zblock(g.nz), slots = 0;
-    if (ws::stream16_slots(ty, &slots) != cudaSuccess) return zb;
-    const long long tiles = (long long)((g.nx + kTile16X - 1) / kTile16X) * ((g.ny + ty - 1) / ty);
-    const long long blocks = std::max<long long>(1, 2LL * slots / tiles);
-    const int zs = (int)std::max<long long>(8, (g.nz + blocks - 1) / blocks);
-    return std::min(zb, std::min(zs, g.nz));
+// Tile height and planes per work item of the 16-bit kernel's next steps: what
+// was chosen, the rest of the smallest estimated step (an SM holds 48 rows of
+// either height, so the estimates compare; see best_zblock).
+ws::StreamTiling pick_tiling16(ws_t ws) {
+    const int fixed = pick_tile16(ws);
+    ws::StreamTiling t{kTile16X, fixed, ws->tiling.zb};
+    if (t.zb > 0) return t;
+    const bool chosen = ws->tile16_y == fixed;
+    ws::StreamTiling &kept = ws->auto16;
+    if (kept.zb > 0 && (kept.ty == fixed || !chosen) && ws->auto16_chosen == chosen) return kept;
+    double best = 0.0;
+    for (int ty : kTile16Ys) {
+        if (chosen) ty = fixed;
+        int slots = 0, sms = 0;
+        if (ws->g.ny < ty || ws::stream16_slots(ty, &slots, &sms) != cudaSuccess) continue;
+        const long long tiles =
+            (long long)((ws->g.nx + kTile16X - 1) / kTile16X) * ((ws->g.ny + ty - 1) / ty);
+        double cost = 0.0;
+        const int zb = best_zblock(ws->g.nz, tiles, slots, sms, kModel16, &cost);
+        if (t.zb <= 0 || cost < best) {
+            best = cost;
+            t.ty = ty;
+            t.zb = zb;
+        }
+    }
+    if (t.zb <= 0) t.zb = default_zblock(ws->g.nz);
+    kept = t;
+    ws->auto16_chosen = chosen;
+    return t;
 }
 
 // FP32 levels (the handle's buffers, or device arrays) -> the 16-bit state
@@ -876,9 +910,7 @@ int ws_step(ws_t ws, int nsteps) {
     ws::StreamTiling tiling{};
     int kern = WS_KERNEL_STREAM;
     if (ws->storage != WS_STORAGE_FP32) {
-        tiling.tx = kTile16X;
-        tiling.ty = pick_tile16(ws);
-        tiling.zb = ws->tiling.zb > 0 ? ws->tiling.zb : default_zblock16(ws->g, tiling.ty);
+        tiling = pick_tiling16(ws);
         if (tiling.ty != ws->t16_ty) {
             int rc = encode_maps16(ws, tiling.ty);
             if (rc != WS_OK) return rc;

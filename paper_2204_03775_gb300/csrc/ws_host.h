@@ -99,6 +99,8 @@ struct ws_handle {
     double wmax = 0.0;         // max (V dt / h)^2 of the model
     ws::FreeBox free_box{};    // cells whose taper is exactly 1, per axis
     int tile16_y = 0;          // 16-bit tile height chosen by ws_set_kernel (0: default)
+    ws::StreamTiling auto16{0, 0, 0};  // the 16-bit tiling a step chose last, and whether
+    bool auto16_chosen = false;        // its height was given
     int t16_ty = 0;            // tile height the 16-bit tensor maps are encoded for
 
     // device scratch of ws_adjoint_gradient, kept for the next call
@@ -163,15 +165,14 @@ int copy_in(ws_t ws, float *dst, const float *src, int on_device, float *dst2 = 
 int copy_out(ws_t ws, float *dst, const float *src, int on_device, float *dst2 = nullptr,
              const float *src2 = nullptr);
 int upload_profiles(ws_t ws);
-// The tile of the 16-bit streaming kernel (64 x ty). The default tile height is the first of kTile16Ys that
-// the grid holds: 24 (two CTAs of 6 warps per SM) measured fastest on the
-// 1024^3 survey (FP16 434.7, BF16 436.5 Gcell/s, against 418 for 48 and 395
-// for 16); 48 is selectable with ws_set_kernel.
+// The tiles of the 16-bit streaming kernel (64 x ty) that a step chooses from:
+// 24 rows (two CTAs of 6 warps per SM) or 16 (three of 4 warps); 48 is
+// selectable with ws_set_kernel (1024^3 about 17 % slower).
 constexpr int kTile16X = 64;
 constexpr int kTile16Ys[] = {24, 16};
 constexpr int kNumTile16Ys = 2;
 int pick_tile16(const ws_t ws);
-int default_zblock16(const ws::Geom &g, int ty);
+ws::StreamTiling pick_tiling16(ws_t ws);
 int encode_maps16(ws_t ws, int ty);
 // FP32 levels (by default the handle's buffers) <-> the 16-bit state.
 int encode_state16(ws_t ws, const ws::Fp32Fields &f);

@@ -219,7 +219,7 @@ struct Weights16 {
 Weights16 zero_sum_weights16();
 bool stream16_tiling_supported(int tx, int ty);
 // SMs x resident CTAs of the 16-bit kernel with 64 x ty tiles.
-cudaError_t stream16_slots(int ty, int *slots);
+cudaError_t stream16_slots(int ty, int *slots, int *sms = nullptr);
 // The tensor maps of a 16-bit step: u: U (16-bit) with box (tx+16, ty+8, 1);
 // d: D and w: the 16-bit model, both with box (tx, ty, 1); u_out receives U'
 // (the other U buffer), D is updated in place at d_io. src_hint: bound on

@@ -880,13 +880,14 @@ bool stream16_tiling_supported(int tx, int ty) {
     return tx == 64 && (ty == 16 || ty == 24 || ty == 48);
 }
 
-cudaError_t stream16_slots(int ty, int *slots) {
+cudaError_t stream16_slots(int ty, int *slots, int *sms) {
     int c = 0, n = 0;
     cudaError_t e = cudaErrorInvalidValue;
     if (ty == 16) e = facts16<Fp16Fmt, 64, 16, 9, 3>(&c, &n);
     if (ty == 24) e = facts16<Fp16Fmt, 64, 24, 9, 3>(&c, &n);
     if (ty == 48) e = facts16<Fp16Fmt, 64, 48, 9, 3>(&c, &n);
     if (e == cudaSuccess) *slots = c * n;
+    if (e == cudaSuccess && sms) *sms = n;
     return e;
 }
 
