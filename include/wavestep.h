@@ -222,8 +222,8 @@ int ws_energy_noalloc(const float *u, const float *u_prev, const float *v, int n
  * again; the handle's state is then left as it is.
  *
  * Needs a velocity model, receivers and FP32 storage, else STATE. Device
- * scratch: about 3 sqrt(N) + 6 padded fields and two
- * trace arrays, allocated by the first call and kept by the handle for the
+ * scratch: about 3 sqrt(N) + 6 padded fields (2 more where the memory holds
+ * them) and two trace arrays, allocated by the first call and kept by the handle for the
  * next ones while N, the receiver count and the tiling stay the same (freed
  * by ws_destroy).
  * Afterwards the handle holds the forward run's final state (step N) and

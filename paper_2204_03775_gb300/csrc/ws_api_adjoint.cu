@@ -73,8 +73,8 @@ int adjoint_prepare(ws_t ws, const char *who, int *kern_out, ws::StreamTiling *t
         int r3 = e == cudaSuccess ? WS_OK : cuda_fail(e, "cudaMalloc adjoint field");
         for (auto &f : ac->ring)
             if (r3 == WS_OK) r3 = field(&f);
-        for (auto &f : ac->rho)
-            if (r3 == WS_OK) r3 = field(&f);
+        for (int q = 0; q < 2; ++q)
+            if (r3 == WS_OK) r3 = field(&ac->rho[q]);
         if (r3 == WS_OK) e = grab(&ac->acc, 2 * fb);   // float2 per cell, padded layout
         if (r3 == WS_OK && e == cudaSuccess) e = grab(&ac->partials, sizeof(double) * (ws::residual_partial_count() + 1));
         if (r3 == WS_OK && e == cudaSuccess) e = grab(&ac->norm, sizeof(double) * (ws::residual_partial_count() + 1));
@@ -86,6 +86,23 @@ int adjoint_prepare(ws_t ws, const char *who, int *kern_out, ws::StreamTiling *t
             delete ws->adj;
             ws->adj = nullptr;
             return r3 != WS_OK ? r3 : cuda_fail(e, "cudaMalloc adjoint scratch");
+        }
+        // more levels of rho, if there is room for them, so that more steps are
+        // imaged together
+        for (int q = 2; q < ws::kMaxImagingSteps; ++q) {
+            if (grab(&ac->rho[q].p, fb) != cudaSuccess) {
+                cudaGetLastError();
+                break;
+            }
+            WS_CUDA(cudaMemsetAsync(ac->rho[q].p, 0, fb, st), "zero adjoint field");
+            if (maps) {
+                const int tx = ws->tiling.tx, ty = ws->tiling.ty;
+                int r4 = encode_map(&ac->rho[q].halo, ac->rho[q].p, g, tx + 2 * ws::kHalo,
+                                    ty + 2 * ws::kHalo);
+                if (r4 == WS_OK) r4 = encode_map(&ac->rho[q].tile, ac->rho[q].p, g, tx, ty);
+                if (r4 != WS_OK) return r4;
+            }
+            ac->nrho = q + 1;
         }
         ac->N = N;
         ac->nrec = ws->nrec;
@@ -159,7 +176,8 @@ struct GradShot {
     float *grad = nullptr;
     bool forward = true;     // run the forward problem (not reused from ws_forward)
     ws::StepArgs a{};
-    int rho_cur = 0;         // rho[rho_cur] = rho^{k+1}
+    ws::ImagingSteps img{};  // steps waiting to be imaged together
+    int pending = 0;
 };
 
 // The gradients of n shots with one grid and one step count, each shot's
@@ -174,7 +192,8 @@ int gradient_run(GradShot *sh, int n, int mode) {
     for (int q = 0; q < n; ++q) {
         GradShot &x = sh[q];
         const cudaStream_t st = x.ws->stream;
-        for (auto &f : x.ac->rho) WS_CUDA(cudaMemsetAsync(f.p, 0, fb, st), "zero adjoint field");
+        for (int k : {N + 1, N + 2})   // rho^{N+1} = rho^{N+2} = 0
+            WS_CUDA(cudaMemsetAsync(x.ac->rho[k % x.ac->nrho].p, 0, fb, st), "zero adjoint field");
         WS_CUDA(cudaMemsetAsync(x.ac->acc, 0, 2 * fb, st), "zero gradient accumulator");
         WS_CUDA(cudaMemcpyAsync(x.ac->rec, x.ws->rec_ijk.data(), sizeof(int) * 3 * x.ws->nrec,
                                 cudaMemcpyHostToDevice, st),
@@ -188,7 +207,6 @@ int gradient_run(GradShot *sh, int n, int mode) {
             if (rc != WS_OK) return rc;
         }
         x.a = base_args(x.ws);
-        x.rho_cur = 0;
     }
 
     // 1. forward from rest, recording the traces and the checkpoints
@@ -246,21 +264,29 @@ int gradient_run(GradShot *sh, int n, int mode) {
             for (int q = 0; q < n; ++q) {
                 GradShot &x = sh[q];
                 ws_t ws = x.ws;
+                const int nr = x.ac->nrho;
                 MappedField *rho = x.ac->rho;
-                MappedField &r1 = rho[x.rho_cur], &r2 = rho[1 - x.rho_cur];
-                int rc = step_fp32(ws, x.a, x.kern, x.tiling, r1.p, &r1.halo, r2.p, &r2.tile, r2.p,
+                MappedField &r1 = rho[(k + 1) % nr], &r2 = rho[(k + 2) % nr];
+                float *out = rho[k % nr].p;
+                int rc = step_fp32(ws, x.a, x.kern, x.tiling, r1.p, &r1.halo, r2.p, &r2.tile, out,
                                    k, false, false);
                 if (rc != WS_OK) return rc;
-                x.rho_cur = 1 - x.rho_cur;   // rho[rho_cur] = rho^k
-                WS_CUDA(ws::launch_inject(rho[x.rho_cur].p, ws->w, ws->gx, ws->gy, ws->gz, g,
-                                          x.ac->rec, ws->nrec, x.ac->r, N, k - 1, ws->stream),
+                WS_CUDA(ws::launch_inject(out, ws->w, ws->gx, ws->gy, ws->gz, g, x.ac->rec,
+                                          ws->nrec, x.ac->r, N, k - 1, ws->stream),
                         "adjoint injection kernel");
+                ws->launches++;
+                // the steps whose rho and L u are alive are imaged together
                 ws::Sources src{};
                 sources_of_step(ws, k - 1, &src);
-                WS_CUDA(ws::launch_imaging(rho[x.rho_cur].p, x.ac->lap[k - 1 - n0], g, src, ws->gx,
-                                           ws->gy, ws->gz, x.ac->acc, ws->stream),
+                x.img.rho[x.pending] = out;
+                x.img.lap[x.pending] = x.ac->lap[k - 1 - n0];
+                for (int s = 0; s < src.n; ++s) x.img.amp[x.pending][s] = src.s[s].amp;
+                if (++x.pending < nr && k > n0 + 1) continue;
+                WS_CUDA(ws::launch_imaging(x.img, x.pending, g, src, ws->gx, ws->gy, ws->gz,
+                                           x.ac->acc, ws->stream),
                         "gradient imaging kernel");
-                ws->launches += 2;
+                x.pending = 0;
+                ws->launches++;
             }
     }
     for (int q = 0; q < n; ++q) {

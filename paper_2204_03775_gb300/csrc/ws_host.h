@@ -128,7 +128,11 @@ struct AdjointCache {
     std::vector<void *> mem;        // everything below, for cudaFree
     std::vector<float *> ck;
     std::vector<float *> lap;       // L u^n of the segment's steps
-    MappedField ring[2], rho[2];    // recomputed u^n / u^{n-1}; rho^{k+1} / rho^{k+2}
+    MappedField ring[2];            // recomputed u^n / u^{n-1}
+    // rho^k in rho[k % nrho]: the steps imaged together stay alive (2 where the
+    // memory does not hold more)
+    MappedField rho[ws::kMaxImagingSteps];
+    int nrho = 2;
     float2 *acc = nullptr;          // compensated FP32 gradient sums, padded layout
     double *partials = nullptr;     // residual partial sums, then the misfit
     double *norm = nullptr;         // gradient-norm partial sums, then the norm

@@ -254,9 +254,15 @@ cudaError_t launch_inject(float *rho, const float *w, const float *gx, const flo
                           const float *gz, const Geom &g, const int *rec_ijk, int nrec,
                           const float *r, int nt, int col, cudaStream_t s);
 // acc (compensated FP32 {sum, correction} per cell, padded layout) +=
-// rho * lapu (the stencil sum L u^n a step stored), plus rho * amp / G at
-// source cells.
-cudaError_t launch_imaging(const float *rho, const float *lapu, const Geom &g, const Sources &src,
+// rho[s] * lap[s] (the stencil sum L u^n a step stored) for the steps s = 0 ..
+// steps-1 in this order, plus rho * amp / G at the cells of src (amp[s][q] for
+// source q). 1 <= steps <= kMaxImagingSteps.
+constexpr int kMaxImagingSteps = 4;
+struct ImagingSteps {
+    const float *rho[kMaxImagingSteps], *lap[kMaxImagingSteps];
+    float amp[kMaxImagingSteps][kMaxSources];
+};
+cudaError_t launch_imaging(const ImagingSteps &st, int steps, const Geom &g, const Sources &src,
                            const float *gx, const float *gy, const float *gz, float2 *acc,
                            cudaStream_t s);
 // out[t] = sum over q < n of src.p[q][t], t < count (FP64 sum in the order of

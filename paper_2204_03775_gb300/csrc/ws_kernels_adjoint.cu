@@ -76,15 +76,16 @@ __global__ void inject_kernel(float *__restrict__ rho, const float *__restrict__
     atomicAdd(&rho[p], w[p] * gd * r[(long long)q * nt + col]);
 }
 
-// acc += rho * (L u) with L u the stencil sum the step kernel stored while
-// recomputing u^{n+1} (the same float value the step used), and at source
-// cells rho * (h^2 s_n) / G. The accumulator is a compensated FP32 sum
-// (Kahan): per cell a float2 {sum, correction} in the padded layout, so a
-// thread's 4 consecutive x cells are one float4 of rho, one of L u and two
-// of acc. GB300 runs FP64 at a small fraction of FP32, which made an FP64
-// accumulator the bottleneck of this pass; the compensated sum keeps the
-// rounding of 800 additions at the level of one. A block covers 128 x 8
-// cells of one plane; one thread finds the block's sources first.
+// For M steps, latest first: acc += rho * (L u) with L u the stencil sum the
+// step kernel stored while recomputing u^{n+1} (the same float value the step
+// used), and at source cells rho * (h^2 s_n) / G. The accumulator is a
+// compensated FP32 sum (Kahan): per cell a float2 {sum, correction} in the
+// padded layout, so a thread's 4 consecutive x cells are one float4 of rho, one
+// of L u and two of acc. GB300 runs FP64 at a small fraction of FP32, which made
+// an FP64 accumulator the bottleneck of this pass; the compensated sum keeps the
+// rounding of 800 additions at the level of one. Bound: HBM, 8 bytes a cell and
+// step and 16 a pass: with M = 4 a step costs 12 bytes, alone 24. A block covers
+// 128 x 8 cells of one plane; one thread finds the block's sources first.
 __device__ __forceinline__ void kahan_add(float &sum, float &corr, float x) {
     const float y = x - corr;
     const float t = sum + y;
@@ -92,9 +93,9 @@ __device__ __forceinline__ void kahan_add(float &sum, float &corr, float x) {
     sum = t;
 }
 
-__global__ void __launch_bounds__(256) imaging_kernel(const float *__restrict__ rho,
-                                                      const float *__restrict__ lapu, Geom g,
-                                                      Sources src, const float *__restrict__ gx,
+template <int M>
+__global__ void __launch_bounds__(256) imaging_kernel(const ImagingSteps st, Geom g, Sources src,
+                                                      const float *__restrict__ gx,
                                                       const float *__restrict__ gy,
                                                       const float *__restrict__ gz,
                                                       float2 *__restrict__ acc) {
@@ -116,23 +117,33 @@ __global__ void __launch_bounds__(256) imaging_kernel(const float *__restrict__ 
     __syncthreads();
     if (i >= g.nx || j >= g.ny) return;
     const long long p = pidx(g, i, j, k);   // a multiple of 4: rows start on 32-cell lines
-    const float4 r4 = *reinterpret_cast<const float4 *>(rho + p);
-    const float4 l4 = __ldcs(reinterpret_cast<const float4 *>(lapu + p));
+    float4 r4[M], l4[M];
+#pragma unroll
+    for (int s = 0; s < M; ++s) {
+        r4[s] = *reinterpret_cast<const float4 *>(st.rho[s] + p);
+        l4[s] = __ldcs(reinterpret_cast<const float4 *>(st.lap[s] + p));
+    }
     float4 a01 = *reinterpret_cast<const float4 *>(acc + p);       // {s0, c0, s1, c1}
     float4 a23 = *reinterpret_cast<const float4 *>(acc + p + 2);   // {s2, c2, s3, c3}
-    float t[4] = {r4.x * l4.x, r4.y * l4.y, r4.z * l4.z, r4.w * l4.w};
-    const float rv[4] = {r4.x, r4.y, r4.z, r4.w};
-    for (unsigned m = mask; m; m &= m - 1) {
-        const SourceSample &ss = src.s[__ffs(m) - 1];
-        const int l = ss.i - i;
-        if (ss.j == j && l >= 0 && l < 4)
-            t[l] = fmaf(rv[l], ss.amp / (gx[ss.i] * gy[j] * gz[k]), t[l]);
+#pragma unroll
+    for (int s = 0; s < M; ++s) {
+        // products rounded by themselves, however many steps a pass takes
+        float t[4] = {__fmul_rn(r4[s].x, l4[s].x), __fmul_rn(r4[s].y, l4[s].y),
+                      __fmul_rn(r4[s].z, l4[s].z), __fmul_rn(r4[s].w, l4[s].w)};
+        const float rv[4] = {r4[s].x, r4[s].y, r4[s].z, r4[s].w};
+        for (unsigned m = mask; m; m &= m - 1) {
+            const int q = __ffs(m) - 1;
+            const SourceSample &ss = src.s[q];
+            const int l = ss.i - i;
+            if (ss.j == j && l >= 0 && l < 4)
+                t[l] = fmaf(rv[l], st.amp[s][q] / (gx[ss.i] * gy[j] * gz[k]), t[l]);
+        }
+        // cells past nx (x padding: zero in rho and in L u) accumulate zeros
+        kahan_add(a01.x, a01.y, t[0]);
+        kahan_add(a01.z, a01.w, t[1]);
+        kahan_add(a23.x, a23.y, t[2]);
+        kahan_add(a23.z, a23.w, t[3]);
     }
-    // cells past nx (x padding: zero in rho and in L u) accumulate zeros
-    kahan_add(a01.x, a01.y, t[0]);
-    kahan_add(a01.z, a01.w, t[1]);
-    kahan_add(a23.x, a23.y, t[2]);
-    kahan_add(a23.z, a23.w, t[3]);
     *reinterpret_cast<float4 *>(acc + p) = a01;
     *reinterpret_cast<float4 *>(acc + p + 2) = a23;
 }
@@ -227,12 +238,18 @@ cudaError_t launch_inject(float *rho, const float *w, const float *gx, const flo
     return cudaGetLastError();
 }
 
-cudaError_t launch_imaging(const float *rho, const float *lapu, const Geom &g, const Sources &src,
+cudaError_t launch_imaging(const ImagingSteps &st, int steps, const Geom &g, const Sources &src,
                            const float *gx, const float *gy, const float *gz, float2 *acc,
                            cudaStream_t s) {
     dim3 block(32, 8, 1);
     dim3 grid((g.nx + 127) / 128, (g.ny + 7) / 8, g.nz);
-    imaging_kernel<<<grid, block, 0, s>>>(rho, lapu, g, src, gx, gy, gz, acc);
+    switch (steps) {
+        case 1: imaging_kernel<1><<<grid, block, 0, s>>>(st, g, src, gx, gy, gz, acc); break;
+        case 2: imaging_kernel<2><<<grid, block, 0, s>>>(st, g, src, gx, gy, gz, acc); break;
+        case 3: imaging_kernel<3><<<grid, block, 0, s>>>(st, g, src, gx, gy, gz, acc); break;
+        case 4: imaging_kernel<4><<<grid, block, 0, s>>>(st, g, src, gx, gy, gz, acc); break;
+        default: return cudaErrorInvalidValue;
+    }
     return cudaGetLastError();
 }
 
