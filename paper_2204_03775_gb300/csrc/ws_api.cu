@@ -492,7 +492,8 @@ ws::StepArgs base_args(const ws_t ws) {
 // One FP32 step of the handle's model (Eq. 1 discretised): out = u^{n+1}
 // from un = u^n (with its halo box map) and unm1 = u^{n-1} (with its tile box
 // map); out may be unm1. Adds the sources of step n when `sources`, records
-// the receivers' trace column n - trace_start when `record`.
+// the receivers' trace column n - trace_start when `record` (with a.inject: adds
+// the residual of that column there instead).
 int step_fp32(ws_t ws, ws::StepArgs &a, int kern, const ws::StreamTiling &tiling, const float *un,
               const CUtensorMap *un_halo, const float *unm1, const CUtensorMap *unm1_tile,
               float *out, long long n, bool sources, bool record) {

@@ -55,13 +55,13 @@ int adjoint_prepare(ws_t ws, const char *who, int *kern_out, ws::StreamTiling *t
             return r2;
         };
         // checkpoints (u^{jC}, u^{jC-1}), j = 1 .. nck-1; segment states; rho
-        ac->ck.assign(2 * size_t(nck - 1), nullptr);
+        ac->ck.assign(2 * size_t(nck - 1), MappedField());
         for (auto &c : ac->ck) {
-            cudaError_t e = grab(&c, fb);
-            if (e != cudaSuccess) {
+            const int r2 = field(&c);
+            if (r2 != WS_OK) {
                 delete ws->adj;
                 ws->adj = nullptr;
-                return cuda_fail(e, "cudaMalloc checkpoint");
+                return r2;
             }
         }
         ac->lap.assign(C, nullptr);
@@ -81,7 +81,6 @@ int adjoint_prepare(ws_t ws, const char *who, int *kern_out, ws::StreamTiling *t
         if (r3 == WS_OK && e == cudaSuccess) e = grab(&ac->r, sizeof(float) * ntr);
         if (r3 == WS_OK && e == cudaSuccess) e = grab(&ac->dd, sizeof(float) * ntr);
         if (r3 == WS_OK && e == cudaSuccess) e = grab(&ac->grad, sizeof(float) * ncell);
-        if (r3 == WS_OK && e == cudaSuccess) e = grab(&ac->rec, sizeof(int) * 3 * ws->nrec);
         if (r3 != WS_OK || e != cudaSuccess) {
             delete ws->adj;
             ws->adj = nullptr;
@@ -116,9 +115,27 @@ int adjoint_prepare(ws_t ws, const char *who, int *kern_out, ws::StreamTiling *t
     return WS_OK;
 }
 
-// The forward run from rest over N steps: traces recorded, checkpoint pairs
-// (u^{jC}, u^{jC-1}) saved; the cache then holds this model version's run.
+// The forward run from rest over N steps, in segments of C: traces recorded,
+// checkpoint pairs (u^{jC}, u^{jC-1}) kept; the cache then holds this model
+// version's run. Nothing is copied for a checkpoint: the steps of segment j
+// write into the pair of checkpoint j + 1 (the last segment's into the handle's
+// fields), the first two out of place, so that the pair they start from stays.
 // forward_begin resets the state, forward_step issues step n.
+struct Level {
+    float *p;
+    const CUtensorMap *halo, *tile;
+};
+
+// Where u^m of the forward run lies, m = -1 .. N (u^0 and u^{-1} are the
+// handle's zeroed fields).
+Level forward_level(ws_t ws, AdjointCache *ac, int m) {
+    const int N = ws->nt_max, C = (int)std::ceil(std::sqrt((double)N)), nck = (N + C - 1) / C;
+    const int b = m & 1, j = m > 0 ? (m - 1) / C + 1 : 0;   // u^m lies in pair j
+    if (j == 0 || j == nck) return Level{ws->buf[b], &ws->tmap_halo[b], &ws->tmap_tile[b]};
+    MappedField &f = ac->ck[2 * (j - 1) + b];
+    return Level{f.p, &f.halo, &f.tile};
+}
+
 int forward_begin(ws_t ws, AdjointCache *ac) {
     const size_t fb = field_bytes(ws->g);
     const size_t ntr = size_t(ws->nrec) * ws->nt_max;
@@ -133,25 +150,19 @@ int forward_begin(ws_t ws, AdjointCache *ac) {
 
 int forward_step(ws_t ws, AdjointCache *ac, int kern, const ws::StreamTiling &tiling,
                  ws::StepArgs &a, int n) {
-    const int C = (int)std::ceil(std::sqrt((double)ws->nt_max));
-    const size_t fb = field_bytes(ws->g);
-    const cudaStream_t st = ws->stream;
-    std::vector<float *> &ck = ac->ck;
-    if (n > 0 && n % C == 0) {
-        const int j = n / C;
-        WS_CUDA(cudaMemcpyAsync(ck[2 * (j - 1)], ws->buf[ws->cur], fb, cudaMemcpyDeviceToDevice, st),
-                "save checkpoint");
-        WS_CUDA(cudaMemcpyAsync(ck[2 * (j - 1) + 1], ws->buf[1 - ws->cur], fb,
-                                cudaMemcpyDeviceToDevice, st),
-                "save checkpoint");
-    }
-    const int c = ws->cur;
-    int rc = step_fp32(ws, a, kern, tiling, ws->buf[c], &ws->tmap_halo[c], ws->buf[1 - c],
-                       &ws->tmap_tile[1 - c], ws->buf[1 - c], n, true, true);
+    const Level un = forward_level(ws, ac, n), um = forward_level(ws, ac, n - 1);
+    const Level out = forward_level(ws, ac, n + 1);
+    int rc = step_fp32(ws, a, kern, tiling, un.p, un.halo, um.p, um.tile, out.p, n, true, true);
     if (rc != WS_OK) return rc;
-    ws->cur = 1 - c;
     ws->step++;
     if (n == ws->nt_max - 1) {
+        // the handle holds u^N and u^{N-1}: the latter too if the last segment
+        // is this step alone
+        ws->cur = ws->nt_max & 1;
+        if (un.p != ws->buf[1 - ws->cur])
+            WS_CUDA(cudaMemcpyAsync(ws->buf[1 - ws->cur], un.p, field_bytes(ws->g),
+                                    cudaMemcpyDeviceToDevice, ws->stream),
+                    "copy the last state");
         ac->fwd_valid = true;
         ac->fwd_version = ws->model_version;
     }
@@ -195,9 +206,6 @@ int gradient_run(GradShot *sh, int n, int mode) {
         for (int k : {N + 1, N + 2})   // rho^{N+1} = rho^{N+2} = 0
             WS_CUDA(cudaMemsetAsync(x.ac->rho[k % x.ac->nrho].p, 0, fb, st), "zero adjoint field");
         WS_CUDA(cudaMemsetAsync(x.ac->acc, 0, 2 * fb, st), "zero gradient accumulator");
-        WS_CUDA(cudaMemcpyAsync(x.ac->rec, x.ws->rec_ijk.data(), sizeof(int) * 3 * x.ws->nrec,
-                                cudaMemcpyHostToDevice, st),
-                "upload receivers");
         // a residual given for the run that ws_forward left in the cache (same
         // model version) needs no new forward run
         x.forward = !(mode == WS_ADJ_RESIDUAL && x.ac->fwd_valid &&
@@ -232,31 +240,23 @@ int gradient_run(GradShot *sh, int n, int mode) {
     // states recomputed from its checkpoint
     for (int j = nck - 1; j >= 0; --j) {
         const int n0 = j * C, n1 = std::min(n0 + C, N);
-        // u^{n0}, u^{n0-1} into the ring, then steps n0 .. n1-1, each storing
-        // L u^n into lap[n - n0] (u^{n1} itself is not needed)
-        for (int q = 0; q < n; ++q) {
-            AdjointCache *ac = sh[q].ac;
-            const cudaStream_t st = sh[q].ws->stream;
-            if (j == 0) {
-                WS_CUDA(cudaMemsetAsync(ac->ring[0].p, 0, fb, st), "zero initial state");
-                WS_CUDA(cudaMemsetAsync(ac->ring[1].p, 0, fb, st), "zero initial state");
-            } else {
-                WS_CUDA(cudaMemcpyAsync(ac->ring[0].p, ac->ck[2 * (j - 1)], fb,
-                                        cudaMemcpyDeviceToDevice, st),
-                        "restore checkpoint");
-                WS_CUDA(cudaMemcpyAsync(ac->ring[1].p, ac->ck[2 * (j - 1) + 1], fb,
-                                        cudaMemcpyDeviceToDevice, st),
-                        "restore checkpoint");
-            }
-        }
-        for (int t = 0; t < n1 - n0; ++t)
+        // steps n0 .. n1-1 from the checkpoint, each storing L u^n into lap[n -
+        // n0] (u^{n1} itself is not needed). The first two read the checkpoint
+        // where it lies; u^m, m > n0, goes to ring[m & 1].
+        if (j == 0)
+            for (int q = 0; q < n; ++q)   // from rest: u^0 = ring[0], u^{-1} = ring[1]
+                for (auto &f : sh[q].ac->ring)
+                    WS_CUDA(cudaMemsetAsync(f.p, 0, fb, sh[q].ws->stream), "zero initial state");
+        for (int m = n0; m < n1; ++m)
             for (int q = 0; q < n; ++q) {
                 GradShot &x = sh[q];
-                const int uc = t & 1;   // ring[uc] = u^{n0+t}
-                MappedField &un = x.ac->ring[uc], &um = x.ac->ring[1 - uc];
-                x.a.lap = x.ac->lap[t];
+                auto level = [&](int l) -> MappedField & {   // u^l
+                    return l <= n0 && j > 0 ? x.ac->ck[2 * (j - 1) + (l & 1)] : x.ac->ring[l & 1];
+                };
+                MappedField &un = level(m), &um = level(m - 1);
+                x.a.lap = x.ac->lap[m - n0];
                 int rc = step_fp32(x.ws, x.a, x.kern, x.tiling, un.p, &un.halo, um.p, &um.tile,
-                                   um.p, n0 + t, true, false);
+                                   level(m + 1).p, m, true, false);
                 x.a.lap = nullptr;
                 if (rc != WS_OK) return rc;
             }
@@ -268,13 +268,12 @@ int gradient_run(GradShot *sh, int n, int mode) {
                 MappedField *rho = x.ac->rho;
                 MappedField &r1 = rho[(k + 1) % nr], &r2 = rho[(k + 2) % nr];
                 float *out = rho[k % nr].p;
+                // rho^k, with W G r^k (trace column k - 1) added at the receivers
+                x.a.inject = x.ac->r;
                 int rc = step_fp32(ws, x.a, x.kern, x.tiling, r1.p, &r1.halo, r2.p, &r2.tile, out,
-                                   k, false, false);
+                                   k - 1 + ws->trace_start, false, true);
+                x.a.inject = nullptr;
                 if (rc != WS_OK) return rc;
-                WS_CUDA(ws::launch_inject(out, ws->w, ws->gx, ws->gy, ws->gz, g, x.ac->rec,
-                                          ws->nrec, x.ac->r, N, k - 1, ws->stream),
-                        "adjoint injection kernel");
-                ws->launches++;
                 // the steps whose rho and L u are alive are imaged together
                 ws::Sources src{};
                 sources_of_step(ws, k - 1, &src);

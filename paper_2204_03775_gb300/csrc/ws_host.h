@@ -126,7 +126,7 @@ struct AdjointCache {
     bool fwd_valid = false;
     unsigned long long fwd_version = 0;
     std::vector<void *> mem;        // everything below, for cudaFree
-    std::vector<float *> ck;
+    std::vector<MappedField> ck;    // checkpoint j: (u^{jC}, u^{jC-1}), u^m in ck[2 (j-1) + (m & 1)]
     std::vector<float *> lap;       // L u^n of the segment's steps
     MappedField ring[2];            // recomputed u^n / u^{n-1}
     // rho^k in rho[k % nrho]: the steps imaged together stay alive (2 where the
@@ -137,7 +137,6 @@ struct AdjointCache {
     double *partials = nullptr;     // residual partial sums, then the misfit
     double *norm = nullptr;         // gradient-norm partial sums, then the norm
     float *r = nullptr, *dd = nullptr, *grad = nullptr;
-    int *rec = nullptr;
     ~AdjointCache() {
         for (void *p : mem) cudaFree(p);
     }
@@ -187,7 +186,8 @@ int decode_state16(ws_t ws);
 void sources_of_step(const ws_t ws, long long n, ws::Sources *out);
 // Step arguments common to every step of the handle's model.
 ws::StepArgs base_args(const ws_t ws);
-// One FP32 step: out = u^{n+1} from un = u^n and unm1 = u^{n-1} (out may be unm1).
+// One FP32 step: out = u^{n+1} from un = u^n and unm1 = u^{n-1} (out may be
+// unm1); record: with the receivers (or a.inject at them).
 int step_fp32(ws_t ws, ws::StepArgs &a, int kern, const ws::StreamTiling &tiling, const float *un,
               const CUtensorMap *un_halo, const float *unm1, const CUtensorMap *unm1_tile,
               float *out, long long n, bool sources, bool record);

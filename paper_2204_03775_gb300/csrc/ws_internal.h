@@ -104,6 +104,8 @@ struct StepArgs {
     long long trace_step;        // column of this step in traces
     unsigned *status;            // device status word
     float *lap;                  // if not null: receives the stencil sum L u^n (padded field)
+    const float *inject;         // if not null: residual [nrec][nt_max]; adds W G r[:, trace_step]
+                                 // at the receivers instead of recording them
     int stall_item;              // test hook: withhold the first copy of this work item (-1: none)
 };
 
@@ -249,10 +251,6 @@ int residual_partial_count();
 // partials holds residual_partial_count() doubles.
 cudaError_t launch_residual(const float *traces, const float *d_obs, long long n, float *r,
                             double *partials, double *misfit, cudaStream_t s);
-// rho[rec] += W G r[:, col] at every receiver (rec_ijk: [nrec][3] device).
-cudaError_t launch_inject(float *rho, const float *w, const float *gx, const float *gy,
-                          const float *gz, const Geom &g, const int *rec_ijk, int nrec,
-                          const float *r, int nt, int col, cudaStream_t s);
 // acc (compensated FP32 {sum, correction} per cell, padded layout) +=
 // rho[s] * lap[s] (the stencil sum L u^n a step stored) for the steps s = 0 ..
 // steps-1 in this order, plus rho * amp / G at the cells of src (amp[s][q] for

@@ -8,8 +8,8 @@
 // backwards:
 //     rho^k = G (2 rho^{k+1} - G rho^{k+2} + W L rho^{k+1}) + W G r^k,
 // r^k the residual at the receivers for the trace sample of u^k; so the
-// step kernels advance rho, and these kernels add W G r^k at the receivers
-// and accumulate the gradient with respect to m = 1/V^2,
+// step kernels advance rho and add W G r^k at the receivers, and these kernels
+// accumulate the gradient with respect to m = 1/V^2,
 //     dJ/dm_i = -V_i^2 sum_n rho^{n+1}_i (L u^n)_i
 //               - [i = s] V_s^2 sum_n rho^{n+1}_s h^2 s_n / G_s.
 #include "ws_internal.h"
@@ -60,20 +60,6 @@ __global__ void __launch_bounds__(kRedThreads) sum_kernel(const double *__restri
         for (int o = 16; o > 0; o >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, o);
         if (threadIdx.x == 0) out[0] = acc;
     }
-}
-
-// rho[rec_r] += W G r[r][col] (atomic: receivers may share a cell).
-__global__ void inject_kernel(float *__restrict__ rho, const float *__restrict__ w,
-                              const float *__restrict__ gx, const float *__restrict__ gy,
-                              const float *__restrict__ gz, Geom g,
-                              const int *__restrict__ rec_ijk, int nrec,
-                              const float *__restrict__ r, int nt, int col) {
-    const int q = blockIdx.x * blockDim.x + threadIdx.x;
-    if (q >= nrec) return;
-    const int i = rec_ijk[3 * q], j = rec_ijk[3 * q + 1], k = rec_ijk[3 * q + 2];
-    const long long p = pidx(g, i, j, k);
-    const float gd = gx[i] * gy[j] * gz[k];
-    atomicAdd(&rho[p], w[p] * gd * r[(long long)q * nt + col]);
 }
 
 // For M steps, latest first: acc += rho * (L u) with L u the stencil sum the
@@ -227,14 +213,6 @@ cudaError_t launch_residual(const float *traces, const float *d_obs, long long n
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     sum_kernel<<<1, kRedThreads, 0, s>>>(partials, blocks, misfit);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_inject(float *rho, const float *w, const float *gx, const float *gy,
-                          const float *gz, const Geom &g, const int *rec_ijk, int nrec,
-                          const float *r, int nt, int col, cudaStream_t s) {
-    inject_kernel<<<(nrec + 255) / 256, 256, 0, s>>>(rho, w, gx, gy, gz, g, rec_ijk, nrec, r, nt,
-                                                     col);
     return cudaGetLastError();
 }
 

@@ -52,9 +52,10 @@ __device__ __forceinline__ void step_cell(const float *u, const float *up, float
 }
 
 // Receivers: a block's entries of its tile's range (sorted by k) on its plane
-// are sampled once all its threads have stored. (As a launch of its own this
+// are sampled, or the residual is added to their cells (atomically: receivers
+// may share one), once all its threads have stored. (As a launch of its own this
 // cost 1 us a step on grids of a few microseconds.)
-__device__ __forceinline__ void record_block(const float *out, const StepArgs &a, int k,
+__device__ __forceinline__ void record_block(float *out, const float *w, const StepArgs &a, int k,
                                              const int *rec_ptr, const RecEntry *rec) {
     const int tile = blockIdx.y * gridDim.x + blockIdx.x;
     const int lo = rec_ptr[tile], hi = rec_ptr[tile + 1];
@@ -64,7 +65,11 @@ __device__ __forceinline__ void record_block(const float *out, const StepArgs &a
     for (int e = lo + tid; e < hi; e += blockDim.x * blockDim.y) {
         if (rec[e].k != k) continue;
         const int i = blockIdx.x * blockDim.x + rec[e].lane, j = blockIdx.y * blockDim.y + rec[e].owner;
-        a.traces[(long long)rec[e].r * a.nt_max + a.trace_step] = out[pidx(a.g, i, j, k)];
+        const long long p = pidx(a.g, i, j, k), t = (long long)rec[e].r * a.nt_max + a.trace_step;
+        if (a.inject)
+            atomicAdd(&out[p], __fmul_rn(__fmul_rn(w[p], a.gx[i] * a.gy[j] * a.gz[k]), a.inject[t]));
+        else
+            a.traces[t] = out[p];
     }
 }
 
@@ -75,7 +80,7 @@ __global__ void __launch_bounds__(256) step_direct_kernel(const float *u,
                                                           const int *rec_ptr, const RecEntry *rec) {
     wait_predecessor();
     step_cell(u, up, out, w, a);
-    if (rec_ptr) record_block(out, a, blockIdx.z, rec_ptr, rec);
+    if (rec_ptr) record_block(out, w, a, blockIdx.z, rec_ptr, rec);
 }
 
 cudaError_t launch_step_direct(const float *u, const float *up, float *out, const float *w,

@@ -99,6 +99,7 @@ struct View {
     const SourceSample *src_;  // this step's source samples
     int nsrc_;
     float *traces_;            // [nrec][nt_max]
+    const float *inject;       // residual [nrec][nt_max] (Mode::kInject)
     int nt_max_;
     long long trace_step_;
     __device__ __forceinline__ const SourceSample *src() const { return src_; }
@@ -109,11 +110,15 @@ struct View {
     __device__ __forceinline__ long long trace_step() const { return trace_step_; }
 };
 
-// Items of one grid; everything comes from kernel parameters. kLap: the
-// launch also stores the stencil sum L u^n (into a.lap).
-template <int TX, int TY, bool kLap>
+// What a launch does besides the step: records the receivers (if any), also
+// stores the stencil sum L u^n (into a.lap), or adds W G r at the receivers
+// (r = a.inject, the adjoint's residual) instead of recording them.
+enum class Mode { kRecord, kLap, kInject };
+
+// Items of one grid; everything comes from kernel parameters.
+template <int TX, int TY, Mode M>
 struct OneGrid {
-    static constexpr bool kStoreLap = kLap;
+    static constexpr Mode kMode = M;
     using V = View;
     const StreamMaps &mp;
     const StepArgs &a;
@@ -139,7 +144,8 @@ struct OneGrid {
         v->trace_step_ = a.trace_step;
         v->u = u;
         v->out = up;
-        v->lap_delta = kLap ? a.lap - up : 0;
+        v->lap_delta = M == Mode::kLap ? a.lap - up : 0;
+        v->inject = M == Mode::kInject ? a.inject : nullptr;
         v->rec_ptr = rec_ptr;
         v->rec_ = rec;
     }
@@ -170,7 +176,7 @@ struct BatchView {
 // the run; shot s reads u^n from buf[cur0 ^ (t & 1)].
 template <int TX, int TY>
 struct ShotBatch {
-    static constexpr bool kStoreLap = false;
+    static constexpr Mode kMode = Mode::kRecord;
     using V = BatchView;
     const BatchShot *shots;
     const int2 *items;
@@ -337,11 +343,49 @@ struct Kern {
         return next;
     }
 
-    // Sources and receivers of plane k (few planes have any).
+    // Adds W G r at the receivers of plane k: lane q takes entry cur + q and
+    // reads its residual; the owning thread adds the entries one after the
+    // other (receivers may share a cell).
     template <class VT>
+    static __device__ __forceinline__ void inject_plane(Walk &wk, const VT &v, int k,
+                                                        float4 (&out)[2], const float4 &w0,
+                                                        const float4 &w1, float gzk) {
+        const int lane = threadIdx.x & 31;
+        int cur = wk.rcur;
+        for (;;) {
+            RecEntry e{INT_MAX, 0, 0, 0};
+            if (cur + lane < wk.rend) e = v.rec()[cur + lane];
+            const bool take = e.k == k;
+            float r = 0.0f;
+            if (take) r = v.inject[(long long)e.r * v.nt_max() + v.trace_step()];
+            const unsigned taken = __ballot_sync(0xffffffffu, take);
+            for (unsigned m = taken; m; m &= m - 1) {
+                const int q = __ffs(m) - 1;
+                const int owner = __shfl_sync(0xffffffffu, e.owner, q) & 31;
+                const int cell = __shfl_sync(0xffffffffu, e.lane, q);
+                const float rq = __shfl_sync(0xffffffffu, r, q);
+                if (lane != owner) continue;
+#pragma unroll
+                for (int c = 0; c < 8; ++c)
+                    if (cell == c) {
+                        const float gd = __fmul_rn(comp(wk.gxy[c / 4], c % 4), gzk);
+                        const float wg = __fmul_rn(comp(c < 4 ? w0 : w1, c % 4), gd);
+                        set_comp(out[c / 4], c % 4,
+                                 __fadd_rn(comp(out[c / 4], c % 4), __fmul_rn(wg, rq)));
+                    }
+            }
+            cur += __popc(taken);
+            if (taken != 0xffffffffu) break;
+        }
+        wk.rcur = cur;
+        wk.rnext_k = cur < wk.rend ? v.rec()[cur].k : INT_MAX;
+    }
+
+    // Sources and receivers of plane k (few planes have any).
+    template <Mode M, class VT>
     static __device__ __forceinline__ void events(Walk &wk, const VT &v, int k, int i, int j,
                                                   float4 (&out)[2], const float4 &w0,
-                                                  const float4 &w1) {
+                                                  const float4 &w1, float gzk) {
         for (unsigned m = wk.src_mask; m; m &= m - 1) {
             const SourceSample ss = v.src()[__ffs(m) - 1];
             if (ss.k != k) continue;
@@ -352,15 +396,19 @@ struct Kern {
                 if (ss.j == j + 1) set_comp(out[1], l, fmaf(comp(w1, l), ss.amp, comp(out[1], l)));
             }
         }
-        if (k == wk.rnext_k)
-            record_plane2(out, k, &wk.rcur, wk.rend, &wk.rnext_k, v.rec(), v.traces(), v.nt_max(),
-                          v.trace_step());
+        if (k == wk.rnext_k) {
+            if constexpr (M == Mode::kInject)
+                inject_plane(wk, v, k, out, w0, w1, gzk);
+            else
+                record_plane2(out, k, &wk.rcur, wk.rend, &wk.rnext_k, v.rec(), v.traces(),
+                              v.nt_max(), v.trace_step());
+        }
         wk.next_event = event_after(wk, v, k);
     }
 
     // Plane k of the item, RQ = (k - z0) mod kTrip (also the stage); parity:
     // of the trip. Returns false when a bounded wait ran out.
-    template <int RQ, bool kLap, class VT>
+    template <int RQ, Mode M, class VT>
     static __device__ __forceinline__ bool plane_step(Walk &wk, B &br, unsigned aOwn, unsigned bOwn,
                                                       unsigned ringA, unsigned ringB, const Job &jb,
                                                       const VT &v, const Coeffs &c, unsigned *status,
@@ -421,9 +469,9 @@ struct Kern {
         const float gzk = v.gz[k];
         float4 out[2] = {update(lap0, wk.q[Q4][0], up0, w0, wk.gxy[0], gzk),
                          update(lap1, wk.q[Q4][1], up1, w1, wk.gxy[1], gzk)};
-        if (k == wk.next_event) events(wk, v, k, i, j, out, w0, w1);
+        if (k == wk.next_event) events<M>(wk, v, k, i, j, out, w0, w1, gzk);
         store_rows(wk, wk.out_k, v.g.pnx, out[0], out[1]);
-        if constexpr (kLap)   // the stencil sum, for the adjoint's imaging
+        if constexpr (M == Mode::kLap)   // the stencil sum, for the adjoint's imaging
             store_rows(wk, wk.out_k + v.lap_delta, v.g.pnx,
                        make_float4(lap0[0].x, lap0[0].y, lap0[1].x, lap0[1].y),
                        make_float4(lap1[0].x, lap1[0].y, lap1[1].x, lap1[1].y));
@@ -562,7 +610,7 @@ __device__ __forceinline__ void stream_body(const S &src, const Coeffs &c, unsig
         for (int kb = it.z0;; kb += kTrip, parity ^= 1u) {
 #define WS_PLANE(RQ)                                                                              \
     if (kb + (RQ) >= it.z1 ||                                                                     \
-        !K::template plane_step<RQ, S::kStoreLap>(wk, br, aOwn, bOwn, ringA, ringB, jb, v, c,     \
+        !K::template plane_step<RQ, S::kMode>(wk, br, aOwn, bOwn, ringA, ringB, jb, v, c,     \
                                                   status, kb + (RQ), i, j, parity, issuer_warp))  \
         break;
             WS_PLANE(0)
@@ -589,13 +637,13 @@ __device__ __forceinline__ void stream_body(const S &src, const Coeffs &c, unsig
     }
 }
 
-template <int TX, int TY, int MINB, bool kLap>
+template <int TX, int TY, int MINB, Mode M>
 __global__ void __launch_bounds__(StreamCfg<TX, TY>::kThreads, MINB)
     step_stream_kernel(const __grid_constant__ StreamMaps maps, const float *u, float *up,
                        const __grid_constant__ StepArgs a, const int zb, const int tiles_x,
                        const int ntiles, const int *__restrict__ rec_ptr,
                        const RecEntry *__restrict__ rec) {
-    const OneGrid<TX, TY, kLap> src{maps, a, u, up, zb, tiles_x, ntiles, rec_ptr, rec};
+    const OneGrid<TX, TY, M> src{maps, a, u, up, zb, tiles_x, ntiles, rec_ptr, rec};
     stream_body<TX, TY>(src, a.c, a.status);
 }
 
@@ -648,11 +696,11 @@ cudaError_t with_tile(int tx, int ty, F &&fn) {
     return cudaErrorInvalidValue;
 }
 
-template <class T, bool kLap>
+template <class T, Mode M>
 cudaError_t launch_grid(const StreamMaps &maps, const float *u, float *up, const StepArgs &a, int zb,
                         const int *rec_ptr, const RecEntry *rec, cudaStream_t s) {
     using Cfg = StreamCfg<T::kX, T::kY>;
-    auto kern = step_stream_kernel<T::kX, T::kY, T::kMin, kLap>;
+    auto kern = step_stream_kernel<T::kX, T::kY, T::kMin, M>;
     static LaunchFacts lf;
     int ctas_per_sm = 0, sms = 0;
     cudaError_t e = occupancy(kern, Cfg::kThreads, Cfg::kSmem, lf, &ctas_per_sm, &sms);
@@ -688,8 +736,9 @@ cudaError_t launch_step_stream(const CUtensorMap *tmap_u, const CUtensorMap *tma
     maps.w = *tmap_w;
     return with_tile(t.tx, t.ty, [&](auto tag) {
         using T = decltype(tag);
-        if (a.lap) return launch_grid<T, true>(maps, u, up, a, t.zb, rec_ptr, rec, s);
-        return launch_grid<T, false>(maps, u, up, a, t.zb, rec_ptr, rec, s);
+        if (a.lap) return launch_grid<T, Mode::kLap>(maps, u, up, a, t.zb, rec_ptr, rec, s);
+        if (a.inject) return launch_grid<T, Mode::kInject>(maps, u, up, a, t.zb, rec_ptr, rec, s);
+        return launch_grid<T, Mode::kRecord>(maps, u, up, a, t.zb, rec_ptr, rec, s);
     });
 }
 
@@ -700,7 +749,7 @@ cudaError_t stream_slots(int tx, int ty, bool batch, int *slots, int *sms) {
         static LaunchFacts lf;
         int c = 0, n = 0;
         cudaError_t e = batch ? batch_facts<T>(&c, &n)
-                              : occupancy(step_stream_kernel<T::kX, T::kY, T::kMin, false>,
+                              : occupancy(step_stream_kernel<T::kX, T::kY, T::kMin, Mode::kRecord>,
                                           Cfg::kThreads, Cfg::kSmem, lf, &c, &n);
         if (e == cudaSuccess) *slots = c * n;
         if (e == cudaSuccess && sms) *sms = n;
