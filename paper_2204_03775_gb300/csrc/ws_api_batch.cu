@@ -298,7 +298,7 @@ int batch_configure(ws_batch_t b, int tx, int ty, int m) {
             int rc = encode_maps(ws);
             if (rc != WS_OK) return rc;
         }
-        int rc = build_rec_tiles(ws, ws::StreamTiling{tx, ty, zb});
+        int rc = build_rec_tiles(ws, ws::StreamTiling{tx, ty, zb}, false, b->stream);
         if (rc != WS_OK) return rc;
         const long long nit = tiles * ((g.nz + zb - 1) / zb);
         for (long long l = 0; l < nit; ++l) {
@@ -343,7 +343,7 @@ int batch_upload(ws_batch_t b, int nsteps) {
             int rc = encode_maps(ws);
             if (rc != WS_OK) return rc;
         }
-        int rc = build_rec_tiles(ws, ws::StreamTiling{b->tx, b->ty, b->zb[q]});
+        int rc = build_rec_tiles(ws, ws::StreamTiling{b->tx, b->ty, b->zb[q]}, false, b->stream);
         if (rc != WS_OK) return rc;
     }
     size_t total = 0;

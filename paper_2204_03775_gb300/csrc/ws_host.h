@@ -71,9 +71,13 @@ struct ws_handle {
     int nrec = 0, nt_max = 0;
     long long trace_start = 0;
     std::vector<int> rec_ijk;
-    float *traces = nullptr;
+    float *traces = nullptr;             // [nrec][nt_max] (kept while large enough)
+    size_t traces_cap = 0;
+    void *rec_table = nullptr;           // rec_ptr, then rec_entries (kept likewise)
+    size_t rec_table_cap = 0;
     int *rec_ptr = nullptr;              // per-tile ranges of rec_entries
     ws::RecEntry *rec_entries = nullptr;
+    float *stage = nullptr;              // planes of an unpadded field, for host arrays
     int rec_tiling_tx = 0, rec_tiling_ty = 0;
     bool rec_direct = false;             // the table is the direct kernel's
 
@@ -159,8 +163,10 @@ int default_zblock(const ws::Geom &g, int tx, int ty);
 // Choose the kernel for the next steps; fills *tiling for the streaming one.
 int pick_kernel(ws_t ws, ws::StreamTiling *tiling);
 void free_receivers(ws_t ws);
-// Receiver table of the streaming kernels, or of the direct kernel, for tile t.
-int build_rec_tiles(ws_t ws, const ws::StreamTiling &t, bool direct = false);
+// Receiver table of the streaming kernels, or of the direct kernel, for tile t,
+// uploaded on `stream` (ordered after the work on the handle's own that may
+// still read the old table).
+int build_rec_tiles(ws_t ws, const ws::StreamTiling &t, bool direct, cudaStream_t stream);
 // Unpadded [nz][ny][nx] user arrays <-> interiors of padded fields, one or
 // two fields a call (src2 / dst2 null: one).
 int copy_in(ws_t ws, float *dst, const float *src, int on_device, float *dst2 = nullptr,

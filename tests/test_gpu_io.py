@@ -133,3 +133,44 @@ def test_16bit_state_of_device_and_host_arrays(storage, nx, offset):
         wsb.ws_read_field(h, ou, ou)
         assert np.array_equal(ou.cpu().numpy(), ref[1])
         assert wsb.ws_test_check_padding(h) == 0
+
+
+def test_host_arrays_larger_than_the_staging():
+    """Host arrays move through the device staging in groups of planes: a field
+    of several groups, the last one short, comes back byte for byte."""
+    nz, ny, nx = 19, 1500, 1001       # 6 MB a plane, 10 planes in 64 MiB
+    rng = np.random.default_rng(0)
+    u, p = (rng.standard_normal((nz, ny, nx)).astype(np.float32) for _ in range(2))
+    h = wsb.ws_create(nx, ny, nz, 10.0, 1e-3)
+    wsb.ws_write_field(h, u, p, 0)
+    du, dp = device_copy(np.zeros_like(u), 0), device_copy(np.zeros_like(u), 0)
+    wsb.ws_read_field(h, du, dp)
+    assert np.array_equal(du.cpu().numpy(), u) and np.array_equal(dp.cpu().numpy(), p)
+    hu, hp = wsb.ws_read_field(h)
+    assert np.array_equal(hu, u) and np.array_equal(hp, p)
+    assert wsb.ws_test_check_padding(h) >= 0
+
+
+def test_receivers_set_again_and_again():
+    """Receiver buffers are kept while large enough: fewer, more, none, and the
+    same again give the traces of a new handle each time."""
+    nx, ny, nz = 70, 30, 20
+    v = np.full((nz, ny, nx), 3000.0, np.float32)
+
+    def handle():
+        h = wsb.ws_create(nx, ny, nz, 10.0, 1e-3)
+        wsb.ws_set_velocity(h, v)
+        wsb.ws_add_source(h, 30, 15, 10, 40.0, 0.0, 1.0)
+        return h
+
+    rng = np.random.default_rng(1)
+    kept = handle()
+    for nrec, nt in ((5, 8), (200, 20), (3, 4), (0, 0), (90, 12), (200, 20)):
+        rec = np.stack([rng.integers(0, n, nrec) for n in (nx, ny, nz)], 1).astype(np.int32)
+        new = handle()
+        for h in (kept, new):
+            wsb.ws_write_field(h, None, None, 0)
+            wsb.ws_set_receivers(h, rec, nt)
+            wsb.ws_step(h, max(nt, 3) - 1)
+        a, b = wsb.ws_read_traces(kept), wsb.ws_read_traces(new)
+        assert np.array_equal(a, b) and (nrec == 0 or not a[:, -1].any())
