@@ -12,14 +12,14 @@
 // GB300 runs FP64 at a 64th of its FP32 rate, and evaluated in FP64 (some 90
 // operations and conversions a cell) the kernel was bound by that pipe: 3.7 ms
 // at 320 x 288 x 256. Instead each cell is summed as pairs of floats, hi + lo,
-// through error-free sums and products (Dekker, Knuth), about 270 FP32
-// operations a cell, and only the threads' totals are FP64:
+// through error-free sums and products (Dekker, Knuth), about 280 FP32
+// operations a cell, and only the threads' totals are FP64 (0.37 ms, issue-bound):
 //  - 5040 h^2 L p = 8064 d1 - 1008 d2 + 128 d3 - 9 d4, d_m the six neighbours at
-//    distance m less 6 p: whole weights, so none is rounded. The pairs p(+m) +
-//    p(-m) and their difference to 2 p are error-free, and on smooth fields the
-//    difference is a single float.
-//  - Values are scaled by a power of two that brings the block's largest to
-//    about 1, so no product underflows that matters.
+//    distance m less 6 p: whole weights, so none is rounded, and sums of floats
+//    of like size leave lo words that are small multiples of one ulp.
+//  - Where the block's largest value is not within 2^-30 .. 2^40, values are
+//    scaled by a power of two that brings it to about 1, so no product underflows
+//    that matters.
 // The error of the sum against 80-bit arithmetic, both forms emulated on the
 // CPU, on smooth fields of 40^3 to 96^3 cells: at most 1.6e-16, FP64 3.0e-16
 // (whose weights are rounded); on white noise both 1 to 3e-16. Blocks out of the scaled range, and threads that meet a
@@ -77,7 +77,7 @@ __device__ __forceinline__ Pair two_prod(float a, float b) {   // a b exactly
 __device__ __forceinline__ Pair add(Pair a, Pair b) {
     const Pair s = two_sum(a.hi, b.hi);
     const float l = __fadd_rn(s.lo, __fadd_rn(a.lo, b.lo));
-    const float h = __fadd_rn(s.hi, l);   // renormalized
+    const float h = __fadd_rn(s.hi, l);
     return Pair{h, __fadd_rn(__fsub_rn(s.hi, h), l)};
 }
 __device__ __forceinline__ Pair mul(Pair a, float b) {
@@ -85,11 +85,14 @@ __device__ __forceinline__ Pair mul(Pair a, float b) {
     return Pair{p.hi, __fmaf_rn(a.lo, b, p.lo)};
 }
 
-// p(+m) + p(-m) - 2 p on one axis.
-__device__ __forceinline__ Pair second_difference(float plus, float minus, float p2) {
-    const Pair s = two_sum(plus, minus);
-    const Pair d = two_sum(s.hi, -p2);
-    return Pair{d.hi, __fadd_rn(d.lo, s.lo)};
+// a + b, lo not folded into hi (it may grow to a few ulps of it).
+__device__ __forceinline__ Pair add_loose(Pair a, Pair b) {
+    const Pair s = two_sum(a.hi, b.hi);
+    return Pair{s.hi, __fadd_rn(s.lo, __fadd_rn(a.lo, b.lo))};
+}
+__device__ __forceinline__ Pair renormalize(Pair a) {
+    const float h = __fadd_rn(a.hi, a.lo);
+    return Pair{h, __fadd_rn(__fsub_rn(a.hi, h), a.lo)};
 }
 
 // The values that a cell's term needs.
@@ -98,7 +101,8 @@ struct Cell {
     float n[4][6];   // p at distance 1 .. 4 on x+, x-, y+, y-, z+, z-
 };
 
-template <class F>
+// kInside: the y and z neighbours lie in the grid.
+template <bool kInside, class F>
 __device__ __forceinline__ Cell load_cell(const F &f, int i, int j, int k, int nx, int ny, int nz) {
     Cell c;
     const long long e = f.at(i, j, k), sy = f.row(), sz = f.plane();
@@ -109,29 +113,33 @@ __device__ __forceinline__ Cell load_cell(const F &f, int i, int j, int k, int n
     for (int m = 1; m <= 4; ++m) {
         c.n[m - 1][0] = f.p_near(e, m, i + m < nx);
         c.n[m - 1][1] = f.p_near(e, -m, i - m >= 0);
-        c.n[m - 1][2] = f.p_near(e, m * sy, j + m < ny);
-        c.n[m - 1][3] = f.p_near(e, -m * sy, j - m >= 0);
-        c.n[m - 1][4] = f.p_near(e, m * sz, k + m < nz);
-        c.n[m - 1][5] = f.p_near(e, -m * sz, k - m >= 0);
+        c.n[m - 1][2] = f.p_near(e, m * sy, kInside || j + m < ny);
+        c.n[m - 1][3] = f.p_near(e, -m * sy, kInside || j - m >= 0);
+        c.n[m - 1][4] = f.p_near(e, m * sz, kInside || k + m < nz);
+        c.n[m - 1][5] = f.p_near(e, -m * sz, kInside || k - m >= 0);
     }
     return c;
 }
 
 // Adds (u - p)^2 / w to *kin + *kin2 and 5040 u h^2 L p to *pot, of the values
-// times s (a power of two).
+// times s (a power of two; kScaled false: s = 1).
+template <bool kScaled>
 __device__ __forceinline__ void add_cell(const Cell &c, float s, Pair *kin, float *kin2, Pair *pot) {
-    const float u = c.u * s, p = c.p * s, p2 = 2.0f * p;
+    auto scaled = [&](float x) { return kScaled ? x * s : x; };
+    const float u = scaled(c.u), p = scaled(c.p);
+    const Pair p6 = two_prod(6.0f, p);
     Pair lap{0.0f, 0.0f};
 #pragma unroll
     for (int m = 4; m >= 1; --m) {
         const float *n = c.n[m - 1];
-        Pair d = second_difference(n[0] * s, n[1] * s, p2);
-        d = add(d, second_difference(n[2] * s, n[3] * s, p2));
-        d = add(d, second_difference(n[4] * s, n[5] * s, p2));
+        Pair d = two_sum(scaled(n[0]), scaled(n[1]));
+        d = add_loose(d, two_sum(scaled(n[2]), scaled(n[3])));
+        d = add_loose(d, two_sum(scaled(n[4]), scaled(n[5])));
+        d = add_loose(d, Pair{-p6.hi, -p6.lo});
         const Pair t = mul(d, m == 1 ? 8064.0f : m == 2 ? -1008.0f : m == 3 ? 128.0f : -9.0f);
-        lap = m == 4 ? t : add(lap, t);
+        lap = m == 4 ? t : add_loose(lap, t);
     }
-    *pot = add(*pot, mul(lap, u));
+    *pot = add(*pot, mul(renormalize(lap), u));
     // u - p = d exactly; (u - p)^2 = q + d.lo^2, the last below 2^-50 of q but
     // never negative, so it is summed apart
     const Pair d = two_sum(u, -p);
@@ -167,10 +175,25 @@ __device__ __noinline__ double cell_fp64(const Cell &c, const Coeffs64 &w, doubl
     return __fma_rn(-uc, lap, __ddiv_rn(__dmul_rn(d, d), vdt2));
 }
 
+// This thread's cells of rows [j0, j1) of plane k, a warp a row at a time;
+// false if one of them has a model out of range.
+template <bool kScaled, bool kInside, class F>
+__device__ __forceinline__ bool sum_rows(const F &f, int j0, int j1, int k, int nx, int ny, int nz,
+                                         float s, Pair *kin, float *kin2, Pair *pot) {
+    bool good = true;
+    for (int j = j0 + (threadIdx.x >> 5); j < j1; j += kThreads / 32)
+        for (int i = threadIdx.x & 31; i < nx; i += 32) {
+            const Cell q = load_cell<kInside>(f, i, j, k, nx, ny, nz);
+            good = good && q.w >= 0x1p-60f;
+            add_cell<kScaled>(q, s, kin, kin2, pot);
+        }
+    return good;
+}
+
 // Block (x = row block jb, y = plane k) sums rows [jb*rows, jb*rows+rows) of
 // plane k into partials[k * gridDim.x + jb]; a warp takes whole rows.
 template <class F>
-__global__ void __launch_bounds__(kThreads)
+__global__ void __launch_bounds__(kThreads, 3)
     energy_partials_kernel(F f, int nx, int ny, int nz, int rows, double h2, Coeffs64 c,
                            double *__restrict__ partials) {
     const int k = blockIdx.y;
@@ -196,25 +219,25 @@ __global__ void __launch_bounds__(kThreads)
     double acc = 0.0;
     if (big != 0u) {   // else every term is zero
         const int ex = (int)(big >> 23) - 127;
-        const int se = max(-60, min(60, -ex));
+        // values near 1 need no scaling; else the block's largest is brought there
+        const bool near1 = ex >= -30 && ex <= 40;
+        const int se = near1 ? 0 : max(-60, min(60, -ex));
         const float s = __int_as_float((se + 127) << 23);
+        const bool inside = j0 >= 4 && j1 + 4 <= ny && k >= 4 && k + 4 < nz;
         Pair kin{0.0f, 0.0f}, pot{0.0f, 0.0f};
         float kin2 = 0.0f;
-        bool fast = abs(ex + se) <= 30;
-        if (fast)
-            for (int j = j0 + warp; j < j1; j += kThreads / 32)
-                for (int i = lane; i < nx; i += 32) {
-                    const Cell q = load_cell(f, i, j, k, nx, ny, nz);
-                    fast = fast && q.w >= 0x1p-60f;
-                    add_cell(q, s, &kin, &kin2, &pot);
-                }
+        bool fast = near1 || abs(ex + se) <= 30;
+        if (near1 && inside)
+            fast = sum_rows<false, true>(f, j0, j1, k, nx, ny, nz, s, &kin, &kin2, &pot);
+        else if (fast)
+            fast = sum_rows<true, false>(f, j0, j1, k, nx, ny, nz, s, &kin, &kin2, &pot);
         const double K = (double)kin.hi + ((double)kin.lo + (double)kin2), Q = (double)pot.hi + (double)pot.lo;
         if (fast && isfinite(K) && isfinite(Q))
             acc = (K - Q / 5040.0) * scalbn(1.0, -2 * se) / h2;
         else
             for (int j = j0 + warp; j < j1; j += kThreads / 32)
                 for (int i = lane; i < nx; i += 32)
-                    acc = __dadd_rn(acc, cell_fp64(load_cell(f, i, j, k, nx, ny, nz), c, h2));
+                    acc = __dadd_rn(acc, cell_fp64(load_cell<false>(f, i, j, k, nx, ny, nz), c, h2));
     }
     // fixed-order block reduction: warp shuffles, then warp 0
 #pragma unroll
