@@ -56,9 +56,7 @@ __device__ __forceinline__ void step_cell(const float *u, const float *up, float
 // may share one), once all its threads have stored. (As a launch of its own this
 // cost 1 us a step on grids of a few microseconds.)
 __device__ __forceinline__ void record_block(float *out, const float *w, const StepArgs &a, int k,
-                                             const int *rec_ptr, const RecEntry *rec) {
-    const int tile = blockIdx.y * gridDim.x + blockIdx.x;
-    const int lo = rec_ptr[tile], hi = rec_ptr[tile + 1];
+                                             int lo, int hi, const RecEntry *rec) {
     if (lo == hi) return;
     __syncthreads();
     const int tid = threadIdx.y * blockDim.x + threadIdx.x;
@@ -78,9 +76,13 @@ __global__ void __launch_bounds__(256) step_direct_kernel(const float *u,
                                                           const float *w,
                                                           const __grid_constant__ StepArgs a,
                                                           const int *rec_ptr, const RecEntry *rec) {
+    // no kernel writes the receiver table: its ranges are read before the
+    // predecessor is waited for
+    const int tile = blockIdx.y * gridDim.x + blockIdx.x;
+    const int lo = rec_ptr ? rec_ptr[tile] : 0, hi = rec_ptr ? rec_ptr[tile + 1] : 0;
     wait_predecessor();
     step_cell(u, up, out, w, a);
-    if (rec_ptr) record_block(out, w, a, blockIdx.z, rec_ptr, rec);
+    record_block(out, w, a, blockIdx.z, lo, hi, rec);
 }
 
 cudaError_t launch_step_direct(const float *u, const float *up, float *out, const float *w,

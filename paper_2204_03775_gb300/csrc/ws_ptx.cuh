@@ -19,8 +19,8 @@ struct LaunchFacts {
 // Overlap of a step with the end of the one before it on the same stream
 // (programmatic dependent launch). A kernel launched with launch_overlapped
 // may start while its predecessor still runs: every thread calls
-// wait_predecessor before it touches global memory (it returns once all
-// earlier work of the stream is complete and visible), then lets its own
+// wait_predecessor before it touches global memory that a kernel writes (it
+// returns once all earlier work of the stream is complete and visible), then lets its own
 // successor start, whose blocks fill the slots that the last wave leaves free.
 // Since the release comes after the wait, at most two kernels of a stream
 // overlap and a successor never runs ahead of anything but its predecessor.
