@@ -1099,8 +1099,11 @@ int ws_write_field(ws_t ws, const float *u, const float *u_prev, long long step,
     // only a missing level needs its buffer cleared
     const size_t fb = field_bytes(ws->g);
     float *un = ws->buf[ws->cur], *um = ws->buf[1 - ws->cur];
-    if (!u) WS_CUDA(cudaMemsetAsync(un, 0, fb, ws->stream), "ws_write_field");
-    if (!u_prev) WS_CUDA(cudaMemsetAsync(um, 0, fb, ws->stream), "ws_write_field");
+    if (!u || !u_prev) {
+        float *first = u ? um : un, *second = u || u_prev ? nullptr : um;
+        WS_CUDA(ws::launch_zero(first, second, fb, ws->stream), "ws_write_field");
+        ws->launches++;
+    }
     int rc = WS_OK;
     if (u)
         rc = copy_in(ws, un, u, on_device, u_prev ? um : nullptr, u_prev);

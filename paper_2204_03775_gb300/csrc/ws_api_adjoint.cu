@@ -141,7 +141,8 @@ int forward_begin(ws_t ws, AdjointCache *ac) {
     const size_t ntr = size_t(ws->nrec) * ws->nt_max;
     const cudaStream_t st = ws->stream;
     ac->fwd_valid = false;
-    for (int b = 0; b < 2; ++b) WS_CUDA(cudaMemsetAsync(ws->buf[b], 0, fb, st), "zero fields");
+    WS_CUDA(ws::launch_zero(ws->buf[0], ws->buf[1], fb, st), "zero fields");
+    ws->launches++;
     WS_CUDA(cudaMemsetAsync(ws->traces, 0, sizeof(float) * ntr, st), "zero traces");
     ws->step = 0;
     ws->trace_start = 0;
@@ -203,9 +204,13 @@ int gradient_run(GradShot *sh, int n, int mode) {
     for (int q = 0; q < n; ++q) {
         GradShot &x = sh[q];
         const cudaStream_t st = x.ws->stream;
-        for (int k : {N + 1, N + 2})   // rho^{N+1} = rho^{N+2} = 0
-            WS_CUDA(cudaMemsetAsync(x.ac->rho[k % x.ac->nrho].p, 0, fb, st), "zero adjoint field");
-        WS_CUDA(cudaMemsetAsync(x.ac->acc, 0, 2 * fb, st), "zero gradient accumulator");
+        // rho^{N+1} = rho^{N+2} = 0
+        WS_CUDA(ws::launch_zero(x.ac->rho[(N + 1) % x.ac->nrho].p, x.ac->rho[(N + 2) % x.ac->nrho].p,
+                                fb, st),
+                "zero adjoint field");
+        WS_CUDA(ws::launch_zero(reinterpret_cast<float *>(x.ac->acc), nullptr, 2 * fb, st),
+                "zero gradient accumulator");
+        x.ws->launches += 2;
         // a residual given for the run that ws_forward left in the cache (same
         // model version) needs no new forward run
         x.forward = !(mode == WS_ADJ_RESIDUAL && x.ac->fwd_valid &&
@@ -244,9 +249,12 @@ int gradient_run(GradShot *sh, int n, int mode) {
         // n0] (u^{n1} itself is not needed). The first two read the checkpoint
         // where it lies; u^m, m > n0, goes to ring[m & 1].
         if (j == 0)
-            for (int q = 0; q < n; ++q)   // from rest: u^0 = ring[0], u^{-1} = ring[1]
-                for (auto &f : sh[q].ac->ring)
-                    WS_CUDA(cudaMemsetAsync(f.p, 0, fb, sh[q].ws->stream), "zero initial state");
+            for (int q = 0; q < n; ++q) {   // from rest: u^0 = ring[0], u^{-1} = ring[1]
+                AdjointCache *ac = sh[q].ac;
+                WS_CUDA(ws::launch_zero(ac->ring[0].p, ac->ring[1].p, fb, sh[q].ws->stream),
+                        "zero initial state");
+                sh[q].ws->launches++;
+            }
         for (int m = n0; m < n1; ++m)
             for (int q = 0; q < n; ++q) {
                 GradShot &x = sh[q];

@@ -158,6 +158,8 @@ inline Fp32Pair<T> dense_pair(T *u, T *up, const Geom &g) {
 // not overlap. Pointers are aligned to 4 bytes.
 cudaError_t launch_copy_in(const float *a, const float *b, float *A, float *B, const Geom &g,
                            cudaStream_t s);
+// bytes (a multiple of 16) of the buffers a and, if not null, b to zero.
+cudaError_t launch_zero(float *a, float *b, size_t bytes, cudaStream_t s);
 cudaError_t launch_copy_out(const float *A, const float *B, float *a, float *b, const Geom &g,
                             cudaStream_t s);
 

@@ -191,6 +191,18 @@ __global__ void __launch_bounds__(kRowThreads)
     }
 }
 
+// Whole buffers (padding included) to zero: n floats of a, and of b if given.
+// One launch for a pair of fields: a memset's call takes the host 11 us, which
+// a run of a few hundred microseconds does not hide.
+__global__ void __launch_bounds__(kRowThreads) zero_kernel(float4 *a, float4 *b, long long n4) {
+    const float4 z = make_float4(0.f, 0.f, 0.f, 0.f);
+    for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < n4;
+         t += (long long)gridDim.x * blockDim.x) {
+        a[t] = z;
+        if (b) b[t] = z;
+    }
+}
+
 bool aligned16(const void *p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
 
 template <bool kIn>
@@ -218,6 +230,14 @@ cudaError_t launch_copy(const Fields &f, const Geom &g, cudaStream_t s) {
 }
 
 }  // namespace
+
+cudaError_t launch_zero(float *a, float *b, size_t bytes, cudaStream_t s) {
+    const long long n4 = (long long)(bytes / sizeof(float4));   // fields are whole 128-byte rows
+    const long long want = (n4 + kRowThreads - 1) / kRowThreads;
+    zero_kernel<<<(unsigned)(want < kCopyBlocks ? want : kCopyBlocks), kRowThreads, 0, s>>>(
+        reinterpret_cast<float4 *>(a), reinterpret_cast<float4 *>(b), n4);
+    return cudaGetLastError();
+}
 
 cudaError_t launch_copy_in(const float *a, const float *b, float *A, float *B, const Geom &g,
                            cudaStream_t s) {
