@@ -290,7 +290,7 @@ int ws_set_storage(ws_t ws, int storage);
  * tile_x x tile_y in {32x8, 32x16, 64x8, 64x16, 64x32} for the FP32 kernel
  * (0, 0 = keep the chosen tile; while none is chosen the step takes 64x16, or
  * 32x16 where 64-cell tiles would be mostly empty, or 8 rows on low grids, and
- * AUTO runs grids of at most 200000 cells with the direct kernel) or in {64x16,
+ * AUTO runs grids of at most 150000 cells with the direct kernel) or in {64x16,
  * 64x24, 64x48} for the 16-bit kernel (64x16 selects both; a 16-bit tile leaves
  * the FP32 tile unchanged and needs nx >= 64 and ny >= tile_y), zblock >= 1
  * planes per work item (0 = default: the block, and for 16-bit storage the tile

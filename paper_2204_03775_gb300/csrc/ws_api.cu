@@ -200,11 +200,12 @@ bool default_tile(const ws::Geom &g, ws::StreamTiling *t) {
 
 // Choose the kernel for the next steps; fills *tiling for the streaming one.
 // Grids of at most kDirectCells cells, left to choose by themselves, take the
-// direct kernel: 101 x 37 x 45 in 2.9 us a step against 3.5 in stream tiles,
-// 48 x 40 x 40 2.3 against 3.4, 191 x 25 x 43 (205 thousand cells) 3.4 either
-// way, 64^3 3.5 against 3.3, 138 x 55 x 138 9.2 against 7.1.
+// direct kernel (steps with receivers): 80 x 40 x 35 in 2.48 us against 2.87 in
+// the best stream tile and block, 48 x 40 x 40 2.30 against 2.84; 218 x 37 x 20
+// (161 thousand cells) 3.43 against 3.20, 101 x 37 x 45 3.44 against 3.27, 64^3
+// 3.48 against 3.18, 138 x 55 x 138 9.2 against 7.1.
 int pick_kernel(ws_t ws, ws::StreamTiling *tiling) {
-    constexpr long long kDirectCells = 200000;
+    constexpr long long kDirectCells = 150000;
     if (ws->kernel == WS_KERNEL_DIRECT) return WS_KERNEL_DIRECT;
     const ws::Geom &g = ws->g;
     ws::StreamTiling t = ws->tiling;

@@ -46,7 +46,7 @@ def test_every_tile_gives_the_direct_kernels_bits(tile, shape):
             assert np.array_equal(r, x)
 
 
-@pytest.mark.parametrize("shape", [(20, 99, 101), (20, 100, 101), (40, 40, 48), (6, 12, 80),
+@pytest.mark.parametrize("shape", [(15, 99, 101), (15, 100, 101), (20, 100, 101), (40, 40, 48), (6, 12, 80),
                                    (7, 40, 33), (3, 5, 300)])
 def test_default_choice_gives_the_direct_kernels_bits(shape):
     """Grids on both sides of the direct kernel's limit, low and narrow ones."""
