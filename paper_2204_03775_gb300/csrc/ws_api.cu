@@ -325,9 +325,28 @@ int build_rec_tiles(ws_t ws, const ws::StreamTiling &t, bool direct, cudaStream_
     return WS_OK;
 }
 
-// Whether the copy kernels may take a device array: float elements on their
-// natural alignment (a 2D copy takes any address).
-static bool kernel_copyable(const void *p) { return (reinterpret_cast<uintptr_t>(p) & 3u) == 0; }
+static bool on_this_device(const char *p) {
+    cudaPointerAttributes a{};
+    int dev = -1;
+    if (cudaPointerGetAttributes(&a, p) != cudaSuccess || cudaGetDevice(&dev) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    return (a.type == cudaMemoryTypeDevice && a.device == dev) || a.type == cudaMemoryTypeManaged;
+}
+
+// Whether kernels may take a caller's device array of an unpadded field (or no
+// array): floats on their natural alignment, in this device's memory from the
+// first byte to the last. A 2D copy takes any address, and returns an error where
+// a kernel would fault. (Asking costs the host 0.5 us an array: two levels of 96^3
+// in and out and a step between them 26.3 -> 28.2 us.)
+static bool kernel_copyable(const ws_t ws, const void *p) {
+    if (!p) return true;
+    const char *c = static_cast<const char *>(p);
+    const size_t bytes = sizeof(float) * size_t(ws->g.nx) * ws->g.ny * ws->g.nz;
+    return (reinterpret_cast<uintptr_t>(p) & 3u) == 0 && on_this_device(c) &&
+           on_this_device(c + bytes - 1);
+}
 
 // The handle's device staging for host arrays: planes of an unpadded field, at
 // most kStageMax bytes (null: not even one plane, or no memory). *planes of them
@@ -341,12 +360,16 @@ static float *host_stage(ws_t ws, int *planes) {
     *planes = (int)std::min<size_t>(g.nz, kStageMax / plane);
     if (*planes < 1) return nullptr;
     if (!ws->stage) {
+        // another thread's capture must not see this allocation
+        cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+        cudaThreadExchangeStreamCaptureMode(&mode);
         cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
         if (cudaStreamIsCapturing(ws->stream, &st) != cudaSuccess ||
             st != cudaStreamCaptureStatusNone || cudaMalloc(&ws->stage, plane * *planes) != cudaSuccess) {
             cudaGetLastError();
             ws->stage = nullptr;
         }
+        cudaThreadExchangeStreamCaptureMode(&mode);
     }
     return ws->stage;
 }
@@ -355,7 +378,7 @@ static float *host_stage(ws_t ws, int *planes) {
 // arrays by one kernel, host arrays through the staging buffer or plane by plane.
 int copy_in(ws_t ws, float *dst, const float *src, int on_device, float *dst2, const float *src2) {
     const ws::Geom &g = ws->g;
-    if (on_device && kernel_copyable(src) && kernel_copyable(src2)) {
+    if (on_device && kernel_copyable(ws, src) && kernel_copyable(ws, src2)) {
         WS_CUDA(ws::launch_copy_in(src, src2, dst, dst2, g, ws->stream), "copy into the padded field");
         ws->launches++;
         return WS_OK;
@@ -388,7 +411,7 @@ int copy_in(ws_t ws, float *dst, const float *src, int on_device, float *dst2, c
 int copy_out(ws_t ws, float *dst, const float *src, int on_device, float *dst2, const float *src2) {
     const ws::Geom &g = ws->g;
     const size_t n = size_t(g.nx) * g.ny * g.nz;
-    if (on_device && kernel_copyable(dst) && kernel_copyable(dst2)) {
+    if (on_device && kernel_copyable(ws, dst) && kernel_copyable(ws, dst2)) {
         // outputs that overlap get their copies one after the other
         const bool both = src2 && (dst2 >= dst + n || dst >= dst2 + n);
         WS_CUDA(ws::launch_copy_out(src, both ? src2 : nullptr, dst, both ? dst2 : nullptr, g,
@@ -771,7 +794,7 @@ int ws_set_velocity(ws_t ws, const float *v, int on_device) {
     if (!ws || !v) return fail(WS_ERR_BADARG, "ws_set_velocity: NULL argument");
     ws->model_version++;
     ws->vel_ok = false;
-    const bool direct = on_device && kernel_copyable(v);
+    const bool direct = on_device && kernel_copyable(ws, v);
     if (!direct) {
         int rc = copy_in(ws, ws->w, v, on_device);
         if (rc != WS_OK) return rc;
@@ -805,7 +828,7 @@ int ws_set_slowness2(ws_t ws, const float *m, int on_device) {
     if (!ws || !m) return fail(WS_ERR_BADARG, "ws_set_slowness2: NULL argument");
     ws->model_version++;
     ws->vel_ok = false;
-    const bool direct = on_device && kernel_copyable(m);
+    const bool direct = on_device && kernel_copyable(ws, m);
     if (!direct) {
         int rc = copy_in(ws, ws->w, m, on_device);
         if (rc != WS_OK) return rc;
@@ -1065,7 +1088,7 @@ int ws_read_field(ws_t ws, float *u, float *u_prev, int on_device) {
     if (!ws) return fail(WS_ERR_BADARG, "ws_read_field: NULL handle");
     int rc = WS_OK;
     if (ws->storage != WS_STORAGE_FP32) {
-        if (on_device && kernel_copyable(u) && kernel_copyable(u_prev)) {
+        if (on_device && kernel_copyable(ws, u) && kernel_copyable(ws, u_prev)) {
             // straight into the caller's arrays; outputs that overlap one
             // after the other
             const size_t n = size_t(ws->g.nx) * ws->g.ny * ws->g.nz;
@@ -1091,8 +1114,8 @@ int ws_read_field(ws_t ws, float *u, float *u_prev, int on_device) {
 int ws_write_field(ws_t ws, const float *u, const float *u_prev, long long step, int on_device) {
     if (!ws) return fail(WS_ERR_BADARG, "ws_write_field: NULL handle");
     if (step < 0) return fail(WS_ERR_BADARG, "ws_write_field: step must be >= 0");
-    if (ws->storage != WS_STORAGE_FP32 && on_device && (u || u_prev) && kernel_copyable(u) &&
-        kernel_copyable(u_prev)) {
+    if (ws->storage != WS_STORAGE_FP32 && on_device && (u || u_prev) && kernel_copyable(ws, u) &&
+        kernel_copyable(ws, u_prev)) {
         ws->step = step;   // straight from the caller's arrays
         return encode_state16(ws, ws::dense_pair(u, u_prev, ws->g));
     }

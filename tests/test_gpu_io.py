@@ -6,6 +6,8 @@ ragged tail, single cells), the alignment of the device array, one field or
 both, and nothing outside the interior may change.
 """
 
+import ctypes
+
 import numpy as np
 import pytest
 
@@ -13,6 +15,7 @@ torch = pytest.importorskip("torch")
 pytestmark = pytest.mark.gpu
 
 import paper_2204_03775_gb300 as wsb  # noqa: E402
+from paper_2204_03775_gb300 import binding  # noqa: E402
 
 
 def device_copy(a, offset):
@@ -174,3 +177,46 @@ def test_receivers_set_again_and_again():
             wsb.ws_step(h, max(nt, 3) - 1)
         a, b = wsb.ws_read_traces(kept), wsb.ws_read_traces(new)
         assert np.array_equal(a, b) and (nrec == 0 or not a[:, -1].any())
+
+
+@pytest.mark.parametrize("kind", ["bytes", "pinned"])
+@pytest.mark.parametrize("storage", [wsb.WS_STORAGE_FP32, wsb.WS_STORAGE_FP16])
+def test_arrays_that_no_kernel_may_take(kind, storage):
+    """Arrays said to be on the device that are not float-aligned, or lie in
+    host memory, go through the copies that take any address: right or refused."""
+    lib = binding.load_library()
+    shape = (5, 17, 67)
+    nz, ny, nx = shape
+    rng = np.random.default_rng(3)
+    u = rng.integers(-64, 64, shape).astype(np.float32)
+    v = np.full(shape, 3000.0, np.float32)
+
+    def handle():
+        h = wsb.ws_create(nx, ny, nz, 10.0, 1e-3)
+        wsb.ws_set_storage(h, storage)
+        return h
+
+    if kind == "bytes":
+        raw = [torch.zeros(u.nbytes + 2, dtype=torch.uint8, device="cuda") for _ in range(3)]
+        views = [r[2:] for r in raw]
+    else:
+        views = [torch.zeros(u.nbytes, dtype=torch.uint8).pin_memory() for _ in range(3)]
+    for t, a in zip(views, (u, v)):
+        t.copy_(torch.from_numpy(a.reshape(-1).view(np.uint8).copy()))
+    torch.cuda.synchronize()
+    pu, pv, po = (ctypes.c_void_p(t.data_ptr()) for t in views)
+    h, ref = handle(), handle()
+    wsb.ws_write_field(ref, u, None, 0)
+    wsb.ws_set_velocity(ref, v)
+    ok = [lib.ws_write_field(h.ptr, pu, None, 0, 1), lib.ws_set_velocity(h.ptr, pv, 1),
+          lib.ws_read_field(ref.ptr, po, None, 1)]
+    wsb.ws_synchronize(h)
+    wsb.ws_synchronize(ref)
+    if kind == "bytes":
+        assert ok == [0, 0, 0]
+    if ok[0] == 0 and ok[1] == 0:
+        for g in (h, ref):
+            wsb.ws_step(g, 2)
+        assert all(np.array_equal(a, b) for a, b in zip(wsb.ws_read_field(h), wsb.ws_read_field(ref)))
+    if ok[2] == 0:
+        assert np.array_equal(views[2].cpu().numpy().view(np.float32).reshape(shape), u)
