@@ -222,10 +222,9 @@ int ws_energy_noalloc(const float *u, const float *u_prev, const float *v, int n
  * again; the handle's state is then left as it is.
  *
  * Needs a velocity model, receivers and FP32 storage, else STATE. Device
- * scratch: about 3 sqrt(N) + 6 padded fields (2 more where the memory holds
- * them) and two trace arrays, allocated by the first call and kept by the handle for the
- * next ones while N, the receiver count and the tiling stay the same (freed
- * by ws_destroy).
+ * scratch: about 3 sqrt(N) + 6 padded fields and two trace arrays, allocated by
+ * the first call and kept by the handle for the next ones while N, the receiver
+ * count and the tiling stay the same (freed by ws_destroy).
  * Afterwards the handle holds the forward run's final state (step N) and
  * its traces. Synchronizes the stream. Errors: BADARG, STATE, OOM, CUDA,
  * TIMEOUT. */
@@ -281,7 +280,7 @@ int ws_forward(ws_t ws);
  * 4.1e-3; BF16 6.1e-3, 2.3e-2, 3.5e-2 (FP32 storage 5.3e-7 ... 1.9e-6): FP16
  * stays within 1e-2, BF16 only for about the first 100 steps (its 8-bit
  * significand's rounding errors add up like a random walk); at 1024^3 after
- * 100 steps FP16 7.6e-4, BF16 5.9e-3. Speed on the 1024^3 survey: 1.28x (FP16
+ * 100 steps FP16 7.6e-4, BF16 5.9e-3. Speed on the 1024^3 survey: 1.20x (FP16
  * and BF16) of FP32 storage. This realizes the reduced-precision
  * storage that the paper contrasts with its FP32-only arithmetic (Section I). */
 int ws_set_storage(ws_t ws, int storage);

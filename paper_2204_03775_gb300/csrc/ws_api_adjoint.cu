@@ -71,10 +71,8 @@ int adjoint_prepare(ws_t ws, const char *who, int *kern_out, ws::StreamTiling *t
             if (e == cudaSuccess) e = cudaMemsetAsync(f, 0, fb, st);
         }
         int r3 = e == cudaSuccess ? WS_OK : cuda_fail(e, "cudaMalloc adjoint field");
-        for (auto &f : ac->ring)
+        for (auto &f : ac->level)
             if (r3 == WS_OK) r3 = field(&f);
-        for (int q = 0; q < 2; ++q)
-            if (r3 == WS_OK) r3 = field(&ac->rho[q]);
         if (r3 == WS_OK) e = grab(&ac->acc, 2 * fb);   // float2 per cell, padded layout
         if (r3 == WS_OK && e == cudaSuccess) e = grab(&ac->partials, sizeof(double) * (ws::residual_partial_count() + 1));
         if (r3 == WS_OK && e == cudaSuccess) e = grab(&ac->norm, sizeof(double) * (ws::residual_partial_count() + 1));
@@ -85,23 +83,6 @@ int adjoint_prepare(ws_t ws, const char *who, int *kern_out, ws::StreamTiling *t
             delete ws->adj;
             ws->adj = nullptr;
             return r3 != WS_OK ? r3 : cuda_fail(e, "cudaMalloc adjoint scratch");
-        }
-        // more levels of rho, if there is room for them, so that more steps are
-        // imaged together
-        for (int q = 2; q < ws::kMaxImagingSteps; ++q) {
-            if (grab(&ac->rho[q].p, fb) != cudaSuccess) {
-                cudaGetLastError();
-                break;
-            }
-            WS_CUDA(cudaMemsetAsync(ac->rho[q].p, 0, fb, st), "zero adjoint field");
-            if (maps) {
-                const int tx = ws->tiling.tx, ty = ws->tiling.ty;
-                int r4 = encode_map(&ac->rho[q].halo, ac->rho[q].p, g, tx + 2 * ws::kHalo,
-                                    ty + 2 * ws::kHalo);
-                if (r4 == WS_OK) r4 = encode_map(&ac->rho[q].tile, ac->rho[q].p, g, tx, ty);
-                if (r4 != WS_OK) return r4;
-            }
-            ac->nrho = q + 1;
         }
         ac->N = N;
         ac->nrec = ws->nrec;
@@ -205,8 +186,7 @@ int gradient_run(GradShot *sh, int n, int mode) {
         GradShot &x = sh[q];
         const cudaStream_t st = x.ws->stream;
         // rho^{N+1} = rho^{N+2} = 0
-        WS_CUDA(ws::launch_zero(x.ac->rho[(N + 1) % x.ac->nrho].p, x.ac->rho[(N + 2) % x.ac->nrho].p,
-                                fb, st),
+        WS_CUDA(ws::launch_zero(x.ac->rho(N + 1).p, x.ac->rho(N + 2).p, fb, st),
                 "zero adjoint field");
         WS_CUDA(ws::launch_zero(reinterpret_cast<float *>(x.ac->acc), nullptr, 2 * fb, st),
                 "zero gradient accumulator");
@@ -247,11 +227,11 @@ int gradient_run(GradShot *sh, int n, int mode) {
         const int n0 = j * C, n1 = std::min(n0 + C, N);
         // steps n0 .. n1-1 from the checkpoint, each storing L u^n into lap[n -
         // n0] (u^{n1} itself is not needed). The first two read the checkpoint
-        // where it lies; u^m, m > n0, goes to ring[m & 1].
+        // where it lies; u^m, m > n0, goes to ring(n1, m).
         if (j == 0)
-            for (int q = 0; q < n; ++q) {   // from rest: u^0 = ring[0], u^{-1} = ring[1]
+            for (int q = 0; q < n; ++q) {   // from rest
                 AdjointCache *ac = sh[q].ac;
-                WS_CUDA(ws::launch_zero(ac->ring[0].p, ac->ring[1].p, fb, sh[q].ws->stream),
+                WS_CUDA(ws::launch_zero(ac->ring(n1, 0).p, ac->ring(n1, 1).p, fb, sh[q].ws->stream),
                         "zero initial state");
                 sh[q].ws->launches++;
             }
@@ -259,7 +239,7 @@ int gradient_run(GradShot *sh, int n, int mode) {
             for (int q = 0; q < n; ++q) {
                 GradShot &x = sh[q];
                 auto level = [&](int l) -> MappedField & {   // u^l
-                    return l <= n0 && j > 0 ? x.ac->ck[2 * (j - 1) + (l & 1)] : x.ac->ring[l & 1];
+                    return l <= n0 && j > 0 ? x.ac->ck[2 * (j - 1) + (l & 1)] : x.ac->ring(n1, l);
                 };
                 MappedField &un = level(m), &um = level(m - 1);
                 x.a.lap = x.ac->lap[m - n0];
@@ -272,10 +252,8 @@ int gradient_run(GradShot *sh, int n, int mode) {
             for (int q = 0; q < n; ++q) {
                 GradShot &x = sh[q];
                 ws_t ws = x.ws;
-                const int nr = x.ac->nrho;
-                MappedField *rho = x.ac->rho;
-                MappedField &r1 = rho[(k + 1) % nr], &r2 = rho[(k + 2) % nr];
-                float *out = rho[k % nr].p;
+                MappedField &r1 = x.ac->rho(k + 1), &r2 = x.ac->rho(k + 2);
+                float *out = x.ac->rho(k).p;
                 // rho^k, with W G r^k (trace column k - 1) added at the receivers
                 x.a.inject = x.ac->r;
                 int rc = step_fp32(ws, x.a, x.kern, x.tiling, r1.p, &r1.halo, r2.p, &r2.tile, out,
@@ -288,7 +266,7 @@ int gradient_run(GradShot *sh, int n, int mode) {
                 x.img.rho[x.pending] = out;
                 x.img.lap[x.pending] = x.ac->lap[k - 1 - n0];
                 for (int s = 0; s < src.n; ++s) x.img.amp[x.pending][s] = src.s[s].amp;
-                if (++x.pending < nr && k > n0 + 1) continue;
+                if (++x.pending < ws::kMaxImagingSteps && k > n0 + 1) continue;
                 WS_CUDA(ws::launch_imaging(x.img, x.pending, g, src, ws->gx, ws->gy, ws->gz,
                                            x.ac->acc, ws->stream),
                         "gradient imaging kernel");

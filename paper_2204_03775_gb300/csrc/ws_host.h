@@ -121,9 +121,10 @@ struct MappedField {
     CUtensorMap halo, tile;
 };
 
-// Scratch of ws_adjoint_gradient: checkpoint pairs, the states of one
-// segment, the two adjoint levels, the gradient accumulator and the trace
-// arrays. Reused while the step count, receivers and tiling stay the same.
+// Scratch of ws_adjoint_gradient: checkpoint pairs, the stencil sums of one
+// segment, four levels of rho and of recomputed states, the gradient accumulator
+// and the trace arrays. Reused while the step count, receivers and tiling stay
+// the same.
 struct AdjointCache {
     int N = -1, nrec = -1, kern = -1, tx = 0, ty = 0;
     // the checkpoints hold the forward run of this model version (ws_forward)
@@ -132,11 +133,13 @@ struct AdjointCache {
     std::vector<void *> mem;        // everything below, for cudaFree
     std::vector<MappedField> ck;    // checkpoint j: (u^{jC}, u^{jC-1}), u^m in ck[2 (j-1) + (m & 1)]
     std::vector<float *> lap;       // L u^n of the segment's steps
-    MappedField ring[2];            // recomputed u^n / u^{n-1}
-    // rho^k in rho[k % nrho]: the steps imaged together stay alive (2 where the
-    // memory does not hold more)
-    MappedField rho[ws::kMaxImagingSteps];
-    int nrho = 2;
+    // rho^k in level[k % 4], so that four steps can be imaged together. Between
+    // two segments only two levels are alive (rho^{n1+1}, rho^{n1+2}; n1 = the
+    // next segment's end): the other two hold its recomputed u^n and u^{n-1}.
+    MappedField level[ws::kMaxImagingSteps];
+    MappedField &rho(int k) { return level[k % ws::kMaxImagingSteps]; }
+    static_assert(ws::kMaxImagingSteps == 4, "the two idle levels below");
+    MappedField &ring(int n1, int m) { return level[(n1 + 3 + (m & 1)) % ws::kMaxImagingSteps]; }
     float2 *acc = nullptr;          // compensated FP32 gradient sums, padded layout
     double *partials = nullptr;     // residual partial sums, then the misfit
     double *norm = nullptr;         // gradient-norm partial sums, then the norm
