@@ -98,3 +98,34 @@ def test_forward_run_for_every_segment_length(nt, shape):
         g, _ = wsb.ws_adjoint_gradient(b, r, wsb.WS_ADJ_RESIDUAL)
         # receivers that share a cell may be added in another order
         assert np.abs(g - own).max() <= 1e-6 * np.abs(own).max()
+
+
+@pytest.mark.parametrize("tile", [(64, 16), (32, 16), (64, 8), (32, 8)])
+@pytest.mark.parametrize("shared", [0, 40])
+def test_injection_of_dense_receivers(tile, shared):
+    """The adjoint step's injection with a receiver on every cell of two planes,
+    in no order (8 a thread, 256 a warp): the direct kernel's bits. With 40 more
+    on one cell, added in another order, to the rounding of such a sum of
+    residuals of one sign (40 half ulps, four times that for the gradient)."""
+    shape = nz, ny, nx = 9, 20, 70
+    vel = synthetic.smooth_random_velocity(shape, 5, 1500.0, 4500.0, spacing=4)
+    rng = np.random.default_rng(shared)
+    rec = np.array([[i, j, k] for k in (2, 5) for j in range(ny) for i in range(nx)], np.int32)
+    rec = np.concatenate([rec[rng.permutation(len(rec))], np.repeat([[66, 17, 5]], shared, 0)])
+    rec = rec.astype(np.int32)
+    nt = 5
+    r = rng.uniform(0.5, 1.0, (len(rec), nt)).astype(np.float32)
+    grads = []
+    for kernel, size in ((wsb.WS_KERNEL_DIRECT, (0, 0)), (wsb.WS_KERNEL_STREAM, tile)):
+        h = wsb.ws_create(nx, ny, nz, 10.0, synthetic.cfl_dt(4500.0, 10.0))
+        wsb.ws_set_kernel(h, kernel, *size, 0)
+        wsb.ws_set_velocity(h, vel)
+        wsb.ws_set_sponge(h, 3, 0.1)
+        wsb.ws_add_source(h, 30, 5, 3, 30.0, 0.0, 1.0)
+        wsb.ws_set_receivers(h, rec, nt)
+        grads.append(wsb.ws_adjoint_gradient(h, r, wsb.WS_ADJ_RESIDUAL)[0])
+    assert np.abs(grads[0]).max() > 0
+    if shared:
+        assert np.abs(grads[0] - grads[1]).max() <= 4 * 40 * 2.0 ** -24 * np.abs(grads[0]).max()
+    else:
+        assert np.array_equal(*grads)
