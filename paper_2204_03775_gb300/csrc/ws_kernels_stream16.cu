@@ -16,32 +16,35 @@
 //
 // A 16-bit stencil is bound by instruction issue long before HBM, so the
 // kernel is built to execute few instructions per cell:
-//  - one CTA per work item (a 64 x 16 tile over a block of planes), 4 warps,
-//    every thread computes 4 x-cells of two rows; no producer warp. Thread 0
+//  - one CTA per work item (a 64 x TY tile over a block of planes; TY = 24:
+//    6 warps, 16: 4 warps), every thread computes 4 x-cells of two rows; no
+//    producer warp. Thread 0
 //    (ring A: U with its halo) and thread 32 (ring B: the D and W tiles)
 //    issue the TMA copies (cp.async.bulk.tensor) of later planes right after
 //    each plane's barrier, which is the point where every thread is done with
 //    the slots being refilled: no "empty" barriers, no polling producer. Each
 //    slot has a "full" mbarrier (transaction bytes).
-//  - ring A has 9 slots and the z loop runs 9 planes per trip, so ring slots,
-//    mbarrier phases and the 9-plane register queue indices are compile-time
-//    constants (no queue rotation); ring B has 3 slots.
+//  - ring A has 9 slots, ring B 3, and the z loop runs 3 planes per trip: the
+//    indices of the 9-plane register queue and ring B's slots are compile-time
+//    constants, ring A's slots and phases are carried from trip to trip, and
+//    the queue is renamed by moves after each trip. (Nine planes per trip need
+//    no renaming, but the body then leaves the instruction caches: 441 against
+//    479 Gcell/s at 1024^3.)
 //  - every value is decoded once: a thread decodes its own cells of plane
 //    k+4 into its register queue and, at plane k, writes them as FP32 into a
 //    double-buffered staging tile; the cells around the tile that the star
-//    stencil reads (not the corners) are decoded into the same tile, 4 cells
-//    per thread above and below the tile and 4 per lane of the last warp
-//    beside it. One barrier per plane (which also ANDs the threads' "no wait
-//    failed" flags, so a bounded wait that gives up stops every warp at the
-//    same plane) separates the staging writes from the neighbour reads
-//    (128-bit loads).
+//    stencil reads (not the corners) are decoded into the same tile in units
+//    of 4 cells, one unit per thread. One barrier per plane (which also ANDs
+//    the threads' "no wait failed" flags, so a bounded wait that gives up
+//    stops every warp at the same plane) separates the staging writes from the
+//    neighbour reads (128-bit loads).
 //  - the stencil sum is c0 u + sum_m c_m s_m with weights whose sum is exact
 //    (zero_sum_weights16: no mass term), symmetric pairs first, two cells per
 //    packed FP32x2 instruction.
 //  - tiles whose cells all have taper 1 (the interior of the absorbing
 //    layer) take d~ = W L + d on planes whose z taper is 1, without the taper
 //    multiplies; the tapered form gives the same bits there.
-//  - 152 registers, 3 CTAs (12 warps) per SM.
+//  - 158 registers (TY = 24): 12 warps per SM, as 2 CTAs of 24 rows or 3 of 16.
 //
 // One power-of-two scale per step for U' and D' (|d| <= |u^{n+1}| + |u^n|,
 // so the same exponent bounds both): stored values are value * 2^e, with e
