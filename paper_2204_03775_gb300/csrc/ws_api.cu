@@ -235,6 +235,13 @@ int pick_kernel(ws_t ws, ws::StreamTiling *tiling) {
     return WS_KERNEL_STREAM;
 }
 
+// The receiver table is of no tile any more (the buffer stays).
+static void forget_rec_tiles(ws_t ws) {
+    ws->rec_ptr = nullptr;
+    ws->rec_entries = nullptr;
+    ws->rec_tiling_tx = ws->rec_tiling_ty = 0;
+}
+
 void free_receivers(ws_t ws) {
     cudaFree(ws->traces);
     cudaFree(ws->rec_table);
@@ -242,9 +249,7 @@ void free_receivers(ws_t ws) {
     ws->traces_cap = 0;
     ws->rec_table = nullptr;
     ws->rec_table_cap = 0;
-    ws->rec_ptr = nullptr;
-    ws->rec_entries = nullptr;
-    ws->rec_tiling_tx = ws->rec_tiling_ty = 0;
+    forget_rec_tiles(ws);
 }
 
 // A device buffer of at least n bytes: *p as it is if it holds them, else a new
@@ -260,8 +265,8 @@ static int keep_or_grow(ws_t ws, void **p, size_t *cap, size_t n, const char *wh
     return WS_OK;
 }
 
-// Uploads from pageable memory that dies after the call: the copy has left it
-// when the call returns, except into a graph. A stream under capture fails here.
+// An upload whose host memory the handle reuses must not be captured into a graph,
+// which would read it again at each launch. A stream under capture fails here.
 static int refuse_capture(ws_t ws, const char *what) {
     cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
     WS_CUDA(cudaStreamIsCapturing(ws->stream, &st), what);
@@ -273,7 +278,10 @@ static int refuse_capture(ws_t ws, const char *what) {
 // entries sorted by k; thread owner = (row pair) * tx/4 + x quad, lane = 4 *
 // (row of the pair) + x cell. Direct kernel (direct): per tile, owner = row,
 // lane = x cell. The upload is issued on `stream`, which the steps that read the
-// table follow.
+// table follow. It is from pageable memory, which the GPU may read in place and
+// behind the work queued before (the driver need not stage it, least of all on a
+// coherent CPU): the host table stays with the handle, and is written again only
+// once the last upload is through, which needs no wait for the queued steps.
 int build_rec_tiles(ws_t ws, const ws::StreamTiling &t, bool direct, cudaStream_t stream) {
     if (ws->nrec == 0) return WS_OK;
     if (ws->rec_tiling_tx == t.tx && ws->rec_tiling_ty == t.ty && ws->rec_direct == direct)
@@ -307,16 +315,25 @@ int build_rec_tiles(ws_t ws, const ws::StreamTiling &t, bool direct, cudaStream_
     // one buffer and one upload: the ranges, then the entries
     const size_t head = (sizeof(int) * (ntiles + 1) + 15) / 16 * 16;
     const size_t bytes = head + sizeof(ws::RecEntry) * ws->nrec;
-    std::vector<char> table(bytes);
-    std::memcpy(table.data(), ptr.data(), sizeof(int) * (ntiles + 1));
-    std::memcpy(table.data() + head, ent.data(), sizeof(ws::RecEntry) * ws->nrec);
     int rc = refuse_capture(ws, "upload receiver table");
-    if (rc == WS_OK)
-        rc = keep_or_grow(ws, &ws->rec_table, &ws->rec_table_cap, bytes, "cudaMalloc receiver table");
     if (rc != WS_OK) return rc;
-    ws->rec_tiling_tx = 0;   // until the upload is issued
-    WS_CUDA(cudaMemcpyAsync(ws->rec_table, table.data(), bytes, cudaMemcpyHostToDevice, stream),
+    forget_rec_tiles(ws);   // until the upload is issued
+    rc = keep_or_grow(ws, &ws->rec_table, &ws->rec_table_cap, bytes, "cudaMalloc receiver table");
+    if (rc != WS_OK) return rc;
+    if (!ws->rec_uploaded)
+        WS_CUDA(cudaEventCreateWithFlags(&ws->rec_uploaded, cudaEventDisableTiming),
+                "upload receiver table");
+    WS_CUDA(cudaEventSynchronize(ws->rec_uploaded), "upload receiver table");
+    ws->rec_host.resize(bytes);
+    std::memcpy(ws->rec_host.data(), ptr.data(), sizeof(int) * (ntiles + 1));
+    std::memcpy(ws->rec_host.data() + head, ent.data(), sizeof(ws::RecEntry) * ws->nrec);
+    WS_CUDA(cudaMemcpyAsync(ws->rec_table, ws->rec_host.data(), bytes, cudaMemcpyHostToDevice, stream),
             "upload receiver table");
+    const cudaError_t e2 = cudaEventRecord(ws->rec_uploaded, stream);
+    if (e2 != cudaSuccess) {
+        cudaStreamSynchronize(stream);   // no event guards the host table
+        return cuda_fail(e2, "upload receiver table");
+    }
     ws->rec_ptr = static_cast<int *>(ws->rec_table);
     ws->rec_entries = reinterpret_cast<ws::RecEntry *>(static_cast<char *>(ws->rec_table) + head);
     ws->rec_tiling_tx = t.tx;
@@ -650,6 +667,10 @@ void destroy(ws_t ws) {
     cudaFree(ws->scale);
     cudaFree(ws->stage);
     free_receivers(ws);
+    if (ws->rec_uploaded) {
+        cudaEventSynchronize(ws->rec_uploaded);   // the upload reads rec_host
+        cudaEventDestroy(ws->rec_uploaded);
+    }
     delete ws->adj;
     delete ws;
 }
@@ -908,7 +929,7 @@ int ws_set_receivers(ws_t ws, int nrec, const int *ijk, int nt_max) {
     ws->model_version++;
     ws->nrec = 0;
     ws->nt_max = 0;
-    ws->rec_tiling_tx = ws->rec_tiling_ty = 0;   // the table is another one
+    forget_rec_tiles(ws);   // the table is another one
     ws->rec_ijk.assign(ijk, ijk + 3 * size_t(nrec));
     ws->trace_start = ws->step;
     if (nrec == 0) {

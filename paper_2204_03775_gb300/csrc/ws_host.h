@@ -77,6 +77,8 @@ struct ws_handle {
     size_t rec_table_cap = 0;
     int *rec_ptr = nullptr;              // per-tile ranges of rec_entries
     ws::RecEntry *rec_entries = nullptr;
+    std::vector<char> rec_host;          // the table's upload reads it until rec_uploaded
+    cudaEvent_t rec_uploaded = nullptr;
     float *stage = nullptr;              // planes of an unpadded field, for host arrays
     int rec_tiling_tx = 0, rec_tiling_ty = 0;
     bool rec_direct = false;             // the table is the direct kernel's

@@ -1,0 +1,49 @@
+"""Receiver tables that are rebuilt while the stream is busy (GPU)."""
+
+import numpy as np
+import pytest
+
+import paper_2204_03775_gb300 as wsb
+from paper_2204_03775_gb300 import synthetic
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("kernel", [wsb.WS_KERNEL_STREAM, wsb.WS_KERNEL_DIRECT])
+def test_table_rebuilt_behind_a_busy_stream(kernel):
+    """A table of 1 MB, set again while some hundred steps are queued: its upload
+    may run long after the call that issued it, so the host memory it comes from
+    has to live on, whatever the host allocates and writes meanwhile. The traces
+    are those of a handle that waits after every call."""
+    nz, ny, nx = 96, 256, 256
+    nt = 150
+    vel = synthetic.smooth_random_velocity((nz, ny, nx), 3, 1500.0, 4500.0, spacing=8)
+    cells = [np.array([[i, j, k] for j in range(ny) for i in range(nx)], np.int32) for k in (9, 30, 40)]
+    rng = np.random.default_rng(5)
+    sets = [c[rng.permutation(len(c))] for c in cells]
+
+    def run(wait):
+        h = wsb.ws_create(nx, ny, nz, 10.0, synthetic.cfl_dt(4500.0, 10.0))
+        wsb.ws_set_velocity(h, vel)
+        wsb.ws_set_kernel(h, kernel)
+        wsb.ws_add_source(h, nx // 2, ny // 2, 20, 30.0, 0.0, 1.0)
+        wsb.ws_set_receivers(h, sets[0], nt)      # the buffers are made here
+        wsb.ws_step(h, 1)
+        wsb.ws_synchronize(h)
+        for rec in sets[1:]:
+            wsb.ws_step(h, nt - 1)
+            if wait:
+                wsb.ws_synchronize(h)
+            wsb.ws_set_receivers(h, rec, nt)
+            wsb.ws_step(h, 1)
+            if wait:
+                wsb.ws_synchronize(h)
+            else:                                 # the host reuses its memory
+                junk = [np.full(rec.size, -1 - q, np.int32) for q in range(16)]
+                del junk
+        wsb.ws_step(h, 1)
+        return wsb.ws_read_traces(h)[:, :2], wsb.ws_read_field(h)[0]
+
+    for a, b in zip(run(False), run(True)):
+        assert np.abs(b).max() > 0
+        assert np.array_equal(a, b)
