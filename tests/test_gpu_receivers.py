@@ -47,3 +47,41 @@ def test_table_rebuilt_behind_a_busy_stream(kernel):
     for a, b in zip(run(False), run(True)):
         assert np.abs(b).max() > 0
         assert np.array_equal(a, b)
+
+
+def test_dense_receivers_on_a_narrow_grid():
+    """Grids narrower than a streaming tile take the direct kernel whatever their
+    size: a receiver on every cell of a vertical plane, some cells shared, is
+    sampled right, and costs a step a few times its own time at most (the scan
+    of a whole column's receivers for each plane took 19 times)."""
+    torch = pytest.importorskip("torch")
+    nz, ny, nx = 6000, 120, 20
+    nt = 72
+    vel = synthetic.smooth_random_velocity((nz, ny, nx), 3, 1500.0, 4500.0, spacing=8)
+    rec = np.array([[7, j, k] for k in range(nz) for j in range(ny)]
+                   + [[7, 60, 750]] * 700 + [[19, 119, nz - 1], [0, 0, 0]], np.int32)
+    rec = rec[np.random.default_rng(2).permutation(len(rec))]
+    h = wsb.ws_create(nx, ny, nz, 10.0, synthetic.cfl_dt(4500.0, 10.0))
+    wsb.ws_set_velocity(h, vel)
+    wsb.ws_add_source(h, 8, 60, 750, 30.0, 0.0, 1.0)
+    stream = torch.cuda.Stream()
+    wsb.ws_set_stream(h, stream)
+
+    def step_ms():
+        wsb.ws_step(h, 4)
+        a, b = (torch.cuda.Event(enable_timing=True) for _ in range(2))
+        a.record(stream)
+        wsb.ws_step(h, 16)
+        b.record(stream)
+        b.synchronize()
+        return a.elapsed_time(b) / 16
+
+    bare = min(step_ms() for _ in range(3))
+    wsb.ws_write_field(h, None, None, 0)
+    wsb.ws_set_receivers(h, rec, nt)
+    for t in range(4):
+        wsb.ws_step(h, 1)
+        u, _ = wsb.ws_read_field(h)
+        assert np.array_equal(wsb.ws_read_traces(h)[:, t], u[rec[:, 2], rec[:, 1], rec[:, 0]])
+    assert np.abs(u).max() > 0
+    assert step_ms() < 8 * bare
