@@ -68,12 +68,17 @@ std::vector<int> zblock_candidates(const ws::Geom &g, int tx, int ty, long long 
     return z;
 }
 
-// Tilings chosen by ws_autotune, keyed by (GPU name, storage, nx, ny, nz):
-// kept in memory and in a text file (one "gpu|storage|nx|ny|nz|tx|ty|zb"
-// line per entry) at $WS_TUNE_CACHE, else $XDG_CACHE_HOME/wavestep/tune.txt,
+// Tilings chosen by ws_autotune, keyed by (GPU name#version, storage, nx, ny,
+// nz): kept in memory and in a text file (one "gpu#version|storage|nx|ny|nz|tx|
+// ty|zb" line per entry) at $WS_TUNE_CACHE, else $XDG_CACHE_HOME/wavestep/tune.txt,
 // else $HOME/.cache/wavestep/tune.txt, so a later process on the same GPU
 // model reuses them. Lines that do not parse are ignored; a file that cannot
 // be written leaves the in-memory cache only.
+// The version is that of the kernel whose steps were timed: raise it with every
+// change of the FP32 streaming kernel or of the candidates that changes their
+// times. Lines of other versions stay in the file, unused. (Those of
+// the first kernel, one row a thread, have none.)
+constexpr const char *kTuneVersion = "#2";
 using TuneKey = std::tuple<std::string, int, int, int, int>;
 std::mutex g_tune_mutex;
 std::map<TuneKey, ws::StreamTiling> g_tune_cache;
@@ -131,7 +136,7 @@ void tune_cache_save() {
     if (!ok || std::rename(tmp.c_str(), path.c_str()) != 0) std::remove(tmp.c_str());
 }
 
-// The name of the current device ("" if it cannot be read), '|' replaced.
+// The cache's name of the current device ("" if it cannot be read), '|' replaced.
 std::string device_name() {
     int dev = 0;
     cudaDeviceProp prop;
@@ -140,7 +145,7 @@ std::string device_name() {
     std::string n(prop.name);
     for (char &c : n)
         if (c == '|' || c == '\n') c = '_';
-    return n;
+    return n + kTuneVersion;
 }
 
 }  // namespace
