@@ -15,6 +15,7 @@ int fail(int code, const char *fmt, ...) {
 }
 
 int cuda_fail(cudaError_t e, const char *what) {
+    cudaGetLastError();   // reported here: later calls, the caller's too, don't find it
     if (e == cudaErrorMemoryAllocation)
         return fail(WS_ERR_OOM, "%s: %s", what, cudaGetErrorString(e));
     return fail(WS_ERR_CUDA, "%s: %s", what, cudaGetErrorString(e));
@@ -789,8 +790,8 @@ int ws_create(ws_t *out, int nx, int ny, int nz, double h, double dt) {
     }
     int rc = upload_profiles(ws);
     if (rc == WS_OK) rc = encode_maps(ws);
-    if (rc == WS_OK && cudaStreamSynchronize(ws->stream) != cudaSuccess)
-        rc = cuda_fail(cudaGetLastError(), "ws_create");
+    if (rc == WS_OK && (e = cudaStreamSynchronize(ws->stream)) != cudaSuccess)
+        rc = cuda_fail(e, "ws_create");
     if (rc != WS_OK) {
         destroy(ws);
         return rc;
@@ -1234,9 +1235,10 @@ long long ws_launch_count(ws_t ws) { return ws ? ws->launches : -1; }
 int ws_test_fill_padding(ws_t ws) {
     if (!ws) return fail(WS_ERR_BADARG, "ws_test_fill_padding: NULL handle");
     int rc = for_each_field(ws, [&](auto *f, auto canary) {
-        fill_pad_kernel<<<kPadGrid, kPadBlock, 0, ws->stream>>>(f, ws->g, canary);
+        using T = std::remove_pointer_t<decltype(f)>;
+        cudaError_t e = ws::launch(fill_pad_kernel<T>, kPadGrid, kPadBlock, 0, ws->stream, f, ws->g,
+                                   canary);
         ws->launches++;
-        cudaError_t e = cudaGetLastError();
         return e == cudaSuccess ? WS_OK : cuda_fail(e, "ws_test_fill_padding");
     });
     if (rc != WS_OK) return rc;
@@ -1252,9 +1254,10 @@ int ws_test_check_padding(ws_t ws, long long *bad) {
     int rc = e == cudaSuccess ? WS_OK : cuda_fail(e, "ws_test_check_padding");
     if (rc == WS_OK)
         rc = for_each_field(ws, [&](auto *f, auto canary) {
-            check_pad_kernel<<<kPadGrid, kPadBlock, 0, ws->stream>>>(f, ws->g, canary, d);
+            using T = std::remove_pointer_t<decltype(f)>;
+            cudaError_t e2 = ws::launch(check_pad_kernel<T>, kPadGrid, kPadBlock, 0, ws->stream, f,
+                                        ws->g, canary, d);
             ws->launches++;
-            cudaError_t e2 = cudaGetLastError();
             return e2 == cudaSuccess ? WS_OK : cuda_fail(e2, "ws_test_check_padding");
         });
     unsigned long long h = 0;

@@ -5,6 +5,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 #include <string>
+#include <utility>
 
 #include "wavestep.h"
 
@@ -12,6 +13,20 @@ namespace ws {
 
 constexpr int kHalo = 4;                 // four neighbours per side (Section II)
 constexpr int kMaxSources = WS_MAX_SOURCES;
+
+// Launches a kernel and returns this launch's own status. (After <<<>>> that is
+// cudaGetLastError, which may be the error of an earlier call, of the library or
+// of its caller, such as an allocation that failed and was dealt with.)
+template <class... Params, class... Args>
+static cudaError_t launch(void (*kern)(Params...), dim3 grid, dim3 block, size_t smem, cudaStream_t s,
+                          Args &&...args) {
+    cudaLaunchConfig_t c{};
+    c.gridDim = grid;
+    c.blockDim = block;
+    c.dynamicSmemBytes = smem;
+    c.stream = s;
+    return cudaLaunchKernelEx(&c, kern, std::forward<Args>(args)...);
+}
 
 // Bits of the device status word.
 constexpr unsigned kStatusTimeout = 1u;

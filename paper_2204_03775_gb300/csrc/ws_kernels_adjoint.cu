@@ -189,31 +189,24 @@ int residual_partial_count() { return 1024; }
 cudaError_t launch_sum_fields(const FieldList &src, int n, long long count, float *out,
                               cudaStream_t s) {
     if (n < 1 || n > kMaxFieldList) return cudaErrorInvalidValue;
-    sum_fields_kernel<<<1216, 256, 0, s>>>(src, n, count, out);
-    return cudaGetLastError();
+    return launch(sum_fields_kernel, 1216, 256, 0, s, src, n, count, out);
 }
 
 cudaError_t launch_norm2(const float *x, long long n, double *partials, double *out,
                          cudaStream_t s) {
     const int blocks = residual_partial_count();
-    norm2_partials_kernel<<<blocks, kRedThreads, 0, s>>>(x, n, partials);
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    sum_kernel<<<1, kRedThreads, 0, s>>>(partials, blocks, out);
-    e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    sqrt_kernel<<<1, 1, 0, s>>>(out);
-    return cudaGetLastError();
+    cudaError_t e = launch(norm2_partials_kernel, blocks, kRedThreads, 0, s, x, n, partials);
+    if (e == cudaSuccess) e = launch(sum_kernel, 1, kRedThreads, 0, s, partials, blocks, out);
+    if (e == cudaSuccess) e = launch(sqrt_kernel, 1, 1, 0, s, out);
+    return e;
 }
 
 cudaError_t launch_residual(const float *traces, const float *d_obs, long long n, float *r,
                             double *partials, double *misfit, cudaStream_t s) {
     const int blocks = residual_partial_count();
-    residual_kernel<<<blocks, kRedThreads, 0, s>>>(traces, d_obs, n, r, partials);
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    sum_kernel<<<1, kRedThreads, 0, s>>>(partials, blocks, misfit);
-    return cudaGetLastError();
+    cudaError_t e = launch(residual_kernel, blocks, kRedThreads, 0, s, traces, d_obs, n, r, partials);
+    if (e == cudaSuccess) e = launch(sum_kernel, 1, kRedThreads, 0, s, partials, blocks, misfit);
+    return e;
 }
 
 cudaError_t launch_imaging(const ImagingSteps &st, int steps, const Geom &g, const Sources &src,
@@ -222,20 +215,18 @@ cudaError_t launch_imaging(const ImagingSteps &st, int steps, const Geom &g, con
     dim3 block(32, 8, 1);
     dim3 grid((g.nx + 127) / 128, (g.ny + 7) / 8, g.nz);
     switch (steps) {
-        case 1: imaging_kernel<1><<<grid, block, 0, s>>>(st, g, src, gx, gy, gz, acc); break;
-        case 2: imaging_kernel<2><<<grid, block, 0, s>>>(st, g, src, gx, gy, gz, acc); break;
-        case 3: imaging_kernel<3><<<grid, block, 0, s>>>(st, g, src, gx, gy, gz, acc); break;
-        case 4: imaging_kernel<4><<<grid, block, 0, s>>>(st, g, src, gx, gy, gz, acc); break;
+        case 1: return launch(imaging_kernel<1>, grid, block, 0, s, st, g, src, gx, gy, gz, acc);
+        case 2: return launch(imaging_kernel<2>, grid, block, 0, s, st, g, src, gx, gy, gz, acc);
+        case 3: return launch(imaging_kernel<3>, grid, block, 0, s, st, g, src, gx, gy, gz, acc);
+        case 4: return launch(imaging_kernel<4>, grid, block, 0, s, st, g, src, gx, gy, gz, acc);
         default: return cudaErrorInvalidValue;
     }
-    return cudaGetLastError();
 }
 
 cudaError_t launch_finalize_gradient(const float2 *acc, const float *w, const Geom &g,
                                      double h_over_dt2, float *grad, cudaStream_t s) {
     dim3 grid((g.nx + 127) / 128, g.ny, g.nz);
-    finalize_kernel<<<grid, 128, 0, s>>>(acc, w, g, h_over_dt2, grad);
-    return cudaGetLastError();
+    return launch(finalize_kernel, grid, 128, 0, s, acc, w, g, h_over_dt2, grad);
 }
 
 }  // namespace ws

@@ -215,18 +215,12 @@ cudaError_t launch_copy(const Fields &f, const Geom &g, cudaStream_t s) {
     dim3 block;
     const unsigned grid = row_grid(g, &block);
     const long long cells = (long long)rows * g.nx;
-#define WS_COPY(AL, NF)                                                                        \
-    copy_rows_kernel<AL, kIn, NF><<<grid, block, 0, s>>>(f, g.nx, g.ny, rows, g.pnx, g.plane, \
-                                                         cells)
-    if (aligned) {
-        if (f.src[1]) WS_COPY(true, 2);
-        else WS_COPY(true, 1);
-    } else {
-        if (f.src[1]) WS_COPY(false, 2);
-        else WS_COPY(false, 1);
-    }
+#define WS_COPY(AL, NF)                                                                   \
+    launch(copy_rows_kernel<AL, kIn, NF>, grid, block, 0, s, f, g.nx, g.ny, rows, g.pnx, \
+           g.plane, cells)
+    if (aligned) return f.src[1] ? WS_COPY(true, 2) : WS_COPY(true, 1);
+    return f.src[1] ? WS_COPY(false, 2) : WS_COPY(false, 1);
 #undef WS_COPY
-    return cudaGetLastError();
 }
 
 }  // namespace
@@ -234,9 +228,8 @@ cudaError_t launch_copy(const Fields &f, const Geom &g, cudaStream_t s) {
 cudaError_t launch_zero(float *a, float *b, size_t bytes, cudaStream_t s) {
     const long long n4 = (long long)(bytes / sizeof(float4));   // fields are whole 128-byte rows
     const long long want = (n4 + kRowThreads - 1) / kRowThreads;
-    zero_kernel<<<(unsigned)(want < kCopyBlocks ? want : kCopyBlocks), kRowThreads, 0, s>>>(
-        reinterpret_cast<float4 *>(a), reinterpret_cast<float4 *>(b), n4);
-    return cudaGetLastError();
+    return launch(zero_kernel, (unsigned)(want < kCopyBlocks ? want : kCopyBlocks), kRowThreads, 0, s,
+                  reinterpret_cast<float4 *>(a), reinterpret_cast<float4 *>(b), n4);
 }
 
 cudaError_t launch_copy_in(const float *a, const float *b, float *A, float *B, const Geom &g,
@@ -349,10 +342,8 @@ cudaError_t launch_model(const float *v, float *w, const Geom &g, double c, unsi
     }
     dim3 block;
     const unsigned grid = row_grid(g, &block);
-    model_kernel<Conv><<<grid, block, 0, s>>>(v, w + pidx(g, 0, 0, 0), g.nx, g.ny,
-                                              (unsigned)g.ny * (unsigned)g.nz, g.pnx, g.plane,
-                                              model_scale(c), extrema);
-    return cudaGetLastError();
+    return launch(model_kernel<Conv>, grid, block, 0, s, v, w + pidx(g, 0, 0, 0), g.nx, g.ny,
+                  (unsigned)g.ny * (unsigned)g.nz, g.pnx, g.plane, model_scale(c), extrema);
 }
 
 }  // namespace

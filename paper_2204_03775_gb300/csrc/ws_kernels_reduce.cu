@@ -275,11 +275,10 @@ cudaError_t launch_energy(const F &f, int nx, int ny, int nz, double h, const Co
                           double *partials, double *out, cudaStream_t s) {
     const int rows = energy_rows_per_block();
     dim3 grid((ny + rows - 1) / rows, nz, 1);
-    energy_partials_kernel<F><<<grid, kThreads, 0, s>>>(f, nx, ny, nz, rows, h * h, c, partials);
-    cudaError_t e = cudaGetLastError();
+    cudaError_t e = launch(energy_partials_kernel<F>, grid, kThreads, 0, s, f, nx, ny, nz, rows, h * h,
+                           c, partials);
     if (e != cudaSuccess) return e;
-    sum_partials_kernel<<<1, kThreads, 0, s>>>(partials, (int)(grid.x * grid.y), out);
-    return cudaGetLastError();
+    return launch(sum_partials_kernel, 1, kThreads, 0, s, partials, (int)(grid.x * grid.y), out);
 }
 
 }  // namespace

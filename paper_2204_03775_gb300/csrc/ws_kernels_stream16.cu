@@ -1116,24 +1116,15 @@ cudaError_t launch_encode16(int storage, const Fp32Fields &f, uint16_t *U, uint1
     const long long o = pidx(g, 0, 0, 0);
     dim3 block;
     const unsigned grid = row_grid(g, &block);
-    if (f.vec)
-        amax2_kernel<true><<<grid, block, 0, s>>>(f, g.nx, g.ny, rows, &sc->amax[slot]);
-    else
-        amax2_kernel<false><<<grid, block, 0, s>>>(f, g.nx, g.ny, rows, &sc->amax[slot]);
-    e = cudaGetLastError();
+    e = launch(f.vec ? amax2_kernel<true> : amax2_kernel<false>, grid, block, 0, s, f, g.nx, g.ny, rows,
+               &sc->amax[slot]);
     if (e != cudaSuccess) return e;
-#define WS_ENCODE(FMT, V)                                                                       \
-    encode_kernel<FMT, V><<<grid, block, 0, s>>>(f, U + o, D + o, g.nx, g.ny, rows, g.pnx, \
-                                                 g.plane, sc, slot)
-    if (storage == WS_STORAGE_BF16) {
-        if (f.vec) WS_ENCODE(Bf16Fmt, true);
-        else WS_ENCODE(Bf16Fmt, false);
-    } else {
-        if (f.vec) WS_ENCODE(Fp16Fmt, true);
-        else WS_ENCODE(Fp16Fmt, false);
-    }
+#define WS_ENCODE(FMT, V)                                                                         \
+    launch(encode_kernel<FMT, V>, grid, block, 0, s, f, U + o, D + o, g.nx, g.ny, rows, g.pnx, \
+           g.plane, sc, slot)
+    if (storage == WS_STORAGE_BF16) return f.vec ? WS_ENCODE(Bf16Fmt, true) : WS_ENCODE(Bf16Fmt, false);
+    return f.vec ? WS_ENCODE(Fp16Fmt, true) : WS_ENCODE(Fp16Fmt, false);
 #undef WS_ENCODE
-    return cudaGetLastError();
 }
 
 cudaError_t launch_decode16(int storage, const uint16_t *U, const uint16_t *D, const Fp32Out &f,
@@ -1142,27 +1133,20 @@ cudaError_t launch_decode16(int storage, const uint16_t *U, const uint16_t *D, c
     const long long o = pidx(g, 0, 0, 0);
     dim3 block;
     const unsigned grid = row_grid(g, &block);
-#define WS_DECODE(FMT, V)                                                                       \
-    decode_kernel<FMT, V><<<grid, block, 0, s>>>(U + o, D + o, f, g.nx, g.ny, rows, g.pnx, \
-                                                 g.plane, sc, slot)
-    if (storage == WS_STORAGE_BF16) {
-        if (f.vec) WS_DECODE(Bf16Fmt, true);
-        else WS_DECODE(Bf16Fmt, false);
-    } else {
-        if (f.vec) WS_DECODE(Fp16Fmt, true);
-        else WS_DECODE(Fp16Fmt, false);
-    }
+#define WS_DECODE(FMT, V)                                                                         \
+    launch(decode_kernel<FMT, V>, grid, block, 0, s, U + o, D + o, f, g.nx, g.ny, rows, g.pnx, \
+           g.plane, sc, slot)
+    if (storage == WS_STORAGE_BF16) return f.vec ? WS_DECODE(Bf16Fmt, true) : WS_DECODE(Bf16Fmt, false);
+    return f.vec ? WS_DECODE(Fp16Fmt, true) : WS_DECODE(Fp16Fmt, false);
 #undef WS_DECODE
-    return cudaGetLastError();
 }
 
 cudaError_t launch_model16(const float *w, uint16_t *w16, const Geom &g, cudaStream_t s) {
     const long long o = pidx(g, 0, 0, 0);
     dim3 block;
     const unsigned grid = row_grid(g, &block);
-    model16_kernel<<<grid, block, 0, s>>>(w + o, w16 + o, g.nx, g.ny,
-                                          (unsigned)g.ny * (unsigned)g.nz, g.pnx, g.plane);
-    return cudaGetLastError();
+    return launch(model16_kernel, grid, block, 0, s, w + o, w16 + o, g.nx, g.ny,
+                  (unsigned)g.ny * (unsigned)g.nz, g.pnx, g.plane);
 }
 
 }  // namespace ws
