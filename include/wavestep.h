@@ -296,7 +296,7 @@ int ws_set_storage(ws_t ws, int storage);
  * height of 24 or 16 rows, whose waves of resident CTAs are estimated to finish
  * first).
  * WS_KERNEL_STREAM needs nx >= tile_x and ny >= tile_y (64 x 8 while no tile is
- * chosen); else BADARG. */
+ * chosen, 32 x 8 once WS_KERNEL_AUTO has stepped the handle); else BADARG. */
 int ws_set_kernel(ws_t ws, int kernel, int tile_x, int tile_y, int zblock);
 
 /* Pick the streaming kernel's tile and z-block for this handle's grid by

@@ -212,7 +212,8 @@ int pick_kernel(ws_t ws, ws::StreamTiling *tiling) {
     ws::StreamTiling t = ws->tiling;
     if (!ws->tile_chosen) {
         const bool automatic = ws->kernel == WS_KERNEL_AUTO;
-        if (!default_tile(g, &t)) return WS_KERNEL_DIRECT;   // AUTO only: STREAM needs 64 x 8
+        if (!default_tile(g, &t)) return WS_KERNEL_DIRECT;   // AUTO only: STREAM needs more
+        if (automatic && !stream_fits(ws, ws->need)) ws->need = t;   // ws_set_kernel: STREAM
         if (automatic && t.zb <= 0 && (long long)g.nx * g.ny * g.nz <= kDirectCells)
             return WS_KERNEL_DIRECT;
     } else if (ws->kernel == WS_KERNEL_AUTO && !stream_fits(ws, t)) {
@@ -994,9 +995,9 @@ int ws_set_kernel(ws_t ws, int kernel, int tile_x, int tile_y, int zblock) {
     if (kernel != WS_KERNEL_AUTO && kernel != WS_KERNEL_DIRECT && kernel != WS_KERNEL_STREAM)
         return fail(WS_ERR_BADARG, "ws_set_kernel: unknown kernel %d", kernel);
     if (zblock < 0) return fail(WS_ERR_BADARG, "ws_set_kernel: zblock must be >= 0");
-    // the streaming tile that must fit: the chosen one, else 64 x 8 (the
-    // smallest that a default may come down to)
-    ws::StreamTiling t = ws->tile_chosen ? ws->tiling : ws::StreamTiling{64, 8, 0};
+    // the streaming tile that must fit: the chosen one, else 64 x 8, or on a
+    // narrower grid that AUTO has stepped the tile it took
+    ws::StreamTiling t = ws->tile_chosen ? ws->tiling : ws->need;
     bool chosen = ws->tile_chosen;
     if (tile_x != 0 || tile_y != 0) {
         const bool fp32 = ws::stream_tiling_supported(tile_x, tile_y);

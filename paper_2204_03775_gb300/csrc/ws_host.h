@@ -86,6 +86,7 @@ struct ws_handle {
     int kernel = WS_KERNEL_AUTO;
     ws::StreamTiling tiling{64, 16, 0};  // tile of the tensor maps; zb 0: default
     bool tile_chosen = false;            // by ws_set_kernel, ws_autotune or a batch
+    ws::StreamTiling need{64, 8, 0};     // what STREAM must fit while none is chosen
     ws::StreamTiling auto_zb{0, 0, 0};   // default z block of the tile last used
     CUtensorMap tmap_halo[2];  // buf[b] with the (tx+8, ty+8, 1) box
     CUtensorMap tmap_tile[2];  // buf[b] with the (tx, ty, 1) box
