@@ -45,6 +45,7 @@ struct PaddedFields {
     // p at offset o from cell e of the array; in: whether that is in the grid
     __device__ float p_near(long long e, long long o, bool) const { return p[e + o]; }
     __device__ float w_at(long long e) const { return w[e]; }
+    __device__ bool surely_positive(long long e) const { return w[e] > 0.0f; }   // w_at, if true
 };
 
 // Unpadded [nz][ny][nx] caller arrays; (V dt / h)^2 is formed from the
@@ -60,6 +61,7 @@ struct DenseFields {
     __device__ long long plane() const { return (long long)nx * ny; }
     __device__ float p_near(long long e, long long o, bool in) const { return in ? p[e + o] : 0.0f; }
     __device__ float w_at(long long e) const { return to_model<FromVelocity>(v[e], scale); }
+    __device__ bool surely_positive(long long e) const { return fabsf(v[e] * scale.hi) >= 0x1p-60f; }
 };
 
 // hi + lo, lo below half an ulp of hi or so.
@@ -217,7 +219,16 @@ __global__ void __launch_bounds__(kThreads, 3)
     __syncthreads();
     big = s_big;
     double acc = 0.0;
-    if (big != 0u) {   // else every term is zero
+    if (big == 0u) {   // every term is zero, or 0 / 0 where the model is bad
+        bool good = true;
+        for (int j = j0 + warp; j < j1; j += kThreads / 32) {
+#pragma unroll 4
+            for (int i = lane; i < nx; i += 32) good &= f.surely_positive(f.at(i, j, k));
+        }
+        for (int j = j0 + warp; !good && j < j1; j += kThreads / 32)
+            for (int i = lane; i < nx; i += 32)
+                if (!(f.w_at(f.at(i, j, k)) > 0.0f)) acc = nan("");
+    } else {
         const int ex = (int)(big >> 23) - 127;
         // values near 1 need no scaling; else the block's largest is brought there
         const bool near1 = ex >= -30 && ex <= 40;
