@@ -296,7 +296,7 @@ cudaError_t launch_norm2(const float *x, long long n, double *partials, double *
 cudaError_t launch_finalize_gradient(const float2 *acc, const float *w, const Geom &g,
                                      double h_over_dt2, float *grad, cudaStream_t s);
 
-// Discrete energy (FP64): partial sums per (row block, plane) into
+// Discrete energy (FP64, as are its terms' precision): partial sums per (row block, plane) into
 // partials[energy_partial_count(ny, nz)], then their fixed-order sum into *out.
 int energy_rows_per_block();
 long long energy_partial_count(int ny, int nz);

@@ -11,20 +11,30 @@
 //
 // GB300 runs FP64 at a 64th of its FP32 rate, and evaluated in FP64 (some 90
 // operations and conversions a cell) the kernel was bound by that pipe: 3.7 ms
-// at 320 x 288 x 256. Instead each cell is summed as pairs of floats, hi + lo,
-// through error-free sums and products (Dekker, Knuth), about 280 FP32
-// operations a cell, and only the threads' totals are FP64 (0.37 ms, issue-bound):
-//  - 5040 h^2 L p = 8064 d1 - 1008 d2 + 128 d3 - 9 d4, d_m the six neighbours at
-//    distance m less 6 p: whole weights, so none is rounded, and sums of floats
-//    of like size leave lo words that are small multiples of one ulp.
-//  - Where the block's largest value is not within 2^-30 .. 2^40, values are
-//    scaled by a power of two that brings it to about 1, so no product underflows
-//    that matters.
-// The error of the sum against 80-bit arithmetic, both forms emulated on the
-// CPU, on smooth fields of 40^3 to 96^3 cells: at most 1.6e-16, FP64 3.0e-16
-// (whose weights are rounded); on white noise both 1 to 3e-16. Blocks out of the scaled range, and threads that meet a
-// value that is not finite or a model below 2^-60, take the FP64 form.
+// at 320 x 288 x 256. Instead the parts of a cell's term are formed exactly, or
+// to more than 53 bits, from floats and integers:
+//  - 5040 h^2 L p = 8064 s1 - 1008 s2 + 128 s3 - 9 s4 - 43050 p, s_m the sum of the
+//    six neighbours at distance m: whole weights, none is rounded. Each value is
+//    cut at two places below the largest of the 25 by adding a constant (error-free
+//    extraction, Rump, Ogita and Oishi): the sum's low bits are a whole number of
+//    22 bits, its remainder is exact. Whole numbers are added and weighted as
+//    integers, without error; the rest, below 2^-44 of the largest value, in floats.
+//    One conversion makes an FP64 number of the 64-bit sum.
+//  - (u - p)^2 / w as three floats, through error-free sums and products (Dekker,
+//    Knuth) and the remainders of two quotients.
+// A thread adds the first in FP64 and the second in three floats. So the sum is
+// as precise as one of FP64 terms, also on a single cell and where neighbouring
+// values differ by any factor. (As pairs of floats throughout, 48 bits, single
+// cells and fields with spikes were off by up to 1e-14 of their parts; FP64: 3e-16
+// to 1e-15.) About 400 instructions a cell, 3 of them FP64, bound by issue (62 % of
+// its slots): ws_energy of 320 x 288 x 256 in 0.43 ms, without allocation 0.49 (the
+// pairs: 0.36, 0.39; FP64 3.8).
+// Where the block's largest value is not within 2^-30 .. 2^40, values are scaled by
+// a power of two that brings it to about 1, so no product underflows that matters.
+// Blocks out of the scaled range, and threads that meet a value that is not finite
+// or a model outside 2^-60 .. 2^30, take the FP64 form.
 #include "ws_model.cuh"
+#include "ws_ptx.cuh"
 
 namespace ws {
 namespace {
@@ -64,7 +74,7 @@ struct DenseFields {
     __device__ bool surely_positive(long long e) const { return fabsf(v[e] * scale.hi) >= 0x1p-60f; }
 };
 
-// hi + lo, lo below half an ulp of hi or so.
+// hi + lo, exactly: the rounded result of a float operation and its error.
 struct Pair {
     float hi, lo;
 };
@@ -76,31 +86,11 @@ __device__ __forceinline__ Pair two_prod(float a, float b) {   // a b exactly
     const float p = __fmul_rn(a, b);
     return Pair{p, __fmaf_rn(a, b, -p)};
 }
-__device__ __forceinline__ Pair add(Pair a, Pair b) {
-    const Pair s = two_sum(a.hi, b.hi);
-    const float l = __fadd_rn(s.lo, __fadd_rn(a.lo, b.lo));
-    const float h = __fadd_rn(s.hi, l);
-    return Pair{h, __fadd_rn(__fsub_rn(s.hi, h), l)};
-}
-__device__ __forceinline__ Pair mul(Pair a, float b) {
-    const Pair p = two_prod(a.hi, b);
-    return Pair{p.hi, __fmaf_rn(a.lo, b, p.lo)};
-}
-
-// a + b, lo not folded into hi (it may grow to a few ulps of it).
-__device__ __forceinline__ Pair add_loose(Pair a, Pair b) {
-    const Pair s = two_sum(a.hi, b.hi);
-    return Pair{s.hi, __fadd_rn(s.lo, __fadd_rn(a.lo, b.lo))};
-}
-__device__ __forceinline__ Pair renormalize(Pair a) {
-    const float h = __fadd_rn(a.hi, a.lo);
-    return Pair{h, __fadd_rn(__fsub_rn(a.hi, h), a.lo)};
-}
 
 // The values that a cell's term needs.
 struct Cell {
     float u, p, w;
-    float n[4][6];   // p at distance 1 .. 4 on x+, x-, y+, y-, z+, z-
+    float2 n[4][3];   // p at distance 1 .. 4 on {x+, x-}, {y+, y-}, {z+, z-}
 };
 
 // kInside: the y and z neighbours lie in the grid.
@@ -113,45 +103,102 @@ __device__ __forceinline__ Cell load_cell(const F &f, int i, int j, int k, int n
     c.w = f.w_at(e);
 #pragma unroll
     for (int m = 1; m <= 4; ++m) {
-        c.n[m - 1][0] = f.p_near(e, m, i + m < nx);
-        c.n[m - 1][1] = f.p_near(e, -m, i - m >= 0);
-        c.n[m - 1][2] = f.p_near(e, m * sy, kInside || j + m < ny);
-        c.n[m - 1][3] = f.p_near(e, -m * sy, kInside || j - m >= 0);
-        c.n[m - 1][4] = f.p_near(e, m * sz, kInside || k + m < nz);
-        c.n[m - 1][5] = f.p_near(e, -m * sz, kInside || k - m >= 0);
+        c.n[m - 1][0] = make_float2(f.p_near(e, m, i + m < nx), f.p_near(e, -m, i - m >= 0));
+        c.n[m - 1][1] = make_float2(f.p_near(e, m * sy, kInside || j + m < ny),
+                                    f.p_near(e, -m * sy, kInside || j - m >= 0));
+        c.n[m - 1][2] = make_float2(f.p_near(e, m * sz, kInside || k + m < nz),
+                                    f.p_near(e, -m * sz, kInside || k - m >= 0));
     }
     return c;
 }
 
-// Adds (u - p)^2 / w to *kin + *kin2 and 5040 u h^2 L p to *pot, of the values
-// times s (a power of two; kScaled false: s = 1).
+// x in FP64, by integer operations (a conversion takes the FP64 pipe). Values
+// below 2^-126 count as zero; x is finite.
+__device__ __forceinline__ double widen(float x) {
+    const unsigned b = __float_as_uint(x), m = b & 0x7fffffffu;
+    return __hiloint2double((int)(m < 0x800000u ? 0u : ((m >> 3) + 0x38000000u) | (b & 0x80000000u)),
+                            (int)(m < 0x800000u ? 0u : b << 29));
+}
+
+// 5040 h^2 L p of a cell's values times s (a power of two; kScaled false: 1), the
+// exact sum rounded to FP64: see the head of this file. *finite: false if one of
+// the values is not.
 template <bool kScaled>
-__device__ __forceinline__ void add_cell(const Cell &c, float s, Pair *kin, float *kin2, Pair *pot) {
-    auto scaled = [&](float x) { return kScaled ? x * s : x; };
-    const float u = scaled(c.u), p = scaled(c.p);
-    const Pair p6 = two_prod(6.0f, p);
-    Pair lap{0.0f, 0.0f};
+__device__ __forceinline__ double stencil_sum(const Cell &c, float s, bool *finite) {
+    auto value = [&](int m, int a) {   // m = 0: p itself
+        const float2 v = m ? c.n[m - 1][a] : make_float2(c.p, 0.0f);
+        return kScaled ? mul2(v, splat(s)) : v;
+    };
+    float big = fabsf(value(0, 0).x);
 #pragma unroll
-    for (int m = 4; m >= 1; --m) {
-        const float *n = c.n[m - 1];
-        Pair d = two_sum(scaled(n[0]), scaled(n[1]));
-        d = add_loose(d, two_sum(scaled(n[2]), scaled(n[3])));
-        d = add_loose(d, two_sum(scaled(n[4]), scaled(n[5])));
-        d = add_loose(d, Pair{-p6.hi, -p6.lo});
-        const Pair t = mul(d, m == 1 ? 8064.0f : m == 2 ? -1008.0f : m == 3 ? 128.0f : -9.0f);
-        lap = m == 4 ? t : add_loose(lap, t);
+    for (int m = 1; m <= 4; ++m)
+#pragma unroll
+        for (int a = 0; a < 3; ++a) big = fmaxf(big, fmaxf(fabsf(value(m, a).x), fabsf(value(m, a).y)));
+    // the largest value's exponent; not below 2^-60 (what is smaller is summed in
+    // the last part), and an infinite one makes both constants NaN
+    const int ex = max(127 - 60, min(253, (int)(__float_as_uint(big) >> 23)));
+    const unsigned c1 = ((unsigned)(ex + 2) << 23) | 0x400000u, c2 = ((unsigned)(ex - 20) << 23) | 0x400000u;
+    const float2 s1 = splat(__uint_as_float(c1)), s2 = splat(__uint_as_float(c2));
+    const float2 m1 = splat(-s1.x), m2 = splat(-s2.x), minus = splat(-1.0f);
+    constexpr int kWeight[5] = {-43050, 8064, -1008, 128, -9};
+    long long sum1 = 0, sum2 = 0;
+    float rest = 0.0f;
+#pragma unroll
+    for (int m = 0; m <= 4; ++m) {
+        unsigned bits1 = 0u, bits2 = 0u;
+        float2 r3 = splat(0.0f);
+#pragma unroll
+        for (int a = 0; a < (m ? 3 : 1); ++a) {
+            const float2 v = value(m, a);
+            const float2 t1 = add2(s1, v), r1 = fma2(add2(t1, m1), minus, v);     // v - (t1 - s1)
+            const float2 t2 = add2(s2, r1), r2 = fma2(add2(t2, m2), minus, r1);   // likewise
+            bits1 += __float_as_uint(t1.x) + __float_as_uint(t1.y);
+            bits2 += __float_as_uint(t2.x) + __float_as_uint(t2.y);
+            r3 = a ? add2(r3, r2) : r2;
+        }
+        const unsigned n = m ? 6u : 2u;   // (m = 0: p, and a zero)
+        sum1 += (long long)kWeight[m] * (int)(bits1 - n * c1);
+        sum2 += (long long)kWeight[m] * (int)(bits2 - n * c2);
+        rest = __fmaf_rn((float)kWeight[m], __fadd_rn(r3.x, r3.y), rest);
     }
-    *pot = add(*pot, mul(renormalize(lap), u));
-    // u - p = d exactly; (u - p)^2 = q + d.lo^2, the last below 2^-50 of q but
-    // never negative, so it is summed apart
-    const Pair d = two_sum(u, -p);
-    Pair q = two_prod(d.hi, d.hi);
-    q.lo = __fmaf_rn(2.0f * d.hi, d.lo, q.lo);
-    // q / w: the nearest quotient, its exact remainder, that one's quotient
-    const float a = __fdiv_rn(q.hi, c.w);
-    const float r = __fadd_rn(__fmaf_rn(-a, c.w, q.hi), q.lo);
-    *kin = add(*kin, Pair{a, __fdividef(r, c.w)});
-    *kin2 = __fadd_rn(*kin2, __fdividef(__fmul_rn(d.lo, d.lo), c.w));
+    const long long sum = (sum1 << 22) + sum2;   // below 2^62, in units of 2^(ex - 170)
+    const double d = __ll2double_rn(sum);
+    const int up = sum ? (ex - 170) * (1 << 20) : 0;   // times 2^(ex - 170), in its exponent
+    *finite = fabsf(rest) < 0x1p126f;
+    return __dadd_rn(__hiloint2double(__double2hiint(d) + up, __double2loint(d)), widen(rest));
+}
+
+// The sums of a thread's cells: kin[0] + kin[1] + kin[2] of (u - p)^2 / w (three
+// floats, more than 70 bits), pot of 5040 u h^2 L p.
+struct Sums {
+    float kin[3] = {0.0f, 0.0f, 0.0f};
+    double pot = 0.0;
+    __device__ double kinetic() const {
+        return __dadd_rn((double)kin[0], __dadd_rn((double)kin[1], (double)kin[2]));
+    }
+};
+
+// Adds a cell, of the values times s; false if a stencil value is not finite.
+template <bool kScaled>
+__device__ __forceinline__ bool add_cell(const Cell &c, float s, Sums *sum) {
+    const float u = kScaled ? c.u * s : c.u, p = kScaled ? c.p * s : c.p;
+    bool finite;
+    const double lap = stencil_sum<kScaled>(c, s, &finite);
+    sum->pot = __fma_rn(widen(u), lap, sum->pot);
+    // u - p = d exactly; (u - p)^2 = q.hi + e.hi + f
+    const Pair d = two_sum(u, -p), q = two_prod(d.hi, d.hi), x = two_prod(2.0f * d.hi, d.lo);
+    const Pair e = two_sum(q.lo, x.hi);
+    const float f = __fmaf_rn(d.lo, d.lo, __fadd_rn(x.lo, e.lo));
+    // the nearest quotient by w, its exact remainder, that one's quotient, and again
+    const float a0 = __fdiv_rn(q.hi, c.w);
+    const Pair r = two_sum(__fmaf_rn(-a0, c.w, q.hi), e.hi);
+    const float a1 = __fdividef(r.hi, c.w);
+    const float a2 = __fdividef(__fadd_rn(__fmaf_rn(-a1, c.w, r.hi), __fadd_rn(r.lo, f)), c.w);
+    const Pair k0 = two_sum(sum->kin[0], a0), k1 = two_sum(sum->kin[1], k0.lo), k2 = two_sum(k1.hi, a1);
+    sum->kin[0] = k0.hi;
+    sum->kin[1] = k2.hi;
+    sum->kin[2] = __fadd_rn(sum->kin[2], __fadd_rn(a2, __fadd_rn(k1.lo, k2.lo)));
+    return finite;
 }
 
 // The term of one cell in FP64: (u - p)^2 / (V dt)^2 - u (L p), every
@@ -166,8 +213,7 @@ __device__ __noinline__ double cell_fp64(const Cell &c, const Coeffs64 &w, doubl
 #pragma unroll
         for (int m = 1; m <= 4; ++m) {
             const double cm = m == 1 ? w.c1 : m == 2 ? w.c2 : m == 3 ? w.c3 : w.c4;
-            l[a] = __fma_rn(cm, __dadd_rn((double)c.n[m - 1][2 * a], (double)c.n[m - 1][2 * a + 1]),
-                            l[a]);
+            l[a] = __fma_rn(cm, __dadd_rn((double)c.n[m - 1][a].x, (double)c.n[m - 1][a].y), l[a]);
         }
     }
     const double lap = __ddiv_rn(__dadd_rn(__dadd_rn(l[0], l[1]), l[2]), h2);
@@ -178,16 +224,15 @@ __device__ __noinline__ double cell_fp64(const Cell &c, const Coeffs64 &w, doubl
 }
 
 // This thread's cells of rows [j0, j1) of plane k, a warp a row at a time;
-// false if one of them has a model out of range.
+// false if one of them has a model or a value out of range.
 template <bool kScaled, bool kInside, class F>
 __device__ __forceinline__ bool sum_rows(const F &f, int j0, int j1, int k, int nx, int ny, int nz,
-                                         float s, Pair *kin, float *kin2, Pair *pot) {
+                                         float s, Sums *sum) {
     bool good = true;
     for (int j = j0 + (threadIdx.x >> 5); j < j1; j += kThreads / 32)
         for (int i = threadIdx.x & 31; i < nx; i += 32) {
             const Cell q = load_cell<kInside>(f, i, j, k, nx, ny, nz);
-            good = good && q.w >= 0x1p-60f;
-            add_cell<kScaled>(q, s, kin, kin2, pot);
+            good = add_cell<kScaled>(q, s, sum) && good && q.w >= 0x1p-60f && q.w <= 0x1p30f;
         }
     return good;
 }
@@ -235,16 +280,15 @@ __global__ void __launch_bounds__(kThreads, 3)
         const int se = near1 ? 0 : max(-60, min(60, -ex));
         const float s = __int_as_float((se + 127) << 23);
         const bool inside = j0 >= 4 && j1 + 4 <= ny && k >= 4 && k + 4 < nz;
-        Pair kin{0.0f, 0.0f}, pot{0.0f, 0.0f};
-        float kin2 = 0.0f;
+        Sums sum;
         bool fast = near1 || abs(ex + se) <= 30;
         if (near1 && inside)
-            fast = sum_rows<false, true>(f, j0, j1, k, nx, ny, nz, s, &kin, &kin2, &pot);
+            fast = sum_rows<false, true>(f, j0, j1, k, nx, ny, nz, s, &sum);
         else if (fast)
-            fast = sum_rows<true, false>(f, j0, j1, k, nx, ny, nz, s, &kin, &kin2, &pot);
-        const double K = (double)kin.hi + ((double)kin.lo + (double)kin2), Q = (double)pot.hi + (double)pot.lo;
-        if (fast && isfinite(K) && isfinite(Q))
-            acc = (K - Q / 5040.0) * scalbn(1.0, -2 * se) / h2;
+            fast = sum_rows<true, false>(f, j0, j1, k, nx, ny, nz, s, &sum);
+        const double kin = sum.kinetic();
+        if (fast && isfinite(kin))
+            acc = (kin - sum.pot / 5040.0) * scalbn(1.0, -2 * se) / h2;
         else
             for (int j = j0 + warp; j < j1; j += kThreads / 32)
                 for (int i = lane; i < nx; i += 32)
