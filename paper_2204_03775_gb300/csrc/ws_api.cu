@@ -58,6 +58,29 @@ PFN_cuTensorMapEncodeTiled_v12000 get_encode_fn() {
     return fn;
 }
 
+cudaError_t HostTables::next(size_t n, char **p) {
+    if (at == 0 && passed[group]) {
+        const cudaError_t e = cudaEventSynchronize(passed[group]);
+        if (e != cudaSuccess) return e;
+    }
+    table[group][at].resize(n);
+    *p = table[group][at].data();
+    return cudaSuccess;
+}
+
+cudaError_t HostTables::upload(void *dst, cudaStream_t stream) {
+    const std::vector<char> &t = table[group][at];
+    cudaError_t e = cudaMemcpyAsync(dst, t.data(), t.size(), cudaMemcpyHostToDevice, stream);
+    if (e != cudaSuccess) return e;
+    if (++at < kGroup && t.size() <= kLarge) return cudaSuccess;
+    if (!passed[group]) e = cudaEventCreateWithFlags(&passed[group], cudaEventDisableTiming);
+    if (e == cudaSuccess) e = cudaEventRecord(passed[group], stream);
+    if (e != cudaSuccess) cudaStreamSynchronize(stream);   // no event guards the group
+    group = 1 - group;
+    at = 0;
+    return e;
+}
+
 size_t field_bytes(const ws::Geom &g) {
     return size_t(g.pnx) * size_t(g.pny) * size_t(g.pnz) * sizeof(float);
 }
@@ -282,8 +305,8 @@ static int refuse_capture(ws_t ws, const char *what) {
 // lane = x cell. The upload is issued on `stream`, which the steps that read the
 // table follow. It is from pageable memory, which the GPU may read in place and
 // behind the work queued before (the driver need not stage it, least of all on a
-// coherent CPU): the host table stays with the handle, and is written again only
-// once the last upload is through, which needs no wait for the queued steps.
+// coherent CPU): the host table stays with the handle until its upload is through,
+// which needs no wait for the queued steps.
 int build_rec_tiles(ws_t ws, const ws::StreamTiling &t, bool direct, cudaStream_t stream) {
     if (ws->nrec == 0) return WS_OK;
     if (ws->rec_tiling_tx == t.tx && ws->rec_tiling_ty == t.ty && ws->rec_direct == direct)
@@ -322,20 +345,11 @@ int build_rec_tiles(ws_t ws, const ws::StreamTiling &t, bool direct, cudaStream_
     forget_rec_tiles(ws);   // until the upload is issued
     rc = keep_or_grow(ws, &ws->rec_table, &ws->rec_table_cap, bytes, "cudaMalloc receiver table");
     if (rc != WS_OK) return rc;
-    if (!ws->rec_uploaded)
-        WS_CUDA(cudaEventCreateWithFlags(&ws->rec_uploaded, cudaEventDisableTiming),
-                "upload receiver table");
-    WS_CUDA(cudaEventSynchronize(ws->rec_uploaded), "upload receiver table");
-    ws->rec_host.resize(bytes);
-    std::memcpy(ws->rec_host.data(), ptr.data(), sizeof(int) * (ntiles + 1));
-    std::memcpy(ws->rec_host.data() + head, ent.data(), sizeof(ws::RecEntry) * ws->nrec);
-    WS_CUDA(cudaMemcpyAsync(ws->rec_table, ws->rec_host.data(), bytes, cudaMemcpyHostToDevice, stream),
-            "upload receiver table");
-    const cudaError_t e2 = cudaEventRecord(ws->rec_uploaded, stream);
-    if (e2 != cudaSuccess) {
-        cudaStreamSynchronize(stream);   // no event guards the host table
-        return cuda_fail(e2, "upload receiver table");
-    }
+    char *table = nullptr;
+    WS_CUDA(ws->rec_host.next(bytes, &table), "upload receiver table");
+    std::memcpy(table, ptr.data(), sizeof(int) * (ntiles + 1));
+    std::memcpy(table + head, ent.data(), sizeof(ws::RecEntry) * ws->nrec);
+    WS_CUDA(ws->rec_host.upload(ws->rec_table, stream), "upload receiver table");
     ws->rec_ptr = static_cast<int *>(ws->rec_table);
     ws->rec_entries = reinterpret_cast<ws::RecEntry *>(static_cast<char *>(ws->rec_table) + head);
     ws->rec_tiling_tx = t.tx;
@@ -669,10 +683,6 @@ void destroy(ws_t ws) {
     cudaFree(ws->scale);
     cudaFree(ws->stage);
     free_receivers(ws);
-    if (ws->rec_uploaded) {
-        cudaEventSynchronize(ws->rec_uploaded);   // the upload reads rec_host
-        cudaEventDestroy(ws->rec_uploaded);
-    }
     delete ws->adj;
     delete ws;
 }

@@ -47,6 +47,28 @@ struct SourceDef {
     double f0, t0, amp;
 };
 
+// Host memory of uploads that may run long after the call: two groups of buffers,
+// each written again only once the event behind its last upload has passed. An
+// event for each upload would cost 2 to 3 us on the way of a call of 27 (a state of
+// 96^3 put back, receivers set, one step, the state out); large tables have one.
+// All uploads are on streams that are ordered one behind the other.
+struct HostTables {
+    static constexpr int kGroup = 4;
+    static constexpr size_t kLarge = 64 << 10;
+    std::vector<char> table[2][kGroup];
+    cudaEvent_t passed[2] = {nullptr, nullptr};
+    int group = 0, at = 0;
+    // The next buffer, of n bytes, free to be written.
+    cudaError_t next(size_t n, char **p);
+    // That buffer to dst, on `stream`.
+    cudaError_t upload(void *dst, cudaStream_t stream);
+    // (the uploads are through)
+    ~HostTables() {
+        for (cudaEvent_t e : passed)
+            if (e) cudaEventDestroy(e);
+    }
+};
+
 // The CUDA driver API's cuTensorMapEncodeTiled (null when unavailable).
 PFN_cuTensorMapEncodeTiled_v12000 get_encode_fn();
 
@@ -77,8 +99,7 @@ struct ws_handle {
     size_t rec_table_cap = 0;
     int *rec_ptr = nullptr;              // per-tile ranges of rec_entries
     ws::RecEntry *rec_entries = nullptr;
-    std::vector<char> rec_host;          // the table's upload reads it until rec_uploaded
-    cudaEvent_t rec_uploaded = nullptr;
+    wsh::HostTables rec_host;            // what the table's uploads read
     float *stage = nullptr;              // planes of an unpadded field, for host arrays
     int rec_tiling_tx = 0, rec_tiling_ty = 0;
     bool rec_direct = false;             // the table is the direct kernel's

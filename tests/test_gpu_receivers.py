@@ -85,3 +85,37 @@ def test_dense_receivers_on_a_narrow_grid():
         assert np.array_equal(wsb.ws_read_traces(h)[:, t], u[rec[:, 2], rec[:, 1], rec[:, 0]])
     assert np.abs(u).max() > 0
     assert step_ms() < 8 * bare
+
+
+@pytest.mark.parametrize("sizes", [[60] * 21, [60, 6000, 60, 60, 6000, 6000, 60, 60, 60, 60, 60, 60, 6000, 60]])
+def test_many_tables_behind_a_busy_stream(sizes):
+    """More tables than the handle keeps host buffers for, small ones and some of
+    more than 64 KB, while steps are queued: each step samples its own cells."""
+    torch = pytest.importorskip("torch")
+    shape = nz, ny, nx = 128, 256, 256
+    rng = np.random.default_rng(1)
+    vel = synthetic.smooth_random_velocity(shape, 3, 1500.0, 4500.0, spacing=8)
+    recs = [np.stack([rng.integers(0, n, m) for n in (nx, ny, nz)], 1).astype(np.int32) for m in sizes]
+
+    def run(wait):
+        h = wsb.ws_create(nx, ny, nz, 10.0, synthetic.cfl_dt(4500.0, 10.0))
+        wsb.ws_set_velocity(h, vel)
+        for k in (20, 60, 100):
+            wsb.ws_add_source(h, nx // 2, ny // 2, k, 30.0, 0.0, 1.0)
+        wsb.ws_set_receivers(h, recs[1], 30)      # the largest buffers
+        wsb.ws_step(h, 30)
+        wsb.ws_synchronize(h)
+        out = []
+        for rec in recs:
+            wsb.ws_set_receivers(h, rec, 30)
+            wsb.ws_step(h, 30)
+            out.append(torch.empty((len(rec), 30), device="cuda"))
+            wsb.ws_read_traces(h, out[-1])
+            if wait:
+                wsb.ws_synchronize(h)
+        wsb.ws_synchronize(h)
+        return [t.cpu().numpy() for t in out]
+
+    for a, b in zip(run(False), run(True)):
+        assert np.abs(b).max() > 0
+        assert np.array_equal(a, b)
