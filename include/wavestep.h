@@ -126,7 +126,10 @@ int ws_clear_sources(ws_t ws);
  * counted from the step at which this call is made (the trace clock
  * restarts here; traces are zeroed). ijk is host memory, [nrec][3] =
  * (i, j, k) per receiver, copied. nrec = 0 removes all receivers. Stepping
- * past nt_max recorded steps fails with STATE. */
+ * past nt_max recorded steps fails with STATE. The device buffers of the traces
+ * and of the receivers' table are kept for the next call while they hold what it
+ * needs, up to four times that (or 16 MiB); nrec = 0 frees them. Fails under
+ * stream capture. Errors: BADARG, OOM, CUDA. */
 int ws_set_receivers(ws_t ws, int nrec, const int *ijk, int nt_max);
 
 /* Advance nsteps steps (asynchronous on the stream). Requires a velocity
@@ -138,7 +141,11 @@ int ws_step(ws_t ws, int nsteps);
 int ws_read_traces(ws_t ws, float *out, int on_device);
 
 /* Copy u^n (into u) and u^{n-1} (into u_prev) as [nz][ny][nx] float32.
- * Either pointer may be NULL. */
+ * Either pointer may be NULL. Host arrays, here, in ws_write_field and in the
+ * model setters, move through a device buffer of up to 64 MiB (whole planes; the
+ * size of a field if that is less), which the first such call allocates and the
+ * handle keeps: it is given back by ws_destroy, or when a later allocation of the
+ * handle finds no memory. Where it cannot be allocated, planes are copied singly. */
 int ws_read_field(ws_t ws, float *u, float *u_prev, int on_device);
 
 /* Replace u^n and u^{n-1} (NULL = zero) and set the step counter to step

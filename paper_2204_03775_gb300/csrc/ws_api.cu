@@ -277,15 +277,29 @@ void free_receivers(ws_t ws) {
     forget_rec_tiles(ws);
 }
 
-// A device buffer of at least n bytes: *p as it is if it holds them, else a new
-// one (the stream drains first: the old one may still be in use).
+// cudaMalloc for a handle: where the memory runs out, its staging for host arrays,
+// which can be made again, is given back first.
+cudaError_t handle_malloc(ws_t ws, void **p, size_t n) {
+    cudaError_t e = cudaMalloc(p, n);
+    if (e != cudaErrorMemoryAllocation || !ws->stage) return e;
+    cudaGetLastError();
+    if ((e = cudaStreamSynchronize(ws->stream)) != cudaSuccess) return e;
+    cudaFree(ws->stage);
+    ws->stage = nullptr;
+    return cudaMalloc(p, n);
+}
+
+// A device buffer of at least n bytes: *p as it is if it holds them and is not far
+// too large (kept: up to four times n, or 16 MiB), else a new one (the stream
+// drains first: the old one may still be in use).
 static int keep_or_grow(ws_t ws, void **p, size_t *cap, size_t n, const char *what) {
-    if (n <= *cap) return WS_OK;
+    constexpr size_t kKeep = 16u << 20;
+    if (n <= *cap && *cap <= std::max(4 * n, kKeep)) return WS_OK;
     WS_CUDA(cudaStreamSynchronize(ws->stream), what);
     cudaFree(*p);
     *p = nullptr;
     *cap = 0;
-    WS_CUDA(cudaMalloc(p, n), what);
+    WS_CUDA(handle_malloc(ws, p, n), what);
     *cap = n;
     return WS_OK;
 }
@@ -381,7 +395,8 @@ static bool kernel_copyable(const ws_t ws, const void *p) {
            on_this_device(c + bytes - 1);
 }
 
-// The handle's device staging for host arrays: planes of an unpadded field, at
+// The handle's device staging for host arrays, made by the first of them and kept
+// until ws_destroy or until the handle runs out of memory: planes of an unpadded field, at
 // most kStageMax bytes (null: not even one plane, or no memory). *planes of them
 // move by one contiguous copy and one kernel instead of a 2D copy per plane, at
 // 9 us or more each from pageable memory: both levels of 101 x 37 x 45 out 819
@@ -981,7 +996,9 @@ int ws_set_storage(ws_t ws, int storage) {
         const size_t hb = size_t(ws->g.pnx) * ws->g.pny * ws->g.pnz * sizeof(uint16_t);
         for (uint16_t **f : {&ws->buf16[0], &ws->buf16[1], &ws->d16, &ws->w16})
             if (!*f) {
-                WS_CUDA(cudaMalloc(f, hb), "cudaMalloc 16-bit field");
+                void *q = nullptr;
+                WS_CUDA(handle_malloc(ws, &q, hb), "cudaMalloc 16-bit field");
+                *f = static_cast<uint16_t *>(q);
                 WS_CUDA(cudaMemsetAsync(*f, 0, hb, ws->stream), "zero 16-bit field");
             }
         ws->w16_ok = false;

@@ -38,7 +38,7 @@ int adjoint_prepare(ws_t ws, const char *who, int *kern_out, ws::StreamTiling *t
         ws->adj = ac;
         auto grab = [&](auto **p, size_t bytes) -> cudaError_t {
             void *q = nullptr;
-            cudaError_t e = cudaMalloc(&q, bytes);
+            cudaError_t e = handle_malloc(ws, &q, bytes);
             if (e == cudaSuccess) {
                 ac->mem.push_back(q);
                 *p = static_cast<std::remove_reference_t<decltype(**p)> *>(q);

@@ -167,7 +167,7 @@ int ws_autotune(ws_t ws, int *tile_x, int *tile_y, int *zblock) {
         if (it != g_tune_cache.end()) best = it->second;
     }
     if (best.tx == 0) {
-        Scratch sc(ws->stream);
+        Scratch sc(ws);
         float *out = nullptr;
         WS_CUDA(sc.alloc(&out, field_bytes(g)), "cudaMalloc tuning field");
         cudaEvent_t e0, e1;

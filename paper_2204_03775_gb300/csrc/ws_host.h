@@ -190,6 +190,8 @@ int default_zblock(const ws::Geom &g, int tx, int ty);
 // Choose the kernel for the next steps; fills *tiling for the streaming one.
 int pick_kernel(ws_t ws, ws::StreamTiling *tiling);
 void free_receivers(ws_t ws);
+// cudaMalloc that gives back the handle's staging when memory runs out.
+cudaError_t handle_malloc(ws_t ws, void **p, size_t n);
 // Receiver table of the streaming kernels, or of the direct kernel, for tile t,
 // uploaded on `stream` (ordered after the work on the handle's own that may
 // still read the old table).
@@ -230,17 +232,17 @@ void destroy(ws_t ws);
 
 // Device scratch of one call: freed, after the stream drains, on every return.
 struct Scratch {
-    cudaStream_t stream;
+    ws_t ws;
     std::vector<void *> ptrs;
-    explicit Scratch(cudaStream_t s) : stream(s) {}
+    explicit Scratch(ws_t w) : ws(w) {}
     ~Scratch() {
-        cudaStreamSynchronize(stream);
+        cudaStreamSynchronize(ws->stream);
         for (void *p : ptrs) cudaFree(p);
     }
     template <class T>
     cudaError_t alloc(T **p, size_t bytes) {
         void *q = nullptr;
-        cudaError_t e = cudaMalloc(&q, bytes);
+        cudaError_t e = handle_malloc(ws, &q, bytes);
         if (e != cudaSuccess) return e;
         ptrs.push_back(q);
         *p = static_cast<T *>(q);
