@@ -396,11 +396,11 @@ static bool kernel_copyable(const ws_t ws, const void *p) {
 }
 
 // The handle's device staging for host arrays, made by the first of them and kept
-// until ws_destroy or until the handle runs out of memory: planes of an unpadded field, at
-// most kStageMax bytes (null: not even one plane, or no memory). *planes of them
-// move by one contiguous copy and one kernel instead of a 2D copy per plane, at
-// 9 us or more each from pageable memory: both levels of 101 x 37 x 45 out 819
-// us, now 38; of 256 x 256 x 200 in 8.3 ms, now 0.65 (pinned 1.38, now 0.56).
+// until ws_destroy or until the handle runs out of memory: planes of an unpadded
+// field, at most kStageMax bytes (null: not even one plane, or no memory). *planes
+// of them move by one contiguous copy and one kernel instead of a 2D copy per
+// plane, at 9 us or more each from pageable memory: both levels of 101 x 37 x 45
+// out 819 us, now 38; of 256 x 256 x 200 in 8.3 ms, now 0.65 (pinned 1.38, now 0.56).
 static float *host_stage(ws_t ws, int *planes) {
     constexpr size_t kStageMax = 64u << 20;
     const ws::Geom &g = ws->g;
@@ -468,8 +468,11 @@ int copy_out(ws_t ws, float *dst, const float *src, int on_device, float *dst2, 
         ws->launches++;
         return src2 && !both ? copy_out(ws, dst2, src2, on_device) : WS_OK;
     }
+    // one plane of long rows comes out in one 2D copy (512 x 512: 22 us, through the
+    // staging 31; 30 x 60000: 268, 62)
+    const bool direct = on_device || (g.nz == 1 && g.nx >= 256);
     int planes = 0;
-    if (float *stage = on_device ? nullptr : host_stage(ws, &planes)) {
+    if (float *stage = direct ? nullptr : host_stage(ws, &planes)) {
         const size_t plane = size_t(g.nx) * g.ny;
         for (int k = 0; k < g.nz; k += planes) {
             ws::Geom part = g;
