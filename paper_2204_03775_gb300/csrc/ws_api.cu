@@ -126,15 +126,11 @@ bool stream_fits(const ws_t ws, const ws::StreamTiling &t) {
     return ws::stream_tiling_supported(t.tx, t.ty) && ws->g.nx >= t.tx && ws->g.ny >= t.ty;
 }
 
-// Planes per work item: long blocks re-read fewer 4-plane halos at their
-// ends, short ones give the in-order dispatch more, smaller items; about 200
-// planes measured best on the 1024^3 survey (five blocks of 205: 389.6
-// Gcell/s against 387.2 at 342 and 376.7 at 64, 64 x 8 tiles). The blocks
-// are cut so that the last one is about a quarter as long as the others:
-// items run in block order, so the launch ends on short items and its tail,
-// when fewer CTAs than SM slots remain, is short (1024^3, four blocks of 241
-// and one of 60: FP32 393.5 against 390.9 Gcell/s for five of 205; 16-bit
-// storage 493 against 485 with equal blocks, 64 x 24 tiles).
+// Planes per work item whatever the GPU: blocks of about 200, the last one about a
+// quarter as long as the others, so that a launch, whose items run in block order,
+// ends on short ones. A candidate of the tuners (a batch of 32 shots of 96 to 320
+// cells a side, 64 x 16 tiles: 870 us a step, the rules for one to six waves of
+// items 876 to 893), and what the estimates below fall back on.
 int default_zblock(int nz) {
     const int blocks = std::max(1, (int)std::lround(nz / 200.0));
     if (blocks == 1) return nz;

@@ -264,8 +264,10 @@ void batch_free(ws_batch_t b) {
     delete b;
 }
 
-// Configure every shot for tile tx x ty with z-blocks for m x slots items
-// (m = 0: each shot's default) and rebuild the item table: longest items
+// Configure every shot for tile tx x ty with z-blocks for m x slots items (m = 0:
+// blocks of about 200 planes), at least 8 planes (two to four shots of 64 to 128
+// cells a side alone would run 8 to 12 % faster with fewer, 16 of them no faster),
+// and rebuild the item table: longest items
 // (most planes) first, so the last wave of the launch holds the shortest
 // ones; among equal lengths, shots in order of decreasing size and each
 // shot's items block-major (neighbouring tiles run together).

@@ -183,8 +183,8 @@ int encode_map(CUtensorMap *map, void *base, const ws::Geom &g, int bx, int by,
 // The handle's maps for its current tiling.
 int encode_maps(ws_t ws);
 bool stream_fits(const ws_t ws, const ws::StreamTiling &t);
-// Planes per work item: the default for nz planes, and the FP32 streaming
-// kernel's for a grid and tile.
+// Planes per work item: about 200, and the FP32 streaming kernel's default for a
+// grid and tile.
 int default_zblock(int nz);
 int default_zblock(const ws::Geom &g, int tx, int ty);
 // Choose the kernel for the next steps; fills *tiling for the streaming one.
