@@ -323,33 +323,34 @@ int build_rec_tiles(ws_t ws, const ws::StreamTiling &t, bool direct, cudaStream_
         return WS_OK;
     const int tiles_x = (ws->g.nx + t.tx - 1) / t.tx;
     const int tiles_y = (ws->g.ny + t.ty - 1) / t.ty;
-    const int warps = direct ? 1 : t.tx / 4 * (t.ty / 2) / 32;
-    const int ntiles = tiles_x * tiles_y * warps;   // (tile, warp) ranges
-    std::vector<std::pair<int, ws::RecEntry>> e(ws->nrec);
-    for (int r = 0; r < ws->nrec; ++r) {
+    const int threads = t.tx / 4 * (t.ty / 2), warps = direct ? 1 : threads / 32;
+    const int ranges = tiles_x * tiles_y * warps;   // (tile, warp)
+    const int nrec = ws->nrec;
+    std::vector<int> range(nrec), order(nrec), next(nrec), ptr;
+    std::vector<ws::RecEntry> e(nrec);
+    for (int r = 0; r < nrec; ++r) {
         const int i = ws->rec_ijk[3 * r], j = ws->rec_ijk[3 * r + 1], k = ws->rec_ijk[3 * r + 2];
         const int tile = (j / t.ty) * tiles_x + (i / t.tx);
         const int li = i - (i / t.tx) * t.tx, lj = j - (j / t.ty) * t.ty;
-        if (direct) {
-            e[r] = {tile, ws::RecEntry{k, lj, li, r}};
-            continue;
-        }
-        const int owner = (lj / 2) * (t.tx / 4) + li / 4;
-        e[r] = {tile * warps + owner / 32, ws::RecEntry{k, owner, (lj % 2) * 4 + li % 4, r}};
+        const int owner = direct ? lj : (lj / 2) * (t.tx / 4) + li / 4;
+        e[r] = ws::RecEntry{k, owner, direct ? li : (lj % 2) * 4 + li % 4, r};
+        range[r] = direct ? tile : tile * warps + owner / 32;
+        order[r] = r;
     }
-    std::stable_sort(e.begin(), e.end(), [](const auto &x, const auto &y) {
-        return x.first != y.first ? x.first < y.first : x.second.k < y.second.k;
-    });
-    std::vector<int> ptr(ntiles + 1, 0);
-    std::vector<ws::RecEntry> ent(ws->nrec);
-    for (int r = 0; r < ws->nrec; ++r) {
-        ptr[e[r].first + 1]++;
-        ent[r] = e[r].second;
-    }
-    for (int tt = 0; tt < ntiles; ++tt) ptr[tt + 1] += ptr[tt];
+    // a stable pass of a counting sort, into `buckets` ranges at ptr
+    auto pass = [&](int buckets, auto &&key) {
+        ptr.assign(buckets + 1, 0);
+        for (int r = 0; r < nrec; ++r) ptr[key(r) + 1]++;
+        for (int b = 0; b < buckets; ++b) ptr[b + 1] += ptr[b];
+        std::vector<int> at(ptr);
+        for (int r : order) next[at[key(r)]++] = r;
+        order.swap(next);
+    };
+    pass(ws->g.nz, [&](int r) { return e[r].k; });
+    pass(ranges, [&](int r) { return range[r]; });
     // one buffer and one upload: the ranges, then the entries
-    const size_t head = (sizeof(int) * (ntiles + 1) + 15) / 16 * 16;
-    const size_t bytes = head + sizeof(ws::RecEntry) * ws->nrec;
+    const size_t head = (sizeof(int) * ptr.size() + 15) / 16 * 16;
+    const size_t bytes = head + sizeof(ws::RecEntry) * nrec;
     int rc = refuse_capture(ws, "upload receiver table");
     if (rc != WS_OK) return rc;
     forget_rec_tiles(ws);   // until the upload is issued
@@ -357,8 +358,9 @@ int build_rec_tiles(ws_t ws, const ws::StreamTiling &t, bool direct, cudaStream_
     if (rc != WS_OK) return rc;
     char *table = nullptr;
     WS_CUDA(ws->rec_host.next(bytes, &table), "upload receiver table");
-    std::memcpy(table, ptr.data(), sizeof(int) * (ntiles + 1));
-    std::memcpy(table + head, ent.data(), sizeof(ws::RecEntry) * ws->nrec);
+    std::memcpy(table, ptr.data(), sizeof(int) * ptr.size());
+    ws::RecEntry *entries = reinterpret_cast<ws::RecEntry *>(table + head);
+    for (int q = 0; q < nrec; ++q) entries[q] = e[order[q]];
     WS_CUDA(ws->rec_host.upload(ws->rec_table, stream), "upload receiver table");
     ws->rec_ptr = static_cast<int *>(ws->rec_table);
     ws->rec_entries = reinterpret_cast<ws::RecEntry *>(static_cast<char *>(ws->rec_table) + head);
