@@ -103,6 +103,7 @@ struct ws_handle {
     float *stage = nullptr;              // planes of an unpadded field, for host arrays
     int rec_tiling_tx = 0, rec_tiling_ty = 0;
     bool rec_direct = false;             // the table is the direct kernel's
+    int rec_planes = 0;                  // and has this many ranges a tile (0: one)
 
     int kernel = WS_KERNEL_AUTO;
     ws::StreamTiling tiling{64, 16, 0};  // tile of the tensor maps; zb 0: default

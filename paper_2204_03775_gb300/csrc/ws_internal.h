@@ -127,11 +127,12 @@ struct StepArgs {
 // Launchers (stream-ordered, no synchronization).
 // out = u^{n+1} from u = u^n and up = u^{n-1}; out may be up (in place).
 // rec_ptr (null: none): per tile of kDirectX x kDirectY columns a range of rec
-// sorted by k, with lane = x and owner = y inside the tile.
+// sorted by k (rec_planes 0), or one for each of its rec_planes planes, with lane = x
+// and owner = y inside the tile.
 constexpr int kDirectX = 32, kDirectY = 8;
 cudaError_t launch_step_direct(const float *u, const float *up, float *out, const float *w,
-                               const StepArgs &a, const int *rec_ptr, const RecEntry *rec,
-                               cudaStream_t s);
+                               const StepArgs &a, const int *rec_ptr, int rec_planes,
+                               const RecEntry *rec, cudaStream_t s);
 // The model (device array [nz][ny][nx], or null: already in w's interior) into
 // the padded w: V -> (V dt / h)^2, m = 1/V^2 -> (dt / h)^2 / m, in double,
 // rounded once. extrema collects {max, min} of the values as float bits; a

@@ -87,34 +87,37 @@ __device__ __forceinline__ void record_block(float *out, const float *w, const S
     }
 }
 
-// A tile's range up to a block's threads is scanned, a longer one searched for
-// the block's plane first. With a receiver on each cell of a vertical plane: 48 x
-// 40 x 40 (320 entries a tile) searched 2.89 us a step, scanned 3.07; 11 x 11 x
-// 1200 (9600) 7.98, 14.4; 20 x 120 x 6000 (48000) 304, 1748 (every block reading
-// its tile's whole range: 3182).
+// Tables without ranges by plane: a tile's range up to a block's threads is scanned,
+// a longer one searched for the block's plane first. With a receiver on each cell
+// of a vertical plane (such a table, for comparison): 48 x 40 x 40 (320 entries a
+// tile) searched 2.89 us a step, scanned 3.07; 11 x 11 x 1200 (9600) 7.98, 14.4; 20
+// x 120 x 6000 (48000) 304, 1748 (every block reading its tile's whole range: 3182).
 constexpr int kScanEntries = 256;
 
 __global__ void __launch_bounds__(256) step_direct_kernel(const float *u,
                                                           const float *up, float *out,
                                                           const float *w,
                                                           const __grid_constant__ StepArgs a,
-                                                          const int *rec_ptr, const RecEntry *rec) {
+                                                          const int *rec_ptr, const int rec_planes,
+                                                          const RecEntry *rec) {
     // no kernel writes the receiver table: its ranges are read before the
     // predecessor is waited for
     const int tile = blockIdx.y * gridDim.x + blockIdx.x;
-    int lo = rec_ptr ? rec_ptr[tile] : 0, hi = rec_ptr ? rec_ptr[tile + 1] : 0;
-    if (hi - lo > kScanEntries) lo = block_first_entry(rec, lo, hi, blockIdx.z);
+    const int range = rec_planes ? tile * rec_planes + blockIdx.z : tile;
+    int lo = rec_ptr ? rec_ptr[range] : 0, hi = rec_ptr ? rec_ptr[range + 1] : 0;
+    if (!rec_planes && hi - lo > kScanEntries) lo = block_first_entry(rec, lo, hi, blockIdx.z);
     wait_predecessor();
     step_cell(u, up, out, w, a);
     record_block(out, w, a, blockIdx.z, lo, hi, rec);
 }
 
 cudaError_t launch_step_direct(const float *u, const float *up, float *out, const float *w,
-                               const StepArgs &a, const int *rec_ptr, const RecEntry *rec,
-                               cudaStream_t s) {
+                               const StepArgs &a, const int *rec_ptr, int rec_planes,
+                               const RecEntry *rec, cudaStream_t s) {
     dim3 block(kDirectX, kDirectY, 1);
     dim3 grid((a.g.nx + kDirectX - 1) / kDirectX, (a.g.ny + kDirectY - 1) / kDirectY, a.g.nz);
-    return launch_overlapped(step_direct_kernel, grid, block, 0, s, u, up, out, w, a, rec_ptr, rec);
+    return launch_overlapped(step_direct_kernel, grid, block, 0, s, u, up, out, w, a, rec_ptr, rec_planes,
+                             rec);
 }
 
 }  // namespace ws
