@@ -214,20 +214,16 @@ static __device__ __forceinline__ int first_entry(const RecEntry *rec, int lo, i
 
 // Receivers of a two-row thread: RecEntry.lane = 4 * row + x cell. Lane q of
 // the warp takes entry cur + q, fetches the owner's 8 values by shuffle and
-// stores the one it names. The next 32 entries are fetched meanwhile.
+// stores the one it names.
 static __device__ __forceinline__ void record_plane2(const float4 (&out)[2], int k, int *rcur, int rend,
                                               int *rnext_k, const RecEntry *rec, float *traces,
                                               int nt_max, long long trace_step) {
     const int lane = threadIdx.x & 31;
     int cur = *rcur;
-    auto entry = [&](int at) {
-        RecEntry e{INT_MAX, 0, 0, 0};
-        if (at + lane < rend) e = rec[at + lane];
-        return e;
-    };
-    RecEntry e = entry(cur);
     for (;;) {
-        const RecEntry e1 = entry(cur + 32);
+        const int idx = cur + lane;
+        RecEntry e{INT_MAX, 0, 0, 0};
+        if (idx < rend) e = rec[idx];
         const bool take = e.k == k;
         const int src = e.owner & 31;
         float v[8];
@@ -248,7 +244,6 @@ static __device__ __forceinline__ void record_plane2(const float4 (&out)[2], int
         const int n = __popc(__ballot_sync(0xffffffffu, take));
         cur += n;
         if (n < 32) break;
-        e = e1;
     }
     *rcur = cur;
     *rnext_k = cur < rend ? rec[cur].k : INT_MAX;
