@@ -506,6 +506,21 @@ int copy_out(ws_t ws, float *dst, const float *src, int on_device, float *dst2, 
     return src2 ? copy_out(ws, dst2, src2, on_device) : WS_OK;
 }
 
+// Whole fields (padding included) to zero: a, and b if not null, by one kernel, or
+// large ones, which a memset writes faster, by memsets (two of 460 MB: 134 us, the
+// kernel 144; of 100 MB: 41.4, 40.3).
+int zero_fields(ws_t ws, float *a, float *b, size_t bytes, const char *what) {
+    constexpr size_t kMemset = 128u << 20;
+    if (bytes <= kMemset) {
+        WS_CUDA(ws::launch_zero(a, b, bytes, ws->stream), what);
+        ws->launches++;
+        return WS_OK;
+    }
+    WS_CUDA(cudaMemsetAsync(a, 0, bytes, ws->stream), what);
+    if (b) WS_CUDA(cudaMemsetAsync(b, 0, bytes, ws->stream), what);
+    return WS_OK;
+}
+
 int upload_profiles(ws_t ws) {
     const ws::Geom &g = ws->g;
     std::vector<float> px(g.nx), py(g.ny), pz(g.nz);
@@ -1188,8 +1203,8 @@ int ws_write_field(ws_t ws, const float *u, const float *u_prev, long long step,
     float *un = ws->buf[ws->cur], *um = ws->buf[1 - ws->cur];
     if (!u || !u_prev) {
         float *first = u ? um : un, *second = u || u_prev ? nullptr : um;
-        WS_CUDA(ws::launch_zero(first, second, fb, ws->stream), "ws_write_field");
-        ws->launches++;
+        const int zc = zero_fields(ws, first, second, fb, "ws_write_field");
+        if (zc != WS_OK) return zc;
     }
     int rc = WS_OK;
     if (u)

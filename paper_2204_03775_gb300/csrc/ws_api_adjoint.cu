@@ -122,8 +122,8 @@ int forward_begin(ws_t ws, AdjointCache *ac) {
     const size_t ntr = size_t(ws->nrec) * ws->nt_max;
     const cudaStream_t st = ws->stream;
     ac->fwd_valid = false;
-    WS_CUDA(ws::launch_zero(ws->buf[0], ws->buf[1], fb, st), "zero fields");
-    ws->launches++;
+    int rc = zero_fields(ws, ws->buf[0], ws->buf[1], fb, "zero fields");
+    if (rc != WS_OK) return rc;
     WS_CUDA(cudaMemsetAsync(ws->traces, 0, sizeof(float) * ntr, st), "zero traces");
     ws->step = 0;
     ws->trace_start = 0;
@@ -184,19 +184,18 @@ int gradient_run(GradShot *sh, int n, int mode) {
     const int np = ws::residual_partial_count();
     for (int q = 0; q < n; ++q) {
         GradShot &x = sh[q];
-        const cudaStream_t st = x.ws->stream;
         // rho^{N+1} = rho^{N+2} = 0
-        WS_CUDA(ws::launch_zero(x.ac->rho(N + 1).p, x.ac->rho(N + 2).p, fb, st),
-                "zero adjoint field");
-        WS_CUDA(ws::launch_zero(reinterpret_cast<float *>(x.ac->acc), nullptr, 2 * fb, st),
-                "zero gradient accumulator");
-        x.ws->launches += 2;
+        int rc = zero_fields(x.ws, x.ac->rho(N + 1).p, x.ac->rho(N + 2).p, fb, "zero adjoint field");
+        if (rc == WS_OK)
+            rc = zero_fields(x.ws, reinterpret_cast<float *>(x.ac->acc), nullptr, 2 * fb,
+                             "zero gradient accumulator");
+        if (rc != WS_OK) return rc;
         // a residual given for the run that ws_forward left in the cache (same
         // model version) needs no new forward run
         x.forward = !(mode == WS_ADJ_RESIDUAL && x.ac->fwd_valid &&
                       x.ac->fwd_version == x.ws->model_version);
         if (x.forward) {
-            int rc = forward_begin(x.ws, x.ac);
+            rc = forward_begin(x.ws, x.ac);
             if (rc != WS_OK) return rc;
         }
         x.a = base_args(x.ws);
@@ -231,9 +230,9 @@ int gradient_run(GradShot *sh, int n, int mode) {
         if (j == 0)
             for (int q = 0; q < n; ++q) {   // from rest
                 AdjointCache *ac = sh[q].ac;
-                WS_CUDA(ws::launch_zero(ac->ring(n1, 0).p, ac->ring(n1, 1).p, fb, sh[q].ws->stream),
-                        "zero initial state");
-                sh[q].ws->launches++;
+                int rc = zero_fields(sh[q].ws, ac->ring(n1, 0).p, ac->ring(n1, 1).p, fb,
+                                     "zero initial state");
+                if (rc != WS_OK) return rc;
             }
         for (int m = n0; m < n1; ++m)
             for (int q = 0; q < n; ++q) {

@@ -203,6 +203,8 @@ int copy_in(ws_t ws, float *dst, const float *src, int on_device, float *dst2 = 
             const float *src2 = nullptr);
 int copy_out(ws_t ws, float *dst, const float *src, int on_device, float *dst2 = nullptr,
              const float *src2 = nullptr);
+// Whole fields to zero (b null: one).
+int zero_fields(ws_t ws, float *a, float *b, size_t bytes, const char *what);
 int upload_profiles(ws_t ws);
 // The tiles of the 16-bit streaming kernel (64 x ty) that a step chooses from:
 // 24 rows (two CTAs of 6 warps per SM) or 16 (three of 4 warps); 48 is

@@ -196,8 +196,7 @@ __global__ void __launch_bounds__(kRowThreads)
 
 // Whole buffers (padding included) to zero: n floats of a, and of b if given.
 // One launch for a pair of fields: a memset's call takes the host 11 us, which
-// a run of a few hundred microseconds does not hide. Memsets write large fields
-// faster (460 MB, two of them: 134 us, this kernel 144; 100 MB: 41.4, 40.3).
+// a run of a few hundred microseconds does not hide.
 __global__ void __launch_bounds__(kRowThreads) zero_kernel(float4 *a, float4 *b, long long n4) {
     const float4 z = make_float4(0.f, 0.f, 0.f, 0.f);
     for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < n4;
@@ -230,11 +229,6 @@ cudaError_t launch_copy(const Fields &f, const Geom &g, cudaStream_t s) {
 }  // namespace
 
 cudaError_t launch_zero(float *a, float *b, size_t bytes, cudaStream_t s) {
-    constexpr size_t kMemset = 128u << 20;
-    if (bytes > kMemset) {
-        const cudaError_t e = cudaMemsetAsync(a, 0, bytes, s);
-        return e == cudaSuccess && b ? cudaMemsetAsync(b, 0, bytes, s) : e;
-    }
     const long long n4 = (long long)(bytes / sizeof(float4));   // fields are whole 128-byte rows
     const long long want = (n4 + kRowThreads - 1) / kRowThreads;
     return launch(zero_kernel, (unsigned)(want < kCopyBlocks ? want : kCopyBlocks), kRowThreads, 0, s,
